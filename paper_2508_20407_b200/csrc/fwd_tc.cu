@@ -40,6 +40,10 @@ static_assert(256 * kSoftmaxRegs + 128 * kOtherRegs <= kThreads * 168, "register
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kPolyPairs = 5;                // of every 16 column pairs, this many get 2^x from the polynomial
+// Keys of a step whose P is handed to the tensor pipe before the rest: their PV products run while the last columns are worked
+// on.  After 64 of 128 keys the pipe ran dry before the rest came; after 96 it does not (64 -> 96: 1.86 -> 1.81 ms at
+// B1 H32 N131072 W1024 d128, 262 -> 257 us at N32768 W512, 437 -> 429 us at B4 H32 N=W=4096 d64).
+constexpr int kFirstKeys = 96;
 constexpr float kRescaleThreshold = 32.0f;  // base-2 units: P stays below 2^32, far inside bf16/fp32 range
 
 // 2^x for a packed pair without the special-function unit: x = n + f with n = floor(x) (taken by adding
@@ -155,7 +159,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
     uint64_t* s_full = bars + 2;      // [2]
     uint64_t* p_full = bars + 4;      // [2]
     uint64_t* pv_done = bars + 6;     // [2]
-    uint64_t* p_half = bars + 8;      // [2]  first 64 keys of P written (PV may start on them)
+    uint64_t* p_first = bars + 8;     // [2]  first kFirstKeys keys of P written (PV may start on them)
     uint64_t* kv_full = bars + 10;    // [kSlots]
     uint64_t* kv_empty = bars + 10 + C::kSlots;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars);
@@ -170,7 +174,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
         for (int i = 0; i < 2; ++i) {
             mbar_init(&s_full[i], 1);
             mbar_init(&p_full[i], kQTile);
-            mbar_init(&p_half[i], kQTile);
+            mbar_init(&p_first[i], kQTile);
             mbar_init(&pv_done[i], 1);
         }
         for (int s = 0; s < C::kSlots; ++s) {
@@ -285,15 +289,16 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                 }
                 commit_lead(lead, &s_full[i]);
             };
-            auto issue_pv_half = [&](int i, uint32_t v_slot, bool accumulate, int half) {
+            // PV of the keys [16 from, 16 to) of a tile
+            auto issue_pv = [&](int i, uint32_t v_slot, bool accumulate, auto from, auto to) {
                 const uint32_t b_lo = v_lo0 + v_slot * (C::kTileBytes >> 4), d = tO0 + i * D, a = tS0 + i * kTileN;
 #pragma unroll
-                for (int k4 = 0; k4 < kTileN / 32; ++k4) {
-                    const int kk = half * (kTileN / 32) + k4;
+                for (int kk = decltype(from)::value; kk < decltype(to)::value; ++kk)
                     mma_ts_lead(lead, d, a + kk * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_pv, (accumulate || kk > 0) ? 1u : 0u);
-                }
-                if (half == 1) commit_lead(lead, &pv_done[i]);
             };
+            constexpr std::integral_constant<int, 0> k_begin{};
+            constexpr std::integral_constant<int, kFirstKeys / 16> k_first{};
+            constexpr std::integral_constant<int, kTileN / 16> k_end{};
             auto walk = make_walker<kBatched>(maps, p, starts);
             Segment s;
             while (ok && walk.next(s)) {
@@ -342,14 +347,15 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                     tc_fence_after();
                     for (int i = 0; i < 2 && ok; ++i) {
                         if (j < cq[i]) {
-                            ok = __all_sync(0xffffffffu, mbar_wait(&p_half[i], n_pv[i] & 1, abort_p));
+                            ok = __all_sync(0xffffffffu, mbar_wait(&p_first[i], n_pv[i] & 1, abort_p));
                             if (!ok) break;
                             tc_fence_after();
-                            issue_pv_half(i, v_slot, j > 0, 0);
+                            issue_pv(i, v_slot, j > 0, k_begin, k_first);
                             ok = __all_sync(0xffffffffu, mbar_wait(&p_full[i], n_pv[i] & 1, abort_p));
                             if (!ok) break;
                             tc_fence_after();
-                            issue_pv_half(i, v_slot, j > 0, 1);
+                            issue_pv(i, v_slot, j > 0, k_first, k_end);
+                            commit_lead(lead, &pv_done[i]);
                             ++n_pv[i];
                         }
                         if (i == 1) commit_lead(lead, &kv_empty[v_slot]);
@@ -470,10 +476,10 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                         pk[e] = pack_bf16x2(p0, p1);
                     }
                     tmem_st16(tS + c * 16, pk);
-                    if (c == kTileN / 64 - 1) {        // first 64 keys are in place: let the PV MMAs start on them
+                    if (c == kFirstKeys / 32 - 1) {    // the first keys are in place: let the PV MMAs start on them
                         tc_wait_st();
                         tc_fence_before();
-                        mbar_arrive(&p_half[i]);
+                        mbar_arrive(&p_first[i]);
                     }
                 }
                 tc_wait_st();
