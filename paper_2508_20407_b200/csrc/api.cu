@@ -265,7 +265,7 @@ static int backward_common(const void* q, const void* k, const void* v, const vo
     const bool tc = !is_f32 && (d == 64 || d == 128) && forward_impl() != 1;
     if (!tc) {
         if (!w.ptr || w.bytes < bwd_workspace_bytes(B, H, W, d)) return TLIN_ERR_WORKSPACE;
-        return launch_bwd_simt(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal_window, is_f32, (float*)w.ptr, sms, st);
+        return launch_bwd_simt(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal_window, is_f32, (float*)w.ptr, st);
     }
     if (tlin_backward_arrangement(B, H, N, W, d) == 2) {
         if (!w.ptr || w.bytes < bwd_fused_workspace_bytes(B, H, W, d)) return TLIN_ERR_WORKSPACE;

@@ -8,37 +8,34 @@
 //   dv_j  = sum_i p_ij dout_i          dp_ij = dout_i . v_j          ds_ij = p_ij (dp_ij - delta_i) / sqrt(d)
 //   dq_i  = sum_j ds_ij k_j            dk_j  = sum_i ds_ij q_i
 //
-// Three kernels.  delta: one warp per query row.  dk/dv: one CTA per block of 32 keys of a (b,h), looping over the
-// query tiles that can see it; every dk/dv element has one owner, so nothing is atomic.  dq: one CTA per tile of 32
-// query rows and per slice of the key range; the slices add their partial dq into an fp32 buffer in the workspace
-// (cleared first), which a last kernel rounds to the output type.
+// delta: one warp per query row.  Main kernel: one CTA per tile of keys of a (b,h), looping over the query tiles that can see
+// it; the scores are computed once per (query, key) tile and give all three gradients: dk/dv stay in registers until the end
+// (one owner each, nothing is atomic), the tile's dq is added to an fp32 dq by vector reductions in L2 (cleared first; the fp32
+// result itself, or a buffer in the workspace that a last kernel rounds to bf16).
 //
-// This is the fp32 path and the path for head sizes other than 64 and 128 (the counterpart of fwd_simt.cu); it is
-// not a roofline target.
+// Bound by the FFMA rate: five products of 2 d FLOP per pair.  64 x 64 tiles (32 x 32 beyond d = 128, where four 64-row tiles do
+// not fit the shared memory), 128 threads up to d = 64 and 256 beyond; a thread holds 4 x 8 (4 x 4) scores and 4 rows of CM
+// columns of each result, 5 to 16 FFMA per shared-memory read.  The kernels before it (two passes over the scores, one score
+// per thread and step, five reads per eight FFMA) against this one, fp32: B8 H12 N1024 W512 d36 2181 -> 448 us (30 TFLOP/s),
+// B4 H12 N1500 W700 d128 6088 -> 1496 us (33 TFLOP/s).
+//
+// This is the fp32 path and the path for bf16 head sizes other than 64 and 128 (the counterpart of fwd_simt.cu).
 #include "tlin_internal.h"
+#include "simt_tiles.cuh"
 #include <math_constants.h>
 
 namespace tlin {
 namespace {
 
-constexpr int kTB = 32;                 // query rows per tile and keys per block
-constexpr int kBwdThreads = 256;
+using namespace simt;
+
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kTR = 16;                 // row groups of a CTA
 
 __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ void from_f(__nv_bfloat16& dst, float x) { dst = __float2bfloat16_rn(x); }
 __device__ __forceinline__ void from_f(float& dst, float x) { dst = x; }
-
-// rows [r0, r0+32) of a [rows_total, d] matrix into padded fp32 shared memory (row stride d+1); rows beyond
-// rows_total become 0
-template <typename T>
-__device__ __forceinline__ void load_tile(float* dst, const T* src, long long r0, long long rows_total, int d) {
-    for (int x = threadIdx.x; x < kTB * d; x += kBwdThreads) {
-        const int r = x / d, c = x - r * d;
-        dst[r * (d + 1) + c] = r0 + r < rows_total ? to_f(src[(r0 + r) * d + c]) : 0.f;
-    }
-}
 
 // delta_i = dout_i . out_i, one warp per row
 template <typename T>
@@ -54,163 +51,153 @@ bwd_delta_kernel(const T* __restrict__ out, const T* __restrict__ dout, float* _
     if (lane == 0) delta[row] = acc;
 }
 
-// shared memory of the two tile kernels: four [32][d+1] tiles, P and dS as [32][33], lse and delta of the rows
-struct BwdSmem {
-    float *Qs, *dOs, *Ks, *Vs, *Ps, *dSs, *lse_s, *delta_s;
-    __device__ BwdSmem(float* base, int d) {
-        const int tile = kTB * (d + 1);
-        Qs = base;
-        dOs = Qs + tile;
-        Ks = dOs + tile;
-        Vs = Ks + tile;
-        Ps = Vs + tile;
-        dSs = Ps + kTB * (kTB + 1);
-        lse_s = dSs + kTB * (kTB + 1);
-        delta_s = lse_s + kTB;
-    }
-};
-size_t bwd_smem_bytes(int d) { return sizeof(float) * (4 * kTB * (d + 1) + 2 * kTB * (kTB + 1) + 2 * kTB); }
+// shared memory: Q, dout, K, V tiles, P and dS as [row][key], lse and delta of the rows
+template <int BT>
+__host__ __device__ constexpr int ld_p() { return BT + 8; }      // 8 modulo 32: four rows x eight keys written by a warp hit 32 banks
+template <int BT>
+size_t bwd_smem_bytes(int d, int slack) { return sizeof(float) * (4 * BT * row_stride(d) + 2 * BT * ld_p<BT>() + 2 * BT + slack); }
 
-// Scores, probabilities and ds of one 32 x 32 (query, key) tile, written to Ps / dSs (both [row][key]).
-// Thread t handles key j = t % 32 and rows i = t / 32 + 8 m: the row operands are warp-uniform (broadcast), the key
-// operands hit 32 different banks thanks to the padding.
-__device__ __forceinline__ void tile_p_ds(const BwdSmem& sm, int d, long long i0, long long j0, long long N, long long W,
-                                          int causal, float scale) {
-    const int j = threadIdx.x & 31, ib = threadIdx.x >> 5, ld = d + 1;
-    float s[4] = {0.f, 0.f, 0.f, 0.f}, dp[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int c = 0; c < d; ++c) {
-        const float kc = sm.Ks[j * ld + c], vc = sm.Vs[j * ld + c];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            s[m] = fmaf(sm.Qs[(ib + 8 * m) * ld + c], kc, s[m]);
-            dp[m] = fmaf(sm.dOs[(ib + 8 * m) * ld + c], vc, dp[m]);
+// acc[i][c] += sum over the BT rows r of A[r][a + i] * B[r][columns]   (A row stride ld_p, B row stride ld)
+template <int BT, int TC, int KA, int CM>
+__device__ __forceinline__ void accumulate_over_rows(float (&acc)[KA][CM], const float* A, const float* B, int ld, int tc) {
+#pragma unroll 2
+    for (int r = 0; r < BT; ++r) {
+        float a[KA], b[CM];
+        if constexpr (KA == 4) {
+            const float4 x = *reinterpret_cast<const float4*>(A + r * ld_p<BT>());
+            a[0] = x.x; a[1] = x.y; a[2] = x.z; a[3] = x.w;
+        } else {
+            const float2 x = *reinterpret_cast<const float2*>(A + r * ld_p<BT>());
+            a[0] = x.x; a[1] = x.y;
         }
-    }
+        load_columns<TC, CM>(b, B + r * ld, tc);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int il = ib + 8 * m;
-        const long long i = i0 + il, jj = j0 + j;
-        const bool ok = i < W && jj < N && (!causal || jj <= (N - W) + i);
-        const float p = ok ? exp2f((s[m] * scale - sm.lse_s[il]) * kLog2e) : 0.f;
-        sm.Ps[il * (kTB + 1) + j] = p;
-        sm.dSs[il * (kTB + 1) + j] = p * (dp[m] - sm.delta_s[il]) * scale;
+        for (int i = 0; i < KA; ++i)
+#pragma unroll
+            for (int c = 0; c < CM; ++c) acc[i][c] = fmaf(a[i], b[c], acc[i][c]);
     }
 }
 
-// MAXM: columns per thread (thread t owns columns t % 8 + 8 m, m < MAXM, below d)
-template <typename T, int MAXM>
-__global__ void __launch_bounds__(kBwdThreads)
-bwd_dkdv_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const T* __restrict__ dout,
-                const float* __restrict__ lse, const float* __restrict__ delta, T* __restrict__ dk, T* __restrict__ dv,
-                long long N, long long W, int d, int causal, float scale) {
-    extern __shared__ __align__(16) float smem_f[];
-    const BwdSmem sm(smem_f, d);
-    const int ld = d + 1;
-    const long long bh = blockIdx.y, j0 = (long long)blockIdx.x * kTB;
-    const T* qb = q + bh * W * d;
-    const T* dob = dout + bh * W * d;
-    load_tile(sm.Ks, k + bh * N * d, j0, N, d);
-    load_tile(sm.Vs, v + bh * N * d, j0, N, d);
-    const int jo = threadIdx.x >> 3, co = threadIdx.x & 7;      // owned key and first owned column
-    float acc_dk[MAXM], acc_dv[MAXM];
+template <typename T, int BT, int TC, int CM>
+__global__ void __launch_bounds__(kTR * TC, CM * TC <= 40 ? 3 : CM * TC <= 64 ? 2 : 1)
+bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const T* __restrict__ dout,
+                const float* __restrict__ lse, const float* __restrict__ delta, float* __restrict__ dq_acc, T* __restrict__ dk,
+                T* __restrict__ dv, int N, int W, int d, int causal, int64_t n_bh, float scale) {
+    constexpr int NT = kTR * TC;
+    constexpr int RI = BT / kTR, KJ = BT / TC, KA = BT / kTR;    // rows and keys of a thread's scores; keys of its dk / dv rows
+    constexpr int LDP = ld_p<BT>();
+    extern __shared__ __align__(16) float smem[];
+    const int ld = row_stride(d);
+    float* Qs = smem;
+    float* dOs = Qs + BT * ld;
+    float* Ks = dOs + BT * ld;
+    float* Vs = Ks + BT * ld;
+    float* Ps = Vs + BT * ld + column_slack<TC, CM>();
+    float* dSs = Ps + BT * LDP;
+    float* lse_s = dSs + BT * LDP;
+    float* delta_s = lse_s + BT;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tc = TC == 8 ? (lane & 7) : (warp & 1) * 8 + (lane & 7);
+    const int tr = (TC == 8 ? warp : warp >> 1) * 4 + (lane >> 3);
+    const int64_t bh = blockIdx.x % n_bh;                        // the key tiles with the most queries go first
+    const int j0 = (int)(blockIdx.x / n_bh) * BT;
+    load_rows<BT, NT>(Ks, ld, k + bh * N * (int64_t)d, j0, N, d);
+    load_rows<BT, NT>(Vs, ld, v + bh * N * (int64_t)d, j0, N, d);
+
+    float acc_dk[KA][CM], acc_dv[KA][CM];
 #pragma unroll
-    for (int m = 0; m < MAXM; ++m) acc_dk[m] = acc_dv[m] = 0.f;
-    // the first query row that may use a key of this block (window rule j <= N-W+i)
-    long long i_first = 0;
-    if (causal) {
-        i_first = j0 - (N - W);
-        if (i_first < 0) i_first = 0;
-    }
-    for (long long i0 = (i_first / kTB) * kTB; i0 < W; i0 += kTB) {
+    for (int i = 0; i < KA; ++i)
+#pragma unroll
+        for (int c = 0; c < CM; ++c) acc_dk[i][c] = acc_dv[i][c] = 0.f;
+    // the first query row that may use a key of this tile (window rule j <= N-W+i)
+    const int i_first = causal ? max(0, j0 - (N - W)) : 0;
+    for (int i0 = i_first / BT * BT; i0 < W; i0 += BT) {
         __syncthreads();
-        load_tile(sm.Qs, qb, i0, W, d);
-        load_tile(sm.dOs, dob, i0, W, d);
-        if (threadIdx.x < kTB) {
-            const long long i = i0 + threadIdx.x;
-            sm.lse_s[threadIdx.x] = i < W ? lse[bh * W + i] : 0.f;
-            sm.delta_s[threadIdx.x] = i < W ? delta[bh * W + i] : 0.f;
+        load_rows<BT, NT>(Qs, ld, q + bh * W * (int64_t)d, i0, W, d);
+        load_rows<BT, NT>(dOs, ld, dout + bh * W * (int64_t)d, i0, W, d);
+        if (threadIdx.x < BT) {
+            const int i = i0 + threadIdx.x;
+            lse_s[threadIdx.x] = i < W ? lse[bh * W + i] : 0.f;
+            delta_s[threadIdx.x] = i < W ? delta[bh * W + i] : 0.f;
+        }
+        cp_async_wait();
+        __syncthreads();
+        // scores -> P and dS, rows tr + 16 i, keys tc + TC j
+        {
+            float s[RI][KJ], dp[RI][KJ];
+#pragma unroll
+            for (int i = 0; i < RI; ++i)
+#pragma unroll
+                for (int j = 0; j < KJ; ++j) s[i][j] = dp[i][j] = 0.f;
+            dot_tile<RI, KJ>(s, Qs + tr * ld, kTR * ld, Ks + tc * ld, TC * ld, d);
+            dot_tile<RI, KJ>(dp, dOs + tr * ld, kTR * ld, Vs + tc * ld, TC * ld, d);
+            const bool edge = i0 + BT > W || j0 + BT > N || (causal && j0 + BT - 1 > N - W + i0);
+#pragma unroll
+            for (int i = 0; i < RI; ++i) {
+                const int row = tr + kTR * i;
+                const float lse_i = lse_s[row], delta_i = delta_s[row];
+                // key tc + TC j of the tile is allowed iff TC j < limit
+                const int limit = i0 + row >= W ? 0 : (causal ? min(N, N - W + i0 + row + 1) : N) - j0 - tc;
+#pragma unroll
+                for (int j = 0; j < KJ; ++j) {
+                    float p = exp2f((s[i][j] * scale - lse_i) * kLog2e);
+                    if (edge && TC * j >= limit) p = 0.f;
+                    Ps[row * LDP + tc + TC * j] = p;
+                    dSs[row * LDP + tc + TC * j] = p * (dp[i][j] - delta_i) * scale;
+                }
+            }
         }
         __syncthreads();
-        tile_p_ds(sm, d, i0, j0, N, W, causal, scale);
-        __syncthreads();
-#pragma unroll 4
-        for (int i = 0; i < kTB; ++i) {
-            const float p = sm.Ps[i * (kTB + 1) + jo], ds = sm.dSs[i * (kTB + 1) + jo];
+        accumulate_over_rows<BT, TC, KA, CM>(acc_dv, Ps + tr * KA, dOs, ld, tc);
+        accumulate_over_rows<BT, TC, KA, CM>(acc_dk, dSs + tr * KA, Qs, ld, tc);
+        // dq of the tile's rows from these keys
+        {
+            float acc[RI][CM];
 #pragma unroll
-            for (int m = 0; m < MAXM; ++m) {
-                const int c = co + 8 * m;
-                if (c < d) {
-                    acc_dv[m] = fmaf(p, sm.dOs[i * ld + c], acc_dv[m]);
-                    acc_dk[m] = fmaf(ds, sm.Qs[i * ld + c], acc_dk[m]);
+            for (int i = 0; i < RI; ++i)
+#pragma unroll
+                for (int c = 0; c < CM; ++c) acc[i][c] = 0.f;
+#pragma unroll 1
+            for (int key = 0; key < BT; key += 4) {
+                float4 a[RI];
+#pragma unroll
+                for (int i = 0; i < RI; ++i) a[i] = *reinterpret_cast<const float4*>(dSs + (tr + kTR * i) * LDP + key);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    float b[CM];
+                    load_columns<TC, CM>(b, Ks + (key + e) * ld, tc);
+#pragma unroll
+                    for (int i = 0; i < RI; ++i)
+#pragma unroll
+                        for (int c = 0; c < CM; ++c) acc[i][c] = fmaf(get(a[i], e), b[c], acc[i][c]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < RI; ++i) {
+                const int row = i0 + tr + kTR * i;
+                if (row >= W) continue;
+                float* dst = dq_acc + (bh * W + row) * d;
+#pragma unroll
+                for (int g = 0; g < CM / 4; ++g) {
+                    const int c = g * 4 * TC + 4 * tc;
+                    if (c < d) atomicAdd(reinterpret_cast<float4*>(dst + c), make_float4(acc[i][g * 4], acc[i][g * 4 + 1], acc[i][g * 4 + 2], acc[i][g * 4 + 3]));
+                }
+#pragma unroll
+                for (int m = CM / 4 * 4; m < CM; ++m) {
+                    const int c = column_of<TC, CM>(m, tc);
+                    if (c < d) atomicAdd(dst + c, acc[i][m]);
                 }
             }
         }
     }
-    if (j0 + jo < N) {
+    cp_async_wait();                            // K and V of a tile that no query may use
 #pragma unroll
-        for (int m = 0; m < MAXM; ++m) {
-            const int c = co + 8 * m;
-            if (c < d) {
-                from_f(dk[(bh * N + j0 + jo) * d + c], acc_dk[m]);
-                from_f(dv[(bh * N + j0 + jo) * d + c], acc_dv[m]);
-            }
-        }
-    }
-}
-
-template <typename T, int MAXM>
-__global__ void __launch_bounds__(kBwdThreads)
-bwd_dq_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const T* __restrict__ dout,
-              const float* __restrict__ lse, const float* __restrict__ delta, float* __restrict__ dq_acc,
-              long long N, long long W, int d, int causal, float scale, int blocks_per_split) {
-    extern __shared__ __align__(16) float smem_f[];
-    const BwdSmem sm(smem_f, d);
-    const int ld = d + 1;
-    const long long bh = blockIdx.y, i0 = (long long)blockIdx.x * kTB;
-    load_tile(sm.Qs, q + bh * W * d, i0, W, d);
-    load_tile(sm.dOs, dout + bh * W * d, i0, W, d);
-    if (threadIdx.x < kTB) {
-        const long long i = i0 + threadIdx.x;
-        sm.lse_s[threadIdx.x] = i < W ? lse[bh * W + i] : 0.f;
-        sm.delta_s[threadIdx.x] = i < W ? delta[bh * W + i] : 0.f;
-    }
-    const int io = threadIdx.x >> 3, co = threadIdx.x & 7;      // owned row and first owned column
-    float acc[MAXM];
-#pragma unroll
-    for (int m = 0; m < MAXM; ++m) acc[m] = 0.f;
-    const long long key_blocks = (N + kTB - 1) / kTB;
-    long long b0 = (long long)blockIdx.z * blocks_per_split, b1 = b0 + blocks_per_split;
-    if (b1 > key_blocks) b1 = key_blocks;
-    if (causal) {                                  // keys beyond the last row's limit are never used by this tile
-        const long long i_last = (i0 + kTB < W ? i0 + kTB : W) - 1;
-        const long long j_lim = (N - W) + i_last;  // last usable key
-        const long long b_lim = j_lim / kTB + 1;
-        if (b1 > b_lim) b1 = b_lim;
-    }
-    for (long long b = b0; b < b1; ++b) {
-        __syncthreads();
-        load_tile(sm.Ks, k + bh * N * d, b * kTB, N, d);
-        load_tile(sm.Vs, v + bh * N * d, b * kTB, N, d);
-        __syncthreads();
-        tile_p_ds(sm, d, i0, b * kTB, N, W, causal, scale);
-        __syncthreads();
-#pragma unroll 4
-        for (int j = 0; j < kTB; ++j) {
-            const float ds = sm.dSs[io * (kTB + 1) + j];
-#pragma unroll
-            for (int m = 0; m < MAXM; ++m) {
-                const int c = co + 8 * m;
-                if (c < d) acc[m] = fmaf(ds, sm.Ks[j * ld + c], acc[m]);
-            }
-        }
-    }
-    if (i0 + io < W && b1 > b0) {
-#pragma unroll
-        for (int m = 0; m < MAXM; ++m) {
-            const int c = co + 8 * m;
-            if (c < d) atomicAdd(&dq_acc[(bh * W + i0 + io) * d + c], acc[m]);
-        }
+    for (int i = 0; i < KA; ++i) {
+        const int key = j0 + tr * KA + i;
+        if (key >= N) continue;
+        store_columns<TC, CM>(dk + (bh * N + key) * d, acc_dk[i], 1.f, tc, d);
+        store_columns<TC, CM>(dv + (bh * N + key) * d, acc_dv[i], 1.f, tc, d);
     }
 }
 
@@ -220,51 +207,45 @@ __global__ void bwd_round_kernel(const float* __restrict__ src, T* __restrict__ 
     if (x < n) from_f(dst[x], src[x]);
 }
 
-template <typename T, int MAXM>
+template <typename T, int BT, int TC, int CM>
 int launch_t(const T* q, const T* k, const T* v, const T* out, const float* lse, const T* dout, T* dq, T* dk, T* dv,
-             int B, int H, int N, int W, int d, int causal, float* ws, int num_sms, cudaStream_t st) {
-    const long long bh = (long long)B * H, rows = bh * W;
+             int B, int H, int N, int W, int d, int causal, float* ws, cudaStream_t st) {
+    const int64_t n_bh = (int64_t)B * H, rows = n_bh * W;
     float* delta = ws;                                  // [B*H*W]
-    float* dq_acc = ws + ((rows + 3) / 4) * 4;          // [B*H*W*d], 16-byte aligned
+    constexpr bool kF32 = sizeof(T) == 4;
+    // fp32: the sums go straight into the result; bf16: [B*H*W*d] fp32 behind delta, 16-byte aligned
+    float* dq_acc = kF32 ? reinterpret_cast<float*>(dq) : ws + ((rows + 3) / 4) * 4;
     const float scale = 1.f / sqrtf((float)d);
-    const size_t smem = bwd_smem_bytes(d);
-    cudaError_t e = cudaFuncSetAttribute(bwd_dkdv_kernel<T, MAXM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem_bytes(8 * MAXM));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(bwd_dq_kernel<T, MAXM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem_bytes(8 * MAXM));
-    TLIN_CUDA_CHECK(e);
-    if (bh > 65535) return TLIN_ERR_UNSUPPORTED;        // grid.y
+    static bool allowed[64] = {};
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_simt_kernel<T, BT, TC, CM>, (int)bwd_smem_bytes<BT>(TC * CM, column_slack<TC, CM>()), allowed));
+    const int64_t ctas = n_bh * ((N + BT - 1) / BT);
+    if (ctas > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
     bwd_delta_kernel<T><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(out, dout, delta, rows, d);
     TLIN_CUDA_CHECK(cudaGetLastError());
     TLIN_CUDA_CHECK(cudaMemsetAsync(dq_acc, 0, (size_t)rows * d * sizeof(float), st));
-    const long long key_blocks = ((long long)N + kTB - 1) / kTB, q_tiles = ((long long)W + kTB - 1) / kTB;
-    bwd_dkdv_kernel<T, MAXM><<<dim3((unsigned)key_blocks, (unsigned)bh), kBwdThreads, smem, st>>>(
-        q, k, v, dout, lse, delta, dk, dv, N, W, d, causal, scale);
+    bwd_simt_kernel<T, BT, TC, CM><<<(unsigned)ctas, kTR * TC, bwd_smem_bytes<BT>(d, column_slack<TC, CM>()), st>>>(
+        q, k, v, dout, lse, delta, dq_acc, dk, dv, N, W, d, causal, n_bh, scale);
     TLIN_CUDA_CHECK(cudaGetLastError());
-    // slices of the key range for dq: enough CTAs for two waves, never more than 65535 (grid.z) or than key blocks
-    long long splits = (2LL * num_sms + q_tiles * bh - 1) / (q_tiles * bh);
-    if (splits < 1) splits = 1;
-    if (splits > key_blocks) splits = key_blocks;
-    if (splits > 65535) splits = 65535;
-    const int blocks_per_split = (int)((key_blocks + splits - 1) / splits);
-    splits = (key_blocks + blocks_per_split - 1) / blocks_per_split;
-    bwd_dq_kernel<T, MAXM><<<dim3((unsigned)q_tiles, (unsigned)bh, (unsigned)splits), kBwdThreads, smem, st>>>(
-        q, k, v, dout, lse, delta, dq_acc, N, W, d, causal, scale, blocks_per_split);
-    TLIN_CUDA_CHECK(cudaGetLastError());
-    bwd_round_kernel<T><<<(unsigned)((rows * d + 255) / 256), 256, 0, st>>>(dq_acc, dq, rows * d);
-    TLIN_CUDA_CHECK(cudaGetLastError());
-    count_launch(4);
+    count_launch(2);
+    if constexpr (!kF32) {
+        bwd_round_kernel<T><<<(unsigned)((rows * d + 255) / 256), 256, 0, st>>>(dq_acc, dq, rows * d);
+        TLIN_CUDA_CHECK(cudaGetLastError());
+        count_launch();
+    }
     return TLIN_OK;
 }
 
 template <typename T>
 int launch_any(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
-               void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, float* ws, int num_sms,
-               cudaStream_t st) {
-    if ((long long)B * H * W * d > (1LL << 40) || (long long)N > 0x7fffffffLL - kTB) return TLIN_ERR_UNSUPPORTED;
+               void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, float* ws, cudaStream_t st) {
+    if ((long long)B * H * W * d > (1LL << 40) || (long long)N > 0x7fffffffLL - 64) return TLIN_ERR_UNSUPPORTED;
     const T *qt = (const T*)q, *kt = (const T*)k, *vt = (const T*)v, *ot = (const T*)out, *dot = (const T*)dout;
-    if (d <= 64) return launch_t<T, 8>(qt, kt, vt, ot, lse, dot, (T*)dq, (T*)dk, (T*)dv, B, H, N, W, d, causal, ws, num_sms, st);
-    if (d <= 128) return launch_t<T, 16>(qt, kt, vt, ot, lse, dot, (T*)dq, (T*)dk, (T*)dv, B, H, N, W, d, causal, ws, num_sms, st);
-    if (d <= 256) return launch_t<T, 32>(qt, kt, vt, ot, lse, dot, (T*)dq, (T*)dk, (T*)dv, B, H, N, W, d, causal, ws, num_sms, st);
+    T *dqt = (T*)dq, *dkt = (T*)dk, *dvt = (T*)dv;
+    if (d <= 40) return launch_t<T, 64, 8, 5>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st);
+    if (d <= 64) return launch_t<T, 64, 8, 8>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st);
+    if (d <= 112) return launch_t<T, 64, 16, 7>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st);
+    if (d <= 128) return launch_t<T, 64, 16, 8>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st);
+    if (d <= 256) return launch_t<T, 32, 16, 16>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st);
     return TLIN_ERR_UNSUPPORTED;
 }
 
@@ -277,9 +258,9 @@ size_t bwd_workspace_bytes(long long B, long long H, long long W, int d) {
 
 int launch_bwd_simt(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                     void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, int is_f32, float* ws,
-                    int num_sms, cudaStream_t st) {
-    if (is_f32) return launch_any<float>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, num_sms, st);
-    return launch_any<__nv_bfloat16>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, num_sms, st);
+                    cudaStream_t st) {
+    if (is_f32) return launch_any<float>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, st);
+    return launch_any<__nv_bfloat16>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, st);
 }
 
 }  // namespace tlin

@@ -278,6 +278,10 @@ def test_backward_other_head_sizes_bf16(B, H, N, W, d, causal):
 
 F32 = [(1, 2, 300, 77, 36, 1), (2, 1, 515, 130, 64, 0), (1, 1, 1000, 200, 128, 1), (1, 3, 97, 97, 100, 1), (1, 1, 1, 1, 4, 1)]
 
+# both tile sizes and both thread counts of the CUDA-core kernel, head sizes at both ends of each column class, tile edges +-1
+F32 += [(1, 2, 64, 64, 40, 1), (1, 1, 65, 63, 44, 0), (2, 1, 129, 65, 64, 1), (1, 1, 63, 63, 68, 1), (1, 1, 130, 64, 112, 0), (1, 1, 100, 65, 116, 1),
+        (1, 2, 33, 31, 132, 0), (1, 1, 97, 64, 256, 1), (1, 1, 300, 20, 36, 1)]
+
 
 @pytest.mark.parametrize("B,H,N,W,d,causal", F32)
 def test_backward_f32(B, H, N, W, d, causal):

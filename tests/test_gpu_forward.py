@@ -549,3 +549,13 @@ def test_chunk_scheduled_forward_with_many_units_is_one_launch():
         if tl.tlin_plan_forward(B, H, n_keys[c], W, d, 1).schedule == 1:
             o1, l1 = run_impl(2, tl.tlin_attn_forward, q[c], k[:, :, :n_keys[c]].contiguous(), v[:, :, :n_keys[c]].contiguous(), causal_window=1)
             assert torch.equal(o1, out[c]) and torch.equal(l1, lse[c])
+
+
+# the register tilings of the CUDA-core kernel (columns per thread: head sizes at both ends of each class; 64 and 65 query rows)
+# and the clusters that share one query tile's keys (few (b,h): 2, 4 and 8 CTAs, some of them without a key under the window rule)
+@pytest.mark.parametrize("B,H,N,W,d,causal", [(1, 2, 130, 64, 40, 1), (1, 2, 130, 65, 44, 1), (2, 1, 193, 129, 64, 0), (1, 1, 127, 70, 68, 1),
+                                              (1, 2, 66, 33, 104, 0), (1, 1, 200, 128, 108, 1), (1, 1, 150, 150, 132, 1), (1, 1, 90, 64, 192, 0),
+                                              (1, 1, 90, 65, 196, 1), (1, 1, 513, 513, 36, 1), (1, 1, 3000, 65, 64, 1), (1, 70, 600, 64, 36, 0),
+                                              (1, 36, 1100, 64, 128, 1), (1, 1, 520, 520, 256, 1)])
+def test_fp32_tilings_and_key_sharing_clusters(B, H, N, W, d, causal):
+    full_compare(synth.Workload("f32 tiles", B, H, d, N, W, seed=40 + N + d, causal_window=causal), 0, kind="f32")
