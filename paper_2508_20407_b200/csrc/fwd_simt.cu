@@ -7,7 +7,7 @@
 // registers (two 16-byte shared loads per 16 to 32 FFMA) and accumulates ROWS x CM output elements; the probabilities pass
 // through shared memory inside the warp only (a row belongs to eight lanes of one warp).  One key scored per lane and one
 // probability per shuffle, as before, spent four shared-memory reads on five FFMA.
-// Measured, fp32: B8 H12 N1024 W512 d36 2059 -> 218 us (25 TFLOP/s), B4 H12 N1500 W700 d128 3229 -> 837 us.
+// Measured, fp32: B8 H12 N1024 W512 d36 2059 -> 210 us (26 TFLOP/s), B4 H12 N1500 W700 d128 3229 -> 837 us.
 //
 // Few (b,h) and query tiles: the CTAs of a cluster (2, 4 or 8) share the keys of one query tile and merge their sums through
 // distributed shared memory, so that no workspace is needed.
@@ -226,14 +226,15 @@ int launch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H,
     return TLIN_OK;
 }
 
-// 8 columns per CM; 128 query rows per CTA while a thread's share of them fits the registers and the call has that many rows
+// 8 columns per CM.  Eight rows per thread instead of four halve the shared-memory reads but need 128 query rows per CTA: worth it
+// for 40 < d <= 64 when that leaves few SMs without a CTA (128 CTAs at B4 H8 N2000 W500 d64: 261 against 285 us); at d <= 40, with three CTAs of
+// either kind per SM, the finer split wins (B8 H12 N1024 W512 d36: 210 against 218 us, B8 H4 N327 W327: 42 against 52 us), and
+// beyond d = 64 the registers do not suffice.
 template <typename T>
 int dispatch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H, int N, int W, int d,
              int causal, long long kv, cudaStream_t st) {
-    if (d <= 64 && W > 64) {
-        if (d <= 40) return launch<T, 8, 5>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
+    if (d > 40 && d <= 64 && (int64_t)B * H * ((W + 127) / 128) >= kDefaultSMs * 3 / 4)
         return launch<T, 8, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
-    }
     if (d <= 40) return launch<T, 4, 5>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
     if (d <= 64) return launch<T, 4, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
     if (d <= 104) return launch<T, 4, 13>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
