@@ -54,9 +54,10 @@ typedef enum {
  *                    iff j <= N-W+i: the history is unmasked and the window is causal (Section 3,
  *                    "Causal Attention", j <= i, aligned to the end).  One softmax runs over the
  *                    union of both key sets.  Requires N >= W.
- * bf16 path: d in {64,128} runs on the tensor cores; any other d that is a multiple of 8 up to 256
- * runs on the CUDA-core kernel.  f32 path: d a multiple of 4 up to 256 (covers the paper's d = 36).
- * Uses the workspace when the plan splits the key range (see tlin_workspace_bytes_forward).
+ * bf16 path: d a multiple of 8 up to 256, on the tensor cores (64 and 128 in tiles of their own, the others in zero-padded
+ * ones).  f32 path: d a multiple of 4 up to 256 (covers the paper's d = 36), CUDA cores.
+ * Uses the workspace when the plan splits the key range (see tlin_workspace_bytes_forward); head sizes other than 64 and 128
+ * also run without one, with whole key ranges.
  */
 int tlin_attn_forward(const void* q, const void* k, const void* v, void* out, float* lse,
                       int B, int H, int N, int W, int d, int causal_window, tlin_stream_t stream);
@@ -281,7 +282,7 @@ int tlin_set_workspace(void* dev_ptr, size_t bytes);
  * (query,key) pairs of a call number W*N without a mask and W*(N-W) + W*(W+1)/2 with the window.
  */
 typedef struct {
-    int32_t tile_m;        /* query rows per CTA                                             */
+    int32_t tile_m;        /* query rows per CTA (CUDA-core path: rows of a unit, a CTA takes several) */
     int32_t tile_n;        /* keys per tile                                                  */
     int32_t q_tiles;       /* ceil(W / tile_m): CTAs that share one key range                */
     int32_t key_tiles;     /* ceil(N / tile_n) per (b,h)                                     */
@@ -348,7 +349,7 @@ int tlin_debug_wait_expires(long long limit_cycles, long long* waited_cycles, tl
 const char* tlin_status_string(int status);
 const char* tlin_version(void);
 /* Which kernel serves tlin_attn_forward: 0 = automatic, 1 = always the CUDA-core kernel,
- * 2 = tensor-core kernel (TLIN_ERR_UNSUPPORTED if the shape does not allow it).  tlin_attn_backward follows the same
+ * 2 = tensor-core kernel (TLIN_ERR_UNSUPPORTED if the shape does not allow it, i.e. in fp32).  tlin_attn_backward follows the same
  * switch (1 = CUDA-core kernels for every head size).  Returns the old value. */
 int tlin_set_forward_impl(int impl);
 /* How the tensor-core kernels of tlin_attn_backward (bf16, d = 64 or 128) are arranged; the chain rule of the Section 3

@@ -116,7 +116,12 @@ static int forward_common(const void* q, const void* k, const void* v, void* out
     float* ws = nullptr;
     if (plan.uses_workspace) {
         const Workspace w = workspace();
-        if (!w.ptr || w.bytes < (size_t)plan.workspace_bytes) return TLIN_ERR_WORKSPACE;
+        if (!w.ptr || w.bytes < (size_t)plan.workspace_bytes) {
+            // head sizes other than 64 and 128 have always run without a workspace: keys are then not split
+            if (d == 64 || d == 128) return TLIN_ERR_WORKSPACE;
+            rc = plan_forward(B, H, N, W, d, causal_window, 0, sms, true, &plan);
+            if (rc != TLIN_OK) return rc;
+        }
         ws = (float*)w.ptr;
     }
     return launch_fwd_tc(q, k, v, out, lse, B, H, N, W, d, causal_window, plan, ws, kv_rows_alloc, st);
@@ -294,7 +299,7 @@ extern "C" int tlin_attn_backward_f32(const float* q, const float* k, const floa
 extern "C" size_t tlin_workspace_bytes_backward(int B, int H, int N, int W, int d) {
     if (B <= 0 || H <= 0 || N <= 0 || W <= 0 || d <= 0) return 0;
     size_t need = bwd_workspace_bytes(B, H, W, d);                 // CUDA-core path
-    for (int causal = 0; causal < 2; ++causal) {
+    for (int causal = 0; causal < 2 && (d == 64 || d == 128); ++causal) {
         tlin_fwd_plan plan;
         if (causal && N < W) continue;
         if (tlin_plan_forward(B, H, N, W, d, causal, 0, 0, &plan) != TLIN_OK || !plan.tensor_path) continue;

@@ -1,5 +1,6 @@
 // CUDA-core forward kernel: exact softmax attention, fp32 arithmetic, any head dimension up to 256.
-// Serves the fp32 entry point (error bar 1e-4) and bf16 shapes the tensor path does not take.
+// Serves the fp32 entry point (error bar 1e-4), and bf16 where tlin_set_forward_impl(1) asks for it or the call has 2^31 query
+// rows or more at a head size other than 64 and 128.
 // Section 3 attention formula; causal rule j <= N-W+i; online (running max / running sum) softmax.
 //
 // Bound by the FFMA rate (128 per clock and SM, 72 TFLOP/s at 1.9 GHz).  A CTA of 128 threads (16 row groups x 8 column

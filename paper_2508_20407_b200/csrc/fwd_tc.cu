@@ -69,13 +69,24 @@ __device__ __forceinline__ void exp2_poly2(uint64_t x2, float& p0, float& p1) {
     p1 = __uint_as_float(y1 + (n1 << 23));
 }
 
+// The kernel's three forms: head size D exactly, one problem or a table of them; or any other head size d <= D that is a multiple
+// of 8.  The last reads its tiles with zero fill beyond d (the tensor maps know the true row length), contracts over ceil(d/16)
+// slices only, and keeps P to 16 mantissa bits as the sum of two bf16 parts, two PV products per step: the CUDA-core kernel that
+// served these sizes before kept P in fp32, and the results are to lose nothing (against 64-bit sums 1.66e-3, the rounding to
+// bf16 alone).  At D = 256 two output accumulators would fill the TMEM, so a CTA works on one Q tile.
+// Measured against that CUDA-core kernel: B2 H9 N3001 W517 d96 2066 -> 45 us, B2 H3 N7791 W968 d40 2582 -> 38 us, B1 H12 N2000
+// W1000 d256 3952 -> 56 us, B4 H12 N370 W96 d32 96 -> 12 us.
+enum { kOneProblem = 0, kTable = 1, kAnyHead = 2 };
+
 template <int D>
 struct Cfg {
+    static constexpr int kTiles = D == 256 ? 1 : 2;            // Q tiles per CTA
+    static constexpr int kRows = kTiles * kQTile;              // query rows per CTA
     static constexpr int kTileBytes = kQTile * D * 2;          // one 128-row tile of Q, K or V
     static constexpr int kBoxes = D / 64;                      // 64-element (128-byte) column blocks per tile
-    static constexpr int kSlots = D == 128 ? 4 : 8;            // K/V ring slots
-    static constexpr int kSmemTiles = (2 + kSlots) * kTileBytes;
-    static constexpr int kStageBytes = 8 * 32 * 128;           // per softmax warp 32 rows x 128 bytes: result rows on their way out
+    static constexpr int kSlots = D == 256 ? 2 : D == 128 ? 4 : 8;            // K/V ring slots
+    static constexpr int kSmemTiles = (kTiles + kSlots) * kTileBytes;
+    static constexpr int kStageBytes = 4 * kTiles * 32 * 128;  // per softmax warp 32 rows x 128 bytes: result rows on their way out
     static constexpr int kNumBars = 10 + 2 * kSlots;
     static constexpr int kSmemBytes = kSmemTiles + kStageBytes + kNumBars * 8 + 16 + 1024;   // + alignment slack
     // TMEM columns: S0, S1 (128 each), O0, O1 (D each)
@@ -107,6 +118,7 @@ struct Params {
     long long total_units;
     int n_groups, q_tiles, key_tiles;
     int N, W, causal;
+    int d;                // head size (row length of every tensor)
     int schedule;         // 0: groups of q_tiles CTAs stream key ranges; 1: every CTA walks whole (b,h,q-tile) problems
     float scale_log2e;
 };
@@ -143,15 +155,19 @@ __device__ __forceinline__ decltype(auto) problem_of(const KernelMaps<kBatched>&
     else return (p);
 }
 
-template <int D, bool kBatched>
+template <int D, int kForm>
 __global__ void __launch_bounds__(kThreads, 1)
-fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_constant__ Params p,
+fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __grid_constant__ Params p,
               const __grid_constant__ GroupStarts starts) {
     using C = Cfg<D>;
+    constexpr bool kBatched = kForm == kTable, kAny = kForm == kAnyHead;
+    constexpr int kTileM = C::kRows;
+    const int d = kAny ? p.d : D;                              // row length; everything below folds where it is D
+    const int boxes = kAny ? (d + 63) / 64 : C::kBoxes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* sQ = smem;                               // 2 tiles
-    uint8_t* sRing = smem + 2 * C::kTileBytes;        // kSlots tiles
+    uint8_t* sQ = smem;                               // kTiles tiles
+    uint8_t* sRing = smem + C::kTiles * C::kTileBytes;        // kSlots tiles
     uint8_t* sStage = smem + C::kSmemTiles;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kSmemTiles + C::kStageBytes);
     uint64_t* q_full = bars + 0;
@@ -219,14 +235,14 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                 if constexpr (kBatched) { map_q_p = &maps.q[s.prob]; map_k_p = &maps.k[s.prob]; map_v_p = &maps.v[s.prob]; }
                 else { map_q_p = &maps.q; map_k_p = &maps.k; map_v_p = &maps.v; }
                 const int row0 = s.qt * kTileM;
-                const int c0 = seg_count(s, tiles_allowed(pr, row0, 0)), c1 = seg_count(s, tiles_allowed(pr, row0, 1));
+                const int c0 = seg_count(s, tiles_allowed(pr, row0, 0)), c1 = C::kTiles > 1 ? seg_count(s, tiles_allowed(pr, row0, 1)) : 0;
                 const int cnt = c0 > c1 ? c0 : c1;
                 if (cnt == 0) continue;
                 if (seg_idx > 0) ok = mbar_wait(q_empty, (seg_idx - 1) & 1, abort_p);
                 if (!ok) break;
-                mbar_arrive_expect_tx(q_full, 2 * C::kTileBytes);
-                for (int i = 0; i < 2; ++i)
-                    for (int b = 0; b < C::kBoxes; ++b)
+                mbar_arrive_expect_tx(q_full, C::kTiles * boxes * (kQTile * 128));
+                for (int i = 0; i < C::kTiles; ++i)
+                    for (int b = 0; b < boxes; ++b)
                         tma_load_3d(sQ + i * C::kTileBytes + b * (kQTile * 128), map_q_p, q_full, b * 64, row0 + i * kQTile, s.bh);
                 for (int j = 0; j < cnt && ok; ++j) {
                     const int t = s.t_begin + j;
@@ -234,9 +250,9 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                         const uint32_t slot = it % C::kSlots, round = it / C::kSlots;
                         ok = mbar_wait(&kv_empty[slot], (round & 1) ^ 1, abort_p);
                         if (!ok) break;
-                        mbar_arrive_expect_tx(&kv_full[slot], C::kTileBytes);
+                        mbar_arrive_expect_tx(&kv_full[slot], boxes * (kQTile * 128));
                         uint8_t* dst = sRing + slot * C::kTileBytes;
-                        for (int b = 0; b < C::kBoxes; ++b)
+                        for (int b = 0; b < boxes; ++b)
                             tma_load_3d(dst + b * (kQTile * 128), kv == 0 ? map_k_p : map_v_p, &kv_full[slot], b * 64, t * kTileN, s.bh);
                         ++it;
                     }
@@ -265,14 +281,15 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
         // instead: 1.88 against 1.83 ms (B1 H32 N131072 W1024 d128), 382 against 361 us (N32768 W1024 d64).
         {
             const uint32_t idesc_qk = make_idesc_bf16(kQTile, kTileN, 0, 0);
-            const uint32_t idesc_pv = make_idesc_bf16(kQTile, D, 0, 1);
+            const uint32_t idesc_pv = make_idesc_bf16(kQTile, kAny ? (d + 15) / 16 * 16 : D, 0, 1);
+            const int slices = kAny ? (d + 15) / 16 : D / 16;         // of the head dimension
             // Descriptors are built once; per MMA only the 14-bit address field of the low word moves
             // (one 32-bit add of a compile-time constant).
             const uint64_t q_desc = make_smem_desc_sw128(smem_u32(sQ), 16, 1024);
             const uint64_t k_desc = make_smem_desc_sw128(smem_u32(sRing), 16, 1024);            // K-major tile (K)
             const uint64_t v_desc = make_smem_desc_sw128(smem_u32(sRing), kQTile * 128, 1024);  // MN-major tile (V)
             const uint32_t desc_hi = (uint32_t)(q_desc >> 32);        // identical for all three
-            const uint32_t q_lo[2] = {(uint32_t)q_desc, (uint32_t)q_desc + (C::kTileBytes >> 4)};
+            const uint32_t q_lo[2] = {(uint32_t)q_desc, (uint32_t)q_desc + (C::kTileBytes >> 4)};      // [1] unused with one Q tile
             const uint32_t k_lo0 = (uint32_t)k_desc, v_lo0 = (uint32_t)v_desc;
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
             const uint32_t tS0 = tmem_u + C::kColS, tO0 = tmem_u + C::kColO;
@@ -281,20 +298,24 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
             uint32_t n_pv[2] = {0, 0};
             bool ok = true;
             auto issue_qk = [&](int i, uint32_t k_slot) {
-                const uint32_t a_lo = q_lo[i], b_lo = k_lo0 + k_slot * (C::kTileBytes >> 4), d = tS0 + i * kTileN;
+                const uint32_t a_lo = q_lo[i], b_lo = k_lo0 + k_slot * (C::kTileBytes >> 4), acc = tS0 + i * kTileN;
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
                     const uint32_t off16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4;
-                    mma_ss_lead(lead, d, a_lo + off16, b_lo + off16, desc_hi, idesc_qk, kk > 0);
+                    mma_ss_lead(!kAny || kk < slices ? lead : 0u, acc, a_lo + off16, b_lo + off16, desc_hi, idesc_qk, kk > 0);
                 }
                 commit_lead(lead, &s_full[i]);
             };
             // PV of the keys [16 from, 16 to) of a tile
             auto issue_pv = [&](int i, uint32_t v_slot, bool accumulate, auto from, auto to) {
-                const uint32_t b_lo = v_lo0 + v_slot * (C::kTileBytes >> 4), d = tO0 + i * D, a = tS0 + i * kTileN;
+                const uint32_t b_lo = v_lo0 + v_slot * (C::kTileBytes >> 4), acc = tO0 + i * D, a = tS0 + i * kTileN;
 #pragma unroll
                 for (int kk = decltype(from)::value; kk < decltype(to)::value; ++kk)
-                    mma_ts_lead(lead, d, a + kk * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_pv, (accumulate || kk > 0) ? 1u : 0u);
+                    mma_ts_lead(lead, acc, a + kk * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_pv, (accumulate || kk > 0) ? 1u : 0u);
+                if constexpr (kAny)        // the low parts of P, 64 columns further
+#pragma unroll
+                    for (int kk = decltype(from)::value; kk < decltype(to)::value; ++kk)
+                        mma_ts_lead(lead, acc, a + 64 + kk * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_pv, 1u);
             };
             constexpr std::integral_constant<int, 0> k_begin{};
             constexpr std::integral_constant<int, kFirstKeys / 16> k_first{};
@@ -304,7 +325,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
             while (ok && walk.next(s)) {
                 const auto& pr = problem_of<kBatched>(maps, p, s);
                 const int row0 = s.qt * kTileM;
-                const int c0 = seg_count(s, tiles_allowed(pr, row0, 0)), c1 = seg_count(s, tiles_allowed(pr, row0, 1));
+                const int c0 = seg_count(s, tiles_allowed(pr, row0, 0)), c1 = C::kTiles > 1 ? seg_count(s, tiles_allowed(pr, row0, 1)) : 0;
                 const int cnt = c0 > c1 ? c0 : c1;
                 if (cnt == 0) continue;
                 const int cq[2] = {c0, c1};
@@ -315,7 +336,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                 ok = __all_sync(0xffffffffu, mbar_wait(&kv_full[k_slot], (it / C::kSlots) & 1, abort_p));
                 if (!ok) break;
                 tc_fence_after();
-                for (int i = 0; i < 2; ++i)
+                for (int i = 0; i < C::kTiles; ++i)
                     if (cq[i] > 0) issue_qk(i, k_slot);
                 commit_lead(lead, &kv_empty[k_slot]);
                 if (cnt == 1) commit_lead(lead, q_empty);      // the segment's last use of Q is issued: its successor may load
@@ -345,7 +366,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                         }
                     }
                     tc_fence_after();
-                    for (int i = 0; i < 2 && ok; ++i) {
+                    for (int i = 0; i < C::kTiles && ok; ++i) {
                         if (j < cq[i]) {
                             ok = __all_sync(0xffffffffu, mbar_wait(&p_first[i], n_pv[i] & 1, abort_p));
                             if (!ok) break;
@@ -358,9 +379,9 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                             commit_lead(lead, &pv_done[i]);
                             ++n_pv[i];
                         }
-                        if (i == 1) commit_lead(lead, &kv_empty[v_slot]);
+                        if (i == C::kTiles - 1) commit_lead(lead, &kv_empty[v_slot]);
                         if (have_next && j + 1 < cq[i]) issue_qk(i, nk_slot);
-                        if (have_next && i == 1) {
+                        if (have_next && i == C::kTiles - 1) {
                             commit_lead(lead, &kv_empty[nk_slot]);
                             // Q is last read by the S of the segment's last key tile: releasing it here lets the
                             // producer fetch the next segment's Q while this one finishes
@@ -376,6 +397,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
     } else {
         // ------------------------------------------------------------------ softmax warpgroups (one per Q tile)
         setmaxnreg_inc<kSoftmaxRegs>();
+        if (C::kTiles > 1 || warp < 4) {
         const int i = warp >> 2;                           // Q tile
         const int r = (warp & 3) * 32 + lane;              // row inside the Q tile == TMEM lane
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
@@ -438,6 +460,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                         tc_fence_after();
 #pragma unroll
                         for (int c = 0; c < D / 8; ++c) {      // narrow pieces: the row of S stays in registers meanwhile
+                            if (kAny && c * 8 >= d) break;
                             uint32_t o[8];
                             tmem_ld8(tO + c * 8, o);
 #pragma unroll
@@ -458,12 +481,12 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                 const uint64_t scale2 = f2_pack(p.scale_log2e, p.scale_log2e), negm2 = f2_pack(-m_use, -m_use);
 #pragma unroll
                 for (int c = 0; c < kTileN / 32; ++c) {
-                    uint32_t pk[16];
+                    uint32_t pk[16], pk_low[kAny ? 16 : 1];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
                         const uint64_t x2 = f2_fma(f2_pack_bits(sv[c][2 * e], sv[c][2 * e + 1]), scale2, negm2);
                         float p0, p1;
-                        if (!kMasked && e * kPolyPairs / 16 != (e + 1) * kPolyPairs / 16) {
+                        if (!kMasked && !kAny && e * kPolyPairs / 16 != (e + 1) * kPolyPairs / 16) {
                             exp2_poly2(x2, p0, p1);
                         } else {
                             float x0, x1;
@@ -474,8 +497,11 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                         sv[c][2 * e] = __float_as_uint(p0);
                         sv[c][2 * e + 1] = __float_as_uint(p1);
                         pk[e] = pack_bf16x2(p0, p1);
+                        if constexpr (kAny)
+                            pk_low[e] = pack_bf16x2(p0 - __uint_as_float(pk[e] << 16), p1 - __uint_as_float(pk[e] & 0xffff0000u));
                     }
                     tmem_st16(tS + c * 16, pk);
+                    if constexpr (kAny) tmem_st16(tS + 64 + c * 16, pk_low);
                     if (c == kFirstKeys / 32 - 1) {    // the first keys are in place: let the PV MMAs start on them
                         tc_wait_st();
                         tc_fence_before();
@@ -517,16 +543,17 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
             const float lse_val = l > 0.f ? (m_ref + log2f(l)) * kLn2 : -CUDART_INF_F;
             const bool store = row < pr.W;
             // partial result -> workspace slot (0: first segment of this CTA's range, 1: a later one)
-            float* pbase = p.ws + ((long long)blockIdx.x * 2 + (s.bh == bh_first ? 0 : 1)) * (long long)kTileM * (D + 1);
+            float* pbase = p.ws + ((long long)blockIdx.x * 2 + (s.bh == bh_first ? 0 : 1)) * (long long)kTileM * (d + 1);
             // A thread holds one row.  Stored straight from the registers a warp's store would touch 32 different lines, so
             // the warp passes its rows through shared memory 128 bytes at a time (16-byte pieces, piece index xor row: no
             // bank conflicts beyond the minimum on either side) and every store instruction writes four whole lines.
             uint8_t* stage = sStage + warp * (32 * 128);
             const int row_warp = row - lane;                   // row of lane 0
             if (whole) {
-                __nv_bfloat16* owarp = reinterpret_cast<__nv_bfloat16*>(pr.out) + ((long long)s.bh * pr.W + row_warp) * D;
+                __nv_bfloat16* owarp = reinterpret_cast<__nv_bfloat16*>(pr.out) + ((long long)s.bh * pr.W + row_warp) * d;
 #pragma unroll
                 for (int h = 0; h < D / 64; ++h) {             // 64 bf16 columns per pass
+                    if (kAny && h * 64 >= d) break;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         uint32_t o[16];
@@ -552,14 +579,15 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                     for (int it = 0; it < 8; ++it) {
                         const int rrow = it * 4 + (lane >> 3), piece = lane & 7;
                         const uint4 w = *reinterpret_cast<const uint4*>(stage + rrow * 128 + ((piece ^ (rrow & 7)) << 4));
-                        if (row_warp + rrow < pr.W) *reinterpret_cast<uint4*>(owarp + (long long)rrow * D + h * 64 + piece * 8) = w;
+                        if (row_warp + rrow < pr.W && (!kAny || h * 64 + piece * 8 < d)) *reinterpret_cast<uint4*>(owarp + (long long)rrow * d + h * 64 + piece * 8) = w;
                     }
                     __syncwarp();
                 }
             } else {
-                float* pwarp = pbase + (long long)(i * kQTile + (warp & 3) * 32) * D;
+                float* pwarp = pbase + (long long)(i * kQTile + (warp & 3) * 32) * d;
 #pragma unroll
                 for (int h = 0; h < D / 32; ++h) {             // 32 fp32 columns per pass
+                    if (kAny && h * 32 >= d) break;
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         uint32_t o[16];
@@ -585,7 +613,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
                     for (int it = 0; it < 8; ++it) {
                         const int rrow = it * 4 + (lane >> 3), piece = lane & 7;
                         const float4 w = *reinterpret_cast<const float4*>(stage + rrow * 128 + ((piece ^ (rrow & 7)) << 4));
-                        *reinterpret_cast<float4*>(pwarp + (long long)rrow * D + h * 32 + piece * 4) = w;
+                        if (!kAny || h * 32 + piece * 4 < d) *reinterpret_cast<float4*>(pwarp + (long long)rrow * d + h * 32 + piece * 4) = w;
                     }
                     __syncwarp();
                 }
@@ -593,9 +621,10 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
             if (whole) {
                 if (store && pr.lse != nullptr) pr.lse[(long long)s.bh * pr.W + row] = lse_val;
             } else {
-                pbase[(long long)kTileM * D + i * kQTile + r] = lse_val;
+                pbase[(long long)kTileM * d + i * kQTile + r] = lse_val;
             }
             tc_fence_before();      // TMEM reads of O are complete before the next segment's arrive lets PV overwrite it
+        }
         }
     }
 
@@ -613,10 +642,12 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kBatched> maps, const __grid_co
 constexpr int kMergeRows = 8;            // one row per warp: many small CTAs hide the latency of the scattered partial reads
 constexpr int kMaxParts = 8;          // more partials than this per row are merged in a slower loop
 
-template <int D>
+template <int D, bool kAny>
 __global__ void __launch_bounds__(256)
 fwd_merge_kernel(const Params p) {
     constexpr int CPL = D / 32;                           // columns per lane
+    constexpr int kTileM = Cfg<D>::kRows;
+    const int d = kAny ? p.d : D;
     const int blocks_per_tile = kTileM / kMergeRows;
     const int quarter = blockIdx.x % blocks_per_tile;
     const int tile_id = blockIdx.x / blocks_per_tile;     // bh * q_tiles + qt
@@ -633,13 +664,14 @@ fwd_merge_kernel(const Params p) {
         for (int g = g_lo; g <= g_hi && g - g_lo < kMaxParts; ++g) {
             const int cta = g * p.q_tiles + qt;
             const int slot = bh == (int)((((unsigned long long)g * U) / G) / T) ? 0 : 1;
-            part_base[g - g_lo] = p.ws + ((long long)cta * 2 + slot) * (long long)kTileM * (D + 1);
+            part_base[g - g_lo] = p.ws + ((long long)cta * 2 + slot) * (long long)kTileM * (d + 1);
         }
     }
     __syncthreads();
     const int n_parts = n_parts_s;
     if (n_parts <= 1) return;                             // written directly by the attention kernel
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool owns = !kAny || lane * CPL < d;            // d is a multiple of 8: a lane's columns are inside or outside as a whole
     for (int rq = warp; rq < kMergeRows; rq += 8) {
         const int rr = quarter * kMergeRows + rq;         // row inside the 256-row tile
         const int row = qt * kTileM + rr;
@@ -649,7 +681,7 @@ fwd_merge_kernel(const Params p) {
             float ls[kMaxParts];
 #pragma unroll
             for (int i = 0; i < kMaxParts; ++i) {
-                ls[i] = i < n_parts ? part_base[i][(long long)kTileM * D + rr] : -CUDART_INF_F;
+                ls[i] = i < n_parts ? part_base[i][(long long)kTileM * d + rr] : -CUDART_INF_F;
                 m = fmaxf(m, ls[i]);
             }
             float z = 0.f, acc[CPL];
@@ -660,16 +692,18 @@ fwd_merge_kernel(const Params p) {
                 if (i < n_parts) {
                     const float w = expf(ls[i] - m);      // -inf (empty part) -> 0
                     z += w;
-                    const float* src = part_base[i] + (long long)rr * D + lane * CPL;
+                    if (!owns) continue;
+                    const float* src = part_base[i] + (long long)rr * d + lane * CPL;
 #pragma unroll
                     for (int e = 0; e < CPL; ++e) acc[e] = fmaf(w, src[e], acc[e]);
                 }
             }
             const float inv = 1.f / z;
-            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)bh * p.W + row) * D + lane * CPL;
+            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)bh * p.W + row) * d + lane * CPL;
 #pragma unroll
             for (int e = 0; e < CPL; e += 2)
-                *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
+                if (owns)
+                    *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
             if (p.lse != nullptr && lane == 0) p.lse[(long long)bh * p.W + row] = m + logf(z);
         } else {
             // many small groups per (b,h): recompute the slot addresses on the fly
@@ -677,55 +711,57 @@ fwd_merge_kernel(const Params p) {
             auto base_of = [&](int g) {
                 const int cta = g * p.q_tiles + qt;
                 const int slot = bh == (int)((((unsigned long long)g * U) / G) / T) ? 0 : 1;
-                return p.ws + ((long long)cta * 2 + slot) * (long long)kTileM * (D + 1);
+                return p.ws + ((long long)cta * 2 + slot) * (long long)kTileM * (d + 1);
             };
-            for (int i = 0; i < n_parts; ++i) m = fmaxf(m, base_of(g_lo_s + i)[(long long)kTileM * D + rr]);
+            for (int i = 0; i < n_parts; ++i) m = fmaxf(m, base_of(g_lo_s + i)[(long long)kTileM * d + rr]);
             float z = 0.f, acc[CPL];
 #pragma unroll
             for (int e = 0; e < CPL; ++e) acc[e] = 0.f;
             for (int i = 0; i < n_parts; ++i) {
                 const float* base = base_of(g_lo_s + i);
-                const float w = expf(base[(long long)kTileM * D + rr] - m);
+                const float w = expf(base[(long long)kTileM * d + rr] - m);
                 z += w;
+                if (!owns) continue;
 #pragma unroll
-                for (int e = 0; e < CPL; ++e) acc[e] = fmaf(w, base[(long long)rr * D + lane * CPL + e], acc[e]);
+                for (int e = 0; e < CPL; ++e) acc[e] = fmaf(w, base[(long long)rr * d + lane * CPL + e], acc[e]);
             }
             const float inv = 1.f / z;
-            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)bh * p.W + row) * D + lane * CPL;
+            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)bh * p.W + row) * d + lane * CPL;
 #pragma unroll
             for (int e = 0; e < CPL; e += 2)
-                *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
+                if (owns)
+                    *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
             if (p.lse != nullptr && lane == 0) p.lse[(long long)bh * p.W + row] = m + logf(z);
         }
     }
 }
 
-template <int D>
+template <int D, int kForm>
 int launch_d(const void* q, const void* k, const void* v, void* out, float* lse, int B, int H, int N, int W,
-             int causal, const tlin_fwd_plan& plan, float* ws, long long kv_rows_alloc, cudaStream_t st) {
+             int d, int causal, const tlin_fwd_plan& plan, float* ws, long long kv_rows_alloc, cudaStream_t st) {
     using C = Cfg<D>;
     const long long bh = (long long)B * H;
     KernelMaps<false> maps;
-    int rc = make_map(&maps.q, q, D, W, bh);
-    if (rc == TLIN_OK) rc = make_map(&maps.k, k, D, N, bh, kQTile, kv_rows_alloc);
-    if (rc == TLIN_OK) rc = make_map(&maps.v, v, D, N, bh, kQTile, kv_rows_alloc);
+    int rc = make_map(&maps.q, q, d, W, bh);
+    if (rc == TLIN_OK) rc = make_map(&maps.k, k, d, N, bh, kQTile, kv_rows_alloc);
+    if (rc == TLIN_OK) rc = make_map(&maps.v, v, d, N, bh, kQTile, kv_rows_alloc);
     if (rc != TLIN_OK) return rc;
     Params p;
     p.out = out; p.lse = lse; p.ws = ws; p.status = status_word();
     if (!p.status) return TLIN_ERR_CUDA;
     p.total_units = plan.total_units; p.n_groups = plan.n_groups; p.q_tiles = plan.q_tiles; p.key_tiles = plan.key_tiles;
-    p.N = N; p.W = W; p.causal = causal; p.schedule = plan.schedule;
-    p.scale_log2e = kLog2e / sqrtf((float)D);
+    p.N = N; p.W = W; p.causal = causal; p.d = d; p.schedule = plan.schedule;
+    p.scale_log2e = kLog2e / sqrtf((float)d);
     static bool smem_allowed[64] = {};
-    TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_tc_kernel<D, false>, C::kSmemBytes, smem_allowed));
+    TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_tc_kernel<D, kForm>, C::kSmemBytes, smem_allowed));
     if (plan.n_groups > kMaxGroups) return TLIN_ERR_UNSUPPORTED;
     GroupStarts starts;
     fwd_group_starts(plan, &starts);
-    fwd_tc_kernel<D, false><<<plan.n_ctas, kThreads, C::kSmemBytes, st>>>(maps, p, starts);
+    fwd_tc_kernel<D, kForm><<<plan.n_ctas, kThreads, C::kSmemBytes, st>>>(maps, p, starts);
     TLIN_CUDA_CHECK(cudaGetLastError());
     count_launch();
     if (plan.uses_workspace) {
-        fwd_merge_kernel<D><<<(unsigned)(bh * plan.q_tiles * (kTileM / kMergeRows)), 256, 0, st>>>(p);
+        fwd_merge_kernel<D, kForm == kAnyHead><<<(unsigned)(bh * plan.q_tiles * (C::kRows / kMergeRows)), 256, 0, st>>>(p);
         TLIN_CUDA_CHECK(cudaGetLastError());
         count_launch();
     }
@@ -765,8 +801,8 @@ int launch_batched_d(const tlin_problem* problems, int n, const long long* start
     GroupStarts starts;
     for (int g = 0; g <= n_ctas; ++g) starts.u[g] = starts_in[g];
     static bool smem_allowed[64] = {};
-    TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_tc_kernel<D, true>, C::kSmemBytes, smem_allowed));
-    fwd_tc_kernel<D, true><<<n_ctas, kThreads, C::kSmemBytes, st>>>(maps, p, starts);
+    TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_tc_kernel<D, kTable>, C::kSmemBytes, smem_allowed));
+    fwd_tc_kernel<D, kTable><<<n_ctas, kThreads, C::kSmemBytes, st>>>(maps, p, starts);
     TLIN_CUDA_CHECK(cudaGetLastError());
     count_launch();
     return TLIN_OK;
@@ -784,10 +820,14 @@ int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long
 int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float* lse,
                   int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& plan,
                   float* ws, long long kv_rows_alloc, cudaStream_t st) {
-    if (plan.tile_m != kTileM || plan.tile_n != kTileN) return TLIN_ERR_UNSUPPORTED;
+    if (plan.tile_m != (d > 128 ? kQTile : kTileM) || plan.tile_n != kTileN) return TLIN_ERR_UNSUPPORTED;
     if ((long long)B * H * W > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
-    if (d == 128) return launch_d<128>(q, k, v, out, lse, B, H, N, W, causal, plan, ws, kv_rows_alloc, st);
-    if (d == 64) return launch_d<64>(q, k, v, out, lse, B, H, N, W, causal, plan, ws, kv_rows_alloc, st);
+    if (d == 128) return launch_d<128, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+    if (d == 64) return launch_d<64, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+    if (d % 8 != 0) return TLIN_ERR_UNSUPPORTED;
+    if (d < 64) return launch_d<64, kAnyHead>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+    if (d < 128) return launch_d<128, kAnyHead>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+    if (d <= 256) return launch_d<256, kAnyHead>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
     return TLIN_ERR_UNSUPPORTED;
 }
 

@@ -39,7 +39,7 @@ void tlin::fwd_group_starts(const tlin_fwd_plan& plan, GroupStarts* starts) {
     thread_local std::vector<long long> prefix;
     prefix.assign((size_t)plan.q_tiles + 1, 0);
     for (int qt = 0; qt < plan.q_tiles; ++qt)
-        prefix[qt + 1] = prefix[qt] + fwd_problem_cost(plan.n_keys, plan.n_queries, plan.key_tiles, qt);
+        prefix[qt + 1] = prefix[qt] + fwd_problem_cost(plan.n_keys, plan.n_queries, plan.key_tiles, qt, plan.tile_m);
     const long long q = plan.q_tiles, n_bh = U / q, per_bh = prefix[q], total = per_bh * n_bh;
     long long biggest = 0;
     for (int qt = 0; qt < q; ++qt) biggest = std::max(biggest, prefix[qt + 1] - prefix[qt]);
@@ -177,12 +177,19 @@ extern "C" int64_t tlin_plan_group_start(const tlin_fwd_plan* plan, int g) {
 
 extern "C" int tlin_plan_forward(int B, int H, int N, int W, int d, int causal_window, int is_f32,
                                  int num_sms, tlin_fwd_plan* plan) {
+    return tlin::plan_forward(B, H, N, W, d, causal_window, is_f32, num_sms, false, plan);
+}
+
+// whole_only: schedule 1 whatever it costs (a tensor-path call whose caller has registered no workspace)
+int tlin::plan_forward(int B, int H, int N, int W, int d, int causal_window, int is_f32, int num_sms, bool whole_only,
+                       tlin_fwd_plan* plan) {
     if (!plan) return TLIN_ERR_INVALID_ARG;
     if (B <= 0 || H <= 0 || N <= 0 || W <= 0 || d <= 0) return TLIN_ERR_INVALID_ARG;
     if (causal_window && N < W) return TLIN_ERR_INVALID_ARG;
     if (num_sms <= 0) num_sms = kDefaultSMs;
     const int impl = forward_impl();
-    const bool tc_shape = !is_f32 && (d == 64 || d == 128);
+    // the tensor kernels count rows in 32 bits; head sizes other than 64 and 128 fall back to the CUDA cores beyond that
+    const bool tc_shape = !is_f32 && (d == 64 || d == 128 || (d % 8 == 0 && d <= 256 && (int64_t)B * H * W <= INT32_MAX));
     if (impl == 2 && !tc_shape) return TLIN_ERR_UNSUPPORTED;
     if (is_f32 ? (d % 4 != 0 || d > 256) : (d % 8 != 0 || d > 256)) return TLIN_ERR_UNSUPPORTED;
     const bool tc = tc_shape && impl != 1;
@@ -207,7 +214,7 @@ extern "C" int tlin_plan_forward(int B, int H, int N, int W, int d, int causal_w
         return TLIN_OK;
     }
     if (num_sms > kMaxGroups) num_sms = kMaxGroups;   // size of the table of group starts handed to the kernels
-    p.tile_m = 256;            // two 128-row Q tiles per CTA
+    p.tile_m = d <= 128 ? 256 : 128;      // two 128-row Q tiles per CTA (one beyond d = 128: TMEM)
     p.tile_n = kTileN;
     p.q_tiles = (W + p.tile_m - 1) / p.tile_m;
     p.key_tiles = (N + p.tile_n - 1) / p.tile_n;
@@ -242,7 +249,7 @@ extern "C" int tlin_plan_forward(int B, int H, int N, int W, int d, int causal_w
             // V exceed L2 the tiles come from HBM at unrelated times: measured about 15 % slower per tile.
             int64_t per_bh = 0, biggest = 0;
             for (int qt = 0; qt < p.q_tiles; ++qt) {
-                const int64_t c = fwd_problem_cost(N, W, p.key_tiles, qt);
+                const int64_t c = fwd_problem_cost(N, W, p.key_tiles, qt, p.tile_m);
                 per_bh += c;
                 if (c > biggest) biggest = c;
             }
@@ -251,7 +258,7 @@ extern "C" int tlin_plan_forward(int B, int H, int N, int W, int d, int causal_w
             if (!kv_in_l2) cost1 += cost1 * 15 / 100;
             allow1 = true;
         }
-        wide = allow1 && cost1 < cost0;
+        wide = whole_only || (allow1 && cost1 < cost0);
     }
     if (wide) {
         p.schedule = 1;

@@ -51,13 +51,14 @@ inline cudaError_t allow_dynamic_smem(Kernel kernel, int bytes, bool (&done)[64]
 // indivisible problems dominate and equal counts do as well).
 constexpr int kMaxGroups = 192;        // groups never exceed the SM count (148 on B200); the planner clamps to this
 struct GroupStarts { long long u[kMaxGroups + 1]; };   // u[g] = first unit of group g, u[n_groups] = total_units
-inline long long fwd_problem_cost(int N, int W, int key_tiles, int qt) {
-    long long rows_end = (long long)(qt + 1) * 256;
+inline long long fwd_problem_cost(int N, int W, int key_tiles, int qt, int tile_m = 256) {
+    long long rows_end = (long long)(qt + 1) * tile_m;
     if (rows_end > W) rows_end = W;
     long long tiles = ((long long)N - W + rows_end + 127) / 128;
     if (tiles > key_tiles) tiles = key_tiles;
     return tiles + 3;
 }
+int plan_forward(int B, int H, int N, int W, int d, int causal_window, int is_f32, int num_sms, bool whole_only, tlin_fwd_plan* plan);
 // fills starts->u[0 .. plan.n_groups]; plan.n_groups <= kMaxGroups
 void fwd_group_starts(const tlin_fwd_plan& plan, GroupStarts* starts);
 

@@ -1,5 +1,6 @@
 """GPU parity of the forward entry points against the CPU oracle (element by element on the same
 seeded inputs; sampled rows at the full benchmark sizes).  Everything goes through the C-ABI."""
+import ctypes
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -559,3 +560,36 @@ def test_chunk_scheduled_forward_with_many_units_is_one_launch():
                                               (1, 36, 1100, 64, 128, 1), (1, 1, 520, 520, 256, 1)])
 def test_fp32_tilings_and_key_sharing_clusters(B, H, N, W, d, causal):
     full_compare(synth.Workload("f32 tiles", B, H, d, N, W, seed=40 + N + d, causal_window=causal), 0, kind="f32")
+
+
+# bf16 head sizes other than 64 and 128 on the tensor cores: the sizes at both ends of each class (8..56, 72..120, 136..256), ragged
+# rows and keys, both schedules, few and many partial results per row, a key prefix of a longer cache
+ANY_HEAD = [(1, 2, 130, 129, 8, 1), (2, 1, 515, 130, 56, 0), (1, 3, 1000, 77, 40, 1), (1, 1, 129, 1, 72, 1), (2, 9, 700, 517, 96, 0),
+            (1, 2, 4000, 300, 120, 1), (1, 1, 128, 128, 136, 1), (1, 2, 3000, 257, 160, 0), (1, 1, 5000, 100, 256, 1), (3, 50, 200, 130, 248, 1),
+            (1, 1, 30000, 64, 80, 1), (2, 40, 600, 600, 112, 1)]
+
+
+@pytest.mark.parametrize("B,H,N,W,d,causal", ANY_HEAD)
+def test_other_head_sizes_on_the_tensor_cores(B, H, N, W, d, causal):
+    wl = synth.Workload("any head", B, H, d, N, W, seed=500 + N + d, causal_window=causal)
+    guarded_compare(wl, 2)
+    q, k, v = synth.forward_inputs(wl, device=DEV)
+    ref, ref_lse = oracle.attn_forward(q.cpu(), k.cpu(), v.cpu(), causal)
+    # Rounding the result to bf16 is an error uniform over the spacing 2^-7 of its binade, 2^-7 / sqrt(12) rms against a mantissa of
+    # 1.35 to 1.55 rms: 1.45e-3 to 1.67e-3.  P keeps 16 mantissa bits (2^-17) and the fp32 sums more, so nothing else of that size may
+    # come in (a P of 8 bits would give 2.3e-3 here).
+    out, _ = tl.tlin_attn_forward(q, k, v, causal_window=causal)
+    e = parity.errors(out.float().cpu().numpy(), ref)
+    assert e["rel_l2"] <= 2.0 ** -9, e
+    # the first N rows of a longer cache, and no registered workspace (keys are then not split)
+    pad = torch.full((B, H, 37, d), float("nan"), dtype=torch.bfloat16, device=DEV)
+    kc, vc = torch.cat([k, pad], 2), torch.cat([v, pad], 2)
+    got = torch.empty_like(q)
+    lse = torch.empty(B, H, W, dtype=torch.float32, device=DEV)
+    tl.set_workspace(None)
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    assert tl.lib().tlin_attn_forward_cache(ptr(q), ptr(kc), ptr(vc), ptr(got), ptr(lse), B, H, N + 37, N, W, d, causal, stream) == tl.TLIN_OK
+    torch.cuda.synchronize()
+    assert tl.tlin_get_status() == 0
+    parity.check(got.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", "cache, no workspace")
