@@ -124,20 +124,38 @@ def _check(rc: int, where: str):
         raise TlinError(rc, where)
 
 
+# The helpers below run several times per call, and a small call is over on the device in about ten microseconds: plain integers
+# instead of ctypes objects, the raw stream handle instead of a Stream object, one test for the case in which all is well.
+_current_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return _current_raw_stream(_current_device()) if stream is None else stream.cuda_stream
 
 
 def _dev(t, dtype, shape, name):
+    if t.is_cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous():
+        return
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
-        raise ValueError(f"{name} must be contiguous {dtype} of shape {tuple(shape)}, got {t.dtype} {tuple(t.shape)}")
+    raise ValueError(f"{name} must be contiguous {dtype} of shape {tuple(shape)}, got {t.dtype} {tuple(t.shape)}")
+
+
+def _out_and_lse(q, out, lse, lse_shape):
+    """The result tensors: allocated here, or the caller's after a check."""
+    if out is None:
+        out = torch.empty_like(q)
+    else:
+        _dev(out, q.dtype, q.shape, "out")
+    if lse is None:
+        lse = torch.empty(lse_shape, dtype=torch.float32, device=q.device)
+    else:
+        _dev(lse, torch.float32, lse_shape, "lse")
+    return out, lse
 
 
 # ------------------------------------------------------------------ workspace
@@ -169,6 +187,8 @@ def ensure_workspace(nbytes: int, device="cuda"):
     """Grows the registered workspace to at least ``nbytes`` (allocation happens here, in torch)."""
     global _workspace_tensor
     cur = 0 if _workspace_tensor is None else _workspace_tensor.numel()
+    if cur > 0 and nbytes <= cur and _workspace_tensor.device == device:
+        return _workspace_tensor
     if nbytes > cur or (_workspace_tensor is not None and str(_workspace_tensor.device) != str(torch.device(device)) and torch.device(device).index is not None):
         set_workspace(torch.empty(max(nbytes, 1 << 20), dtype=torch.uint8, device=device))
     return _workspace_tensor
@@ -182,12 +202,7 @@ def tlin_attn_forward(q, k, v, out=None, lse=None, causal_window=1, stream=None)
     _dev(q, torch.bfloat16, (B, H, W, d), "q")
     _dev(k, torch.bfloat16, (B, H, N, d), "k")
     _dev(v, torch.bfloat16, (B, H, N, d), "v")
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((B, H, W), dtype=torch.float32, device=q.device)
-    _dev(out, torch.bfloat16, (B, H, W, d), "out")
-    _dev(lse, torch.float32, (B, H, W), "lse")
+    out, lse = _out_and_lse(q, out, lse, (B, H, W))
     ensure_workspace(workspace_bytes_forward(B, H, N, W, d, causal_window), q.device)
     _check(lib().tlin_attn_forward(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, N, W, d,
                                    int(causal_window), _stream(stream)), "tlin_attn_forward")
@@ -206,12 +221,7 @@ def tlin_attn_forward_prefixes(q, k, v, n_keys, out=None, lse=None, causal_windo
     _dev(q, torch.bfloat16, (C, B, H, W, d), "q")
     _dev(k, torch.bfloat16, (B, H, L, d), "k")
     _dev(v, torch.bfloat16, (B, H, L, d), "v")
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((C, B, H, W), dtype=torch.float32, device=q.device)
-    _dev(out, torch.bfloat16, (C, B, H, W, d), "out")
-    _dev(lse, torch.float32, (C, B, H, W), "lse")
+    out, lse = _out_and_lse(q, out, lse, (C, B, H, W))
     arr = (ctypes.c_int32 * C)(*n_keys)
     ensure_workspace(int(lib().tlin_workspace_bytes_forward_prefixes(B, H, W, d, C, arr, int(causal_window))), q.device)
     _check(lib().tlin_attn_forward_prefixes(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, L, W, d, C, arr,
@@ -226,12 +236,7 @@ def tlin_attn_forward_cache(q, k_cache, v_cache, n_keys, out=None, lse=None, cau
     _dev(q, torch.bfloat16, (B, H, W, d), "q")
     _dev(k_cache, torch.bfloat16, (B, H, Ncap, d), "k_cache")
     _dev(v_cache, torch.bfloat16, (B, H, Ncap, d), "v_cache")
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((B, H, W), dtype=torch.float32, device=q.device)
-    _dev(out, torch.bfloat16, (B, H, W, d), "out")
-    _dev(lse, torch.float32, (B, H, W), "lse")
+    out, lse = _out_and_lse(q, out, lse, (B, H, W))
     ensure_workspace(workspace_bytes_forward(B, H, int(n_keys), W, d, causal_window), q.device)
     _check(lib().tlin_attn_forward_cache(_ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(out), _ptr(lse), B, H, Ncap, int(n_keys),
                                          W, d, int(causal_window), _stream(stream)), "tlin_attn_forward_cache")
@@ -243,21 +248,23 @@ def make_problem_table(problems):
     k, v [B,H,rows,d] with rows >= n_keys (n_keys None: all rows)."""
     arr = (Problem * len(problems))()
     keep = []
+    bf16 = torch.bfloat16
     for i, (q, k, v, out, lse, n_keys, causal) in enumerate(problems):
-        d = q.shape[-1]
-        W = q.shape[-2]
+        q_shape, k_shape = q.shape, k.shape
+        W, d = q_shape[-2], q_shape[-1]
         bh = q.numel() // (W * d)
-        rows = k.shape[-2]
+        rows = k_shape[-2]
         n_keys = rows if n_keys is None else int(n_keys)
-        for t, name in ((q, "q"), (k, "k"), (v, "v"), (out, "out")):
-            if not t.is_cuda or t.dtype != torch.bfloat16 or not t.is_contiguous():
+        for t in (q, k, v, out):
+            if t.dtype is not bf16 or not t.is_contiguous() or not t.is_cuda:
+                name = next(n for n, x in (("q", q), ("k", k), ("v", v), ("out", out)) if x is t)
                 raise ValueError(f"problem {i}: {name} must be a contiguous bf16 CUDA tensor")
-        if k.numel() != bh * rows * d or v.shape != k.shape or out.shape != q.shape:
+        if k.numel() != bh * rows * d or v.shape != k_shape or out.shape != q_shape:
             raise ValueError(f"problem {i}: shape mismatch")
-        if lse is not None and (lse.dtype != torch.float32 or lse.numel() != bh * W or not lse.is_contiguous()):
+        if lse is not None and (lse.dtype is not torch.float32 or lse.numel() != bh * W or not lse.is_contiguous()):
             raise ValueError(f"problem {i}: lse must be contiguous fp32 of {bh * W} elements")
-        arr[i] = Problem(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
-                         bh, n_keys, rows if rows != n_keys else 0, W, int(causal), 0)
+        arr[i] = (q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
+                  bh, n_keys, rows if rows != n_keys else 0, W, int(causal), 0)
         keep.append((q, k, v, out, lse))
     return arr, keep
 
@@ -285,12 +292,7 @@ def tlin_attn_forward_f32(q, k, v, out=None, lse=None, causal_window=1, stream=N
     _dev(q, torch.float32, (B, H, W, d), "q")
     _dev(k, torch.float32, (B, H, N, d), "k")
     _dev(v, torch.float32, (B, H, N, d), "v")
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((B, H, W), dtype=torch.float32, device=q.device)
-    _dev(out, torch.float32, (B, H, W, d), "out")
-    _dev(lse, torch.float32, (B, H, W), "lse")
+    out, lse = _out_and_lse(q, out, lse, (B, H, W))
     _check(lib().tlin_attn_forward_f32(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, N, W, d,
                                        int(causal_window), _stream(stream)), "tlin_attn_forward_f32")
     return out, lse

@@ -76,8 +76,13 @@ Workspace workspace() {
 }
 void reset_launches() { t_launches = 0; }
 int* status_word() {
-    int* p = nullptr;
+    static std::atomic<int*> at[kMaxDevices];             // the address is fixed per device: asked for once
+    const int dev = current_device_slot();
+    if (dev < 0) return nullptr;
+    int* p = at[dev].load(std::memory_order_acquire);
+    if (p) return p;
     if (cudaGetSymbolAddress((void**)&p, g_status_word) != cudaSuccess) return nullptr;
+    at[dev].store(p, std::memory_order_release);
     return p;
 }
 void count_launch(int n) { t_launches += n; }
@@ -105,8 +110,10 @@ static int forward_common(const void* q, const void* k, const void* v, void* out
     if (rc != TLIN_OK) return rc;
     rc = device_info(&sms);
     if (rc != TLIN_OK) return rc;
-    rc = tlin_plan_forward(B, H, N, W, d, causal_window, is_f32, sms, &plan);
-    if (rc != TLIN_OK) return rc;
+    if (sms != kDefaultSMs) {
+        rc = tlin_plan_forward(B, H, N, W, d, causal_window, is_f32, sms, &plan);
+        if (rc != TLIN_OK) return rc;
+    }
     if (log_plans()) log_fwd_plan(is_f32 ? "forward (fp32)" : "forward", B, H, N, W, d, causal_window, plan);
     if (is_f32)
         return launch_fwd_simt_f32((const float*)q, (const float*)k, (const float*)v, (float*)out, lse, B, H, N, W, d, causal_window,
