@@ -22,9 +22,11 @@ constexpr int kUnroll = 4;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
+// Not the non-coherent form, and no pointer of these kernels is __restrict__: a kernel may be resident while the one before it in the
+// stream still writes (launch_overlapped), and nothing may be read ahead of after_previous().
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
     return r;
 }
@@ -68,8 +70,8 @@ __device__ __forceinline__ void combine(float& m, float& l, float (&a)[8], float
 // appended in this launch, or -1) is taken from k_new / v_new instead of the cache.  Returns, in threads 0..D-1, column
 // c = threadIdx.x of the un-normalised result `a`, the row sum `ll` and the running maximum `mm` (log2 units).
 template <int D>
-__device__ __forceinline__ void attend_key_range(const uint4* __restrict__ q_row, const uint4* __restrict__ kn, const uint4* __restrict__ vn,
-                                                 const uint4* __restrict__ kc, const uint4* __restrict__ vc, int j0, int j1, int pos,
+__device__ __forceinline__ void attend_key_range(const uint4* q_row, const uint4* kn, const uint4* vn,
+                                                 const uint4* kc, const uint4* vc, int j0, int j1, int pos,
                                                  float scale_log2e, float& a, float& ll, float& mm) {
     constexpr int LPR = D / 8;           // lanes (16-byte chunks) per row
     constexpr int RPW = 32 / LPR;        // rows per warp-load
@@ -166,14 +168,16 @@ __device__ __forceinline__ void attend_key_range(const uint4* __restrict__ q_row
 
 template <int D>
 __global__ void __launch_bounds__(kWarps * 32, kDecodeCtasPerSM)
-decode_splitk_kernel(const uint4* __restrict__ q_new, const uint4* __restrict__ k_new, const uint4* __restrict__ v_new,
-                     uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
-                     float* __restrict__ part_o, float* __restrict__ part_lse,
-                     int Ncap, int pos_all, const int* __restrict__ pos_per_seq, int H, int* __restrict__ status,
+decode_splitk_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_new,
+                     uint4* k_cache, uint4* v_cache,
+                     float* part_o, float* part_lse,
+                     int Ncap, int pos_all, const int* pos_per_seq, int H, int* status,
                      int splits, int kps, float scale_log2e) {
     constexpr int LPR = D / 8;           // lanes (16-byte chunks) per row
     const int bh = blockIdx.x / splits, sp = blockIdx.x - bh * splits;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    after_previous();
+    let_next_start();
     // one position for the whole batch, or one per sequence read from device memory (ragged batch)
     int pos = pos_all;
     if (pos_per_seq != nullptr) {
@@ -229,6 +233,8 @@ template <int D>
 __global__ void __launch_bounds__(kWarps * 32, kDecodeCtasPerSM)
 decode_table_kernel(const __grid_constant__ DecodeTable tbl, float scale_log2e) {
     constexpr int LPR = D / 8;
+    after_previous();
+    let_next_start();
     int pi = 0;
     while (pi + 1 < tbl.n && (int)blockIdx.x >= tbl.prob[pi + 1].cta0) ++pi;
     const DecodeProblemDev& pr = tbl.prob[pi];
@@ -257,9 +263,11 @@ decode_table_kernel(const __grid_constant__ DecodeTable tbl, float scale_log2e) 
 // One CTA per (b,h): out = sum_s w_s o_s / sum_s w_s with w_s = exp(lse_s - max lse).
 template <int D>
 __global__ void __launch_bounds__(D)
-decode_merge_kernel(const float* __restrict__ part_o, const float* __restrict__ part_lse,
-                    __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int splits) {
+decode_merge_kernel(const float* part_o, const float* part_lse,
+                    __nv_bfloat16* out, float* lse, int splits) {
     const int bh = blockIdx.x, c = threadIdx.x;
+    after_previous();
+    let_next_start();
     const float* pl = part_lse + (int64_t)bh * splits;
     float mm = -CUDART_INF_F;
     for (int s = 0; s < splits; ++s) mm = fmaxf(mm, pl[s]);
@@ -351,10 +359,10 @@ __device__ __forceinline__ uint4 quantise16(const uint4& lo8, const uint4& hi8, 
 
 template <int D>
 __global__ void __launch_bounds__(kWarps * 32, kDecodeCtasPerSM)
-decode_fp8_splitk_kernel(const uint4* __restrict__ q_new, const uint4* __restrict__ k_new, const uint4* __restrict__ v_new,
-                         uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
-                         const float* __restrict__ k_scale, const float* __restrict__ v_scale,
-                         float* __restrict__ part_o, float* __restrict__ part_lse,
+decode_fp8_splitk_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_new,
+                         uint4* k_cache, uint4* v_cache,
+                         const float* k_scale, const float* v_scale,
+                         float* part_o, float* part_lse,
                          int Ncap, int pos, int splits, int kps, float scale_log2e) {
     constexpr int LPR = D / 16;          // lanes (16-byte chunks of codes) per row
     constexpr int RPW = 32 / LPR;        // rows per warp-load
@@ -364,6 +372,8 @@ decode_fp8_splitk_kernel(const uint4* __restrict__ q_new, const uint4* __restric
     const int sub = lane % LPR, rsel = lane / LPR;
     const int L = pos + 1;
     const int j0 = sp * kps, j1 = min(L, j0 + kps);
+    after_previous();
+    let_next_start();
     const float ks = k_scale[bh], vs = v_scale[bh];
 
     const uint4* kc = k_cache + (int64_t)bh * Ncap * LPR;
@@ -487,12 +497,10 @@ int launch_d(const void* q_new, const void* k_new, const void* v_new, void* k_ca
     float* part_o = ws;
     float* part_lse = ws + bh * kDecodeMaxSplits * D;
     const float scale_log2e = kLog2e / sqrtf((float)D);
-    decode_splitk_kernel<D><<<plan.n_ctas, kWarps * 32, 0, st>>>(
+    TLIN_CUDA_CHECK(launch_overlapped(decode_splitk_kernel<D>, plan.n_ctas, kWarps * 32, 0, st,
         (const uint4*)q_new, (const uint4*)k_new, (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache,
-        part_o, part_lse, Ncap, pos, pos_per_seq, H, status_word(), plan.splits, plan.keys_per_split, scale_log2e);
-    TLIN_CUDA_CHECK(cudaGetLastError());
-    decode_merge_kernel<D><<<(unsigned)bh, D, 0, st>>>(part_o, part_lse, (__nv_bfloat16*)out, lse, plan.splits);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+        part_o, part_lse, Ncap, pos, pos_per_seq, H, status_word(), plan.splits, plan.keys_per_split, scale_log2e));
+    TLIN_CUDA_CHECK(launch_overlapped(decode_merge_kernel<D>, (unsigned)bh, D, 0, st, part_o, part_lse, (__nv_bfloat16*)out, lse, plan.splits));
     count_launch(2);
     return TLIN_OK;
 }
@@ -505,12 +513,10 @@ int launch_fp8_d(const void* q_new, const void* k_new, const void* v_new, void* 
     float* part_o = ws;
     float* part_lse = ws + bh * kDecodeMaxSplits * D;
     const float scale_log2e = kLog2e / sqrtf((float)D);
-    decode_fp8_splitk_kernel<D><<<plan.n_ctas, kWarps * 32, 0, st>>>(
+    TLIN_CUDA_CHECK(launch_overlapped(decode_fp8_splitk_kernel<D>, plan.n_ctas, kWarps * 32, 0, st,
         (const uint4*)q_new, (const uint4*)k_new, (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, k_scale, v_scale,
-        part_o, part_lse, Ncap, pos, plan.splits, plan.keys_per_split, scale_log2e);
-    TLIN_CUDA_CHECK(cudaGetLastError());
-    decode_merge_kernel<D><<<(unsigned)bh, D, 0, st>>>(part_o, part_lse, (__nv_bfloat16*)out, lse, plan.splits);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+        part_o, part_lse, Ncap, pos, plan.splits, plan.keys_per_split, scale_log2e));
+    TLIN_CUDA_CHECK(launch_overlapped(decode_merge_kernel<D>, (unsigned)bh, D, 0, st, part_o, part_lse, (__nv_bfloat16*)out, lse, plan.splits));
     count_launch(2);
     return TLIN_OK;
 }
@@ -531,8 +537,7 @@ int launch_table_d(const tlin_decode_problem* problems, int n, cudaStream_t st) 
         ctas += pb.BH;
     }
     if (ctas > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
-    decode_table_kernel<D><<<(unsigned)ctas, kWarps * 32, 0, st>>>(tbl, kLog2e / sqrtf((float)D));
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(decode_table_kernel<D>, (unsigned)ctas, kWarps * 32, 0, st, tbl, kLog2e / sqrtf((float)D)));
     count_launch();
     return TLIN_OK;
 }

@@ -211,6 +211,8 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
         }
     }
     tc_fence_before();
+    after_previous();
+    let_next_start();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
@@ -652,6 +654,8 @@ fwd_merge_kernel(const Params p) {
     const int quarter = blockIdx.x % blocks_per_tile;
     const int tile_id = blockIdx.x / blocks_per_tile;     // bh * q_tiles + qt
     const int bh = tile_id / p.q_tiles, qt = tile_id - bh * p.q_tiles;
+    after_previous();
+    let_next_start();
     __shared__ const float* part_base[kMaxParts];
     __shared__ int n_parts_s, g_lo_s;
     if (threadIdx.x == 0) {
@@ -757,12 +761,10 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
     if (plan.n_groups > kMaxGroups) return TLIN_ERR_UNSUPPORTED;
     GroupStarts starts;
     fwd_group_starts(plan, &starts);
-    fwd_tc_kernel<D, kForm><<<plan.n_ctas, kThreads, C::kSmemBytes, st>>>(maps, p, starts);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(fwd_tc_kernel<D, kForm>, plan.n_ctas, kThreads, C::kSmemBytes, st, maps, p, starts));
     count_launch();
     if (plan.uses_workspace) {
-        fwd_merge_kernel<D, kForm == kAnyHead><<<(unsigned)(bh * plan.q_tiles * (C::kRows / kMergeRows)), 256, 0, st>>>(p);
-        TLIN_CUDA_CHECK(cudaGetLastError());
+        TLIN_CUDA_CHECK(launch_overlapped(fwd_merge_kernel<D, kForm == kAnyHead>, (unsigned)(bh * plan.q_tiles * (C::kRows / kMergeRows)), 256, 0, st, p));
         count_launch();
     }
     return TLIN_OK;
@@ -802,8 +804,7 @@ int launch_batched_d(const tlin_problem* problems, int n, const long long* start
     for (int g = 0; g <= n_ctas; ++g) starts.u[g] = starts_in[g];
     static bool smem_allowed[64] = {};
     TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_tc_kernel<D, kTable>, C::kSmemBytes, smem_allowed));
-    fwd_tc_kernel<D, kTable><<<n_ctas, kThreads, C::kSmemBytes, st>>>(maps, p, starts);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(fwd_tc_kernel<D, kTable>, n_ctas, kThreads, C::kSmemBytes, st, maps, p, starts));
     count_launch();
     return TLIN_OK;
 }

@@ -104,6 +104,30 @@ __host__ __device__ inline long long bwd_first_unit_of_share(int N, int W, int c
 constexpr int kMaxBatch = 24;          // problems per launch of the batched kernel (its table travels as a launch parameter)
 void balanced_run_starts(const long long* prefix, long long units, int n_ctas, long long* starts);
 
+// Launches of one call, and of successive calls, overlap their starts: a kernel launched here may begin while the kernel before it
+// in the stream is still finishing (programmatic dependent launch), sets up what needs no memory, and waits in after_previous()
+// until that kernel has completed and its writes are visible.  Every kernel launched this way calls after_previous() in all
+// threads before it touches global memory, which also makes completion transitive along the stream.  let_next_start() allows
+// the kernel behind it to be brought in.
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+template <class... Params, class... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
+}
+
 #define TLIN_CUDA_CHECK(expr)                                                              \
     do {                                                                                   \
         cudaError_t e__ = (expr);                                                          \
