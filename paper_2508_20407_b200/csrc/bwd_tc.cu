@@ -20,11 +20,9 @@
 //   the same TMEM columns -> dS (bf16, in place) -> dQ += dS K with K read MN-major.  The work is scheduled like the
 //   forward (groups that split the key range write fp32 partial dQ to the workspace; a small kernel adds them).
 //
-// bwd_fused_tc_kernel  (d = 128, on request)  The dK/dV kernel with a third accumulating product per chain step,
-//   dQ^T_x = K^T dS^T_x (K read MN-major, dS^T_x also written to shared memory as the B operand) into the chain's dead
-//   dP^T_x columns, which the chain's threads read back and add to an fp32 dQ buffer with reductions in L2; a small kernel
-//   scales and rounds it.  Five matrix products instead of seven, but 32 KB of reductions per chain step, and an SM gets
-//   about 25 bytes per clock of those: measured within +-10 % of the two kernels.
+// bwd_fused_tc_kernel  (d = 128, chosen for small and middle-sized calls)  The dK/dV kernel with a third accumulating product,
+//   dQ^T = K^T dS^T, which a warpgroup of its own adds to an fp32 dQ buffer with reductions in L2; a small kernel scales and
+//   rounds it.  Five matrix products instead of seven.
 //
 // A preparation kernel writes lse*log2(e) and delta per query row, padded to a multiple of 128 rows per (b,h) with
 // +inf / 0: a padded row then gives p = 0 without any test.
@@ -34,6 +32,7 @@
 #include "sm100_ptx.cuh"
 #include "tc_common.cuh"
 #include <math_constants.h>
+#include <type_traits>
 
 namespace tlin {
 namespace {
@@ -72,8 +71,10 @@ __host__ __device__ constexpr int prep_rows_per_block() { return 8 * (32 / (D / 
 
 template <int D>
 __global__ void __launch_bounds__(256)
-bwd_prep_kernel(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ dout, const float* __restrict__ lse,
-                float* __restrict__ lse2, float* __restrict__ delta, int W, int Wpad, long long rows_padded) {
+bwd_prep_kernel(const __nv_bfloat16* out, const __nv_bfloat16* dout, const float* lse, float* lse2, float* delta, float* dq32,
+                int W, int Wpad, long long rows_padded) {
+    after_previous();
+    let_next_start();
     constexpr int LPR = D / 8;              // lanes per row
     constexpr int RPP = 32 / LPR;           // rows per pass of a warp
     const int lane = threadIdx.x & 31, sub = lane / LPR, l = lane % LPR;
@@ -86,6 +87,10 @@ bwd_prep_kernel(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __re
         const long long bh = prow / Wpad;
         const int i = (int)(prow - bh * Wpad);
         row[ps] = (prow < rows_padded && i < W) ? bh * W + i : -1;
+        if (dq32 != nullptr && prow < rows_padded) {            // the fp32 dQ sums of the one-kernel arrangement start at zero
+            float4* z = reinterpret_cast<float4*>(dq32 + prow * D) + l;
+            z[0] = z[LPR] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
         a[ps] = b[ps] = make_uint4(0u, 0u, 0u, 0u);
         if (row[ps] >= 0) {
             a[ps] = *reinterpret_cast<const uint4*>(out + row[ps] * D + l * 8);
@@ -462,32 +467,65 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 }
 
 // ------------------------------------------------------------------------------------------ dK / dV / dQ in one kernel
-// The dK/dV kernel with a third accumulating product per chain step: dQ^T_x = K^T dS^T_x goes into the chain's dead dP^T_x
-// columns (dS^T_x now sits beside P^T_x over S^T_x), is read back by the chain's threads and added to an fp32 dQ buffer in the
-// workspace with reductions in L2.  Scores are computed once: five matrix products per (query, key) pair instead of seven.
-// Columns of a chain: [P^T q0-31 | dS^T q0-31 | P^T q32-63 | dS^T q32-63] (16 each, written over S^T_x half by half) and dQ^T_x (64).
+// A CTA owns one 128-key tile at a time and walks the 128-row query tiles that may see it; five products per step, all 128 wide:
+//   S^T = K Q^T, dP^T = V dout^T (TMEM lane = key, column = query), dV += P^T dout, dK += dS^T Q (P^T, dS^T bf16 in TMEM, written
+//   over S^T and dP^T), dQ^T = K^T dS^T (K read MN-major; dS^T once more in shared memory; over dP^T, whose dS^T dK has consumed).
+// TMEM is full with S^T, dP^T, dK and dV, so a step's products follow one another; what keeps the tensor pipe busy is the order:
+//   dK(j), dQ(j) | dP(j+1) once dQ(j) has been taken out of TMEM | dV(j+1), S(j+2) once P(j+1) is there
+// The exponentials of step j+1 run while dK(j) and dQ(j) do, dS(j+1) while dV(j+1) and S(j+2) do.
+// Three warpgroups work on a step: two take 64 queries each (thread = key row) through P and dS, the third takes dQ^T into
+// registers (thread = column of dQ) and adds it to the fp32 dQ in the workspace, 128 consecutive bytes per reduction, while the
+// others go on.  An SM has about 25 bytes of reductions per clock accepted, 2600 clocks for a step's 64 KB: with the reductions in
+// the threads that also form P and dS, and score products 64 queries wide, the training chunk (B4 H32 N8192 W1024) took 1543 us at
+// full clock and 1759 us under the power cap, now 1405 and 1601; B1 H32 N8192 W1024 449 -> 399 us, B2 H16 N4096 W512 132 -> 116 us,
+// B1 H4 N700 W300 28 -> 18 us (two launches fewer to wait for).
 template <int D>
-__global__ void __launch_bounds__(ACfg<D>::kThreads, 1)
-bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do, const BwdParams p) {
-    using C = ACfg<D>;
+struct FCfg {
     static_assert(D == 128, "the transposed dQ accumulator needs M = d = 128");
+    static constexpr int kTileBytes = kQTile * D * 2;          // one 128-row tile (K, V, Q or dout)
+    static constexpr int kBoxes = D / 64;
+    static constexpr int kOffK = 0, kOffV = kTileBytes;
+    static constexpr int kOffQ = 2 * kTileBytes;               // 2 slots
+    static constexpr int kOffDO = 4 * kTileBytes;              // 2 slots
+    static constexpr int kOffStage = 6 * kTileBytes;           // dS^T tile: two blocks of 128 keys x 64 queries; dK / dV rows on their way out
+    static constexpr int kOffStats = 7 * kTileBytes;           // 2 slots: lse2 of 128 rows, delta of 128 rows
+    static constexpr int kOffBars = kOffStats + 2 * 1024;
+    static constexpr int kNumBars = 20;
+    static constexpr int kSmemBytes = kOffBars + kNumBars * 8 + 16;
+    static constexpr uint32_t kColDK = 0, kColDV = D, kColS = 2 * D, kColDP = 2 * D + 128;
+    static constexpr int kThreads = 32 * 16;
+    static constexpr int kDqWarp = 8, kProducer = 12, kMma = 13, kKv = 14;      // warps 0 to 7: P and dS
+    // setmaxnreg moves registers between warpgroups; the CTA starts with 128 per thread, and an increase beyond what the others
+    // released would wait for ever
+    static constexpr int kComputeRegs = 144, kDqRegs = 152, kOtherRegs = 64;
+    static_assert(256 * kComputeRegs + 128 * kDqRegs + 128 * kOtherRegs <= kThreads * 128, "register budget of the CTA exceeded");
+};
+
+template <int D>
+__global__ void __launch_bounds__(FCfg<D>::kThreads, 1)
+bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do, const BwdParams p) {
+    using C = FCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* sKV = smem + C::kOffKV;          // K, V
-    uint8_t* sRing = smem + C::kOffRing;      // [kSlots][Q 64 rows | dout 64 rows]
-    float* sStats = reinterpret_cast<float*>(smem + C::kOffStats);   // [kSlots][lse2 64 | delta 64]
+    float* sStats = reinterpret_cast<float*>(smem + C::kOffStats);   // [2][lse2 128 | delta 128]
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
-    uint64_t* kv_full = bars + 0;
-    uint64_t* kv_empty = bars + 1;
-    uint64_t* sdp_full = bars + 2;    // [2] S^T_x and dP^T_x of a step are in TMEM
-    uint64_t* pds_full = bars + 4;    // [2] the chain's threads have stored P^T_x and dS^T_x
-    uint64_t* acc_full = bars + 6;    // dK, dV of the key tile are complete
-    uint64_t* acc_empty = bars + 7;   // all threads have read them
-    uint64_t* slot_full = bars + 8;   // [kSlots]
-    uint64_t* slot_empty = slot_full + C::kSlots;
-    uint64_t* dqt_full = bars + C::kNumBars;        // [2] dQ^T_x of a chain step is in TMEM
-    uint64_t* dq_drained = dqt_full + 2;            // [2] the chain's threads hold it in registers: its columns are free
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars + 4);
+    uint64_t* q_full = bars + 0;      // [2] Q and the row statistics of a step
+    uint64_t* q_empty = bars + 2;     // [2]
+    uint64_t* do_full = bars + 4;     // [2]
+    uint64_t* do_empty = bars + 6;    // [2]
+    uint64_t* k_full = bars + 8;
+    uint64_t* k_empty = bars + 9;
+    uint64_t* v_full = bars + 10;
+    uint64_t* v_empty = bars + 11;
+    uint64_t* s_full = bars + 12;     // S^T of a step is in TMEM
+    uint64_t* p_full = bars + 13;     // P^T is written
+    uint64_t* dp_full = bars + 14;    // dP^T is in TMEM
+    uint64_t* ds_full = bars + 15;    // dS^T is written (TMEM and shared memory)
+    uint64_t* dq_full = bars + 16;    // dQ^T is in TMEM
+    uint64_t* dq_drained = bars + 17; // the dQ warpgroup holds it in registers
+    uint64_t* acc_full = bars + 18;   // dK, dV of the key tile are complete
+    uint64_t* acc_empty = bars + 19;  // all threads have read them
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -495,33 +533,23 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
     if (threadIdx.x == 0) {
         *abort_flag = base_ok ? 0 : 1;
-        mbar_init(kv_full, 1);
-        mbar_init(kv_empty, 1);
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&sdp_full[i], 1);
-            mbar_init(&pds_full[i], 128);
-            mbar_init(&dqt_full[i], 1);
-            mbar_init(&dq_drained[i], 128);
-        }
-        for (int i = 0; i < C::kSlots; ++i) {
-            mbar_init(&slot_full[i], 1);
-            mbar_init(&slot_empty[i], 1);
-        }
-        mbar_init(acc_full, 1);
-        mbar_init(acc_empty, 256);
+        for (int i = 0; i < C::kNumBars; ++i)
+            mbar_init(&bars[i], &bars[i] == p_full || &bars[i] == ds_full || &bars[i] == acc_empty ? 256 : &bars[i] == dq_drained ? 128 : 1);
         fence_mbar_init();
     }
-    if (warp == kMmaWarp) {
+    if (warp == C::kMma) {
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
-    if (warp == kProducerWarp && lane == 0) {
+    if (warp == C::kProducer && lane == 0) {
         prefetch_tensormap(&map_q);
         prefetch_tensormap(&map_k);
         prefetch_tensormap(&map_v);
         prefetch_tensormap(&map_do);
     }
     tc_fence_before();
+    after_previous();
+    let_next_start();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
@@ -533,44 +561,48 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     // turn spreads those evenly.
     const long long u_begin = blockIdx.x, u_end = p.total_units, u_step = gridDim.x;
 
-    if (warp == kProducerWarp) {
-        // ------------------------------------------------------------------ TMA producer: Q / dout / row statistics ring
-        // The ring runs ahead of the key tiles: the first chain steps of the next key tile are loaded while the
-        // current one is still being worked on.
+    if (warp >= C::kProducer) {
+    setmaxnreg_dec<C::kOtherRegs>();
+    if (warp == C::kProducer) {
+        // ------------------------------------------------------------------ TMA producer: Q, dout and row statistics of the steps
         if (lane == 0) {
             bool ok = base_ok;
-            uint32_t hh = 0;                // chain steps (64 queries each) issued
+            uint32_t nq = 0, ndo = 0;       // tiles armed
             for (long long u = u_begin; u < u_end && ok; u += u_step) {
                 const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
-                const int row_first = first_q_tile(p, t) * kQTile, row_end = p.q_tiles128 * kQTile;
-                for (int row = row_first; row < row_end && ok; row += 64, ++hh) {
-                    const uint32_t slot = hh % C::kSlots, round = hh / C::kSlots;
-                    ok = mbar_wait(&slot_empty[slot], (round & 1) ^ 1, abort_p);
+                for (int i = first_q_tile(p, t); i < p.q_tiles128; ++i) {
+                    const uint32_t slot = nq & 1, par = ((nq >> 1) & 1) ^ 1;
+                    const int row = i * kQTile;
+                    ok = mbar_wait(&q_empty[slot], par, abort_p);
                     if (!ok) break;
-                    uint8_t* dst = sRing + slot * C::kSlotBytes;
-                    mbar_arrive_expect_tx(&slot_full[slot], C::kSlotBytes + 512);
-                    for (int x = 0; x < C::kBoxes; ++x) {
-                        tma_load_3d(dst + x * (64 * 128), &map_q, &slot_full[slot], x * 64, row, bh);
-                        tma_load_3d(dst + C::kHalfBytes + x * (64 * 128), &map_do, &slot_full[slot], x * 64, row, bh);
-                    }
-                    bulk_load_1d(sStats + slot * 128, p.lse2 + (long long)bh * p.Wpad + row, 256, &slot_full[slot]);
-                    bulk_load_1d(sStats + slot * 128 + 64, p.delta + (long long)bh * p.Wpad + row, 256, &slot_full[slot]);
+                    mbar_arrive_expect_tx(&q_full[slot], C::kTileBytes + 1024);
+                    ++nq;
+                    for (int x = 0; x < C::kBoxes; ++x)
+                        tma_load_3d(smem + C::kOffQ + slot * C::kTileBytes + x * (kQTile * 128), &map_q, &q_full[slot], x * 64, row, bh);
+                    bulk_load_1d(sStats + slot * 256, p.lse2 + (long long)bh * p.Wpad + row, 512, &q_full[slot]);
+                    bulk_load_1d(sStats + slot * 256 + 128, p.delta + (long long)bh * p.Wpad + row, 512, &q_full[slot]);
+                    ok = mbar_wait(&do_empty[slot], par, abort_p);
+                    if (!ok) break;
+                    mbar_arrive_expect_tx(&do_full[slot], C::kTileBytes);
+                    ++ndo;
+                    for (int x = 0; x < C::kBoxes; ++x)
+                        tma_load_3d(smem + C::kOffDO + slot * C::kTileBytes + x * (kQTile * 128), &map_do, &do_full[slot], x * 64, row, bh);
                 }
             }
             if (!ok && base_ok) {
                 int dummy = 0;              // leave no copy in flight: the barriers armed last must complete (bounded)
-                for (uint32_t back = 1; back <= (uint32_t)C::kSlots && back <= hh; ++back) {
-                    const uint32_t id = hh - back;
-                    mbar_wait(&slot_full[id % C::kSlots], (id / C::kSlots) & 1, &dummy, 200000000LL);
+                for (uint32_t back = 1; back <= 2; ++back) {
+                    if (back <= nq) mbar_wait(&q_full[(nq - back) & 1], ((nq - back) >> 1) & 1, &dummy, 200000000LL);
+                    if (back <= ndo) mbar_wait(&do_full[(ndo - back) & 1], ((ndo - back) >> 1) & 1, &dummy, 200000000LL);
                 }
             }
         }
-    } else if (warp == kKvWarp) {
+    } else if (warp == C::kKv) {
         // ------------------------------------------------------------------ TMA producer: K, V of the key tiles
         if (lane == 0) {
             bool ok = base_ok;
-            uint32_t n = 0;
-            for (long long u = u_begin; u < u_end && ok; u += u_step, ++n) {
+            uint32_t nk = 0, nv = 0;        // tiles armed
+            for (long long u = u_begin; u < u_end && ok; u += u_step) {
                 const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
                 if (u + u_step < u_end) {   // K, V have one buffer: the next tile's rows come as far as L2 meanwhile
                     const int bh_n = (int)((u + u_step) / p.key_tiles), t_n = (int)(u + u_step - (long long)bh_n * p.key_tiles);
@@ -579,179 +611,204 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                         tma_prefetch_l2_3d(&map_v, x * 64, t_n * kTileN, bh_n);
                     }
                 }
-                ok = mbar_wait(kv_empty, (n & 1) ^ 1, abort_p);
+                ok = mbar_wait(v_empty, (nv & 1) ^ 1, abort_p);      // V is read for the last time before K is
                 if (!ok) break;
-                mbar_arrive_expect_tx(kv_full, 2 * C::kTileBytes);
-                for (int x = 0; x < C::kBoxes; ++x) {
-                    tma_load_3d(sKV + x * (kQTile * 128), &map_k, kv_full, x * 64, t * kTileN, bh);
-                    tma_load_3d(sKV + C::kTileBytes + x * (kQTile * 128), &map_v, kv_full, x * 64, t * kTileN, bh);
-                }
+                mbar_arrive_expect_tx(v_full, C::kTileBytes);
+                ++nv;
+                for (int x = 0; x < C::kBoxes; ++x) tma_load_3d(smem + C::kOffV + x * (kQTile * 128), &map_v, v_full, x * 64, t * kTileN, bh);
+                ok = mbar_wait(k_empty, (nk & 1) ^ 1, abort_p);
+                if (!ok) break;
+                mbar_arrive_expect_tx(k_full, C::kTileBytes);
+                ++nk;
+                for (int x = 0; x < C::kBoxes; ++x) tma_load_3d(smem + C::kOffK + x * (kQTile * 128), &map_k, k_full, x * 64, t * kTileN, bh);
             }
-            if (!ok && base_ok && n > 0) {
+            if (!ok && base_ok) {
                 int dummy = 0;
-                mbar_wait(kv_full, (n - 1) & 1, &dummy, 200000000LL);
+                if (nv > 0) mbar_wait(v_full, (nv - 1) & 1, &dummy, 200000000LL);
+                if (nk > 0) mbar_wait(k_full, (nk - 1) & 1, &dummy, 200000000LL);
             }
         }
-    } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------------ MMA issuer (all lanes walk, one issues)
-        const uint32_t idesc_st = make_idesc_bf16(kQTile, 64, 0, 0);         // S^T, dP^T of a chain: M = keys, N = 64 queries
+    } else if (warp == C::kMma) {
+        // ------------------------------------------------------------------ MMA issuer (all lanes walk, the lane elected once issues)
+        const uint32_t idesc_s = make_idesc_bf16(kQTile, kQTile, 0, 0);      // S^T, dP^T: M = keys, N = 128 queries
         const uint32_t idesc_acc = make_idesc_bf16(kQTile, D, 0, 1);         // dV, dK: A in TMEM, B MN-major
-        const uint32_t idesc_dqt = make_idesc_bf16(D, 64, 1, 1);             // dQ^T_x = K^T dS^T_x: M = d, N = 64 queries, K = keys; both MN-major
+        const uint32_t idesc_dqt = make_idesc_bf16(D, kQTile, 1, 1);         // dQ^T: M = d, N = 128 queries, K = keys; both MN-major
         const uint64_t kmaj = make_smem_desc_sw128(smem_u32(smem), 16, 1024);
-        const uint64_t mnmaj = make_smem_desc_sw128(smem_u32(smem), 64 * 128, 1024);   // 64-row tiles: 8 KB between column blocks
+        const uint64_t mnmaj = make_smem_desc_sw128(smem_u32(smem), kQTile * 128, 1024);   // 16 KB between 64-element column blocks
         const uint32_t desc_hi = (uint32_t)(kmaj >> 32);
         const uint32_t kmaj_lo = (uint32_t)kmaj, mnmaj_lo = (uint32_t)mnmaj;
-        const uint32_t mnmaj128_lo = (uint32_t)make_smem_desc_sw128(smem_u32(smem), kQTile * 128, 1024);   // 128-row tile: 16 KB between column blocks
-        const uint32_t ds_off = (uint32_t)(C::kOffStage >> 4);              // dS^T_x tiles: chain x at + x * 16 KB
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint32_t tDK = tmem_u + C::kColDK, tDV = tmem_u + C::kColDV;
-        const uint32_t k_off = (uint32_t)(C::kOffKV >> 4), v_off = (uint32_t)((C::kOffKV + C::kTileBytes) >> 4);
-        // [S^T_x | dP^T_x] = [K Q_x^T | V dout_x^T]: A a 128-row K-major tile, B the 64-row K-major tile of the slot
-        auto issue_sdp = [&](int x, uint32_t slot) {
-            const uint32_t q_off = (uint32_t)((C::kOffRing + slot * C::kSlotBytes) >> 4), do_off = q_off + (uint32_t)(C::kHalfBytes >> 4);
-            const uint32_t d = tmem_u + C::kColR + x * 128;
+        const uint32_t tDK = tmem_u + C::kColDK, tDV = tmem_u + C::kColDV, tS = tmem_u + C::kColS, tDP = tmem_u + C::kColDP;
+        const uint32_t lead = elect_one() ? 1u : 0u;
+        // [keys x 128 queries] = A B^T over d, both K-major 128-row tiles
+        auto issue_scores = [&](uint32_t acc, uint32_t a_off, uint32_t b_off) {
+            const uint32_t a_lo = kmaj_lo + (a_off >> 4), b_lo = kmaj_lo + (b_off >> 4);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
-                const uint32_t a16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4, b16 = ((kk >> 2) * (64 * 128) + (kk & 3) * 32) >> 4;
-                if (elect_one()) mma_ss_parts(d, kmaj_lo + k_off + a16, kmaj_lo + q_off + b16, desc_hi, idesc_st, kk > 0);
+                const uint32_t off16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4;
+                mma_ss_lead(lead, acc, a_lo + off16, b_lo + off16, desc_hi, idesc_s, kk > 0);
             }
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-                const uint32_t a16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4, b16 = ((kk >> 2) * (64 * 128) + (kk & 3) * 32) >> 4;
-                if (elect_one()) mma_ss_parts(d + 64, kmaj_lo + v_off + a16, kmaj_lo + do_off + b16, desc_hi, idesc_st, kk > 0);
-            }
-            commit_elected(&sdp_full[x]);
         };
-        // dV += P^T_x dout_x, dK += dS^T_x Q_x: A in TMEM (64 queries = 32 columns), B the slot's 64-row tile read MN-major
-        auto issue_acc = [&](int x, uint32_t slot, bool accumulate) {
-            const uint32_t q_off = (uint32_t)((C::kOffRing + slot * C::kSlotBytes) >> 4), do_off = q_off + (uint32_t)(C::kHalfBytes >> 4);
-            const uint32_t a = tmem_u + C::kColR + x * 128;
-            // dQ^T_x (d x 64 queries, over the dead dP^T_x columns) = K^T (the K tile read MN-major) dS^T_x (shared memory,
-            // MN-major); first, so that the chain's threads can take it away while dV and dK are in the pipe
+        // dV or dK += (bf16 [keys x 128 queries] in TMEM: 64 queries in the first 32 columns of each 64) x (128-row tile read MN-major)
+        auto issue_acc = [&](uint32_t acc, uint32_t a, uint32_t b_off, bool accumulate) {
+            const uint32_t b_lo = mnmaj_lo + (b_off >> 4);
 #pragma unroll
-            for (int kk = 0; kk < kTileN / 16; ++kk)
-                if (elect_one()) mma_ss_parts(a + 64, mnmaj128_lo + k_off + kk * (2048 >> 4), mnmaj_lo + ds_off + x * (16384 >> 4) + kk * (2048 >> 4),
-                                              desc_hi, idesc_dqt, kk > 0 ? 1u : 0u);
-            commit_elected(&dqt_full[x]);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                if (elect_one()) mma_ts_parts(tDV, a + (kk >> 1) * 32 + (kk & 1) * 8, mnmaj_lo + do_off + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                if (elect_one()) mma_ts_parts(tDK, a + (kk >> 1) * 32 + 16 + (kk & 1) * 8, mnmaj_lo + q_off + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
-            commit_elected(&slot_empty[slot]);
+            for (int kk = 0; kk < kQTile / 16; ++kk)
+                mma_ts_lead(lead, acc, a + (kk >> 2) * 64 + (kk & 3) * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
         };
         bool ok = base_ok;
-        uint32_t g = 0, n = 0;              // 128-query steps done, key tiles done; chain x of step g uses ring entry 2g + x
+        uint32_t g = 0, n = 0;              // steps and key tiles done; step g uses Q / dout slot g & 1
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_p));
+            return ok;
+        };
         for (long long u = u_begin; u < u_end && ok; u += u_step, ++n) {
-            const int t = (int)(u % p.key_tiles);
-            const int steps = p.q_tiles128 - first_q_tile(p, t);
-            ok = __all_sync(0xffffffffu, mbar_wait(kv_full, n & 1, abort_p));
-            if (!ok) break;
-            for (int x = 0; x < 2 && ok; ++x) {
-                const uint32_t hh = 2 * g + x;
-                ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[hh % C::kSlots], (hh / C::kSlots) & 1, abort_p));
-                if (!ok) break;
-                if (g > 0) {                                // dP^T_x is written over the chain's previous dQ^T_x
-                    ok = __all_sync(0xffffffffu, mbar_wait(&dq_drained[x], (g - 1) & 1, abort_p));
-                    if (!ok) break;
-                }
-                issue_sdp(x, hh % C::kSlots);
-            }
-            if (!ok) break;
-            for (int s = 0; s < steps && ok; ++s, ++g) {
+            const int steps = p.q_tiles128 - first_q_tile(p, (int)(u % p.key_tiles));
+            if (!wait(k_full, n & 1) || !wait(&q_full[g & 1], (g >> 1) & 1)) break;
+            tc_fence_after();
+            issue_scores(tS, C::kOffK, C::kOffQ + (g & 1) * C::kTileBytes);
+            commit_lead(lead, s_full);
+            if (!wait(v_full, n & 1) || !wait(&do_full[g & 1], (g >> 1) & 1)) break;
+            if (g > 0 && !wait(dq_drained, (g - 1) & 1)) break;             // dP^T goes over the previous step's dQ^T
+            tc_fence_after();
+            issue_scores(tDP, C::kOffV, C::kOffDO + (g & 1) * C::kTileBytes);
+            commit_lead(lead, dp_full);
+            if (steps == 1) commit_lead(lead, v_empty);
+            for (int s = 0; s < steps; ++s, ++g) {
+                const uint32_t slot = g & 1, next = slot ^ 1, next_par = ((g + 1) >> 1) & 1;
                 const bool have_next = s + 1 < steps;
-                for (int x = 0; x < 2 && ok; ++x) {
-                    const uint32_t hh = 2 * g + x;
-                    ok = __all_sync(0xffffffffu, mbar_wait(&pds_full[x], g & 1, abort_p));
-                    if (!ok) break;
-                    if (s == 0 && x == 0 && n > 0) {        // the previous key tile's dK, dV must have been read out
-                        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty, (n - 1) & 1, abort_p));
-                        if (!ok) break;
-                    }
+                if (!wait(p_full, g & 1)) break;
+                if (s == 0 && n > 0 && !wait(acc_empty, (n - 1) & 1)) break;   // the previous key tile's dK, dV must have been read out
+                tc_fence_after();
+                issue_acc(tDV, tS, C::kOffDO + slot * C::kTileBytes, s > 0);
+                commit_lead(lead, &do_empty[slot]);
+                if (have_next) {
+                    if (!wait(&q_full[next], next_par)) break;
                     tc_fence_after();
-                    issue_acc(x, hh % C::kSlots, s > 0 || x > 0);
+                    issue_scores(tS, C::kOffK, C::kOffQ + next * C::kTileBytes);
+                    commit_lead(lead, s_full);
                 }
-                if (!ok) break;
-                if (!have_next) commit_elected(kv_empty);   // K (read by the dQ^T products) and V are free for the next key tile
-                // the next score products of a chain overwrite its dQ^T_x: they follow its drain, which runs while the
-                // other chain's products are in the pipe
-                for (int x = 0; x < 2 && ok && have_next; ++x) {
-                    const uint32_t hn = 2 * g + x + 2;
-                    ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[hn % C::kSlots], (hn / C::kSlots) & 1, abort_p));
-                    if (!ok) break;
-                    ok = __all_sync(0xffffffffu, mbar_wait(&dq_drained[x], g & 1, abort_p));
-                    if (!ok) break;
+                if (!wait(ds_full, g & 1)) break;
+                tc_fence_after();
+                issue_acc(tDK, tDP, C::kOffQ + slot * C::kTileBytes, s > 0);
+                commit_lead(lead, &q_empty[slot]);
+#pragma unroll
+                for (int kk = 0; kk < kTileN / 16; ++kk)
+                    mma_ss_lead(lead, tDP, mnmaj_lo + (C::kOffK >> 4) + kk * (2048 >> 4), mnmaj_lo + (C::kOffStage >> 4) + kk * (2048 >> 4), desc_hi, idesc_dqt, kk > 0);
+                commit_lead(lead, dq_full);
+                if (have_next) {
+                    if (!wait(&do_full[next], next_par) || !wait(dq_drained, g & 1)) break;
                     tc_fence_after();
-                    issue_sdp(x, hn % C::kSlots);
+                    issue_scores(tDP, C::kOffV, C::kOffDO + next * C::kTileBytes);
+                    commit_lead(lead, dp_full);
+                    if (s + 2 == steps) commit_lead(lead, v_empty);
+                } else {
+                    commit_lead(lead, k_empty);
+                    commit_lead(lead, acc_full);
                 }
-                if (!ok) break;
             }
-            if (!ok) break;
-            commit_elected(acc_full);
         }
-    } else if (warp < 8) {
-        // ------------------------------------------------------------------ elementwise threads
-        const int wg = warp >> 2;                              // chain: which 64 queries of every tile
+    }
+    } else if (warp >= C::kDqWarp) {
+        // ------------------------------------------------------------------ dQ^T -> fp32 dQ (reductions in L2)
+        setmaxnreg_inc<C::kDqRegs>();
+        const int r = (warp & 3) * 32 + lane;                  // column of dQ == TMEM lane
+        const uint32_t tDQ = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + C::kColDP;
+        bool ok = base_ok;
+        uint32_t g = 0;
+        for (long long u = u_begin; u < u_end && ok; u += u_step) {
+            const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
+            for (int i = first_q_tile(p, t); i < p.q_tiles128; ++i, ++g) {
+                ok = __all_sync(0xffffffffu, mbar_wait(dq_full, g & 1, abort_p));
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t o[4][32];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) tmem_ld32_async(tDQ + c * 32, o[c]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) tmem_wait_ld(o[c]);
+                tc_fence_before();
+                mbar_arrive(dq_drained);
+                // for one query the 32 lanes of a warp hold 32 consecutive floats of its row: 128 bytes per reduction
+                float* drow = p.ws + ((long long)bh * p.Wpad + i * kQTile) * D + r;
+#pragma unroll
+                for (int e = 0; e < kQTile; ++e) atomicAdd(drow + e * D, __uint_as_float(o[e >> 5][e & 31]));
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ P and dS
+        setmaxnreg_inc<C::kComputeRegs>();
+        const int wg = warp >> 2;                              // which 64 queries of every tile
         const int r = (warp & 3) * 32 + lane;                  // key row inside the tile == TMEM lane
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tS = tmem_base + lane_addr + C::kColR + wg * 128;
-        const uint32_t tDP = tS + 64;
+        const uint32_t tS = tmem_base + lane_addr + C::kColS + wg * 64, tDP = tmem_base + lane_addr + C::kColDP + wg * 64;
+        uint8_t* ds_row = smem + C::kOffStage + wg * 16384 + r * 128;       // this key's row of the dS^T tile
         bool ok = base_ok;
-        // the second half of a step's dQ^T_x values waits in registers and is handed to L2 while the next step's products run
-        uint32_t held[32];
-        float* held_row = nullptr;
         uint32_t g = 0, n = 0;
         for (long long u = u_begin; u < u_end && ok; u += u_step, ++n) {
             const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
             const int key = t * kTileN + r;
-            const int i_first = first_q_tile(p, t);
             const long long shift = (long long)p.N - p.W;       // query q may use key k iff q >= k - shift
             const int q_min = p.causal ? (int)((long long)key - shift) : -0x7fffffff;
             const int q_min_warp = p.causal ? (int)((long long)key - lane + 31 - shift) : -0x7fffffff;   // largest in the warp
-            for (int i = i_first; i < p.q_tiles128; ++i, ++g) {
-                const uint32_t hh = 2 * g + wg, slot = hh % C::kSlots;
-                const float* st = sStats + slot * 128;
-                const int q0 = i * kQTile + wg * 64;              // first query of this thread's columns
-                ok = __all_sync(0xffffffffu, mbar_wait(&sdp_full[wg], g & 1, abort_p));
-                if (!ok) break;
+            auto step = [&](int q0, auto masked_tag) {
+                constexpr bool kMasked = decltype(masked_tag)::value;
+                const float* st = sStats + (g & 1) * 256 + wg * 64;
+                ok = __all_sync(0xffffffffu, mbar_wait(s_full, g & 1, abort_p));
+                if (!ok) return;
                 // already complete (the MMAs waited for it); observing it here orders the bulk-copied lse2 / delta
                 // before this thread's reads
-                ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[slot], (hh / C::kSlots) & 1, abort_p));
-                if (!ok) break;
+                ok = __all_sync(0xffffffffu, mbar_wait(&q_full[g & 1], (g >> 1) & 1, abort_p));
+                if (!ok) return;
                 tc_fence_after();
-                const bool masked = q0 < q_min_warp;              // warp-uniform: some element of some lane is masked
-                // 32 queries at a time: P^T and dS^T of a half go over the 32 columns of S^T_x that have just been read
-                uint8_t* ds_row = smem + C::kOffStage + wg * 16384 + r * 128;       // this key's row of the dS^T_x tile
+                uint32_t pe[2][32];
+                tmem_ld32_async(tS, pe[0]);
+                tmem_ld32_async(tS + 32, pe[1]);
+                tmem_wait_ld(pe[0]);
+                tmem_wait_ld(pe[1]);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    uint32_t sv[32], dv_[32];
-                    tmem_ld32_async(tS + h * 32, sv);
-                    tmem_ld32_async(tDP + h * 32, dv_);
-                    tmem_wait_ld(sv);
-                    tmem_wait_ld(dv_);
-                    uint32_t pk[16], dk_[16];
+                    uint32_t pk[16];
 #pragma unroll
                     for (int c = 0; c < 32; c += 4) {
                         const float4 l4 = *reinterpret_cast<const float4*>(st + h * 32 + c);
-                        const float4 d4 = *reinterpret_cast<const float4*>(st + 64 + h * 32 + c);
-                        const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, dlv[4] = {d4.x, d4.y, d4.z, d4.w};
-                        float pe[4], de[4];
+                        const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
+                        float x[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            pe[e] = ex2(fmaf(__uint_as_float(sv[c + e]), p.scale_log2e, -lv[e]));
-                            if (masked && q0 + h * 32 + c + e < q_min) pe[e] = 0.f;
-                            de[e] = pe[e] * (__uint_as_float(dv_[c + e]) - dlv[e]);
+                            x[e] = ex2(fmaf(__uint_as_float(pe[h][c + e]), p.scale_log2e, -lv[e]));
+                            if (kMasked && q0 + h * 32 + c + e < q_min) x[e] = 0.f;
+                            pe[h][c + e] = __float_as_uint(x[e]);
                         }
-                        pk[c / 2] = pack_bf16x2(pe[0], pe[1]);
-                        pk[c / 2 + 1] = pack_bf16x2(pe[2], pe[3]);
+                        pk[c / 2] = pack_bf16x2(x[0], x[1]);
+                        pk[c / 2 + 1] = pack_bf16x2(x[2], x[3]);
+                    }
+                    tmem_st16(tS + h * 16, pk);
+                }
+                tc_wait_st();
+                tc_fence_before();
+                mbar_arrive(p_full);
+                ok = __all_sync(0xffffffffu, mbar_wait(dp_full, g & 1, abort_p));
+                if (!ok) return;
+                tc_fence_after();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t dp[32], dk_[16];
+                    tmem_ld32_async(tDP + h * 32, dp);
+                    tmem_wait_ld(dp);
+#pragma unroll
+                    for (int c = 0; c < 32; c += 4) {
+                        const float4 d4 = *reinterpret_cast<const float4*>(st + 128 + h * 32 + c);
+                        const float dlv[4] = {d4.x, d4.y, d4.z, d4.w};
+                        float de[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) de[e] = __uint_as_float(pe[h][c + e]) * (__uint_as_float(dp[c + e]) - dlv[e]);
                         dk_[c / 2] = pack_bf16x2(de[0], de[1]);
                         dk_[c / 2 + 1] = pack_bf16x2(de[2], de[3]);
                     }
-                    tmem_st16(tS + h * 32, pk);
-                    tmem_st16(tS + h * 32 + 16, dk_);
-                    // and dS^T_x once more as the B operand of the dQ^T product: row = key, 64 queries = 128 bytes, 16-byte
-                    // pieces at (piece xor row mod 8), the layout the 128-byte swizzle of the descriptors expects
+                    tmem_st16(tDP + h * 16, dk_);          // over columns of dP^T that are already in registers
+                    // and once more as the B operand of the dQ^T product: row = key, 64 queries = 128 bytes, 16-byte pieces at
+                    // (piece xor row mod 8), the layout the 128-byte swizzle of the descriptors expects
 #pragma unroll
                     for (int c4 = 0; c4 < 4; ++c4)
                         *reinterpret_cast<uint4*>(ds_row + (((h * 4 + c4) ^ (r & 7)) << 4)) =
@@ -760,31 +817,12 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 tc_wait_st();
                 fence_proxy_async_smem();             // the tile was written with ordinary stores and is read by the MMA
                 tc_fence_before();
-                mbar_arrive(&pds_full[wg]);
-                // ------------------------------------------------------------ dQ^T_x -> fp32 dQ (reductions in L2)
-                // For one query the 32 lanes of a warp hold 32 consecutive floats of its row of the fp32 dQ buffer: one
-                // reduction instruction adds 128 consecutive bytes.  The half kept from the previous step goes first, while
-                // this step's products are in the pipe.
-                if (held_row != nullptr) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) atomicAdd(held_row + (long long)e * D, __uint_as_float(held[e]));
-                }
-                ok = __all_sync(0xffffffffu, mbar_wait(&dqt_full[wg], g & 1, abort_p));
-                if (!ok) break;
-                tc_fence_after();
-                // TMEM lane = column of dQ (this thread: r), TMEM column = query.  Once the values are in registers the columns
-                // are free for the chain's next score products.
-                uint32_t o[32];
-                tmem_ld32_async(tDP, o);
-                tmem_ld32_async(tDP + 32, held);
-                tmem_wait_ld(o);
-                tmem_wait_ld(held);
-                tc_fence_before();
-                mbar_arrive(&dq_drained[wg]);
-                float* drow = p.ws + ((long long)bh * p.Wpad + q0) * D + r;
-#pragma unroll
-                for (int e = 0; e < 32; ++e) atomicAdd(drow + (long long)e * D, __uint_as_float(o[e]));
-                held_row = drow + 32LL * D;
+                mbar_arrive(ds_full);
+            };
+            for (int i = first_q_tile(p, t); i < p.q_tiles128 && ok; ++i, ++g) {
+                const int q0 = i * kQTile + wg * 64;              // first query of this thread's columns
+                if (q0 < q_min_warp) step(q0, std::true_type{});  // warp-uniform: some element of some lane is masked
+                else step(q0, std::false_type{});
             }
             if (!ok) break;
             // ---------------------------------------------------------------- dK, dV of this key tile
@@ -793,7 +831,8 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             tc_fence_after();
             // Each thread holds half a row (D/2 columns) of dK and of dV.  Written straight from the registers a warp's store
             // would touch 32 different lines; the warp passes its 32 x D bytes through shared memory (16-byte pieces, piece
-            // index xor row so that neither side has bank conflicts beyond the minimum) and stores whole lines instead.
+            // index xor row so that neither side has bank conflicts beyond the minimum) and stores whole lines instead.  Its
+            // part of the buffer is where its own rows of dS^T go, so no other warp is in the way.
             constexpr int kPieces = D / 16;                    // 16-byte pieces per half row
             constexpr int kRowsPerStore = 32 / kPieces;
             uint8_t* stage = smem + C::kOffStage + warp * (32 * D);
@@ -817,6 +856,10 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                         *reinterpret_cast<uint4*>(stage + lane * D + ((piece ^ (lane & (kPieces - 1))) << 4)) = w;
                     }
                 }
+                if (which == 1) {                              // both accumulators have been read
+                    tc_fence_before();
+                    mbar_arrive(acc_empty);
+                }
                 __syncwarp();
                 __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(which == 0 ? p.dk : p.dv) +
                                      ((long long)bh * p.N + key_warp) * D + wg * (D / 2);
@@ -828,19 +871,13 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 }
                 __syncwarp();
             }
-            tc_fence_before();
-            mbar_arrive(acc_empty);
-        }
-        if (held_row != nullptr) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) atomicAdd(held_row + (long long)e * D, __uint_as_float(held[e]));
         }
     }
 
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) atomicExch(p.status, base_ok ? (int)TLIN_ERR_TIMEOUT : (int)TLIN_ERR_CUDA);
-    if (warp == kMmaWarp) {
+    if (warp == C::kMma) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
     }
@@ -1288,9 +1325,8 @@ int launch_d(const void* q, const void* k, const void* v, const void* out, const
     TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dkdv_tc_kernel<D>, ACfg<D>::kSmemBytes, smem_allowed_a));
     TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dq_tc_kernel<D>, BCfg<D>::kSmemBytes, smem_allowed_b));
     const long long rows_padded = bh * Wpad;
-    bwd_prep_kernel<D><<<(unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st>>>(
-        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, W, Wpad, rows_padded);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(bwd_prep_kernel<D>, (unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st,
+        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, (float*)nullptr, W, Wpad, rows_padded));
     // dK, dV: the units are (b,h,key tile); a CTA takes a contiguous run of them
     BwdParams pa = p;
     pa.total_units = bh * p.key_tiles;
@@ -1318,7 +1354,9 @@ int launch_d(const void* q, const void* k, const void* v, const void* out, const
 // fp32 dQ sums (rows padded to 128 per (b,h)) -> scaled bf16 dQ; 8 elements per thread
 template <int D>
 __global__ void __launch_bounds__(256)
-bwd_dq_convert_kernel(const float* __restrict__ dq32, __nv_bfloat16* __restrict__ dq, int W, int Wpad, long long rows, float scale) {
+bwd_dq_convert_kernel(const float* dq32, __nv_bfloat16* dq, int W, int Wpad, long long rows, float scale) {
+    after_previous();
+    let_next_start();
     constexpr int TPR = D / 8;              // threads per row
     const long long idx = (long long)blockIdx.x * 256 + threadIdx.x;
     const long long row = idx / TPR;
@@ -1342,11 +1380,11 @@ int launch_fused_128(const void* q, const void* k, const void* v, const void* ou
     constexpr int D = 128;
     const long long bh = (long long)B * H;
     const int Wpad = (W + kQTile - 1) / kQTile * kQTile;
-    CUtensorMap mk, mv, mq64, mdo64;
+    CUtensorMap mk, mv, mq, mdo;
     int rc = make_map(&mk, k, D, N, bh);
     if (rc == TLIN_OK) rc = make_map(&mv, v, D, N, bh);
-    if (rc == TLIN_OK) rc = make_map(&mq64, q, D, W, bh, 64);
-    if (rc == TLIN_OK) rc = make_map(&mdo64, dout, D, W, bh, 64);
+    if (rc == TLIN_OK) rc = make_map(&mq, q, D, W, bh);
+    if (rc == TLIN_OK) rc = make_map(&mdo, dout, D, W, bh);
     if (rc != TLIN_OK) return rc;
     BwdParams p;
     float* lse2 = ws;
@@ -1365,19 +1403,14 @@ int launch_fused_128(const void* q, const void* k, const void* v, const void* ou
     p.total_units = bh * p.key_tiles;
     p.n_groups = 0; p.q_tiles = 0; p.schedule = 0;
     static bool smem_allowed[64] = {};
-    constexpr int kSmem = ACfg<D>::kSmemBytes + 32;             // four more barriers than the dK/dV kernel
-    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_fused_tc_kernel<D>, kSmem, smem_allowed));
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_fused_tc_kernel<D>, FCfg<D>::kSmemBytes, smem_allowed));
     const long long rows_padded = bh * Wpad;
-    bwd_prep_kernel<D><<<(unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st>>>(
-        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, W, Wpad, rows_padded);
-    TLIN_CUDA_CHECK(cudaGetLastError());
-    TLIN_CUDA_CHECK(cudaMemsetAsync(dq32, 0, (size_t)rows_padded * D * sizeof(float), st));
+    TLIN_CUDA_CHECK(launch_overlapped(bwd_prep_kernel<D>, (unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st,
+        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, dq32, W, Wpad, rows_padded));
     const long long ctas = p.total_units < num_sms ? p.total_units : num_sms;
-    bwd_fused_tc_kernel<D><<<(unsigned)ctas, ACfg<D>::kThreads, kSmem, st>>>(mq64, mk, mv, mdo64, p);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(bwd_fused_tc_kernel<D>, (unsigned)ctas, FCfg<D>::kThreads, FCfg<D>::kSmemBytes, st, mq, mk, mv, mdo, p));
     const long long rows = bh * W, threads = rows * (D / 8);
-    bwd_dq_convert_kernel<D><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(dq32, (__nv_bfloat16*)dq, W, Wpad, rows, p.scale);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(bwd_dq_convert_kernel<D>, (unsigned)((threads + 255) / 256), 256, 0, st, dq32, (__nv_bfloat16*)dq, W, Wpad, rows, p.scale));
     count_launch(3);
     return TLIN_OK;
 }
