@@ -474,11 +474,12 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 //   dK(j), dQ(j) | dP(j+1) once dQ(j) has been taken out of TMEM | dV(j+1), S(j+2) once P(j+1) is there
 // The exponentials of step j+1 run while dK(j) and dQ(j) do, dS(j+1) while dV(j+1) and S(j+2) do.
 // Three warpgroups work on a step: two take 64 queries each (thread = key row) through P and dS, the third takes dQ^T into
-// registers (thread = column of dQ) and adds it to the fp32 dQ in the workspace, 128 consecutive bytes per reduction, while the
-// others go on.  An SM has about 25 bytes of reductions per clock accepted, 2600 clocks for a step's 64 KB: with the reductions in
-// the threads that also form P and dS, and score products 64 queries wide, the training chunk (B4 H32 N8192 W1024) took 1543 us at
-// full clock and 1759 us under the power cap, now 1405 and 1601; B1 H32 N8192 W1024 449 -> 399 us, B2 H16 N4096 W512 132 -> 116 us,
-// B1 H4 N700 W300 28 -> 18 us (two launches fewer to wait for).
+// registers (thread = column of dQ), passes it through shared memory and has the copy engine add the rows to the fp32 dQ in the
+// workspace.  That is 64 KB of reductions per step, which L2 takes at about 6 TB/s: 0.68 of the 1.28 ms below.
+// Measured at B4 H32 N8192 W1024 (full clock / under the power cap): reductions in the threads that form P and dS, scores 64
+// queries wide 1543 / 1759 us; 128 wide, a warpgroup of its own with red instructions 1405 / 1601 us (they fill the load/store
+// unit that P and dS need); through the copy engine 1278 / 1397 us.  B1 H32 N8192 W1024 449 -> 354 us, B1 H32 N32768 W512
+// 942 -> 804 us, B2 H16 N4096 W512 132 -> 108 us, B1 H4 N700 W300 28 -> 18 us.
 template <int D>
 struct FCfg {
     static_assert(D == 128, "the transposed dQ accumulator needs M = d = 128");
@@ -486,19 +487,21 @@ struct FCfg {
     static constexpr int kBoxes = D / 64;
     static constexpr int kOffK = 0, kOffV = kTileBytes;
     static constexpr int kOffQ = 2 * kTileBytes;               // 2 slots
-    static constexpr int kOffDO = 4 * kTileBytes;              // 2 slots
-    static constexpr int kOffStage = 6 * kTileBytes;           // dS^T tile: two blocks of 128 keys x 64 queries; dK / dV rows on their way out
+    static constexpr int kOffDO = 4 * kTileBytes;
+    static constexpr int kOffStage = 5 * kTileBytes;           // dS^T tile: two blocks of 128 keys x 64 queries; dK / dV rows on their way out
+    static constexpr int kOffDQ = 6 * kTileBytes;              // 4 buffers of 16 queries x D fp32: dQ rows on their way to L2
+    static constexpr int kDqRows = 16;
     static constexpr int kOffStats = 7 * kTileBytes;           // 2 slots: lse2 of 128 rows, delta of 128 rows
     static constexpr int kOffBars = kOffStats + 2 * 1024;
-    static constexpr int kNumBars = 20;
+    static constexpr int kNumBars = 18;
     static constexpr int kSmemBytes = kOffBars + kNumBars * 8 + 16;
     static constexpr uint32_t kColDK = 0, kColDV = D, kColS = 2 * D, kColDP = 2 * D + 128;
     static constexpr int kThreads = 32 * 16;
     static constexpr int kDqWarp = 8, kProducer = 12, kMma = 13, kKv = 14;      // warps 0 to 7: P and dS
-    // setmaxnreg moves registers between warpgroups; the CTA starts with 128 per thread, and an increase beyond what the others
-    // released would wait for ever
-    static constexpr int kComputeRegs = 144, kDqRegs = 152, kOtherRegs = 64;
-    static_assert(256 * kComputeRegs + 128 * kDqRegs + 128 * kOtherRegs <= kThreads * 128, "register budget of the CTA exceeded");
+    // setmaxnreg moves registers between warpgroups; the CTA starts with 128 per thread (which the P and dS warps keep).  An
+    // increase beyond what the others released would wait for ever, one below the count at launch is an illegal instruction.
+    static constexpr int kLaunchRegs = 128, kDqRegs = 152, kOtherRegs = 104;
+    static_assert(128 * kDqRegs + 128 * kOtherRegs <= 256 * kLaunchRegs && kDqRegs > kLaunchRegs && kOtherRegs < kLaunchRegs, "register budget");
 };
 
 template <int D>
@@ -511,20 +514,20 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
     uint64_t* q_full = bars + 0;      // [2] Q and the row statistics of a step
     uint64_t* q_empty = bars + 2;     // [2]
-    uint64_t* do_full = bars + 4;     // [2]
-    uint64_t* do_empty = bars + 6;    // [2]
-    uint64_t* k_full = bars + 8;
-    uint64_t* k_empty = bars + 9;
-    uint64_t* v_full = bars + 10;
-    uint64_t* v_empty = bars + 11;
-    uint64_t* s_full = bars + 12;     // S^T of a step is in TMEM
-    uint64_t* p_full = bars + 13;     // P^T is written
-    uint64_t* dp_full = bars + 14;    // dP^T is in TMEM
-    uint64_t* ds_full = bars + 15;    // dS^T is written (TMEM and shared memory)
-    uint64_t* dq_full = bars + 16;    // dQ^T is in TMEM
-    uint64_t* dq_drained = bars + 17; // the dQ warpgroup holds it in registers
-    uint64_t* acc_full = bars + 18;   // dK, dV of the key tile are complete
-    uint64_t* acc_empty = bars + 19;  // all threads have read them
+    uint64_t* do_full = bars + 4;
+    uint64_t* do_empty = bars + 5;
+    uint64_t* k_full = bars + 6;
+    uint64_t* k_empty = bars + 7;
+    uint64_t* v_full = bars + 8;
+    uint64_t* v_empty = bars + 9;
+    uint64_t* s_full = bars + 10;     // S^T of a step is in TMEM
+    uint64_t* p_full = bars + 11;     // P^T is written
+    uint64_t* dp_full = bars + 12;    // dP^T is in TMEM
+    uint64_t* ds_full = bars + 13;    // dS^T is written (TMEM and shared memory)
+    uint64_t* dq_full = bars + 14;    // dQ^T is in TMEM
+    uint64_t* dq_drained = bars + 15; // the dQ warpgroup holds it in registers
+    uint64_t* acc_full = bars + 16;   // dK, dV of the key tile are complete
+    uint64_t* acc_empty = bars + 17;  // all threads have read them
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
@@ -581,20 +584,18 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                         tma_load_3d(smem + C::kOffQ + slot * C::kTileBytes + x * (kQTile * 128), &map_q, &q_full[slot], x * 64, row, bh);
                     bulk_load_1d(sStats + slot * 256, p.lse2 + (long long)bh * p.Wpad + row, 512, &q_full[slot]);
                     bulk_load_1d(sStats + slot * 256 + 128, p.delta + (long long)bh * p.Wpad + row, 512, &q_full[slot]);
-                    ok = mbar_wait(&do_empty[slot], par, abort_p);
+                    ok = mbar_wait(do_empty, (ndo & 1) ^ 1, abort_p);
                     if (!ok) break;
-                    mbar_arrive_expect_tx(&do_full[slot], C::kTileBytes);
+                    mbar_arrive_expect_tx(do_full, C::kTileBytes);
                     ++ndo;
-                    for (int x = 0; x < C::kBoxes; ++x)
-                        tma_load_3d(smem + C::kOffDO + slot * C::kTileBytes + x * (kQTile * 128), &map_do, &do_full[slot], x * 64, row, bh);
+                    for (int x = 0; x < C::kBoxes; ++x) tma_load_3d(smem + C::kOffDO + x * (kQTile * 128), &map_do, do_full, x * 64, row, bh);
                 }
             }
             if (!ok && base_ok) {
                 int dummy = 0;              // leave no copy in flight: the barriers armed last must complete (bounded)
-                for (uint32_t back = 1; back <= 2; ++back) {
-                    if (back <= nq) mbar_wait(&q_full[(nq - back) & 1], ((nq - back) >> 1) & 1, &dummy, 200000000LL);
-                    if (back <= ndo) mbar_wait(&do_full[(ndo - back) & 1], ((ndo - back) >> 1) & 1, &dummy, 200000000LL);
-                }
+                for (uint32_t back = 1; back <= 2 && back <= nq; ++back)
+                    mbar_wait(&q_full[(nq - back) & 1], ((nq - back) >> 1) & 1, &dummy, 200000000LL);
+                if (ndo > 0) mbar_wait(do_full, (ndo - 1) & 1, &dummy, 200000000LL);
             }
         }
     } else if (warp == C::kKv) {
@@ -657,7 +658,7 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 mma_ts_lead(lead, acc, a + (kk >> 2) * 64 + (kk & 3) * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
         };
         bool ok = base_ok;
-        uint32_t g = 0, n = 0;              // steps and key tiles done; step g uses Q / dout slot g & 1
+        uint32_t g = 0, n = 0;              // steps and key tiles done; step g uses Q slot g & 1
         auto wait = [&](uint64_t* bar, uint32_t parity) {
             ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_p));
             return ok;
@@ -668,10 +669,10 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             tc_fence_after();
             issue_scores(tS, C::kOffK, C::kOffQ + (g & 1) * C::kTileBytes);
             commit_lead(lead, s_full);
-            if (!wait(v_full, n & 1) || !wait(&do_full[g & 1], (g >> 1) & 1)) break;
+            if (!wait(v_full, n & 1) || !wait(do_full, g & 1)) break;
             if (g > 0 && !wait(dq_drained, (g - 1) & 1)) break;             // dP^T goes over the previous step's dQ^T
             tc_fence_after();
-            issue_scores(tDP, C::kOffV, C::kOffDO + (g & 1) * C::kTileBytes);
+            issue_scores(tDP, C::kOffV, C::kOffDO);
             commit_lead(lead, dp_full);
             if (steps == 1) commit_lead(lead, v_empty);
             for (int s = 0; s < steps; ++s, ++g) {
@@ -680,8 +681,8 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 if (!wait(p_full, g & 1)) break;
                 if (s == 0 && n > 0 && !wait(acc_empty, (n - 1) & 1)) break;   // the previous key tile's dK, dV must have been read out
                 tc_fence_after();
-                issue_acc(tDV, tS, C::kOffDO + slot * C::kTileBytes, s > 0);
-                commit_lead(lead, &do_empty[slot]);
+                issue_acc(tDV, tS, C::kOffDO, s > 0);
+                commit_lead(lead, do_empty);
                 if (have_next) {
                     if (!wait(&q_full[next], next_par)) break;
                     tc_fence_after();
@@ -697,9 +698,9 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     mma_ss_lead(lead, tDP, mnmaj_lo + (C::kOffK >> 4) + kk * (2048 >> 4), mnmaj_lo + (C::kOffStage >> 4) + kk * (2048 >> 4), desc_hi, idesc_dqt, kk > 0);
                 commit_lead(lead, dq_full);
                 if (have_next) {
-                    if (!wait(&do_full[next], next_par) || !wait(dq_drained, g & 1)) break;
+                    if (!wait(do_full, (g + 1) & 1) || !wait(dq_drained, g & 1)) break;
                     tc_fence_after();
-                    issue_scores(tDP, C::kOffV, C::kOffDO + next * C::kTileBytes);
+                    issue_scores(tDP, C::kOffV, C::kOffDO);
                     commit_lead(lead, dp_full);
                     if (s + 2 == steps) commit_lead(lead, v_empty);
                 } else {
@@ -714,6 +715,7 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         setmaxnreg_inc<C::kDqRegs>();
         const int r = (warp & 3) * 32 + lane;                  // column of dQ == TMEM lane
         const uint32_t tDQ = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + C::kColDP;
+        const bool issuer = threadIdx.x == C::kDqWarp * 32;
         bool ok = base_ok;
         uint32_t g = 0;
         for (long long u = u_begin; u < u_end && ok; u += u_step) {
@@ -729,15 +731,27 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 for (int c = 0; c < 4; ++c) tmem_wait_ld(o[c]);
                 tc_fence_before();
                 mbar_arrive(dq_drained);
-                // for one query the 32 lanes of a warp hold 32 consecutive floats of its row: 128 bytes per reduction
-                float* drow = p.ws + ((long long)bh * p.Wpad + i * kQTile) * D + r;
+                // rows of dQ (consecutive in the workspace) through shared memory, 16 at a time, added by the copy engine
+                float* drow = p.ws + ((long long)bh * p.Wpad + i * kQTile) * D;
 #pragma unroll
-                for (int e = 0; e < kQTile; ++e) atomicAdd(drow + e * D, __uint_as_float(o[e >> 5][e & 31]));
+                for (int c = 0; c < kQTile / C::kDqRows; ++c) {
+                    float* buf = reinterpret_cast<float*>(smem + C::kOffDQ + (c & 3) * (C::kDqRows * D * 4));
+                    if (issuer) bulk_wait_read<3>();              // the buffer's previous rows have been read
+                    named_barrier(1, 128);
+#pragma unroll
+                    for (int e = 0; e < C::kDqRows; ++e) buf[e * D + r] = __uint_as_float(o[c >> 1][(c & 1) * 16 + e]);
+                    fence_proxy_async_smem();
+                    named_barrier(1, 128);
+                    if (issuer) {
+                        bulk_add_f32(drow + c * C::kDqRows * D, buf, C::kDqRows * D * 4);
+                        bulk_commit();
+                    }
+                }
             }
         }
+        if (issuer) bulk_wait_all();
     } else {
         // ------------------------------------------------------------------ P and dS
-        setmaxnreg_inc<C::kComputeRegs>();
         const int wg = warp >> 2;                              // which 64 queries of every tile
         const int r = (warp & 3) * 32 + lane;                  // key row inside the tile == TMEM lane
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
