@@ -5,7 +5,9 @@
 //   p = exp(q k^T / sqrt(d) - lse)    dp = dout v^T    ds = p * (dp - delta) / sqrt(d),  delta_i = dout_i . out_i
 //   dv = p^T dout      dk = ds^T q      dq = ds k
 //
-// Two kernels, neither with atomics, both recomputing p from the saved lse (the default):
+// Two kernels, neither with atomics, both recomputing p from the saved lse (what the one kernel below does not serve).  Steps with
+// masked elements have a copy of the code of their own and the MMA warps elect their issuing lane once: B3 H12 N=W=1999 d64 175 ->
+// 160 us, B2 H8 N1961 W578 d64 62 -> 53 us, B4 H32 N8192 W1024 d64 1.31 -> 1.20 ms.
 //
 // bwd_dkdv_tc_kernel   A CTA owns one 128-key tile of a (b,h) at a time and walks the 128-row query tiles that may
 //   see it.  Scores are computed TRANSPOSED (S^T = K Q^T, dP^T = V dout^T: TMEM lane = key, column = query) so that
@@ -197,6 +199,8 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         prefetch_tensormap(&map_do);
     }
     tc_fence_before();
+    after_previous();
+    let_next_start();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
@@ -267,7 +271,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
         }
     } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------------ MMA issuer (all lanes walk, one issues)
+        // ------------------------------------------------------------------ MMA issuer (all lanes walk, the lane elected once issues)
         const uint32_t idesc_st = make_idesc_bf16(kQTile, 64, 0, 0);         // S^T, dP^T of a chain: M = keys, N = 64 queries
         const uint32_t idesc_acc = make_idesc_bf16(kQTile, D, 0, 1);         // dV, dK: A in TMEM, B MN-major
         const uint64_t kmaj = make_smem_desc_sw128(smem_u32(smem), 16, 1024);
@@ -275,6 +279,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const uint32_t desc_hi = (uint32_t)(kmaj >> 32);
         const uint32_t kmaj_lo = (uint32_t)kmaj, mnmaj_lo = (uint32_t)mnmaj;
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+        const uint32_t lead = elect_one() ? 1u : 0u;
         const uint32_t tDK = tmem_u + C::kColDK, tDV = tmem_u + C::kColDV;
         const uint32_t k_off = (uint32_t)(C::kOffKV >> 4), v_off = (uint32_t)((C::kOffKV + C::kTileBytes) >> 4);
         // [S^T_x | dP^T_x] = [K Q_x^T | V dout_x^T]: A a 128-row K-major tile, B the 64-row K-major tile of the slot
@@ -284,14 +289,14 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t a16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4, b16 = ((kk >> 2) * (64 * 128) + (kk & 3) * 32) >> 4;
-                if (elect_one()) mma_ss_parts(d, kmaj_lo + k_off + a16, kmaj_lo + q_off + b16, desc_hi, idesc_st, kk > 0);
+                mma_ss_lead(lead, d, kmaj_lo + k_off + a16, kmaj_lo + q_off + b16, desc_hi, idesc_st, kk > 0);
             }
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t a16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4, b16 = ((kk >> 2) * (64 * 128) + (kk & 3) * 32) >> 4;
-                if (elect_one()) mma_ss_parts(d + 64, kmaj_lo + v_off + a16, kmaj_lo + do_off + b16, desc_hi, idesc_st, kk > 0);
+                mma_ss_lead(lead, d + 64, kmaj_lo + v_off + a16, kmaj_lo + do_off + b16, desc_hi, idesc_st, kk > 0);
             }
-            commit_elected(&sdp_full[x]);
+            commit_lead(lead, &sdp_full[x]);
         };
         // dV += P^T_x dout_x, dK += dS^T_x Q_x: A in TMEM (64 queries = 32 columns), B the slot's 64-row tile read MN-major
         auto issue_acc = [&](int x, uint32_t slot, bool accumulate) {
@@ -299,11 +304,11 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const uint32_t a = tmem_u + C::kColR + x * 128;
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-                if (elect_one()) mma_ts_parts(tDV, a + kk * 8, mnmaj_lo + do_off + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
+                mma_ts_lead(lead, tDV, a + kk * 8, mnmaj_lo + do_off + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-                if (elect_one()) mma_ts_parts(tDK, a + 64 + kk * 8, mnmaj_lo + q_off + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
-            commit_elected(&slot_empty[slot]);
+                mma_ts_lead(lead, tDK, a + 64 + kk * 8, mnmaj_lo + q_off + kk * (2048 >> 4), desc_hi, idesc_acc, (accumulate || kk > 0) ? 1u : 0u);
+            commit_lead(lead, &slot_empty[slot]);
         };
         bool ok = base_ok;
         uint32_t g = 0, n = 0;              // 128-query steps done, key tiles done; chain x of step g uses ring entry 2g + x
@@ -319,7 +324,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 issue_sdp(x, hh % C::kSlots);
             }
             if (!ok) break;
-            if (steps == 1) commit_elected(kv_empty);       // K, V have been read for the last time: the next tile's may load
+            if (steps == 1) commit_lead(lead, kv_empty);       // K, V have been read for the last time: the next tile's may load
             for (int s = 0; s < steps && ok; ++s, ++g) {
                 const bool have_next = s + 1 < steps;
                 for (int x = 0; x < 2 && ok; ++x) {
@@ -340,10 +345,10 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                 }
                 if (!ok) break;
-                if (have_next && s + 2 == steps) commit_elected(kv_empty);
+                if (have_next && s + 2 == steps) commit_lead(lead, kv_empty);
             }
             if (!ok) break;
-            commit_elected(acc_full);
+            commit_lead(lead, acc_full);
         }
     } else if (warp < 8) {
         // ------------------------------------------------------------------ elementwise threads
@@ -365,18 +370,18 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const long long shift = (long long)p.N - p.W;       // query q may use key k iff q >= k - shift
             const int q_min = p.causal ? (int)((long long)key - shift) : -0x7fffffff;
             const int q_min_warp = p.causal ? (int)((long long)key - lane + 31 - shift) : -0x7fffffff;   // largest in the warp
-            for (int i = i_first; i < p.q_tiles128; ++i, ++g) {
+            // a copy of the step for the tiles with masked elements: conditions in the loop cut it into short blocks
+            auto step = [&](int q0, auto masked_tag) {
+                constexpr bool kMasked = decltype(masked_tag)::value;
                 const uint32_t hh = 2 * g + wg, slot = hh % C::kSlots;
                 const float* st = sStats + slot * 128;
-                const int q0 = i * kQTile + wg * 64;              // first query of this thread's columns
                 ok = __all_sync(0xffffffffu, mbar_wait(&sdp_full[wg], g & 1, abort_p));
-                if (!ok) break;
+                if (!ok) return;
                 // already complete (the MMAs waited for it); observing it here orders the bulk-copied lse2 / delta
                 // before this thread's reads
                 ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[slot], (hh / C::kSlots) & 1, abort_p));
-                if (!ok) break;
+                if (!ok) return;
                 tc_fence_after();
-                const bool masked = q0 < q_min_warp;              // warp-uniform: some element of some lane is masked
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     uint32_t sv[32], dv_[32];
@@ -394,7 +399,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             pe[e] = ex2(fmaf(__uint_as_float(sv[c + e]), p.scale_log2e, -lv[e]));
-                            if (masked && q0 + h * 32 + c + e < q_min) pe[e] = 0.f;
+                            if (kMasked && q0 + h * 32 + c + e < q_min) pe[e] = 0.f;
                             de[e] = pe[e] * (__uint_as_float(dv_[c + e]) - dlv[e]);
                         }
                         pk[c / 2] = pack_bf16x2(pe[0], pe[1]);
@@ -409,6 +414,11 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 tc_wait_st();
                 tc_fence_before();
                 mbar_arrive(&pds_full[wg]);
+            };
+            for (int i = i_first; i < p.q_tiles128 && ok; ++i, ++g) {
+                const int q0 = i * kQTile + wg * 64;              // first query of this thread's columns
+                if (q0 < q_min_warp) step(q0, std::true_type{});  // warp-uniform: some element of some lane is masked
+                else step(q0, std::false_type{});
             }
             if (!ok) break;
             // ---------------------------------------------------------------- dK, dV of this key tile
@@ -981,6 +991,8 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         prefetch_tensormap(&map_do);
     }
     tc_fence_before();
+    after_previous();
+    let_next_start();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
@@ -1045,7 +1057,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             }
         }
     } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------------ MMA issuer (all lanes walk, one issues)
+        // ------------------------------------------------------------------ MMA issuer (all lanes walk, the lane elected once issues)
         const uint32_t idesc_s = make_idesc_bf16(kQTile, kTileN, 0, 0);      // S, dP: M = queries, N = keys
         const uint32_t idesc_dq = make_idesc_bf16(kQTile, D, 0, 1);          // dQ: A = dS in TMEM, B = K MN-major
         const uint64_t kmaj = make_smem_desc_sw128(smem_u32(smem), 16, 1024);
@@ -1053,13 +1065,14 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t desc_hi = (uint32_t)(kmaj >> 32);
         const uint32_t kmaj_lo = (uint32_t)kmaj, mnmaj_lo = (uint32_t)mnmaj;
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+        const uint32_t lead = elect_one() ? 1u : 0u;
         auto issue_r = [&](int i, int a_byte_off, int b_byte_off) {        // R_i = A B^T (contraction over d)
             const uint32_t a_lo = kmaj_lo + (uint32_t)(a_byte_off >> 4), b_lo = kmaj_lo + (uint32_t)(b_byte_off >> 4);
             const uint32_t d = tmem_u + C::kColR + i * kTileN;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t off16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4;
-                if (elect_one()) mma_ss_parts(d, a_lo + off16, b_lo + off16, desc_hi, idesc_s, kk > 0);
+                mma_ss_lead(lead, d, a_lo + off16, b_lo + off16, desc_hi, idesc_s, kk > 0);
             }
         };
         auto issue_dq = [&](int i, int k_byte_off, bool accumulate) {       // dQ_i += dS_i K (contraction over keys)
@@ -1067,7 +1080,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const uint32_t d = tmem_u + C::kColDQ + i * D, a = tmem_u + C::kColR + i * kTileN;
 #pragma unroll
             for (int kk = 0; kk < kTileN / 16; ++kk)
-                if (elect_one()) mma_ts_parts(d, a + kk * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_dq, (accumulate || kk > 0) ? 1u : 0u);
+                mma_ts_lead(lead, d, a + kk * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_dq, (accumulate || kk > 0) ? 1u : 0u);
         };
         uint32_t kit = 0, vit = 0, seg_idx = 0;
         uint32_t n_step[2] = {0, 0};
@@ -1089,7 +1102,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             for (int i = 0; i < 2; ++i)
                 if (cq[i] > 0) {
                     issue_r(i, C::kOffQ + i * C::kTileBytes, C::kOffK + ks * C::kTileBytes);
-                    commit_elected(&s_full[i]);
+                    commit_lead(lead, &s_full[i]);
                 }
             for (int j = 0; j < cnt && ok; ++j) {
                 const uint32_t vs = vit % C::kVSlots;
@@ -1102,13 +1115,13 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                         if (!ok) break;
                         tc_fence_after();
                         issue_r(i, C::kOffDO + i * C::kTileBytes, C::kOffV + vs * C::kTileBytes);   // dP over S
-                        commit_elected(&dp_full[i]);
+                        commit_lead(lead, &dp_full[i]);
                     }
                 }
                 if (!ok) break;
-                commit_elected(&v_empty[vs]);
+                commit_lead(lead, &v_empty[vs]);
                 const bool have_next = j + 1 < cnt;
-                if (!have_next) commit_elected(qdo_empty);       // Q and dout of this segment have been read for the last time
+                if (!have_next) commit_lead(lead, qdo_empty);       // Q and dout of this segment have been read for the last time
                 uint32_t nks = 0;
                 if (have_next) {
                     nks = (kit + 1) % C::kKSlots;
@@ -1126,16 +1139,16 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     if (have_next && j + 1 < cq[i]) {
                         tc_fence_after();
                         issue_r(i, C::kOffQ + i * C::kTileBytes, C::kOffK + nks * C::kTileBytes);
-                        commit_elected(&s_full[i]);
+                        commit_lead(lead, &s_full[i]);
                     }
                 }
                 if (!ok) break;
-                commit_elected(&k_empty[ks]);
+                commit_lead(lead, &k_empty[ks]);
                 ++kit;
                 ks = nks;
             }
             if (!ok) break;
-            commit_elected(dq_done);
+            commit_lead(lead, dq_done);
             ++seg_idx;
         }
     }
@@ -1168,13 +1181,13 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const bool row_ok = row < p.W;
             const float l2 = row_ok ? p.lse2[(long long)s.bh * p.Wpad + row] : CUDART_INF_F;
             const float dl = row_ok ? p.delta[(long long)s.bh * p.Wpad + row] : 0.f;
-            for (int j = 0; j < cnt_i; ++j) {
+            // a copy of the step for the tiles with masked columns (the last ones of a segment)
+            auto step = [&](int j, auto masked_tag) {
+                constexpr bool kMasked = decltype(masked_tag)::value;
                 ok = __all_sync(0xffffffffu, mbar_wait(&s_full[i], n & 1, abort_p));
-                if (!ok) break;
+                if (!ok) return;
                 tc_fence_after();
-                const int k0 = (s.t_begin + j) * kTileN;
-                const bool masked = k0 + kTileN > lim_warp;
-                const int nvalid = lim_row - k0;
+                const int nvalid = lim_row - (s.t_begin + j) * kTileN;
                 uint32_t sv[kTileN / 32][32];
 #pragma unroll
                 for (int c = 0; c < kTileN / 32; ++c) tmem_ld32_async(tR + c * 32, sv[c]);
@@ -1186,11 +1199,11 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
                 for (int e = 0; e < kTileN; ++e) {
                     float pe = ex2(fmaf(__uint_as_float(sv[e >> 5][e & 31]), p.scale_log2e, -l2));
-                    if (masked && e >= nvalid) pe = 0.f;
+                    if (kMasked && e >= nvalid) pe = 0.f;
                     sv[e >> 5][e & 31] = __float_as_uint(pe);
                 }
                 ok = __all_sync(0xffffffffu, mbar_wait(&dp_full[i], n & 1, abort_p));
-                if (!ok) break;
+                if (!ok) return;
                 tc_fence_after();
 #pragma unroll
                 for (int c = 0; c < kTileN / 16; ++c) {
@@ -1210,7 +1223,12 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 tc_fence_before();
                 mbar_arrive(&ds_full[i]);
                 ++n;
-            }
+            };
+            int n_open = lim_warp / kTileN - s.t_begin;            // steps before the first one with a masked column
+            n_open = n_open < 0 ? 0 : (n_open < cnt_i ? n_open : cnt_i);
+            int j = 0;
+            for (; j < n_open && ok; ++j) step(j, std::false_type{});
+            for (; j < cnt_i && ok; ++j) step(j, std::true_type{});
             if (!ok) break;
             const uint32_t my_seg = seg_idx;
             if (!skipped) ++seg_idx;
@@ -1277,6 +1295,8 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 template <int D>
 __global__ void __launch_bounds__(256)
 bwd_dq_reduce_kernel(const BwdParams p) {
+    after_previous();
+    let_next_start();
     constexpr int CPL = D / 32;
     const int blocks_per_tile = kTileM / 8;
     const int part = blockIdx.x % blocks_per_tile;
@@ -1346,20 +1366,17 @@ int launch_d(const void* q, const void* k, const void* v, const void* out, const
     pa.total_units = bh * p.key_tiles;
     pa.n_groups = 0; pa.q_tiles = 0; pa.schedule = 0;
     const long long ctas_a = pa.total_units < num_sms ? pa.total_units : num_sms;
-    bwd_dkdv_tc_kernel<D><<<(unsigned)ctas_a, ACfg<D>::kThreads, ACfg<D>::kSmemBytes, st>>>(mq64, mk, mv, mdo64, pa);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(bwd_dkdv_tc_kernel<D>, (unsigned)ctas_a, ACfg<D>::kThreads, ACfg<D>::kSmemBytes, st, mq64, mk, mv, mdo64, pa));
     // dQ: the forward's plan
     BwdParams pb = p;
     pb.total_units = plan.total_units; pb.n_groups = plan.n_groups; pb.q_tiles = plan.q_tiles; pb.schedule = plan.schedule;
     if (plan.n_groups > kMaxGroups) return TLIN_ERR_UNSUPPORTED;
     GroupStarts starts;
     fwd_group_starts(plan, &starts);
-    bwd_dq_tc_kernel<D><<<plan.n_ctas, BCfg<D>::kThreads, BCfg<D>::kSmemBytes, st>>>(mq, mk, mv, mdo, pb, starts);
-    TLIN_CUDA_CHECK(cudaGetLastError());
+    TLIN_CUDA_CHECK(launch_overlapped(bwd_dq_tc_kernel<D>, plan.n_ctas, BCfg<D>::kThreads, BCfg<D>::kSmemBytes, st, mq, mk, mv, mdo, pb, starts));
     count_launch(3);
     if (plan.uses_workspace) {
-        bwd_dq_reduce_kernel<D><<<(unsigned)(bh * plan.q_tiles * (kTileM / 8)), 256, 0, st>>>(pb);
-        TLIN_CUDA_CHECK(cudaGetLastError());
+        TLIN_CUDA_CHECK(launch_overlapped(bwd_dq_reduce_kernel<D>, (unsigned)(bh * plan.q_tiles * (kTileM / 8)), 256, 0, st, pb));
         count_launch();
     }
     return TLIN_OK;
