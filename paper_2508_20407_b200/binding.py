@@ -2,17 +2,22 @@
 
 Argument marshalling only: every function takes torch tensors (device memory, streams) and hands
 raw pointers and sizes to libtlin.so.  No attention arithmetic happens here and there is no
-fallback: if the shared library is missing or a call fails, an exception is raised.
+fallback: if the shared library is missing or a call fails, an exception is raised.  The entry
+points that are called per layer and token are marshalled by the extension module ``_fastcall``
+(csrc/fastcall.cpp), the others through ctypes.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libtlin.so")
+FASTCALL_PATH = os.path.join(_HERE, "_fastcall.so")
 
 TLIN_OK = 0
 ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_ARCH = -1, -2, -3, -4, -5, -6
@@ -111,6 +116,23 @@ def lib():
     return _lib
 
 
+_fast = None
+
+
+def _native():
+    """The extension module that marshals the hot entry points; raises if it has not been built."""
+    global _fast
+    if _fast is None:
+        lib()
+        if not os.path.exists(FASTCALL_PATH):
+            raise RuntimeError(f"{FASTCALL_PATH} is missing: build it with `python -m paper_2508_20407_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("_fastcall", FASTCALL_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_fastcall", FASTCALL_PATH, loader=loader))
+        loader.exec_module(module)
+        _fast = module
+    return _fast
+
+
 def status_string(status: int) -> str:
     return lib().tlin_status_string(status).decode()
 
@@ -197,15 +219,12 @@ def ensure_workspace(nbytes: int, device="cuda"):
 # ------------------------------------------------------------------ compute
 def tlin_attn_forward(q, k, v, out=None, lse=None, causal_window=1, stream=None):
     """bf16 forward.  q [B,H,W,d], k,v [B,H,N,d] -> (out [B,H,W,d] bf16, lse [B,H,W] fp32)."""
-    B, H, W, d = q.shape
-    N = k.shape[2]
-    _dev(q, torch.bfloat16, (B, H, W, d), "q")
-    _dev(k, torch.bfloat16, (B, H, N, d), "k")
-    _dev(v, torch.bfloat16, (B, H, N, d), "v")
-    out, lse = _out_and_lse(q, out, lse, (B, H, W))
-    ensure_workspace(workspace_bytes_forward(B, H, N, W, d, causal_window), q.device)
-    _check(lib().tlin_attn_forward(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, N, W, d,
-                                   int(causal_window), _stream(stream)), "tlin_attn_forward")
+    n, causal = _fast or _native(), int(causal_window)
+    if q.is_cuda:
+        ensure_workspace(n.workspace_forward(q, k, -1, causal), q.device)
+    rc, out, lse = n.forward(0, q, k, v, 0, out, lse, causal, stream)
+    if rc:
+        raise TlinError(rc, "tlin_attn_forward")
     return out, lse
 
 
@@ -231,15 +250,12 @@ def tlin_attn_forward_prefixes(q, k, v, n_keys, out=None, lse=None, causal_windo
 
 def tlin_attn_forward_cache(q, k_cache, v_cache, n_keys, out=None, lse=None, causal_window=1, stream=None):
     """Cache-miss forward over the first ``n_keys`` rows of decode caches [B,H,Ncap,d], in place."""
-    B, H, W, d = q.shape
-    Ncap = k_cache.shape[2]
-    _dev(q, torch.bfloat16, (B, H, W, d), "q")
-    _dev(k_cache, torch.bfloat16, (B, H, Ncap, d), "k_cache")
-    _dev(v_cache, torch.bfloat16, (B, H, Ncap, d), "v_cache")
-    out, lse = _out_and_lse(q, out, lse, (B, H, W))
-    ensure_workspace(workspace_bytes_forward(B, H, int(n_keys), W, d, causal_window), q.device)
-    _check(lib().tlin_attn_forward_cache(_ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(out), _ptr(lse), B, H, Ncap, int(n_keys),
-                                         W, d, int(causal_window), _stream(stream)), "tlin_attn_forward_cache")
+    n, causal, n_keys = _fast or _native(), int(causal_window), int(n_keys)
+    if q.is_cuda and n_keys > 0:
+        ensure_workspace(n.workspace_forward(q, k_cache, n_keys, causal), q.device)
+    rc, out, lse = n.forward(2, q, k_cache, v_cache, n_keys, out, lse, causal, stream)
+    if rc:
+        raise TlinError(rc, "tlin_attn_forward_cache")
     return out, lse
 
 
@@ -271,9 +287,9 @@ def make_problem_table(problems):
 
 def tlin_attn_forward_batched(problems, stream=None):
     """One launch for a list of problems (q, k, v, out, lse, n_keys, causal_window) sharing one head size."""
-    arr, _keep = make_problem_table(problems)
-    d = problems[0][0].shape[-1]
-    _check(lib().tlin_attn_forward_batched(ctypes.cast(arr, ctypes.c_void_p), len(problems), d, _stream(stream)), "tlin_attn_forward_batched")
+    rc = (_fast or _native()).forward_batched(problems, stream)
+    if rc:
+        raise TlinError(rc, "tlin_attn_forward_batched")
 
 
 def tlin_plan_batched(problem_array, num_sms=0):
@@ -287,33 +303,19 @@ def tlin_plan_batched(problem_array, num_sms=0):
 
 def tlin_attn_forward_f32(q, k, v, out=None, lse=None, causal_window=1, stream=None):
     """fp32 forward (CUDA-core kernel)."""
-    B, H, W, d = q.shape
-    N = k.shape[2]
-    _dev(q, torch.float32, (B, H, W, d), "q")
-    _dev(k, torch.float32, (B, H, N, d), "k")
-    _dev(v, torch.float32, (B, H, N, d), "v")
-    out, lse = _out_and_lse(q, out, lse, (B, H, W))
-    _check(lib().tlin_attn_forward_f32(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, N, W, d,
-                                       int(causal_window), _stream(stream)), "tlin_attn_forward_f32")
+    rc, out, lse = (_fast or _native()).forward(1, q, k, v, 0, out, lse, int(causal_window), stream)
+    if rc:
+        raise TlinError(rc, "tlin_attn_forward_f32")
     return out, lse
 
 
-def _backward(fn_name, dtype, q, k, v, out, lse, dout, dq, dk, dv, causal_window, stream):
-    B, H, W, d = q.shape
-    N = k.shape[2]
-    for t, shape, name in ((q, (B, H, W, d), "q"), (k, (B, H, N, d), "k"), (v, (B, H, N, d), "v"),
-                           (out, (B, H, W, d), "out"), (dout, (B, H, W, d), "dout")):
-        _dev(t, dtype, shape, name)
-    _dev(lse, torch.float32, (B, H, W), "lse")
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(k) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    _dev(dq, dtype, (B, H, W, d), "dq")
-    _dev(dk, dtype, (B, H, N, d), "dk")
-    _dev(dv, dtype, (B, H, N, d), "dv")
-    ensure_workspace(workspace_bytes_backward(B, H, N, W, d), q.device)
-    _check(getattr(lib(), fn_name)(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), _ptr(dout), _ptr(dq), _ptr(dk),
-                                   _ptr(dv), B, H, N, W, d, int(causal_window), _stream(stream)), fn_name)
+def _backward(f32, q, k, v, out, lse, dout, dq, dk, dv, causal_window, stream):
+    if q.is_cuda and q.dim() == 4:
+        B, H, W, d = q.shape
+        ensure_workspace(workspace_bytes_backward(B, H, k.shape[2], W, d), q.device)
+    rc, dq, dk, dv = (_fast or _native()).backward(f32, q, k, v, out, lse, dout, dq, dk, dv, int(causal_window), stream)
+    if rc:
+        raise TlinError(rc, "tlin_attn_backward_f32" if f32 else "tlin_attn_backward")
     return dq, dk, dv
 
 
@@ -321,12 +323,12 @@ def tlin_attn_backward(q, k, v, out, lse, dout, dq=None, dk=None, dv=None, causa
     """bf16 backward of ``tlin_attn_forward``: (dq [B,H,W,d], dk, dv [B,H,N,d]) for the loss gradient ``dout``.
 
     ``out`` and ``lse`` are the forward's results for the same q, k, v and causal_window."""
-    return _backward("tlin_attn_backward", torch.bfloat16, q, k, v, out, lse, dout, dq, dk, dv, causal_window, stream)
+    return _backward(False, q, k, v, out, lse, dout, dq, dk, dv, causal_window, stream)
 
 
 def tlin_attn_backward_f32(q, k, v, out, lse, dout, dq=None, dk=None, dv=None, causal_window=1, stream=None):
     """fp32 backward of ``tlin_attn_forward_f32`` (CUDA-core kernels)."""
-    return _backward("tlin_attn_backward_f32", torch.float32, q, k, v, out, lse, dout, dq, dk, dv, causal_window, stream)
+    return _backward(True, q, k, v, out, lse, dout, dq, dk, dv, causal_window, stream)
 
 
 def tlin_attn_forward_host(q_h, k_h, v_h, out_h, lse_h, q_d, k_d, v_d, out_d, lse_d, causal_window=1, stream=None):
@@ -345,59 +347,36 @@ def tlin_attn_forward_host(q_h, k_h, v_h, out_h, lse_h, q_d, k_d, v_d, out_d, ls
 
 def tlin_decode_step(q_new, k_new, v_new, k_cache, v_cache, pos, out=None, lse=None, stream=None):
     """One cached decode step: appends k_new/v_new at row pos, attends q_new over rows [0,pos]."""
-    B, H, Ncap, d = k_cache.shape
-    for t, n in ((q_new, "q_new"), (k_new, "k_new"), (v_new, "v_new")):
-        _dev(t, torch.bfloat16, (B, H, 1, d), n)
-    _dev(k_cache, torch.bfloat16, (B, H, Ncap, d), "k_cache")
-    _dev(v_cache, torch.bfloat16, (B, H, Ncap, d), "v_cache")
-    if out is None:
-        out = torch.empty_like(q_new)
-    if lse is None:
-        lse = torch.empty((B, H), dtype=torch.float32, device=q_new.device)
-    ensure_workspace(workspace_bytes_decode(B, H, Ncap, d), q_new.device)
-    _check(lib().tlin_decode_step(_ptr(q_new), _ptr(k_new), _ptr(v_new), _ptr(k_cache), _ptr(v_cache),
-                                  _ptr(out), _ptr(lse), B, H, Ncap, int(pos), d, _stream(stream)), "tlin_decode_step")
+    n = _fast or _native()
+    if q_new.is_cuda:
+        ensure_workspace(n.workspace_decode(k_cache), q_new.device)
+    rc, out, lse = n.decode(0, q_new, k_new, v_new, k_cache, v_cache, None, None, int(pos), out, lse, stream)
+    if rc:
+        raise TlinError(rc, "tlin_decode_step")
     return out, lse
 
 
 def tlin_decode_step_fp8(q_new, k_new, v_new, k_cache, v_cache, k_scale, v_scale, pos, out=None, lse=None, stream=None):
     """Decode step over an 8-bit cache: k_cache, v_cache are uint8 [B,H,Ncap,d] (E4M3 codes), value = code * scale[b,h];
     k_scale, v_scale fp32 device tensors [B,H]."""
-    B, H, Ncap, d = k_cache.shape
-    for t, n in ((q_new, "q_new"), (k_new, "k_new"), (v_new, "v_new")):
-        _dev(t, torch.bfloat16, (B, H, 1, d), n)
-    _dev(k_cache, torch.uint8, (B, H, Ncap, d), "k_cache")
-    _dev(v_cache, torch.uint8, (B, H, Ncap, d), "v_cache")
-    _dev(k_scale, torch.float32, (B, H), "k_scale")
-    _dev(v_scale, torch.float32, (B, H), "v_scale")
-    if out is None:
-        out = torch.empty_like(q_new)
-    if lse is None:
-        lse = torch.empty((B, H), dtype=torch.float32, device=q_new.device)
-    ensure_workspace(workspace_bytes_decode(B, H, Ncap, d), q_new.device)
-    _check(lib().tlin_decode_step_fp8(_ptr(q_new), _ptr(k_new), _ptr(v_new), _ptr(k_cache), _ptr(v_cache), _ptr(k_scale),
-                                      _ptr(v_scale), _ptr(out), _ptr(lse), B, H, Ncap, int(pos), d, _stream(stream)),
-           "tlin_decode_step_fp8")
+    n = _fast or _native()
+    if q_new.is_cuda:
+        ensure_workspace(n.workspace_decode(k_cache), q_new.device)
+    rc, out, lse = n.decode(1, q_new, k_new, v_new, k_cache, v_cache, k_scale, v_scale, int(pos), out, lse, stream)
+    if rc:
+        raise TlinError(rc, "tlin_decode_step_fp8")
     return out, lse
 
 
 def tlin_decode_step_ragged(q_new, k_new, v_new, k_cache, v_cache, pos, max_pos, out=None, lse=None, stream=None):
     """Decode step with one cache length per sequence: ``pos`` is an int32 device tensor of shape [B],
     ``max_pos`` a host-side upper bound of its entries."""
-    B, H, Ncap, d = k_cache.shape
-    for t, n in ((q_new, "q_new"), (k_new, "k_new"), (v_new, "v_new")):
-        _dev(t, torch.bfloat16, (B, H, 1, d), n)
-    _dev(k_cache, torch.bfloat16, (B, H, Ncap, d), "k_cache")
-    _dev(v_cache, torch.bfloat16, (B, H, Ncap, d), "v_cache")
-    _dev(pos, torch.int32, (B,), "pos")
-    if out is None:
-        out = torch.empty_like(q_new)
-    if lse is None:
-        lse = torch.empty((B, H), dtype=torch.float32, device=q_new.device)
-    ensure_workspace(workspace_bytes_decode(B, H, Ncap, d), q_new.device)
-    _check(lib().tlin_decode_step_ragged(_ptr(q_new), _ptr(k_new), _ptr(v_new), _ptr(k_cache), _ptr(v_cache),
-                                         _ptr(out), _ptr(lse), B, H, Ncap, _ptr(pos), int(max_pos), d, _stream(stream)),
-           "tlin_decode_step_ragged")
+    n = _fast or _native()
+    if q_new.is_cuda:
+        ensure_workspace(n.workspace_decode(k_cache), q_new.device)
+    rc, out, lse = n.decode(2, q_new, k_new, v_new, k_cache, v_cache, pos, None, int(max_pos), out, lse, stream)
+    if rc:
+        raise TlinError(rc, "tlin_decode_step_ragged")
     return out, lse
 
 

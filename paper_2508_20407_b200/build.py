@@ -1,14 +1,18 @@
-"""Builds libtlin.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libtlin.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the Python extension module _fastcall.so
+that marshals its hot entry points."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "_build")
 LIB = os.path.join(HERE, "libtlin.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")
 SOURCES = ["api.cu", "plan.cu", "fwd_simt.cu", "fwd_tc.cu", "decode.cu", "merge.cu", "bwd_simt.cu", "bwd_tc.cu", "debug.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -54,6 +58,18 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run([nvcc, "-shared", "-o", LIB] + objs + ["-cudart", "static"], capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("link failed:\n" + r.stdout + r.stderr)
+    source = os.path.join(CSRC, "fastcall.cpp")
+    if force or _stale(FASTCALL, [source, headers[-1]]):
+        torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+        cuda = os.path.dirname(os.path.dirname(nvcc)) if os.path.sep in nvcc else "/usr/local/cuda"
+        cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-o", FASTCALL, source,
+               "-I" + os.path.join(torch_dir, "include"), "-I" + os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+               "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"], "-L" + os.path.join(torch_dir, "lib"),
+               "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lc10", "-lc10_cuda", "-L" + HERE, "-l:libtlin.so",
+               "-Wl,-rpath,$ORIGIN"]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError("g++ failed: " + " ".join(cmd) + "\n" + r.stdout + r.stderr)
     return LIB
 
 
