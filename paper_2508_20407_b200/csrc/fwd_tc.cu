@@ -639,104 +639,114 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
     }
 }
 
-// Combines the partial results of every (b,h) whose key tiles were split between groups.
-// One CTA per 8 query rows of a (b,h, q-tile pair): 8 warps, one row each, 4 (or 2) columns per lane.
-constexpr int kMergeRows = 8;            // one row per warp: many small CTAs hide the latency of the scattered partial reads
-constexpr int kMaxParts = 8;          // more partials than this per row are merged in a slower loop
+// Combines the partial results of every (b,h) whose key tiles were split between groups.  Bound by the latency of its scattered
+// reads (the partials are in L2): a row belongs to the fewest lanes that read it 16 bytes at a time, four parts of a row are on
+// their way at once, a warp takes kPasses groups of rows, and nothing is shared between threads.
+// Against one row per warp, 4- to 8-byte reads and the list of parts worked out by one thread before a barrier, whole calls: B1 H4
+// N1024 W128 d64 10.0 -> 8.2 us, B4 H16 N8192 W256 d64 60 -> 56 us, B4 H32 N8192 W1024 d128 520 -> 503 us.  One pass is best while
+// the CTAs are few (10.0 -> 8.2 us against 11.1 with four, d40 33.5 against 35.7); four from 65536 rows on (503 against 510 us).
+constexpr int kMergeParts = 4;           // parts read at once
+template <int D, int kPasses>
+struct MergeCfg {
+    static constexpr int kLanes = D / 4 < 32 ? D / 4 : 32;            // lanes per row
+    static constexpr int kVecs = D / 4 / kLanes;                      // 16-byte pieces per lane
+    static constexpr int kWarpRows = 32 / kLanes;
+    static constexpr int kRows = 8 * kWarpRows * kPasses;             // rows per CTA
+};
 
-template <int D, bool kAny>
+template <int D, bool kAny, int kPasses>
 __global__ void __launch_bounds__(256)
-fwd_merge_kernel(const Params p) {
-    constexpr int CPL = D / 32;                           // columns per lane
+fwd_merge_kernel(const __grid_constant__ Params p, const __grid_constant__ GroupStarts starts) {
+    using M = MergeCfg<D, kPasses>;
     constexpr int kTileM = Cfg<D>::kRows;
+    static_assert(kTileM % M::kRows == 0, "a CTA's rows lie in one tile");
+    constexpr int kBlocksPerTile = kTileM / M::kRows;
     const int d = kAny ? p.d : D;
-    const int blocks_per_tile = kTileM / kMergeRows;
-    const int quarter = blockIdx.x % blocks_per_tile;
-    const int tile_id = blockIdx.x / blocks_per_tile;     // bh * q_tiles + qt
+    const int tile_id = blockIdx.x / kBlocksPerTile;                  // bh * q_tiles + qt
     const int bh = tile_id / p.q_tiles, qt = tile_id - bh * p.q_tiles;
+    // groups holding the first and the last unit of this (b,h): largest g with starts.u[g] <= x
+    const long long x0 = (long long)bh * p.key_tiles, x1 = x0 + p.key_tiles - 1;
+    int g_lo = (int)((float)x0 * (float)p.n_groups / (float)p.total_units);
+    while (g_lo > 0 && starts.u[g_lo] > x0) --g_lo;
+    while (g_lo + 1 < p.n_groups && starts.u[g_lo + 1] <= x0) ++g_lo;
+    int g_hi = g_lo;
+    while (g_hi + 1 < p.n_groups && starts.u[g_hi + 1] <= x1) ++g_hi;
     after_previous();
     let_next_start();
-    __shared__ const float* part_base[kMaxParts];
-    __shared__ int n_parts_s, g_lo_s;
-    if (threadIdx.x == 0) {
-        const unsigned long long T = (unsigned long long)p.key_tiles, U = (unsigned long long)p.total_units, G = (unsigned)p.n_groups;
-        // groups holding the first and the last unit of this (b,h): largest g with floor(g*U/G) <= x
-        const unsigned long long x0 = (unsigned long long)bh * T, x1 = x0 + T - 1;
-        const int g_lo = (int)(((x0 + 1) * G - 1) / U), g_hi = (int)(((x1 + 1) * G - 1) / U);
-        g_lo_s = g_lo;
-        n_parts_s = g_hi - g_lo + 1;
-        for (int g = g_lo; g <= g_hi && g - g_lo < kMaxParts; ++g) {
-            const int cta = g * p.q_tiles + qt;
-            const int slot = bh == (int)((((unsigned long long)g * U) / G) / T) ? 0 : 1;
-            part_base[g - g_lo] = p.ws + ((long long)cta * 2 + slot) * (long long)kTileM * (d + 1);
-        }
+    if (g_hi == g_lo) return;                             // written directly by the attention kernel
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, piece = lane % M::kLanes;
+    const int rr0 = (blockIdx.x % kBlocksPerTile) * M::kRows + warp * (M::kWarpRows * kPasses) + lane / M::kLanes;
+    // slot 0 of a CTA holds its group's first segment (the group starts in this (b,h)), slot 1 a later one
+    auto part_of = [&](int g) { return p.ws + ((long long)(g * p.q_tiles + qt) * 2 + (starts.u[g] >= x0 ? 0 : 1)) * (long long)kTileM * (d + 1); };
+    float m[kPasses], z[kPasses];
+    float4 acc[kPasses][M::kVecs];
+#pragma unroll
+    for (int ps = 0; ps < kPasses; ++ps) {
+        m[ps] = -CUDART_INF_F;
+        z[ps] = 0.f;
+#pragma unroll
+        for (int v = 0; v < M::kVecs; ++v) acc[ps][v] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    __syncthreads();
-    const int n_parts = n_parts_s;
-    if (n_parts <= 1) return;                             // written directly by the attention kernel
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool owns = !kAny || lane * CPL < d;            // d is a multiple of 8: a lane's columns are inside or outside as a whole
-    for (int rq = warp; rq < kMergeRows; rq += 8) {
-        const int rr = quarter * kMergeRows + rq;         // row inside the 256-row tile
-        const int row = qt * kTileM + rr;
-        if (row >= p.W) break;
-        float m = -CUDART_INF_F;
-        if (n_parts <= kMaxParts) {
-            float ls[kMaxParts];
+    for (int g0 = g_lo; g0 <= g_hi; g0 += kMergeParts) {
+        const float* base[kMergeParts];
 #pragma unroll
-            for (int i = 0; i < kMaxParts; ++i) {
-                ls[i] = i < n_parts ? part_base[i][(long long)kTileM * d + rr] : -CUDART_INF_F;
-                m = fmaxf(m, ls[i]);
-            }
-            float z = 0.f, acc[CPL];
+        for (int i = 0; i < kMergeParts; ++i) base[i] = g0 + i <= g_hi ? part_of(g0 + i) : nullptr;
 #pragma unroll
-            for (int e = 0; e < CPL; ++e) acc[e] = 0.f;
+        for (int ps = 0; ps < kPasses; ++ps) {
+            const int rr = rr0 + ps * M::kWarpRows;
+            if (qt * kTileM + rr >= p.W) continue;
+            float ls[kMergeParts];
+            float4 x[kMergeParts][M::kVecs];
 #pragma unroll
-            for (int i = 0; i < kMaxParts; ++i) {
-                if (i < n_parts) {
-                    const float w = expf(ls[i] - m);      // -inf (empty part) -> 0
-                    z += w;
-                    if (!owns) continue;
-                    const float* src = part_base[i] + (long long)rr * d + lane * CPL;
+            for (int i = 0; i < kMergeParts; ++i) {
+                ls[i] = -CUDART_INF_F;
 #pragma unroll
-                    for (int e = 0; e < CPL; ++e) acc[e] = fmaf(w, src[e], acc[e]);
+                for (int v = 0; v < M::kVecs; ++v) x[i][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (base[i] != nullptr) {
+                    ls[i] = base[i][(long long)kTileM * d + rr];
+#pragma unroll
+                    for (int v = 0; v < M::kVecs; ++v) {
+                        const int c = (v * M::kLanes + piece) * 4;
+                        if (!kAny || c < d) x[i][v] = *reinterpret_cast<const float4*>(base[i] + (long long)rr * d + c);
+                    }
                 }
             }
-            const float inv = 1.f / z;
-            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)bh * p.W + row) * d + lane * CPL;
+            float mn = m[ps];
 #pragma unroll
-            for (int e = 0; e < CPL; e += 2)
-                if (owns)
-                    *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
-            if (p.lse != nullptr && lane == 0) p.lse[(long long)bh * p.W + row] = m + logf(z);
-        } else {
-            // many small groups per (b,h): recompute the slot addresses on the fly
-            const unsigned long long T = (unsigned long long)p.key_tiles, U = (unsigned long long)p.total_units, G = (unsigned)p.n_groups;
-            auto base_of = [&](int g) {
-                const int cta = g * p.q_tiles + qt;
-                const int slot = bh == (int)((((unsigned long long)g * U) / G) / T) ? 0 : 1;
-                return p.ws + ((long long)cta * 2 + slot) * (long long)kTileM * (d + 1);
-            };
-            for (int i = 0; i < n_parts; ++i) m = fmaxf(m, base_of(g_lo_s + i)[(long long)kTileM * d + rr]);
-            float z = 0.f, acc[CPL];
+            for (int i = 0; i < kMergeParts; ++i) mn = fmaxf(mn, ls[i]);
+            if (mn == -CUDART_INF_F) continue;            // every part so far is empty
+            const float old = expf(m[ps] - mn);
+            m[ps] = mn;
+            z[ps] *= old;
 #pragma unroll
-            for (int e = 0; e < CPL; ++e) acc[e] = 0.f;
-            for (int i = 0; i < n_parts; ++i) {
-                const float* base = base_of(g_lo_s + i);
-                const float w = expf(base[(long long)kTileM * d + rr] - m);
-                z += w;
-                if (!owns) continue;
+            for (int v = 0; v < M::kVecs; ++v) { acc[ps][v].x *= old; acc[ps][v].y *= old; acc[ps][v].z *= old; acc[ps][v].w *= old; }
 #pragma unroll
-                for (int e = 0; e < CPL; ++e) acc[e] = fmaf(w, base[(long long)rr * d + lane * CPL + e], acc[e]);
+            for (int i = 0; i < kMergeParts; ++i) {
+                const float w = expf(ls[i] - mn);         // -inf (empty part) -> 0
+                z[ps] += w;
+#pragma unroll
+                for (int v = 0; v < M::kVecs; ++v) {
+                    acc[ps][v].x = fmaf(w, x[i][v].x, acc[ps][v].x);
+                    acc[ps][v].y = fmaf(w, x[i][v].y, acc[ps][v].y);
+                    acc[ps][v].z = fmaf(w, x[i][v].z, acc[ps][v].z);
+                    acc[ps][v].w = fmaf(w, x[i][v].w, acc[ps][v].w);
+                }
             }
-            const float inv = 1.f / z;
-            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)bh * p.W + row) * d + lane * CPL;
-#pragma unroll
-            for (int e = 0; e < CPL; e += 2)
-                if (owns)
-                    *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
-            if (p.lse != nullptr && lane == 0) p.lse[(long long)bh * p.W + row] = m + logf(z);
         }
+    }
+#pragma unroll
+    for (int ps = 0; ps < kPasses; ++ps) {
+        const int row = qt * kTileM + rr0 + ps * M::kWarpRows;
+        if (row >= p.W) continue;
+        const float inv = 1.f / z[ps];
+        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)bh * p.W + row) * d;
+#pragma unroll
+        for (int v = 0; v < M::kVecs; ++v) {
+            const int c = (v * M::kLanes + piece) * 4;
+            if (!kAny || c < d)
+                *reinterpret_cast<uint2*>(dst + c) = make_uint2(pack_bf16x2(acc[ps][v].x * inv, acc[ps][v].y * inv), pack_bf16x2(acc[ps][v].z * inv, acc[ps][v].w * inv));
+        }
+        if (p.lse != nullptr && piece == 0) p.lse[(long long)bh * p.W + row] = m[ps] + logf(z[ps]);
     }
 }
 
@@ -764,7 +774,12 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
     TLIN_CUDA_CHECK(launch_overlapped(fwd_tc_kernel<D, kForm>, plan.n_ctas, kThreads, C::kSmemBytes, st, maps, p, starts));
     count_launch();
     if (plan.uses_workspace) {
-        TLIN_CUDA_CHECK(launch_overlapped(fwd_merge_kernel<D, kForm == kAnyHead>, (unsigned)(bh * plan.q_tiles * (C::kRows / kMergeRows)), 256, 0, st, p));
+        constexpr bool kAny = kForm == kAnyHead;
+        const long long tiles = bh * plan.q_tiles;
+        if (tiles * C::kRows >= 65536)
+            TLIN_CUDA_CHECK(launch_overlapped(fwd_merge_kernel<D, kAny, 4>, (unsigned)(tiles * (C::kRows / MergeCfg<D, 4>::kRows)), 256, 0, st, p, starts));
+        else
+            TLIN_CUDA_CHECK(launch_overlapped(fwd_merge_kernel<D, kAny, 1>, (unsigned)(tiles * (C::kRows / MergeCfg<D, 1>::kRows)), 256, 0, st, p, starts));
         count_launch();
     }
     return TLIN_OK;

@@ -593,3 +593,17 @@ def test_other_head_sizes_on_the_tensor_cores(B, H, N, W, d, causal):
     torch.cuda.synchronize()
     assert tl.tlin_get_status() == 0
     parity.check(got.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", "cache, no workspace")
+
+
+# the merge of split key ranges with many rows (several groups of rows per warp): ragged rows, both head sizes, another head size
+@pytest.mark.parametrize("B,H,N,W,d,causal", [(33, 10, 1300, 200, 64, 1), (19, 10, 900, 300, 128, 0), (19, 10, 900, 300, 96, 0), (259, 2, 2000, 100, 136, 0)])
+def test_merge_of_many_rows(B, H, N, W, d, causal):
+    plan = tl.tlin_plan_forward(B, H, N, W, d, causal)
+    assert plan.schedule == 0 and plan.uses_workspace and B * H * plan.q_tiles * plan.tile_m >= 65536
+    wl = synth.Workload("many rows", B, H, d, N, W, seed=60 + N, causal_window=causal)
+    q, k, v = synth.forward_inputs(wl, device=DEV)
+    out, lse = tl.tlin_attn_forward(q, k, v, causal_window=causal)
+    assert tl.tlin_get_status() == 0 and bool(torch.isfinite(out.float()).all()) and bool(torch.isfinite(lse).all())
+    for b, h in ((0, 0), (B // 2, H // 2), (B - 1, H - 1)):
+        ref, ref_lse = oracle.attn_forward(q[b:b + 1, h:h + 1].cpu(), k[b:b + 1, h:h + 1].cpu(), v[b:b + 1, h:h + 1].cpu(), causal)
+        parity.check(out[b:b + 1, h:h + 1].float().cpu().numpy(), lse[b:b + 1, h:h + 1].cpu().numpy(), ref, ref_lse, "bf16", f"b{b} h{h}")
