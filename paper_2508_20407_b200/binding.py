@@ -311,8 +311,7 @@ def tlin_attn_forward_f32(q, k, v, out=None, lse=None, causal_window=1, stream=N
 
 def _backward(f32, q, k, v, out, lse, dout, dq, dk, dv, causal_window, stream):
     if q.is_cuda and q.dim() == 4:
-        B, H, W, d = q.shape
-        ensure_workspace(workspace_bytes_backward(B, H, k.shape[2], W, d), q.device)
+        ensure_workspace((_fast or _native()).workspace_backward(q, k), q.device)
     rc, dq, dk, dv = (_fast or _native()).backward(f32, q, k, v, out, lse, dout, dq, dk, dv, int(causal_window), stream)
     if rc:
         raise TlinError(rc, "tlin_attn_backward_f32" if f32 else "tlin_attn_backward")
@@ -494,31 +493,10 @@ def tlin_last_launch_count() -> int:
     return int(lib().tlin_last_launch_count())
 
 
-# ------------------------------------------------------------------ autograd glue (marshalling only)
-class _AttentionFunction(torch.autograd.Function):
-    """Lets PyTorch's autograd call the library's forward and backward entry points; nothing is computed here."""
-
-    @staticmethod
-    def forward(ctx, q, k, v, causal_window):
-        f32 = q.dtype == torch.float32
-        q, k, v = q.contiguous(), k.contiguous(), v.contiguous()
-        out, lse = (tlin_attn_forward_f32 if f32 else tlin_attn_forward)(q, k, v, causal_window=causal_window)
-        ctx.save_for_backward(q, k, v, out, lse)
-        ctx.causal_window = int(causal_window)
-        ctx.f32 = f32
-        ctx.mark_non_differentiable(lse)
-        return out, lse
-
-    @staticmethod
-    def backward(ctx, dout, _dlse):
-        q, k, v, out, lse = ctx.saved_tensors
-        fn = tlin_attn_backward_f32 if ctx.f32 else tlin_attn_backward
-        dq, dk, dv = fn(q, k, v, out, lse, dout.contiguous(), causal_window=ctx.causal_window)
-        return dq, dk, dv, None
-
-
+# ------------------------------------------------------------------ autograd
 def attention(q, k, v, causal_window=1):
     """Differentiable attention for PyTorch training code: (out, lse) = tlin_attn_forward(q, k, v); gradients of `out`
     with respect to q, k, v come from tlin_attn_backward (lse is returned for merging and is not differentiable).
-    bf16 or fp32 tensors, shapes as in tlin_attn_forward."""
-    return _AttentionFunction.apply(q, k, v, causal_window)
+    bf16 or fp32 tensors, shapes as in tlin_attn_forward.  The differentiable operation is in the extension module, so that a
+    backward pass does not wait for the interpreter."""
+    return (_fast or _native()).attention(q, k, v, int(causal_window))

@@ -1,6 +1,7 @@
 // Argument marshalling of the hot entry points as a Python extension module: checks the tensors, allocates the results and calls
 // the C functions of include/tlin.h, nothing else.  A small call is over on the device in about ten microseconds; the same checks
 // and calls through Python attributes and ctypes took sixteen.
+#include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/utils/pybind.h>
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
@@ -45,7 +46,8 @@ Tensor given_or_fresh(const Opt& t, at::IntArrayRef shape, at::ScalarType dtype,
     return *t;
 }
 template <class F>
-int without_gil(F&& f) {
+int without_gil(F&& f) {                 // called with the lock held (from Python) or without it (from autograd's threads)
+    if (!PyGILState_Check()) return f();
     py::gil_scoped_release release;
     return f();
 }
@@ -58,15 +60,14 @@ size_t workspace_forward(const Tensor& q, const Tensor& k, int64_t n_keys, int c
                                         as_int(q.size(3)), causal);
 }
 // kind: 0 bf16, 1 fp32, 2 bf16 over the first n_keys rows of a cache
-Result forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, int64_t n_keys, const Opt& out_, const Opt& lse_, int causal,
-               const py::object& stream) {
+Result run_forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, int64_t n_keys, const Opt& out_, const Opt& lse_, int causal,
+                   tlin_stream_t st) {
     const int64_t B = four_dims(q, "q").size(0), H = q.size(1), W = q.size(2), d = q.size(3), N = four_dims(k, "k").size(2);
     const at::ScalarType dt = kind == 1 ? at::kFloat : at::kBFloat16;
     check(q, dt, {B, H, W, d}, "q");
     check(k, dt, {B, H, N, d}, kind == 2 ? "k_cache" : "k");
     check(v, dt, {B, H, N, d}, kind == 2 ? "v_cache" : "v");
     const Tensor out = given_or_fresh(out_, {B, H, W, d}, dt, q, "out"), lse = given_or_fresh(lse_, {B, H, W}, at::kFloat, q, "lse");
-    const tlin_stream_t st = stream_of(stream);
     const int b = as_int(B), h = as_int(H), n = as_int(N), w = as_int(W), dd = as_int(d), nk = as_int(n_keys);
     const int rc = without_gil([&] {
         const void *qp = q.data_ptr(), *kp = k.data_ptr(), *vp = v.data_ptr();
@@ -78,8 +79,14 @@ Result forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, int6
     return {rc, out, lse};
 }
 
-std::tuple<int, Tensor, Tensor, Tensor> backward(bool f32, const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out, const Tensor& lse,
-                                                 const Tensor& dout, const Opt& dq_, const Opt& dk_, const Opt& dv_, int causal, const py::object& stream) {
+Result forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, int64_t n_keys, const Opt& out, const Opt& lse, int causal,
+               const py::object& stream) {
+    return run_forward(kind, q, k, v, n_keys, out, lse, causal, stream_of(stream));
+}
+
+using Gradients = std::tuple<int, Tensor, Tensor, Tensor>;
+Gradients run_backward(bool f32, const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out, const Tensor& lse,
+                                                 const Tensor& dout, const Opt& dq_, const Opt& dk_, const Opt& dv_, int causal, tlin_stream_t st) {
     const int64_t B = four_dims(q, "q").size(0), H = q.size(1), W = q.size(2), d = q.size(3), N = four_dims(k, "k").size(2);
     const at::ScalarType dt = f32 ? at::kFloat : at::kBFloat16;
     check(q, dt, {B, H, W, d}, "q");
@@ -90,7 +97,6 @@ std::tuple<int, Tensor, Tensor, Tensor> backward(bool f32, const Tensor& q, cons
     check(lse, at::kFloat, {B, H, W}, "lse");
     const Tensor dq = given_or_fresh(dq_, {B, H, W, d}, dt, q, "dq"), dk = given_or_fresh(dk_, {B, H, N, d}, dt, q, "dk"),
                  dv = given_or_fresh(dv_, {B, H, N, d}, dt, q, "dv");
-    const tlin_stream_t st = stream_of(stream);
     const int b = as_int(B), h = as_int(H), n = as_int(N), w = as_int(W), dd = as_int(d);
     const int rc = without_gil([&] {
         if (f32)
@@ -101,6 +107,64 @@ std::tuple<int, Tensor, Tensor, Tensor> backward(bool f32, const Tensor& q, cons
                                   dk.data_ptr(), dv.data_ptr(), b, h, n, w, dd, causal, st);
     });
     return {rc, dq, dk, dv};
+}
+
+Gradients backward(bool f32, const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out, const Tensor& lse, const Tensor& dout, const Opt& dq,
+                   const Opt& dk, const Opt& dv, int causal, const py::object& stream) {
+    return run_backward(f32, q, k, v, out, lse, dout, dq, dk, dv, causal, stream_of(stream));
+}
+size_t workspace_backward(const Tensor& q, const Tensor& k) {
+    four_dims(q, "q");
+    four_dims(k, "k");
+    return tlin_workspace_bytes_backward(as_int(q.size(0)), as_int(q.size(1)), as_int(k.size(2)), as_int(q.size(2)), as_int(q.size(3)));
+}
+
+// ---- autograd: the forward and the backward entry point as one differentiable operation (nothing is computed here)
+// The Python side owns the workspace and the exception type.
+void raise(int rc, const char* where) {
+    if (rc == TLIN_OK) return;
+    py::gil_scoped_acquire lock;
+    const py::object type = py::module_::import("paper_2508_20407_b200.binding").attr("TlinError");
+    PyErr_SetObject(type.ptr(), type(rc, where).ptr());
+    throw py::error_already_set();
+}
+void ensure_workspace(size_t bytes, const Tensor& like) {
+    py::gil_scoped_acquire lock;
+    py::module_::import("paper_2508_20407_b200.binding").attr("ensure_workspace")(bytes, like.device());
+}
+
+struct Attention : public torch::autograd::Function<Attention> {
+    static torch::autograd::variable_list forward(torch::autograd::AutogradContext* ctx, const Tensor& q_in, const Tensor& k_in, const Tensor& v_in,
+                                                  int64_t causal) {
+        const Tensor q = q_in.contiguous(), k = k_in.contiguous(), v = v_in.contiguous();
+        const bool f32 = q.scalar_type() == at::kFloat;
+        if (!f32 && q.is_cuda()) ensure_workspace(workspace_forward(q, k, -1, (int)causal), q);
+        const auto [rc, out, lse] = run_forward(f32 ? 1 : 0, q, k, v, 0, std::nullopt, std::nullopt, (int)causal, (tlin_stream_t)c10::cuda::getCurrentCUDAStream().stream());
+        raise(rc, f32 ? "tlin_attn_forward_f32" : "tlin_attn_forward");
+        ctx->save_for_backward({q, k, v, out, lse});
+        ctx->saved_data["causal"] = causal;
+        ctx->mark_non_differentiable({lse});
+        return {out, lse};
+    }
+    static torch::autograd::variable_list backward(torch::autograd::AutogradContext* ctx, torch::autograd::variable_list grads) {
+        const auto saved = ctx->get_saved_variables();
+        const Tensor &q = saved[0], &k = saved[1];
+        const bool f32 = q.scalar_type() == at::kFloat;
+        const Tensor dout = grads[0].defined() ? grads[0].contiguous() : at::zeros_like(saved[3]);
+        const int causal = (int)ctx->saved_data["causal"].toInt();
+        const auto st = (tlin_stream_t)c10::cuda::getCurrentCUDAStream().stream();
+        auto [rc, dq, dk, dv] = run_backward(f32, q, k, saved[2], saved[3], saved[4], dout, std::nullopt, std::nullopt, std::nullopt, causal, st);
+        if (rc == TLIN_ERR_WORKSPACE) {      // too small so far: asking first would cost this thread a turn of the interpreter (20 us)
+            ensure_workspace(workspace_backward(q, k), q);
+            std::tie(rc, dq, dk, dv) = run_backward(f32, q, k, saved[2], saved[3], saved[4], dout, dq, dk, dv, causal, st);
+        }
+        raise(rc, f32 ? "tlin_attn_backward_f32" : "tlin_attn_backward");
+        return {dq, dk, dv, Tensor()};
+    }
+};
+std::tuple<Tensor, Tensor> attention(const Tensor& q, const Tensor& k, const Tensor& v, int64_t causal) {
+    const auto r = Attention::apply(q, k, v, causal);
+    return {r[0], r[1]};
 }
 
 size_t workspace_decode(const Tensor& k_cache) {
@@ -178,6 +242,8 @@ PYBIND11_MODULE(_fastcall, m) {
     m.def("workspace_forward", &workspace_forward);
     m.def("forward", &forward);
     m.def("backward", &backward);
+    m.def("workspace_backward", &workspace_backward);
+    m.def("attention", &attention);
     m.def("workspace_decode", &workspace_decode);
     m.def("decode", &decode);
     m.def("forward_batched", &forward_batched);

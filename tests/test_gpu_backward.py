@@ -398,3 +398,25 @@ def test_backward_both_kernel_families_agree_on_every_head_of_the_training_chunk
         assert bool((worst <= gate).all()), f"{name}: worst (b,h) ratio {float((worst / gate).max()):.3f}"
         rel = (diff.double().pow(2).sum(dim=(2, 3)) / b.double().pow(2).sum(dim=(2, 3)).clamp_min(1e-30)).sqrt()
         assert bool((rel <= REL_L2).all()), f"{name}: rel L2 {float(rel.max()):.3e}"
+
+
+def test_autograd_backward_gets_its_workspace_and_reports_errors():
+    # the differentiable operation runs its backward without the interpreter as long as the registered workspace suffices; here it
+    # does not exist when the backward starts, on a stream of its own, and the gradients equal the entry point's
+    g = torch.Generator(device="cpu").manual_seed(5)
+    q, k, v = (torch.randn(1, 3, n, 128, generator=g).to(torch.bfloat16).to(DEV).requires_grad_() for n in (200, 700, 700))
+    dout = torch.randn(1, 3, 200, 128, generator=g).to(torch.bfloat16).to(DEV)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        out, lse = tl.attention(q, k, v, 1)
+        tl.set_workspace(None)
+        got = torch.autograd.grad(out, (q, k, v), dout)
+    torch.cuda.current_stream().wait_stream(side)
+    want = tl.tlin_attn_backward(q.detach(), k.detach(), v.detach(), out.detach(), lse, dout, causal_window=1)
+    torch.cuda.synchronize()
+    assert torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+    assert float((got[0].float() - want[0].float()).abs().max()) <= 2.0 ** -7 * float(want[0].float().abs().max())
+    odd = torch.zeros(1, 1, 8, 36, dtype=torch.bfloat16, device=DEV, requires_grad=True)
+    with pytest.raises(tl.TlinError):
+        tl.attention(odd, odd, odd, 1)
