@@ -316,12 +316,15 @@ int tlin_plan_decode(int B, int H, int L, int d, int num_sms, tlin_decode_plan* 
 /* Work sharing of the tensor-core dK/dV kernel of tlin_attn_backward: its units are (b,h,128-key tile) in that order and
  * CTA `share` of `n_shares` starts at the unit returned here (share = n_shares gives the unit count B*H*ceil(N/128)).  The
  * shares are balanced by the number of 128-row query tiles each key tile has to visit, which under the window rule falls
- * towards the end of a (b,h).  -1 on bad arguments. */
+ * towards the end of a (b,h).  -1 on bad arguments.  Under the window rule, calls with few key tiles per CTA and a window that is a
+ * large part of the keys take the key tiles in descending order of cost instead, one round after the other. */
 int64_t tlin_plan_backward_share_start(int B, int H, int N, int W, int causal_window, int share, int n_shares);
 /* First unit of group g.  floor(g * total_units / n_groups), except under schedule 1 with the window rule: there a
  * (b,h,query tile) problem costs the key tiles its rows may use (+3 for starting and finishing it and for its masked steps), which grows with the
  * query tile, and when there are at least three problems per group the groups take contiguous runs of problems whose
- * costliest run is as cheap as contiguous runs allow (long problems) and which stay close to equal shares of the cost. */
+ * costliest run is as cheap as contiguous runs allow (long problems) and which stay close to equal shares of the cost.  A launch
+ * whose K and V stay in L2 (64 MiB) takes the problems of that schedule in descending order of cost instead, one round of CTAs
+ * after the other, every other round backwards: the same problems, more evenly shared. */
 int64_t tlin_plan_group_start(const tlin_fwd_plan* plan, int g);
 /* Mask predicate: may query i (0 <= i < W) use key j?  1 or 0. */
 int tlin_allowed(int64_t i, int64_t j, int64_t N, int64_t W, int causal_window);

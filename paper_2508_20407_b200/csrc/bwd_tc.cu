@@ -141,6 +141,53 @@ struct ACfg {
     static constexpr int kThreads = 32 * 11;
 };
 
+// Order in which the CTAs of the key-tile kernels take the (b,h,key tile) units.  With the window rule key tile t is visited by
+// fewer query tiles the later it is.
+enum { kUnitRuns = 0,      // contiguous runs of equal cost: a CTA stays on one or two (b,h) (dK/dV kernel)
+       kUnitTurns = 1,     // in turn (CTA c: c, c + CTAs, ...): all CTAs work on the key tiles of two or three (b,h) at any time, so the
+                           // rows of the fp32 dQ buffer they add to, and the Q / dout tiles they read, stay in L2 whatever the size
+                           // of the call (one-kernel arrangement)
+       kUnitDealt = 2 };   // by descending cost over all (b,h) (dealt_position)
+// A CTA walks u = begin, begin + step, ... below end; unit(u, bh, t) says which (b,h) and key tile that is.
+template <int kOrder>
+struct UnitOrder {
+    long long begin, end, step;
+    int T;
+    __device__ UnitOrder(const BwdParams& p) : T(p.key_tiles) {
+        if constexpr (kOrder == kUnitRuns) {
+            begin = bwd_first_unit_of_share(p.N, p.W, p.causal, p.total_units, p.key_tiles, blockIdx.x, gridDim.x);
+            end = bwd_first_unit_of_share(p.N, p.W, p.causal, p.total_units, p.key_tiles, blockIdx.x + 1, gridDim.x);
+            step = 1;
+        } else if constexpr (kOrder == kUnitTurns) {
+            begin = blockIdx.x;
+            end = p.total_units;
+            step = gridDim.x;
+        } else {                        // u counts rounds
+            begin = 0;
+            const int full = (int)(p.total_units / gridDim.x);
+            end = full + (dealt_position(full) < p.total_units ? 1 : 0);
+            step = 1;
+        }
+    }
+    __device__ void unit(const BwdParams& p, long long u, int& bh, int& t) const {
+        if constexpr (kOrder == kUnitDealt) {
+            const unsigned pos = (unsigned)dealt_position((int)u), n_bh = (unsigned)p.total_units / (unsigned)T;
+            t = (int)(pos / n_bh);
+            bh = (int)(pos - (unsigned)t * n_bh);
+        } else {
+            bh = (int)(u / T);
+            t = (int)(u - (long long)bh * T);
+        }
+    }
+};
+// Dealing pays where runs and turns come out uneven, i.e. with few units per CTA and a window that is a large part of the keys (units
+// per CTA x N / W up to 32: costliest CTA 8 to 100 % above the mean against 1 to 10 %), and costs about 5 % of locality otherwise
+// (B1 H32 N32768 W512 817 -> 867 us); it needs the tensors that the units of a (b,h) share in L2 for all (b,h) at once.
+// Measured: B3 H12 N=W=1999 d64 161 -> 119 us (two kernels), B1 H16 N=W=2000 d128 84 -> 61 us (one kernel).
+bool deal_units(long long bh, int N, int W, int causal, int key_tiles, long long shared_bytes, int num_sms) {
+    return causal && shared_bytes <= (140LL << 20) && bh * key_tiles * N <= 32LL * num_sms * W;
+}
+
 // first 128-row query tile that may use a key of key tile t
 __device__ __forceinline__ int first_q_tile(const BwdParams& p, int t) {
     if (!p.causal) return 0;
@@ -148,7 +195,7 @@ __device__ __forceinline__ int first_q_tile(const BwdParams& p, int t) {
     return f <= 0 ? 0 : (int)(f / kQTile);
 }
 
-template <int D>
+template <int D, int kOrder>
 __global__ void __launch_bounds__(ACfg<D>::kThreads, 1)
 bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do, const BwdParams p) {
@@ -205,11 +252,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     volatile int* abort_p = abort_flag;
-
-    // The CTAs share the (b,h,key tile) units by cost (query tiles a key tile has to visit), not by count: with the
-    // window rule the last key tiles of a (b,h) are cheaper, down to one step.
-    const long long u_begin = bwd_first_unit_of_share(p.N, p.W, p.causal, p.total_units, p.key_tiles, blockIdx.x, gridDim.x);
-    const long long u_end = bwd_first_unit_of_share(p.N, p.W, p.causal, p.total_units, p.key_tiles, blockIdx.x + 1, gridDim.x);
+    const UnitOrder<kOrder> order(p);
 
     if (warp == kProducerWarp) {
         // ------------------------------------------------------------------ TMA producer: Q / dout / row statistics ring
@@ -218,8 +261,9 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (lane == 0) {
             bool ok = base_ok;
             uint32_t hh = 0;                // chain steps (64 queries each) issued
-            for (long long u = u_begin; u < u_end && ok; ++u) {
-                const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
+            for (long long u = order.begin; u < order.end && ok; u += order.step) {
+                int bh, t;
+                order.unit(p, u, bh, t);
                 const int row_first = first_q_tile(p, t) * kQTile, row_end = p.q_tiles128 * kQTile;
                 for (int row = row_first; row < row_end && ok; row += 64, ++hh) {
                     const uint32_t slot = hh % C::kSlots, round = hh / C::kSlots;
@@ -248,10 +292,11 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (lane == 0) {
             bool ok = base_ok;
             uint32_t n = 0;
-            for (long long u = u_begin; u < u_end && ok; ++u, ++n) {
-                const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
-                if (u + 1 < u_end) {        // K, V have one buffer: the next tile's rows come as far as L2 meanwhile
-                    const int bh_n = (int)((u + 1) / p.key_tiles), t_n = (int)(u + 1 - (long long)bh_n * p.key_tiles);
+            for (long long u = order.begin; u < order.end && ok; u += order.step, ++n) {
+                int bh, t, bh_n, t_n;
+                order.unit(p, u, bh, t);
+                if (u + order.step < order.end) {   // K, V have one buffer: the next tile's rows come as far as L2 meanwhile
+                    order.unit(p, u + order.step, bh_n, t_n);
                     for (int x = 0; x < C::kBoxes; ++x) {
                         tma_prefetch_l2_3d(&map_k, x * 64, t_n * kTileN, bh_n);
                         tma_prefetch_l2_3d(&map_v, x * 64, t_n * kTileN, bh_n);
@@ -312,8 +357,9 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         };
         bool ok = base_ok;
         uint32_t g = 0, n = 0;              // 128-query steps done, key tiles done; chain x of step g uses ring entry 2g + x
-        int t = (int)(u_begin % p.key_tiles);
-        for (long long u = u_begin; u < u_end && ok; ++u, ++n, t = t + 1 == p.key_tiles ? 0 : t + 1) {
+        for (long long u = order.begin; u < order.end && ok; u += order.step, ++n) {
+            int bh, t;
+            order.unit(p, u, bh, t);
             const int steps = p.q_tiles128 - first_q_tile(p, t);
             ok = __all_sync(0xffffffffu, mbar_wait(kv_full, n & 1, abort_p));
             if (!ok) break;
@@ -359,12 +405,9 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const uint32_t tDP = tS + 64;
         bool ok = base_ok;
         uint32_t g = 0, n = 0;
-        int bh = (int)(u_begin / p.key_tiles), t = (int)(u_begin - (long long)bh * p.key_tiles);
-        for (long long u = u_begin; u < u_end && ok; ++u, ++n, ++t) {
-            if (t == p.key_tiles) {
-                t = 0;
-                ++bh;
-            }
+        for (long long u = order.begin; u < order.end && ok; u += order.step, ++n) {
+            int bh, t;
+            order.unit(p, u, bh, t);
             const int key = t * kTileN + r;
             const int i_first = first_q_tile(p, t);
             const long long shift = (long long)p.N - p.W;       // query q may use key k iff q >= k - shift
@@ -514,7 +557,7 @@ struct FCfg {
     static_assert(128 * kDqRegs + 128 * kOtherRegs <= 256 * kLaunchRegs && kDqRegs > kLaunchRegs && kOtherRegs < kLaunchRegs, "register budget");
 };
 
-template <int D>
+template <int D, int kOrder>
 __global__ void __launch_bounds__(FCfg<D>::kThreads, 1)
 bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                     const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do, const BwdParams p) {
@@ -567,12 +610,7 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     volatile int* abort_p = abort_flag;
-
-    // The CTAs take the (b,h,key tile) units in turn (CTA c: units c, c + CTAs, ...), so that at any time all of them work on
-    // the key tiles of two or three (b,h): the rows of the fp32 dQ buffer they add to, and the Q / dout tiles they read, then
-    // stay in L2 whatever the size of the call.  With the window rule the last key tiles of a (b,h) are cheaper; taking units in
-    // turn spreads those evenly.
-    const long long u_begin = blockIdx.x, u_end = p.total_units, u_step = gridDim.x;
+    const UnitOrder<kOrder> order(p);
 
     if (warp >= C::kProducer) {
     setmaxnreg_dec<C::kOtherRegs>();
@@ -581,8 +619,9 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         if (lane == 0) {
             bool ok = base_ok;
             uint32_t nq = 0, ndo = 0;       // tiles armed
-            for (long long u = u_begin; u < u_end && ok; u += u_step) {
-                const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
+            for (long long u = order.begin; u < order.end && ok; u += order.step) {
+                int bh, t;
+                order.unit(p, u, bh, t);
                 for (int i = first_q_tile(p, t); i < p.q_tiles128; ++i) {
                     const uint32_t slot = nq & 1, par = ((nq >> 1) & 1) ^ 1;
                     const int row = i * kQTile;
@@ -613,10 +652,11 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         if (lane == 0) {
             bool ok = base_ok;
             uint32_t nk = 0, nv = 0;        // tiles armed
-            for (long long u = u_begin; u < u_end && ok; u += u_step) {
-                const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
-                if (u + u_step < u_end) {   // K, V have one buffer: the next tile's rows come as far as L2 meanwhile
-                    const int bh_n = (int)((u + u_step) / p.key_tiles), t_n = (int)(u + u_step - (long long)bh_n * p.key_tiles);
+            for (long long u = order.begin; u < order.end && ok; u += order.step) {
+                int bh, t, bh_n, t_n;
+                order.unit(p, u, bh, t);
+                if (u + order.step < order.end) {   // K, V have one buffer: the next tile's rows come as far as L2 meanwhile
+                    order.unit(p, u + order.step, bh_n, t_n);
                     for (int x = 0; x < C::kBoxes; ++x) {
                         tma_prefetch_l2_3d(&map_k, x * 64, t_n * kTileN, bh_n);
                         tma_prefetch_l2_3d(&map_v, x * 64, t_n * kTileN, bh_n);
@@ -673,8 +713,10 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_p));
             return ok;
         };
-        for (long long u = u_begin; u < u_end && ok; u += u_step, ++n) {
-            const int steps = p.q_tiles128 - first_q_tile(p, (int)(u % p.key_tiles));
+        for (long long u = order.begin; u < order.end && ok; u += order.step, ++n) {
+            int bh, t;
+            order.unit(p, u, bh, t);
+            const int steps = p.q_tiles128 - first_q_tile(p, t);
             if (!wait(k_full, n & 1) || !wait(&q_full[g & 1], (g >> 1) & 1)) break;
             tc_fence_after();
             issue_scores(tS, C::kOffK, C::kOffQ + (g & 1) * C::kTileBytes);
@@ -728,8 +770,9 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const bool issuer = threadIdx.x == C::kDqWarp * 32;
         bool ok = base_ok;
         uint32_t g = 0;
-        for (long long u = u_begin; u < u_end && ok; u += u_step) {
-            const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
+        for (long long u = order.begin; u < order.end && ok; u += order.step) {
+            int bh, t;
+            order.unit(p, u, bh, t);
             for (int i = first_q_tile(p, t); i < p.q_tiles128; ++i, ++g) {
                 ok = __all_sync(0xffffffffu, mbar_wait(dq_full, g & 1, abort_p));
                 if (!ok) break;
@@ -769,8 +812,9 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         uint8_t* ds_row = smem + C::kOffStage + wg * 16384 + r * 128;       // this key's row of the dS^T tile
         bool ok = base_ok;
         uint32_t g = 0, n = 0;
-        for (long long u = u_begin; u < u_end && ok; u += u_step, ++n) {
-            const int bh = (int)(u / p.key_tiles), t = (int)(u - (long long)bh * p.key_tiles);
+        for (long long u = order.begin; u < order.end && ok; u += order.step, ++n) {
+            int bh, t;
+            order.unit(p, u, bh, t);
             const int key = t * kTileN + r;
             const long long shift = (long long)p.N - p.W;       // query q may use key k iff q >= k - shift
             const int q_min = p.causal ? (int)((long long)key - shift) : -0x7fffffff;
@@ -930,7 +974,7 @@ struct BCfg {
     static_assert(256 * kComputeRegs + 128 * kOtherRegs <= kThreads * 168, "register budget of the CTA exceeded");
 };
 
-template <int D>
+template <int D, bool kDeal>
 __global__ void __launch_bounds__(BCfg<D>::kThreads, 1)
 bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do, const BwdParams p,
@@ -1005,7 +1049,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (lane == 0) {
             uint32_t kit = 0, vit = 0, seg_idx = 0;
             bool ok = base_ok;
-            SegmentWalker walk(p, starts);
+            std::conditional_t<kDeal, DealtWalker, SegmentWalker> walk(p, starts);
             Segment s;
             while (ok && walk.next(s)) {
                 const int row0 = s.qt * kTileM;
@@ -1085,7 +1129,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         uint32_t kit = 0, vit = 0, seg_idx = 0;
         uint32_t n_step[2] = {0, 0};
         bool ok = base_ok;
-        SegmentWalker walk(p, starts);
+        std::conditional_t<kDeal, DealtWalker, SegmentWalker> walk(p, starts);
         Segment s;
         while (ok && walk.next(s)) {
             const int row0 = s.qt * kTileM;
@@ -1162,8 +1206,9 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t tDQ = tmem_base + lane_addr + C::kColDQ + i * D;
         uint32_t n = 0, seg_idx = 0;
         bool ok = base_ok;
-        SegmentWalker walk(p, starts);
-        const int bh_first = (int)(walk.u / p.key_tiles);     // (b,h) of this CTA's first unit (used under schedule 0 only)
+        std::conditional_t<kDeal, DealtWalker, SegmentWalker> walk(p, starts);
+        int bh_first = 0;                                     // (b,h) of this CTA's first unit (used under schedule 0 only)
+        if constexpr (!kDeal) bh_first = (int)(walk.u / p.key_tiles);
         Segment s;
         while (ok && walk.next(s)) {
             const int row0 = s.qt * kTileM;
@@ -1355,9 +1400,11 @@ int launch_d(const void* q, const void* k, const void* v, const void* out, const
     p.scale = 1.f / sqrtf((float)D);
     p.scale_log2e = kLog2e * p.scale;
     p.wide_stores = ((reinterpret_cast<uintptr_t>(dq) | reinterpret_cast<uintptr_t>(ws)) & 31u) == 0;
-    static bool smem_allowed_a[64] = {}, smem_allowed_b[64] = {};
-    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dkdv_tc_kernel<D>, ACfg<D>::kSmemBytes, smem_allowed_a));
-    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dq_tc_kernel<D>, BCfg<D>::kSmemBytes, smem_allowed_b));
+    static bool smem_allowed[4][64] = {};
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dkdv_tc_kernel<D, kUnitRuns>, ACfg<D>::kSmemBytes, smem_allowed[0]));
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dkdv_tc_kernel<D, kUnitDealt>, ACfg<D>::kSmemBytes, smem_allowed[1]));
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dq_tc_kernel<D, false>, BCfg<D>::kSmemBytes, smem_allowed[2]));
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dq_tc_kernel<D, true>, BCfg<D>::kSmemBytes, smem_allowed[3]));
     const long long rows_padded = bh * Wpad;
     TLIN_CUDA_CHECK(launch_overlapped(bwd_prep_kernel<D>, (unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st,
         (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, (float*)nullptr, W, Wpad, rows_padded));
@@ -1365,15 +1412,16 @@ int launch_d(const void* q, const void* k, const void* v, const void* out, const
     BwdParams pa = p;
     pa.total_units = bh * p.key_tiles;
     pa.n_groups = 0; pa.q_tiles = 0; pa.schedule = 0;
+    const auto kernel_a = deal_units(bh, N, W, causal, p.key_tiles, bh * (long long)W * D * 4, num_sms) ? bwd_dkdv_tc_kernel<D, kUnitDealt> : bwd_dkdv_tc_kernel<D, kUnitRuns>;
     const long long ctas_a = pa.total_units < num_sms ? pa.total_units : num_sms;
-    TLIN_CUDA_CHECK(launch_overlapped(bwd_dkdv_tc_kernel<D>, (unsigned)ctas_a, ACfg<D>::kThreads, ACfg<D>::kSmemBytes, st, mq64, mk, mv, mdo64, pa));
+    TLIN_CUDA_CHECK(launch_overlapped(kernel_a, (unsigned)ctas_a, ACfg<D>::kThreads, ACfg<D>::kSmemBytes, st, mq64, mk, mv, mdo64, pa));
     // dQ: the forward's plan
     BwdParams pb = p;
     pb.total_units = plan.total_units; pb.n_groups = plan.n_groups; pb.q_tiles = plan.q_tiles; pb.schedule = plan.schedule;
     if (plan.n_groups > kMaxGroups) return TLIN_ERR_UNSUPPORTED;
     GroupStarts starts;
     fwd_group_starts(plan, &starts);
-    TLIN_CUDA_CHECK(launch_overlapped(bwd_dq_tc_kernel<D>, plan.n_ctas, BCfg<D>::kThreads, BCfg<D>::kSmemBytes, st, mq, mk, mv, mdo, pb, starts));
+    TLIN_CUDA_CHECK(launch_overlapped(dealt(plan, bh, D) ? bwd_dq_tc_kernel<D, true> : bwd_dq_tc_kernel<D, false>, plan.n_ctas, BCfg<D>::kThreads, BCfg<D>::kSmemBytes, st, mq, mk, mv, mdo, pb, starts));
     count_launch(3);
     if (plan.uses_workspace) {
         TLIN_CUDA_CHECK(launch_overlapped(bwd_dq_reduce_kernel<D>, (unsigned)(bh * plan.q_tiles * (kTileM / 8)), 256, 0, st, pb));
@@ -1433,13 +1481,15 @@ int launch_fused_128(const void* q, const void* k, const void* v, const void* ou
     p.wide_stores = 0;
     p.total_units = bh * p.key_tiles;
     p.n_groups = 0; p.q_tiles = 0; p.schedule = 0;
-    static bool smem_allowed[64] = {};
-    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_fused_tc_kernel<D>, FCfg<D>::kSmemBytes, smem_allowed));
+    const auto kernel = deal_units(bh, N, W, causal, p.key_tiles, bh * (long long)Wpad * D * 8, num_sms) ? bwd_fused_tc_kernel<D, kUnitDealt> : bwd_fused_tc_kernel<D, kUnitTurns>;
+    static bool smem_allowed[2][64] = {};
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_fused_tc_kernel<D, kUnitTurns>, FCfg<D>::kSmemBytes, smem_allowed[0]));
+    TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_fused_tc_kernel<D, kUnitDealt>, FCfg<D>::kSmemBytes, smem_allowed[1]));
     const long long rows_padded = bh * Wpad;
     TLIN_CUDA_CHECK(launch_overlapped(bwd_prep_kernel<D>, (unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st,
         (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, dq32, W, Wpad, rows_padded));
     const long long ctas = p.total_units < num_sms ? p.total_units : num_sms;
-    TLIN_CUDA_CHECK(launch_overlapped(bwd_fused_tc_kernel<D>, (unsigned)ctas, FCfg<D>::kThreads, FCfg<D>::kSmemBytes, st, mq, mk, mv, mdo, p));
+    TLIN_CUDA_CHECK(launch_overlapped(kernel, (unsigned)ctas, FCfg<D>::kThreads, FCfg<D>::kSmemBytes, st, mq, mk, mv, mdo, p));
     const long long rows = bh * W, threads = rows * (D / 8);
     TLIN_CUDA_CHECK(launch_overlapped(bwd_dq_convert_kernel<D>, (unsigned)((threads + 255) / 256), 256, 0, st, dq32, (__nv_bfloat16*)dq, W, Wpad, rows, p.scale));
     count_launch(3);
@@ -1457,7 +1507,7 @@ size_t bwd_fused_workspace_bytes(long long B, long long H, long long W, int d) {
 int launch_bwd_fused(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                      void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, float* ws, int num_sms, cudaStream_t st) {
     if (d != 128) return TLIN_ERR_UNSUPPORTED;
-    if ((long long)B * H * W > 0x7fffffffLL || (long long)B * H > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
+    if ((long long)B * H * W > 0x7fffffffLL || (long long)B * H > 0x7fffffffLL || (long long)B * H * ((N + kTileN - 1LL) / kTileN) > 0x7fff0000LL) return TLIN_ERR_UNSUPPORTED;
     return launch_fused_128(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, causal, ws, num_sms, st);
 }
 
@@ -1473,7 +1523,7 @@ int launch_bwd_tc(const void* q, const void* k, const void* v, const void* out, 
                   void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& plan,
                   float* ws, int num_sms, cudaStream_t st) {
     if (plan.tile_m != tc::kTileM || plan.tile_n != kTileN || !plan.tensor_path) return TLIN_ERR_UNSUPPORTED;
-    if ((long long)B * H * W > 0x7fffffffLL || (long long)B * H > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
+    if ((long long)B * H * W > 0x7fffffffLL || (long long)B * H > 0x7fffffffLL || (long long)B * H * ((N + kTileN - 1LL) / kTileN) > 0x7fff0000LL) return TLIN_ERR_UNSUPPORTED;
     if (d == 128) return launch_d<128>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, causal, plan, ws, num_sms, st);
     if (d == 64) return launch_d<64>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, causal, plan, ws, num_sms, st);
     return TLIN_ERR_UNSUPPORTED;

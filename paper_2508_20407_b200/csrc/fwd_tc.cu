@@ -69,14 +69,16 @@ __device__ __forceinline__ void exp2_poly2(uint64_t x2, float& p0, float& p1) {
     p1 = __uint_as_float(y1 + (n1 << 23));
 }
 
-// The kernel's three forms: head size D exactly, one problem or a table of them; or any other head size d <= D that is a multiple
+// The kernel's forms: head size D exactly, one problem or a table of them; or any other head size d <= D that is a multiple
 // of 8.  The last reads its tiles with zero fill beyond d (the tensor maps know the true row length), contracts over ceil(d/16)
 // slices only, and keeps P to 16 mantissa bits as the sum of two bf16 parts, two PV products per step: the CUDA-core kernel that
 // served these sizes before kept P in fp32, and the results are to lose nothing (against 64-bit sums 1.66e-3, the rounding to
 // bf16 alone).  At D = 256 two output accumulators would fill the TMEM, so a CTA works on one Q tile.
 // Measured against that CUDA-core kernel: B2 H9 N3001 W517 d96 2066 -> 45 us, B2 H3 N7791 W968 d40 2582 -> 38 us, B1 H12 N2000
 // W1000 d256 3952 -> 56 us, B4 H12 N370 W96 d32 96 -> 12 us.
-enum { kOneProblem = 0, kTable = 1, kAnyHead = 2 };
+// kDealt and kAnyDealt are the first and the last with problems dealt out by cost (DealtWalker; a form of their own because the
+// choice at run time costs the others 1 to 2 %).
+enum { kOneProblem = 0, kTable = 1, kAnyHead = 2, kDealt = 3, kAnyDealt = 4 };
 
 template <int D>
 struct Cfg {
@@ -143,9 +145,10 @@ struct BatchWalker {
         return true;
     }
 };
-template <bool kBatched>
-__device__ __forceinline__ auto make_walker(const KernelMaps<kBatched>& m, const Params& p, const GroupStarts& starts) {
-    if constexpr (kBatched) return BatchWalker(m, starts);
+template <int kForm>
+__device__ __forceinline__ auto make_walker(const KernelMaps<kForm == kTable>& m, const Params& p, const GroupStarts& starts) {
+    if constexpr (kForm == kTable) return BatchWalker(m, starts);
+    else if constexpr (kForm == kDealt || kForm == kAnyDealt) return DealtWalker(p, starts);
     else return SegmentWalker(p, starts);
 }
 // shape (N, W, causal, key_tiles) and result pointers of the problem a segment belongs to
@@ -160,7 +163,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __grid_constant__ Params p,
               const __grid_constant__ GroupStarts starts) {
     using C = Cfg<D>;
-    constexpr bool kBatched = kForm == kTable, kAny = kForm == kAnyHead;
+    constexpr bool kBatched = kForm == kTable, kAny = kForm == kAnyHead || kForm == kAnyDealt, kWhole = kForm == kTable || kForm >= kDealt;   // kWhole: no split keys
     constexpr int kTileM = C::kRows;
     const int d = kAny ? p.d : D;                              // row length; everything below folds where it is D
     const int boxes = kAny ? (d + 63) / 64 : C::kBoxes;
@@ -227,7 +230,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             uint32_t it = 0;           // ring counter
             uint32_t seg_idx = 0;
             bool ok = true;
-            auto walk = make_walker<kBatched>(maps, p, starts);
+            auto walk = make_walker<kForm>(maps, p, starts);
             Segment s;
             while (ok && walk.next(s)) {
                 const auto& pr = problem_of<kBatched>(maps, p, s);
@@ -322,7 +325,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             constexpr std::integral_constant<int, 0> k_begin{};
             constexpr std::integral_constant<int, kFirstKeys / 16> k_first{};
             constexpr std::integral_constant<int, kTileN / 16> k_end{};
-            auto walk = make_walker<kBatched>(maps, p, starts);
+            auto walk = make_walker<kForm>(maps, p, starts);
             Segment s;
             while (ok && walk.next(s)) {
                 const auto& pr = problem_of<kBatched>(maps, p, s);
@@ -407,9 +410,9 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
         const uint32_t tO = tmem_base + lane_addr + C::kColO + i * D;
         uint32_t n = 0;     // tiles processed by this warpgroup (phase counter of s_full/p_full/pv_done)
         bool ok = true;
-        auto walk = make_walker<kBatched>(maps, p, starts);
+        auto walk = make_walker<kForm>(maps, p, starts);
         int bh_first = 0;                                  // (b,h) of this CTA's first unit (used under schedule 0 only)
-        if constexpr (!kBatched) bh_first = (int)(walk.u / p.key_tiles);
+        if constexpr (!kWhole) bh_first = (int)(walk.u / p.key_tiles);
         Segment s;
         while (ok && walk.next(s)) {
             const auto& pr = problem_of<kBatched>(maps, p, s);
@@ -527,7 +530,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             if (!ok) break;
             if (allowed_i == 0) continue;                  // this Q tile does not exist: nothing to write
             // ---------------------------------------------------------------- epilogue of the segment
-            const bool whole = kBatched || (s.t_begin == 0 && s.t_end == p.key_tiles);
+            const bool whole = kWhole || (s.t_begin == 0 && s.t_end == p.key_tiles);
             if (cnt_i > 0) {
                 ok = mbar_wait(&pv_done[i], (n - 1) & 1, abort_p);
                 ok = __all_sync(0xffffffffu, ok);
@@ -773,7 +776,7 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
     fwd_group_starts(plan, &starts);
     TLIN_CUDA_CHECK(launch_overlapped(fwd_tc_kernel<D, kForm>, plan.n_ctas, kThreads, C::kSmemBytes, st, maps, p, starts));
     count_launch();
-    if (plan.uses_workspace) {
+    if constexpr (kForm == kOneProblem || kForm == kAnyHead) if (plan.uses_workspace) {
         constexpr bool kAny = kForm == kAnyHead;
         const long long tiles = bh * plan.q_tiles;
         if (tiles * C::kRows >= 65536)
@@ -837,10 +840,16 @@ int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float*
                   int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& plan,
                   float* ws, long long kv_rows_alloc, cudaStream_t st) {
     if (plan.tile_m != (d > 128 ? kQTile : kTileM) || plan.tile_n != kTileN) return TLIN_ERR_UNSUPPORTED;
-    if ((long long)B * H * W > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
+    if ((long long)B * H * W > 0x7fffffffLL || d % 8 != 0 || d > 256) return TLIN_ERR_UNSUPPORTED;
+    if (dealt(plan, (long long)B * H, d)) {
+        if (d == 128) return launch_d<128, kDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+        if (d == 64) return launch_d<64, kDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+        if (d < 64) return launch_d<64, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+        if (d < 128) return launch_d<128, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+        return launch_d<256, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+    }
     if (d == 128) return launch_d<128, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
     if (d == 64) return launch_d<64, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
-    if (d % 8 != 0) return TLIN_ERR_UNSUPPORTED;
     if (d < 64) return launch_d<64, kAnyHead>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
     if (d < 128) return launch_d<128, kAnyHead>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
     if (d <= 256) return launch_d<256, kAnyHead>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);

@@ -51,6 +51,35 @@ struct SegmentWalker {
     }
 };
 
+// Under the window rule the problems of schedule 1 (and the key tiles of the backward) differ in cost by up to the number of query
+// tiles.  Contiguous runs of them leave the costliest CTA far above the mean when a CTA has only a few (B3 H12 N=W=1999: 36 against
+// 23 key-tile times); dealt out in descending order of cost, every other round backwards, they do not (24).  Measured, forward: B3
+// H12 N=W=1999 d64 54.7 -> 38.0 us, B2 H16 N=W=1500 d128 48.2 -> 30.8 us, B1 H16 N=W=3000 d64 75 -> 43 us.  The price is that
+// neighbouring CTAs work on different (b,h), so this is for calls whose shared tensors stay in L2.
+// Position of this CTA's r-th item in the list sorted by cost; at or beyond the list's length: nothing left.
+__device__ __forceinline__ long long dealt_position(int r) {
+    return (long long)r * gridDim.x + ((r & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+}
+// The problems of schedule 1 by descending cost: the last query tiles see the most keys.
+struct DealtWalker {
+    long long total;
+    int T, q_tiles, n_bh, round;
+    template <class P>
+    __device__ DealtWalker(const P& p, const GroupStarts&)
+        : total(p.total_units), T(p.key_tiles), q_tiles(p.q_tiles), n_bh((int)(p.total_units / p.q_tiles)), round(0) {}
+    __device__ bool next(Segment& s) {
+        const long long pos = dealt_position(round++);
+        if (pos >= total) return false;
+        const int rank = (int)(pos / n_bh);
+        s.prob = 0;
+        s.bh = (int)(pos - (long long)rank * n_bh);
+        s.qt = q_tiles - 1 - rank;
+        s.t_begin = 0;
+        s.t_end = T;
+        return true;
+    }
+};
+
 __device__ __forceinline__ void commit_elected(uint64_t* bar) {
     if (elect_one()) tc_commit(bar);
 }
@@ -86,6 +115,12 @@ inline EncodeTiledFn encode_fn() {
             fn = reinterpret_cast<EncodeTiledFn>(f);
     });
     return fn;
+}
+
+// Does a launch that follows this plan deal its problems out by cost?  K and V are read by the query tiles of a (b,h) at unrelated
+// times, so they have to stay in L2 (the bound the planner uses for schedule 1).
+inline bool dealt(const tlin_fwd_plan& plan, long long bh, int d) {
+    return plan.schedule == 1 && plan.causal_window && plan.q_tiles > 1 && 2 * bh * plan.n_keys * (long long)d * 2 <= (64LL << 20);
 }
 
 // [BH, rows, D] bf16, box = 64 elements x box_rows rows x 1, 128-byte swizzle, zero fill outside.  rows_alloc > rows: only

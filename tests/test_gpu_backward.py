@@ -420,3 +420,16 @@ def test_autograd_backward_gets_its_workspace_and_reports_errors():
     odd = torch.zeros(1, 1, 8, 36, dtype=torch.bfloat16, device=DEV, requires_grad=True)
     with pytest.raises(tl.TlinError):
         tl.attention(odd, odd, odd, 1)
+
+
+# key tiles dealt out by cost, in both arrangements: one incomplete round, exactly one round of 148 CTAs, one unit more, several rounds
+DEALT = [(1, 1, 300, 300, 128), (1, 37, 512, 512, 128), (1, 149, 128, 100, 128), (1, 75, 390, 300, 64), (1, 37, 512, 512, 64), (2, 30, 1000, 640, 128)]
+
+
+@pytest.mark.parametrize("arrangement", [1, 2])
+@pytest.mark.parametrize("B,H,N,W,d", DEALT)
+def test_backward_key_tiles_dealt_by_cost(B, H, N, W, d, arrangement):
+    if d != 128 and arrangement == 2:
+        pytest.skip("one kernel only at d = 128")
+    assert B * H * -(-N // 128) * N <= 32 * 148 * W                                        # what the dispatch asks
+    run_case(B, H, N, W, d, 1, seed=900 + N + W, impl=0, guarded=True, arrangement=arrangement)

@@ -607,3 +607,15 @@ def test_merge_of_many_rows(B, H, N, W, d, causal):
     for b, h in ((0, 0), (B // 2, H // 2), (B - 1, H - 1)):
         ref, ref_lse = oracle.attn_forward(q[b:b + 1, h:h + 1].cpu(), k[b:b + 1, h:h + 1].cpu(), v[b:b + 1, h:h + 1].cpu(), causal)
         parity.check(out[b:b + 1, h:h + 1].float().cpu().numpy(), lse[b:b + 1, h:h + 1].cpu().numpy(), ref, ref_lse, "bf16", f"b{b} h{h}")
+
+
+# problems dealt out by cost (window rule, several query tiles, K and V in L2): one incomplete round, exactly one round, one item more,
+# an odd and an even number of rounds, N > W, a head size in padded tiles
+DEALT = [(1, 1, 300, 300, 64, 1), (1, 37, 900, 900, 64, 1), (1, 149, 260, 257, 128, 1), (2, 40, 600, 513, 64, 1), (1, 100, 700, 600, 96, 1), (1, 60, 300, 300, 200, 1)]
+
+
+@pytest.mark.parametrize("B,H,N,W,d,causal", DEALT)
+def test_forward_problems_dealt_by_cost(B, H, N, W, d, causal):
+    plan = tl.tlin_plan_forward(B, H, N, W, d, causal)
+    assert plan.schedule == 1 and plan.q_tiles > 1 and 4 * B * H * N * d <= 64 << 20      # what the dispatch asks
+    guarded_compare(synth.Workload("dealt", B, H, d, N, W, seed=70 + N, causal_window=causal), 2)
