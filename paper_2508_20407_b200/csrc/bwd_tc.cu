@@ -13,9 +13,9 @@
 //   see it.  Scores are computed TRANSPOSED (S^T = K Q^T, dP^T = V dout^T: TMEM lane = key, column = query) so that
 //   P^T and dS^T, written back to TMEM as bf16, are directly the A operands of dV += P^T dout and dK += dS^T Q, whose
 //   B operands are the dout / Q tiles already in shared memory (read MN-major).  dK and dV stay in TMEM for the whole
-//   key tile and are written once.  Each 128-query tile is worked on as two independent chains of 64 queries, one per
-//   warpgroup (thread = key row): [S^T_x | dP^T_x] by the tensor pipe, then P^T_x and dS^T_x written over them in
-//   place, then the two accumulating MMAs; while one chain does its elementwise work the tensor pipe serves the other.
+//   key tile and are written once.  The queries are worked on as independent chains of 64, two (d = 128) or three (d = 64), one
+//   per warpgroup (thread = key row): [S^T_x | dP^T_x] by the tensor pipe, then P^T_x and dS^T_x written over them in
+//   place, then the two accumulating MMAs; while one chain does its elementwise work the tensor pipe serves the others.
 //
 // bwd_dq_tc_kernel     The forward's structure: a CTA owns 256 query rows (two Q tiles, one warpgroup each, one
 //   thread per row) and streams 128-key tiles; per tile S = Q K^T -> p (kept in registers), then dP = dout V^T into
@@ -44,7 +44,6 @@ using namespace tc;
 
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;
-constexpr int kKvWarp = 10;                 // dK/dV kernel only
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct BwdParams {
@@ -126,19 +125,30 @@ struct ACfg {
     static constexpr int kTileBytes = kQTile * D * 2;          // one 128-row tile (K or V)
     static constexpr int kHalfBytes = 64 * D * 2;              // one 64-row tile (Q or dout of a chain step)
     static constexpr int kBoxes = D / 64;
+    // Chains of 64 queries, one warpgroup each: as many as TMEM has columns for beside dK and dV.  A chain's products and its
+    // elementwise work follow one another and leave both pipes half idle at d = 64; a third chain fills them better.  Backward
+    // with two / three, microseconds: 36 x 1999^2 causal 111.5 / 101.6, 128 x 1024 x 8192 1232 / 1160, 16 x 2000^2 68.5 / 65.4.
+    static constexpr int kChains = D == 128 ? 2 : 3;
+    static constexpr int kProducer = 4 * kChains, kMma = kProducer + 1, kKv = kProducer + 2;      // warps below: P and dS
+    static constexpr int kThreads = D == 128 ? 32 * 11 : 32 * 16;
+    // d = 64: setmaxnreg moves registers from the fourth warpgroup to the chains; the CTA starts with 128 per thread.  An increase
+    // beyond what was released would wait for ever, one below the count at launch is an illegal instruction.
+    static constexpr int kComputeRegs = 136, kOtherRegs = 104;
+    static_assert(384 * kComputeRegs + 128 * kOtherRegs <= 512 * 128 && kComputeRegs > 128 && kOtherRegs < 128, "register budget");
+    // columns of a result row that a thread writes out: half a row of dK and of dV, or (three chains) a whole row of one of them
+    static constexpr int kOutCols = kChains == 2 ? D / 2 : D;
     static constexpr int kSlots = D == 128 ? 4 : 8;            // ring of chain steps: Q (64 rows), dout (64 rows), 64 lse2 + 64 delta
     static constexpr int kSlotBytes = 2 * kHalfBytes;
     static constexpr int kOffKV = 0;
     static constexpr int kOffRing = 2 * kTileBytes;
     static constexpr int kOffStats = kOffRing + kSlots * kSlotBytes;
-    static constexpr int kOffStage = kOffStats + kSlots * 512;  // per compute warp 32 rows x D bytes: dK / dV rows on their way out
-    static constexpr int kOffBars = kOffStage + 8 * 32 * D;
-    static constexpr int kNumBars = 8 + 2 * kSlots;
+    static constexpr int kOffStage = kOffStats + kSlots * 512;  // per writing warp 32 rows of kOutCols: dK / dV on their way out
+    static constexpr int kOffBars = kOffStage + 8 * 32 * kOutCols * 2;
+    static constexpr int kNumBars = 4 + 2 * kChains + 2 * kSlots;
     static constexpr int kSmemBytes = kOffBars + kNumBars * 8 + 16;
     // TMEM columns: dK, dV (D each); per chain x (64 queries of the tile) 128 columns: S^T_x (64 fp32) and dP^T_x
     // (64 fp32); P^T_x and dS^T_x (bf16, 32 columns each) are written over the first half of S^T_x and dP^T_x
     static constexpr uint32_t kColDK = 0, kColDV = D, kColR = 2 * D;
-    static constexpr int kThreads = 32 * 11;
 };
 
 // Order in which the CTAs of the key-tile kernels take the (b,h,key tile) units.  With the window rule key tile t is visited by
@@ -207,11 +217,11 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
     uint64_t* kv_full = bars + 0;
     uint64_t* kv_empty = bars + 1;
-    uint64_t* sdp_full = bars + 2;    // [2] S^T_x and dP^T_x of a step are in TMEM
-    uint64_t* pds_full = bars + 4;    // [2] the chain's threads have stored P^T_x and dS^T_x
-    uint64_t* acc_full = bars + 6;    // dK, dV of the key tile are complete
-    uint64_t* acc_empty = bars + 7;   // all threads have read them
-    uint64_t* slot_full = bars + 8;   // [kSlots]
+    uint64_t* acc_full = bars + 2;    // dK, dV of the key tile are complete
+    uint64_t* acc_empty = bars + 3;   // all threads have read them
+    uint64_t* sdp_full = bars + 4;    // [kChains] S^T_x and dP^T_x of a chain step are in TMEM
+    uint64_t* pds_full = sdp_full + C::kChains;   // [kChains] the chain's threads have stored P^T_x and dS^T_x
+    uint64_t* slot_full = pds_full + C::kChains;  // [kSlots]
     uint64_t* slot_empty = slot_full + C::kSlots;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars);
     int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
@@ -223,7 +233,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         *abort_flag = base_ok ? 0 : 1;
         mbar_init(kv_full, 1);
         mbar_init(kv_empty, 1);
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < C::kChains; ++i) {
             mbar_init(&sdp_full[i], 1);
             mbar_init(&pds_full[i], 128);
         }
@@ -235,11 +245,11 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         mbar_init(acc_empty, 256);
         fence_mbar_init();
     }
-    if (warp == kMmaWarp) {
+    if (warp == C::kMma) {
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
-    if (warp == kProducerWarp && lane == 0) {
+    if (warp == C::kProducer && lane == 0) {
         prefetch_tensormap(&map_q);
         prefetch_tensormap(&map_k);
         prefetch_tensormap(&map_v);
@@ -254,7 +264,8 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     volatile int* abort_p = abort_flag;
     const UnitOrder<kOrder> order(p);
 
-    if (warp == kProducerWarp) {
+    if constexpr (C::kChains == 3) setmaxnreg_dec<C::kOtherRegs>();
+    if (warp == C::kProducer) {
         // ------------------------------------------------------------------ TMA producer: Q / dout / row statistics ring
         // The ring runs ahead of the key tiles: the first chain steps of the next key tile are loaded while the
         // current one is still being worked on.
@@ -287,7 +298,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
             }
         }
-    } else if (warp == kKvWarp) {
+    } else if (warp == C::kKv) {
         // ------------------------------------------------------------------ TMA producer: K, V of the key tiles
         if (lane == 0) {
             bool ok = base_ok;
@@ -315,7 +326,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 mbar_wait(kv_full, (n - 1) & 1, &dummy, 200000000LL);
             }
         }
-    } else if (warp == kMmaWarp) {
+    } else if (warp == C::kMma) {
         // ------------------------------------------------------------------ MMA issuer (all lanes walk, the lane elected once issues)
         const uint32_t idesc_st = make_idesc_bf16(kQTile, 64, 0, 0);         // S^T, dP^T of a chain: M = keys, N = 64 queries
         const uint32_t idesc_acc = make_idesc_bf16(kQTile, D, 0, 1);         // dV, dK: A in TMEM, B MN-major
@@ -356,47 +367,42 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             commit_lead(lead, &slot_empty[slot]);
         };
         bool ok = base_ok;
-        uint32_t g = 0, n = 0;              // 128-query steps done, key tiles done; chain x of step g uses ring entry 2g + x
+        uint32_t hh = 0, n = 0;             // chain steps and key tiles done; chain step h belongs to chain h mod kChains and ring slot h mod kSlots
         for (long long u = order.begin; u < order.end && ok; u += order.step, ++n) {
             int bh, t;
             order.unit(p, u, bh, t);
-            const int steps = p.q_tiles128 - first_q_tile(p, t);
+            const uint32_t first = hh, end = hh + 2 * (uint32_t)(p.q_tiles128 - first_q_tile(p, t));
             ok = __all_sync(0xffffffffu, mbar_wait(kv_full, n & 1, abort_p));
             if (!ok) break;
-            for (int x = 0; x < 2 && ok; ++x) {
-                const uint32_t hh = 2 * g + x;
-                ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[hh % C::kSlots], (hh / C::kSlots) & 1, abort_p));
+            for (uint32_t h = first; h < first + C::kChains && h < end; ++h) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[h % C::kSlots], (h / C::kSlots) & 1, abort_p));
                 if (!ok) break;
-                issue_sdp(x, hh % C::kSlots);
+                issue_sdp(h % C::kChains, h % C::kSlots);
             }
             if (!ok) break;
-            if (steps == 1) commit_lead(lead, kv_empty);       // K, V have been read for the last time: the next tile's may load
-            for (int s = 0; s < steps && ok; ++s, ++g) {
-                const bool have_next = s + 1 < steps;
-                for (int x = 0; x < 2 && ok; ++x) {
-                    const uint32_t hh = 2 * g + x;
-                    ok = __all_sync(0xffffffffu, mbar_wait(&pds_full[x], g & 1, abort_p));
-                    if (!ok) break;
-                    if (s == 0 && x == 0 && n > 0) {        // the previous key tile's dK, dV must have been read out
-                        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty, (n - 1) & 1, abort_p));
-                        if (!ok) break;
-                    }
-                    tc_fence_after();
-                    issue_acc(x, hh % C::kSlots, s > 0 || x > 0);
-                    if (have_next) {
-                        const uint32_t hn = hh + 2;
-                        ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[hn % C::kSlots], (hn / C::kSlots) & 1, abort_p));
-                        if (!ok) break;
-                        issue_sdp(x, hn % C::kSlots);
-                    }
-                }
+            if (end - first <= C::kChains) commit_lead(lead, kv_empty);     // K, V have been read for the last time: the next tile's may load
+            for (; hh < end; ++hh) {
+                const uint32_t x = hh % C::kChains, hn = hh + C::kChains;
+                ok = __all_sync(0xffffffffu, mbar_wait(&pds_full[x], (hh / C::kChains) & 1, abort_p));
                 if (!ok) break;
-                if (have_next && s + 2 == steps) commit_lead(lead, kv_empty);
+                if (hh == first && n > 0) {                 // the previous key tile's dK, dV must have been read out
+                    ok = __all_sync(0xffffffffu, mbar_wait(acc_empty, (n - 1) & 1, abort_p));
+                    if (!ok) break;
+                }
+                tc_fence_after();
+                issue_acc(x, hh % C::kSlots, hh > first);
+                if (hn < end) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[hn % C::kSlots], (hn / C::kSlots) & 1, abort_p));
+                    if (!ok) break;
+                    issue_sdp(x, hn % C::kSlots);
+                    if (hn + 1 == end) commit_lead(lead, kv_empty);
+                }
             }
             if (!ok) break;
             commit_lead(lead, acc_full);
         }
-    } else if (warp < 8) {
+    } else if (warp < C::kProducer) {
+        if constexpr (C::kChains == 3) setmaxnreg_inc<C::kComputeRegs>();
         // ------------------------------------------------------------------ elementwise threads
         const int wg = warp >> 2;                              // chain: which 64 queries of every tile
         const int r = (warp & 3) * 32 + lane;                  // key row inside the tile == TMEM lane
@@ -404,7 +410,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const uint32_t tS = tmem_base + lane_addr + C::kColR + wg * 128;
         const uint32_t tDP = tS + 64;
         bool ok = base_ok;
-        uint32_t g = 0, n = 0;
+        uint32_t hh = 0, n = 0;                                // first chain step of the key tile, key tiles done
         for (long long u = order.begin; u < order.end && ok; u += order.step, ++n) {
             int bh, t;
             order.unit(p, u, bh, t);
@@ -414,35 +420,35 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const int q_min = p.causal ? (int)((long long)key - shift) : -0x7fffffff;
             const int q_min_warp = p.causal ? (int)((long long)key - lane + 31 - shift) : -0x7fffffff;   // largest in the warp
             // a copy of the step for the tiles with masked elements: conditions in the loop cut it into short blocks
-            auto step = [&](int q0, auto masked_tag) {
+            auto step = [&](uint32_t h, int q0, auto masked_tag) {
                 constexpr bool kMasked = decltype(masked_tag)::value;
-                const uint32_t hh = 2 * g + wg, slot = hh % C::kSlots;
+                const uint32_t slot = h % C::kSlots;
                 const float* st = sStats + slot * 128;
-                ok = __all_sync(0xffffffffu, mbar_wait(&sdp_full[wg], g & 1, abort_p));
+                ok = __all_sync(0xffffffffu, mbar_wait(&sdp_full[wg], (h / C::kChains) & 1, abort_p));
                 if (!ok) return;
                 // already complete (the MMAs waited for it); observing it here orders the bulk-copied lse2 / delta
                 // before this thread's reads
-                ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[slot], (hh / C::kSlots) & 1, abort_p));
+                ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[slot], (h / C::kSlots) & 1, abort_p));
                 if (!ok) return;
                 tc_fence_after();
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t sv[32], dv_[32];
-                    tmem_ld32_async(tS + h * 32, sv);
-                    tmem_ld32_async(tDP + h * 32, dv_);
-                    tmem_wait_ld(sv);
-                    tmem_wait_ld(dv_);
-                    uint32_t pk[16], dk_[16];
+                for (int part = 0; part < 4; ++part) {       // 16 columns at a time: 32 spill at three chains and gain nothing at two
+                    uint32_t sv[16], dv_[16];
+                    tmem_ld16_async(tS + part * 16, sv);
+                    tmem_ld16_async(tDP + part * 16, dv_);
+                    tmem_wait_ld16(sv);
+                    tmem_wait_ld16(dv_);
+                    uint32_t pk[8], dk_[8];
 #pragma unroll
-                    for (int c = 0; c < 32; c += 4) {
-                        const float4 l4 = *reinterpret_cast<const float4*>(st + h * 32 + c);
-                        const float4 d4 = *reinterpret_cast<const float4*>(st + 64 + h * 32 + c);
+                    for (int c = 0; c < 16; c += 4) {
+                        const float4 l4 = *reinterpret_cast<const float4*>(st + part * 16 + c);
+                        const float4 d4 = *reinterpret_cast<const float4*>(st + 64 + part * 16 + c);
                         const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, dlv[4] = {d4.x, d4.y, d4.z, d4.w};
                         float pe[4], de[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             pe[e] = ex2(fmaf(__uint_as_float(sv[c + e]), p.scale_log2e, -lv[e]));
-                            if (kMasked && q0 + h * 32 + c + e < q_min) pe[e] = 0.f;
+                            if (kMasked && q0 + part * 16 + c + e < q_min) pe[e] = 0.f;
                             de[e] = pe[e] * (__uint_as_float(dv_[c + e]) - dlv[e]);
                         }
                         pk[c / 2] = pack_bf16x2(pe[0], pe[1]);
@@ -451,36 +457,40 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         dk_[c / 2 + 1] = pack_bf16x2(de[2], de[3]);
                     }
                     // bf16 P^T over columns of S^T, dS^T over columns of dP^T, that are already in registers
-                    tmem_st16(tS + h * 16, pk);
-                    tmem_st16(tDP + h * 16, dk_);
+                    tmem_st8(tS + part * 8, pk);
+                    tmem_st8(tDP + part * 8, dk_);
                 }
                 tc_wait_st();
                 tc_fence_before();
                 mbar_arrive(&pds_full[wg]);
             };
-            for (int i = i_first; i < p.q_tiles128 && ok; ++i, ++g) {
-                const int q0 = i * kQTile + wg * 64;              // first query of this thread's columns
-                if (q0 < q_min_warp) step(q0, std::true_type{});  // warp-uniform: some element of some lane is masked
-                else step(q0, std::false_type{});
+            const uint32_t end = hh + 2 * (uint32_t)(p.q_tiles128 - i_first);
+            for (uint32_t h = hh + ((uint32_t)wg + C::kChains - hh % C::kChains) % C::kChains; h < end && ok; h += C::kChains) {
+                const int q0 = i_first * kQTile + (int)(h - hh) * 64;   // first query of this thread's columns
+                if (q0 < q_min_warp) step(h, q0, std::true_type{});     // warp-uniform: some element of some lane is masked
+                else step(h, q0, std::false_type{});
             }
+            hh = end;
             if (!ok) break;
+            if (wg >= 2) continue;                                 // the third chain leaves the results to the other two
             // ---------------------------------------------------------------- dK, dV of this key tile
             ok = __all_sync(0xffffffffu, mbar_wait(acc_full, n & 1, abort_p));
             if (!ok) break;
             tc_fence_after();
-            // Each thread holds half a row (D/2 columns) of dK and of dV.  Written straight from the registers a warp's store
-            // would touch 32 different lines; the warp passes its 32 x D bytes through shared memory (16-byte pieces, piece
-            // index xor row so that neither side has bank conflicts beyond the minimum) and stores whole lines instead.
-            constexpr int kPieces = D / 16;                    // 16-byte pieces per half row
+            // Each thread holds half a row of dK and of dV (three chains: a whole row of one of them).  Written straight from the
+            // registers a warp's store would touch 32 different lines; the warp passes its rows through shared memory (16-byte
+            // pieces, piece index xor row so that neither side has bank conflicts beyond the minimum) and stores whole lines.
+            constexpr int kCols = C::kOutCols, kPieces = kCols / 8;   // 16-byte pieces per row
             constexpr int kRowsPerStore = 32 / kPieces;
-            uint8_t* stage = smem + C::kOffStage + warp * (32 * D);
+            uint8_t* stage = smem + C::kOffStage + warp * (32 * kCols * 2);
             const int key_warp = t * kTileN + (warp & 3) * 32;     // key of lane 0
 #pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                const uint32_t tA = tmem_base + lane_addr + (which == 0 ? C::kColDK : C::kColDV) + wg * (D / 2);
+            for (int part = 0; part < (C::kChains == 2 ? 2 : 1); ++part) {
+                const int which = C::kChains == 2 ? part : wg, col = C::kChains == 2 ? wg * kCols : 0;
+                const uint32_t tA = tmem_base + lane_addr + (which == 0 ? C::kColDK : C::kColDV) + col;
                 const float f = which == 0 ? p.scale : 1.f;
 #pragma unroll
-                for (int c = 0; c < D / 64; ++c) {
+                for (int c = 0; c < kCols / 32; ++c) {
                     uint32_t o[32];
                     tmem_ld32(tA + c * 32, o);
 #pragma unroll
@@ -491,16 +501,15 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         w.z = pack_bf16x2(__uint_as_float(o[v4 * 8 + 4]) * f, __uint_as_float(o[v4 * 8 + 5]) * f);
                         w.w = pack_bf16x2(__uint_as_float(o[v4 * 8 + 6]) * f, __uint_as_float(o[v4 * 8 + 7]) * f);
                         const int piece = c * 4 + v4;
-                        *reinterpret_cast<uint4*>(stage + lane * D + ((piece ^ (lane & (kPieces - 1))) << 4)) = w;
+                        *reinterpret_cast<uint4*>(stage + lane * (kCols * 2) + ((piece ^ (lane & (kPieces - 1))) << 4)) = w;
                     }
                 }
                 __syncwarp();
-                __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(which == 0 ? p.dk : p.dv) +
-                                     ((long long)bh * p.N + key_warp) * D + wg * (D / 2);
+                __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(which == 0 ? p.dk : p.dv) + ((long long)bh * p.N + key_warp) * D + col;
 #pragma unroll
                 for (int it = 0; it < 32 / kRowsPerStore; ++it) {
                     const int rrow = it * kRowsPerStore + lane / kPieces, piece = lane % kPieces;
-                    const uint4 w = *reinterpret_cast<const uint4*>(stage + rrow * D + ((piece ^ (rrow & (kPieces - 1))) << 4));
+                    const uint4 w = *reinterpret_cast<const uint4*>(stage + rrow * (kCols * 2) + ((piece ^ (rrow & (kPieces - 1))) << 4));
                     if (key_warp + rrow < p.N) *reinterpret_cast<uint4*>(dst + (long long)rrow * D + piece * 8) = w;
                 }
                 __syncwarp();
@@ -513,7 +522,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) atomicExch(p.status, base_ok ? (int)TLIN_ERR_TIMEOUT : (int)TLIN_ERR_CUDA);
-    if (warp == kMmaWarp) {
+    if (warp == C::kMma) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
     }

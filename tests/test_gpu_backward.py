@@ -433,3 +433,13 @@ def test_backward_key_tiles_dealt_by_cost(B, H, N, W, d, arrangement):
         pytest.skip("one kernel only at d = 128")
     assert B * H * -(-N // 128) * N <= 32 * 148 * W                                        # what the dispatch asks
     run_case(B, H, N, W, d, 1, seed=900 + N + W, impl=0, guarded=True, arrangement=arrangement)
+
+
+# d = 64 has three chains of 64 queries per key tile: tiles of 2 (fewer steps than chains), 4 and many steps, and several key tiles per
+# CTA, so that they begin with any chain; with and without the window rule, whole and ragged tiles
+THREE_CHAINS = [(1, 300, 128, 128, 1), (4, 80, 257, 65, 0), (3, 60, 640, 200, 1), (1, 50, 1000, 700, 0), (1, 3, 1283, 1283, 1)]
+
+
+@pytest.mark.parametrize("B,H,N,W,causal", THREE_CHAINS)
+def test_backward_chains_of_key_tiles_at_head_size_64(B, H, N, W, causal):
+    run_case(B, H, N, W, 64, causal, seed=1300 + N + W, impl=0, guarded=True, arrangement=1)
