@@ -7,7 +7,9 @@
 //
 // Two kernels, neither with atomics, both recomputing p from the saved lse (what the one kernel below does not serve).  Steps with
 // masked elements have a copy of the code of their own and the MMA warps elect their issuing lane once: B3 H12 N=W=1999 d64 175 ->
-// 160 us, B2 H8 N1961 W578 d64 62 -> 53 us, B4 H32 N8192 W1024 d64 1.31 -> 1.20 ms.
+// 160 us, B2 H8 N1961 W578 d64 62 -> 53 us, B4 H32 N8192 W1024 d64 1.31 -> 1.20 ms.  Their elementwise arithmetic runs on packed
+// pairs of floats, the same operations in half the instructions (101.6 -> 97.0 us, 65.8 -> 63.1 us, 1.14 -> 1.09 ms for the first,
+// 16 x 2000^2 and the last); the one kernel keeps single floats, as pairs there gain nothing and spill.
 //
 // bwd_dkdv_tc_kernel   A CTA owns one 128-key tile of a (b,h) at a time and walks the 128-row query tiles that may
 //   see it.  Scores are computed TRANSPOSED (S^T = K Q^T, dP^T = V dout^T: TMEM lane = key, column = query) so that
@@ -47,7 +49,7 @@ constexpr int kMmaWarp = 9;
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct BwdParams {
-    const float* lse2;        // [B*H, Wpad]  lse * log2(e), +inf beyond W
+    const float* neg_lse2;        // [B*H, Wpad]  -lse * log2(e), -inf beyond W
     const float* delta;       // [B*H, Wpad]  dout . out,   0 beyond W
     void* dq;                 // [B*H, W, D] bf16
     void* dk;                 // [B*H, N, D] bf16
@@ -63,7 +65,7 @@ struct BwdParams {
 };
 
 // ------------------------------------------------------------------------------------------ preparation
-// Row statistics of the backward pass: lse2 = lse * log2(e) and delta = sum_c out*dout, on rows padded to 128 per (b,h)
+// Row statistics of the backward pass: neg_lse2 = -lse * log2(e) and delta = sum_c out*dout, on rows padded to 128 per (b,h)
 // (padding rows: +inf and 0).  D/8 lanes share a row with one 16-byte load per tensor each; a warp keeps kPrepPasses
 // groups of rows in flight, so that enough bytes are outstanding to stream at HBM speed.
 constexpr int kPrepPasses = 4;
@@ -72,7 +74,7 @@ __host__ __device__ constexpr int prep_rows_per_block() { return 8 * (32 / (D / 
 
 template <int D>
 __global__ void __launch_bounds__(256)
-bwd_prep_kernel(const __nv_bfloat16* out, const __nv_bfloat16* dout, const float* lse, float* lse2, float* delta, float* dq32,
+bwd_prep_kernel(const __nv_bfloat16* out, const __nv_bfloat16* dout, const float* lse, float* neg_lse2, float* delta, float* dq32,
                 int W, int Wpad, long long rows_padded) {
     after_previous();
     let_next_start();
@@ -113,7 +115,7 @@ bwd_prep_kernel(const __nv_bfloat16* out, const __nv_bfloat16* dout, const float
         for (int o = LPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         const long long prow = first + ps * RPP;
         if (l == 0 && prow < rows_padded) {
-            lse2[prow] = row[ps] >= 0 ? lse[row[ps]] * kLog2e : CUDART_INF_F;
+            neg_lse2[prow] = row[ps] >= 0 ? -lse[row[ps]] * kLog2e : -CUDART_INF_F;
             delta[prow] = row[ps] >= 0 ? acc : 0.f;
         }
     }
@@ -137,7 +139,7 @@ struct ACfg {
     static_assert(384 * kComputeRegs + 128 * kOtherRegs <= 512 * 128 && kComputeRegs > 128 && kOtherRegs < 128, "register budget");
     // columns of a result row that a thread writes out: half a row of dK and of dV, or (three chains) a whole row of one of them
     static constexpr int kOutCols = kChains == 2 ? D / 2 : D;
-    static constexpr int kSlots = D == 128 ? 4 : 8;            // ring of chain steps: Q (64 rows), dout (64 rows), 64 lse2 + 64 delta
+    static constexpr int kSlots = D == 128 ? 4 : 8;            // ring of chain steps: Q (64 rows), dout (64 rows), 64 neg_lse2 + 64 delta
     static constexpr int kSlotBytes = 2 * kHalfBytes;
     static constexpr int kOffKV = 0;
     static constexpr int kOffRing = 2 * kTileBytes;
@@ -213,7 +215,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sKV = smem + C::kOffKV;          // K, V
     uint8_t* sRing = smem + C::kOffRing;      // [kSlots][Q 64 rows | dout 64 rows]
-    float* sStats = reinterpret_cast<float*>(smem + C::kOffStats);   // [kSlots][lse2 64 | delta 64]
+    float* sStats = reinterpret_cast<float*>(smem + C::kOffStats);   // [kSlots][neg_lse2 64 | delta 64]
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
     uint64_t* kv_full = bars + 0;
     uint64_t* kv_empty = bars + 1;
@@ -286,7 +288,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         tma_load_3d(dst + x * (64 * 128), &map_q, &slot_full[slot], x * 64, row, bh);
                         tma_load_3d(dst + C::kHalfBytes + x * (64 * 128), &map_do, &slot_full[slot], x * 64, row, bh);
                     }
-                    bulk_load_1d(sStats + slot * 128, p.lse2 + (long long)bh * p.Wpad + row, 256, &slot_full[slot]);
+                    bulk_load_1d(sStats + slot * 128, p.neg_lse2 + (long long)bh * p.Wpad + row, 256, &slot_full[slot]);
                     bulk_load_1d(sStats + slot * 128 + 64, p.delta + (long long)bh * p.Wpad + row, 256, &slot_full[slot]);
                 }
             }
@@ -419,6 +421,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const long long shift = (long long)p.N - p.W;       // query q may use key k iff q >= k - shift
             const int q_min = p.causal ? (int)((long long)key - shift) : -0x7fffffff;
             const int q_min_warp = p.causal ? (int)((long long)key - lane + 31 - shift) : -0x7fffffff;   // largest in the warp
+            const uint64_t scale2 = f2_pack(p.scale_log2e, p.scale_log2e);
             // a copy of the step for the tiles with masked elements: conditions in the loop cut it into short blocks
             auto step = [&](uint32_t h, int q0, auto masked_tag) {
                 constexpr bool kMasked = decltype(masked_tag)::value;
@@ -426,7 +429,7 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 const float* st = sStats + slot * 128;
                 ok = __all_sync(0xffffffffu, mbar_wait(&sdp_full[wg], (h / C::kChains) & 1, abort_p));
                 if (!ok) return;
-                // already complete (the MMAs waited for it); observing it here orders the bulk-copied lse2 / delta
+                // already complete (the MMAs waited for it); observing it here orders the bulk-copied neg_lse2 / delta
                 // before this thread's reads
                 ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[slot], (h / C::kSlots) & 1, abort_p));
                 if (!ok) return;
@@ -441,20 +444,20 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     uint32_t pk[8], dk_[8];
 #pragma unroll
                     for (int c = 0; c < 16; c += 4) {
-                        const float4 l4 = *reinterpret_cast<const float4*>(st + part * 16 + c);
-                        const float4 d4 = *reinterpret_cast<const float4*>(st + 64 + part * 16 + c);
-                        const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, dlv[4] = {d4.x, d4.y, d4.z, d4.w};
-                        float pe[4], de[4];
+                        const ulonglong2 l4 = *reinterpret_cast<const ulonglong2*>(st + part * 16 + c);        // two pairs of floats
+                        const ulonglong2 d4 = *reinterpret_cast<const ulonglong2*>(st + 64 + part * 16 + c);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            pe[e] = ex2(fmaf(__uint_as_float(sv[c + e]), p.scale_log2e, -lv[e]));
-                            if (kMasked && q0 + part * 16 + c + e < q_min) pe[e] = 0.f;
-                            de[e] = pe[e] * (__uint_as_float(dv_[c + e]) - dlv[e]);
+                        for (int e = 0; e < 4; e += 2) {
+                            float p0, p1, d0, d1;
+                            f2_unpack(f2_fma(f2_pack_bits(sv[c + e], sv[c + e + 1]), scale2, e == 0 ? l4.x : l4.y), p0, p1);
+                            p0 = ex2(p0);
+                            p1 = ex2(p1);
+                            if (kMasked && q0 + part * 16 + c + e < q_min) p0 = 0.f;
+                            if (kMasked && q0 + part * 16 + c + e + 1 < q_min) p1 = 0.f;
+                            f2_unpack(f2_mul(f2_pack(p0, p1), f2_sub(f2_pack_bits(dv_[c + e], dv_[c + e + 1]), e == 0 ? d4.x : d4.y)), d0, d1);
+                            pk[(c + e) / 2] = pack_bf16x2(p0, p1);
+                            dk_[(c + e) / 2] = pack_bf16x2(d0, d1);
                         }
-                        pk[c / 2] = pack_bf16x2(pe[0], pe[1]);
-                        pk[c / 2 + 1] = pack_bf16x2(pe[2], pe[3]);
-                        dk_[c / 2] = pack_bf16x2(de[0], de[1]);
-                        dk_[c / 2 + 1] = pack_bf16x2(de[2], de[3]);
                     }
                     // bf16 P^T over columns of S^T, dS^T over columns of dP^T, that are already in registers
                     tmem_st8(tS + part * 8, pk);
@@ -553,7 +556,7 @@ struct FCfg {
     static constexpr int kOffStage = 5 * kTileBytes;           // dS^T tile: two blocks of 128 keys x 64 queries; dK / dV rows on their way out
     static constexpr int kOffDQ = 6 * kTileBytes;              // 4 buffers of 16 queries x D fp32: dQ rows on their way to L2
     static constexpr int kDqRows = 16;
-    static constexpr int kOffStats = 7 * kTileBytes;           // 2 slots: lse2 of 128 rows, delta of 128 rows
+    static constexpr int kOffStats = 7 * kTileBytes;           // 2 slots: neg_lse2 of 128 rows, delta of 128 rows
     static constexpr int kOffBars = kOffStats + 2 * 1024;
     static constexpr int kNumBars = 18;
     static constexpr int kSmemBytes = kOffBars + kNumBars * 8 + 16;
@@ -572,7 +575,7 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do, const BwdParams p) {
     using C = FCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    float* sStats = reinterpret_cast<float*>(smem + C::kOffStats);   // [2][lse2 128 | delta 128]
+    float* sStats = reinterpret_cast<float*>(smem + C::kOffStats);   // [2][neg_lse2 128 | delta 128]
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
     uint64_t* q_full = bars + 0;      // [2] Q and the row statistics of a step
     uint64_t* q_empty = bars + 2;     // [2]
@@ -640,7 +643,7 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     ++nq;
                     for (int x = 0; x < C::kBoxes; ++x)
                         tma_load_3d(smem + C::kOffQ + slot * C::kTileBytes + x * (kQTile * 128), &map_q, &q_full[slot], x * 64, row, bh);
-                    bulk_load_1d(sStats + slot * 256, p.lse2 + (long long)bh * p.Wpad + row, 512, &q_full[slot]);
+                    bulk_load_1d(sStats + slot * 256, p.neg_lse2 + (long long)bh * p.Wpad + row, 512, &q_full[slot]);
                     bulk_load_1d(sStats + slot * 256 + 128, p.delta + (long long)bh * p.Wpad + row, 512, &q_full[slot]);
                     ok = mbar_wait(do_empty, (ndo & 1) ^ 1, abort_p);
                     if (!ok) break;
@@ -833,7 +836,7 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 const float* st = sStats + (g & 1) * 256 + wg * 64;
                 ok = __all_sync(0xffffffffu, mbar_wait(s_full, g & 1, abort_p));
                 if (!ok) return;
-                // already complete (the MMAs waited for it); observing it here orders the bulk-copied lse2 / delta
+                // already complete (the MMAs waited for it); observing it here orders the bulk-copied neg_lse2 / delta
                 // before this thread's reads
                 ok = __all_sync(0xffffffffu, mbar_wait(&q_full[g & 1], (g >> 1) & 1, abort_p));
                 if (!ok) return;
@@ -853,7 +856,7 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                         float x[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            x[e] = ex2(fmaf(__uint_as_float(pe[h][c + e]), p.scale_log2e, -lv[e]));
+                            x[e] = ex2(fmaf(__uint_as_float(pe[h][c + e]), p.scale_log2e, lv[e]));
                             if (kMasked && q0 + h * 32 + c + e < q_min) x[e] = 0.f;
                             pe[h][c + e] = __float_as_uint(x[e]);
                         }
@@ -1233,8 +1236,9 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const long long lim_warp_ll = p.causal ? (long long)p.N - p.W + (row - lane) + 1 : (long long)p.N;
             const int lim_warp = (int)(lim_warp_ll < p.N ? lim_warp_ll : p.N);
             const bool row_ok = row < p.W;
-            const float l2 = row_ok ? p.lse2[(long long)s.bh * p.Wpad + row] : CUDART_INF_F;
+            const float l2 = row_ok ? p.neg_lse2[(long long)s.bh * p.Wpad + row] : -CUDART_INF_F;
             const float dl = row_ok ? p.delta[(long long)s.bh * p.Wpad + row] : 0.f;
+            const uint64_t l22 = f2_pack(l2, l2), dl2 = f2_pack(dl, dl), scale2 = f2_pack(p.scale_log2e, p.scale_log2e);
             // a copy of the step for the tiles with masked columns (the last ones of a segment)
             auto step = [&](int j, auto masked_tag) {
                 constexpr bool kMasked = decltype(masked_tag)::value;
@@ -1251,10 +1255,15 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 mbar_arrive(&p_ready[i]);                      // S is in registers: dP may overwrite it
                 // p = 2^(s*scale*log2e - lse*log2e), kept as fp32 in the registers that held s
 #pragma unroll
-                for (int e = 0; e < kTileN; ++e) {
-                    float pe = ex2(fmaf(__uint_as_float(sv[e >> 5][e & 31]), p.scale_log2e, -l2));
-                    if (kMasked && e >= nvalid) pe = 0.f;
-                    sv[e >> 5][e & 31] = __float_as_uint(pe);
+                for (int e = 0; e < kTileN; e += 2) {
+                    float p0, p1;
+                    f2_unpack(f2_fma(f2_pack_bits(sv[e >> 5][e & 31], sv[e >> 5][(e & 31) + 1]), scale2, l22), p0, p1);
+                    p0 = ex2(p0);
+                    p1 = ex2(p1);
+                    if (kMasked && e >= nvalid) p0 = 0.f;
+                    if (kMasked && e + 1 >= nvalid) p1 = 0.f;
+                    sv[e >> 5][e & 31] = __float_as_uint(p0);
+                    sv[e >> 5][(e & 31) + 1] = __float_as_uint(p1);
                 }
                 ok = __all_sync(0xffffffffu, mbar_wait(&dp_full[i], n & 1, abort_p));
                 if (!ok) return;
@@ -1267,8 +1276,9 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     uint32_t pk[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const float d0 = __uint_as_float(sv[c >> 1][(c & 1) * 16 + 2 * e]) * (__uint_as_float(dp[2 * e]) - dl);
-                        const float d1 = __uint_as_float(sv[c >> 1][(c & 1) * 16 + 2 * e + 1]) * (__uint_as_float(dp[2 * e + 1]) - dl);
+                        const uint64_t p2 = f2_pack_bits(sv[c >> 1][(c & 1) * 16 + 2 * e], sv[c >> 1][(c & 1) * 16 + 2 * e + 1]);
+                        float d0, d1;
+                        f2_unpack(f2_mul(p2, f2_sub(f2_pack_bits(dp[2 * e], dp[2 * e + 1]), dl2)), d0, d1);
                         pk[e] = pack_bf16x2(d0, d1);
                     }
                     tmem_st8(tR + c * 8, pk);                 // bf16 dS over columns of dP that are already in registers
@@ -1397,9 +1407,9 @@ int launch_d(const void* q, const void* k, const void* v, const void* out, const
     if (rc == TLIN_OK) rc = make_map(&mdo64, dout, D, W, bh, 64);
     if (rc != TLIN_OK) return rc;
     BwdParams p;
-    float* lse2 = ws;
+    float* neg_lse2 = ws;
     float* delta = ws + bh * Wpad;
-    p.lse2 = lse2; p.delta = delta; p.dq = dq; p.dk = dk; p.dv = dv;
+    p.neg_lse2 = neg_lse2; p.delta = delta; p.dq = dq; p.dk = dk; p.dv = dv;
     p.ws = ws + 2 * bh * Wpad;
     p.status = status_word();
     if (!p.status) return TLIN_ERR_CUDA;
@@ -1416,7 +1426,7 @@ int launch_d(const void* q, const void* k, const void* v, const void* out, const
     TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_dq_tc_kernel<D, true>, BCfg<D>::kSmemBytes, smem_allowed[3]));
     const long long rows_padded = bh * Wpad;
     TLIN_CUDA_CHECK(launch_overlapped(bwd_prep_kernel<D>, (unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st,
-        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, (float*)nullptr, W, Wpad, rows_padded));
+        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, neg_lse2, delta, (float*)nullptr, W, Wpad, rows_padded));
     // dK, dV: the units are (b,h,key tile); a CTA takes a contiguous run of them
     BwdParams pa = p;
     pa.total_units = bh * p.key_tiles;
@@ -1475,10 +1485,10 @@ int launch_fused_128(const void* q, const void* k, const void* v, const void* ou
     if (rc == TLIN_OK) rc = make_map(&mdo, dout, D, W, bh);
     if (rc != TLIN_OK) return rc;
     BwdParams p;
-    float* lse2 = ws;
+    float* neg_lse2 = ws;
     float* delta = ws + bh * Wpad;
     float* dq32 = ws + 2 * bh * Wpad;
-    p.lse2 = lse2; p.delta = delta; p.dq = dq; p.dk = dk; p.dv = dv;
+    p.neg_lse2 = neg_lse2; p.delta = delta; p.dq = dq; p.dk = dk; p.dv = dv;
     p.ws = dq32;
     p.status = status_word();
     if (!p.status) return TLIN_ERR_CUDA;
@@ -1496,7 +1506,7 @@ int launch_fused_128(const void* q, const void* k, const void* v, const void* ou
     TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_fused_tc_kernel<D, kUnitDealt>, FCfg<D>::kSmemBytes, smem_allowed[1]));
     const long long rows_padded = bh * Wpad;
     TLIN_CUDA_CHECK(launch_overlapped(bwd_prep_kernel<D>, (unsigned)((rows_padded + prep_rows_per_block<D>() - 1) / prep_rows_per_block<D>()), 256, 0, st,
-        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, lse2, delta, dq32, W, Wpad, rows_padded));
+        (const __nv_bfloat16*)out, (const __nv_bfloat16*)dout, lse, neg_lse2, delta, dq32, W, Wpad, rows_padded));
     const long long ctas = p.total_units < num_sms ? p.total_units : num_sms;
     TLIN_CUDA_CHECK(launch_overlapped(kernel, (unsigned)ctas, FCfg<D>::kThreads, FCfg<D>::kSmemBytes, st, mq, mk, mv, mdo, p));
     const long long rows = bh * W, threads = rows * (D / 8);
@@ -1507,7 +1517,7 @@ int launch_fused_128(const void* q, const void* k, const void* v, const void* ou
 
 }  // namespace
 
-// row statistics (lse2, delta, padded) + the fp32 dQ sums, rows padded to 128 per (b,h)
+// row statistics (neg_lse2, delta, padded) + the fp32 dQ sums, rows padded to 128 per (b,h)
 size_t bwd_fused_workspace_bytes(long long B, long long H, long long W, int d) {
     const long long bh = B * H, Wpad = (W + tc::kQTile - 1) / tc::kQTile * tc::kQTile;
     return (size_t)(2 * bh * Wpad + bh * Wpad * d) * sizeof(float);
@@ -1520,7 +1530,7 @@ int launch_bwd_fused(const void* q, const void* k, const void* v, const void* ou
     return launch_fused_128(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, causal, ws, num_sms, st);
 }
 
-// row statistics (lse2, delta, padded) + the dQ kernel's partial slots
+// row statistics (neg_lse2, delta, padded) + the dQ kernel's partial slots
 size_t bwd_tc_workspace_bytes(long long B, long long H, long long W, int d, const tlin_fwd_plan& plan) {
     const long long bh = B * H, Wpad = (W + tc::kQTile - 1) / tc::kQTile * tc::kQTile;
     long long floats = 2 * bh * Wpad;
