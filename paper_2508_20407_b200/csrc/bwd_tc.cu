@@ -434,13 +434,19 @@ bwd_dkdv_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 ok = __all_sync(0xffffffffu, mbar_wait(&slot_full[slot], (h / C::kSlots) & 1, abort_p));
                 if (!ok) return;
                 tc_fence_after();
+                uint32_t svb[2][16], dvb[2][16];
+                tmem_ld16_async(tS, svb[0]);
+                tmem_ld16_async(tDP, dvb[0]);
 #pragma unroll
                 for (int part = 0; part < 4; ++part) {       // 16 columns at a time: 32 spill at three chains and gain nothing at two
-                    uint32_t sv[16], dv_[16];
-                    tmem_ld16_async(tS + part * 16, sv);
-                    tmem_ld16_async(tDP + part * 16, dv_);
+                    uint32_t (&sv)[16] = svb[part & 1];
+                    uint32_t (&dv_)[16] = dvb[part & 1];
                     tmem_wait_ld16(sv);
                     tmem_wait_ld16(dv_);
+                    if (part < 3) {                          // in flight during the arithmetic
+                        tmem_ld16_async(tS + (part + 1) * 16, svb[(part + 1) & 1]);
+                        tmem_ld16_async(tDP + (part + 1) * 16, dvb[(part + 1) & 1]);
+                    }
                     uint32_t pk[8], dk_[8];
 #pragma unroll
                     for (int c = 0; c < 16; c += 4) {
@@ -975,10 +981,17 @@ struct BCfg {
     static constexpr int kOffK = 4 * kTileBytes;
     static constexpr int kOffV = (4 + kKSlots) * kTileBytes;
     static constexpr int kOffBars = (4 + kKSlots + kVSlots) * kTileBytes;
-    static constexpr int kNumBars = 11 + 2 * kKSlots + 2 * kVSlots;
+    // Score buffers.  A step of one Q tile (item) holds one from its S to its dQ; the items take them in turn, in the order
+    // (key tile, Q tile).  TMEM has room for a third at d = 64: S of a later step is then ready when a warpgroup has handed over
+    // its dS.  With the TMEM reads of both kernels issued one chunk ahead: 16 x 2000^2 backward 63.3 -> 60.6 us, B4 H32 N8192 W1024
+    // 1.09 -> 1.06 ms, B3 H12 1999^2 96.8 -> 95.2 us.
+    static constexpr int kBufs = D == 128 ? 2 : 3;
+    static constexpr int kAhead = kBufs - 1;                   // S runs at most this many key tiles ahead (K slots: these and the current one)
+    static_assert(kAhead < kKSlots, "S of a later key tile would wait for the slot of the current one");
+    static constexpr int kNumBars = 9 + kBufs + 2 * kKSlots + 2 * kVSlots;
     static constexpr int kSmemBytes = kOffBars + kNumBars * 8 + 32;   // + TMEM slot, abort flag, unit range
-    // TMEM columns: R0, R1 (S, then dP, then dS as bf16; 128 each), dQ0, dQ1 (D each)
-    static constexpr uint32_t kColR = 0, kColDQ = 256;
+    // TMEM columns: the score buffers (S, then dP, then dS as bf16; 128 each), dQ0, dQ1 (D each)
+    static constexpr uint32_t kColR = 0, kColDQ = kBufs * kTileN;
     static constexpr int kThreads = 32 * 12;                   // warps 10 and 11 only lend their registers
     // setmaxnreg moves registers between warpgroups; the CTA starts with 168 per thread (65536 / 384, rounded down to a
     // multiple of 8), and an increase beyond what the other warpgroup released would wait for ever
@@ -1001,11 +1014,11 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     uint64_t* qdo_full = bars + 0;
     uint64_t* qdo_empty = bars + 1;
     uint64_t* dq_done = bars + 2;
-    uint64_t* s_full = bars + 3;      // [2]
-    uint64_t* p_ready = bars + 5;     // [2]  every thread of the tile has read S
-    uint64_t* dp_full = bars + 7;     // [2]
-    uint64_t* ds_full = bars + 9;     // [2]
-    uint64_t* k_full = bars + 11;
+    uint64_t* p_ready = bars + 3;     // [2]  every thread of the Q tile has read S
+    uint64_t* dp_full = bars + 5;     // [2]
+    uint64_t* ds_full = bars + 7;     // [2]
+    uint64_t* s_full = bars + 9;      // [kBufs] by buffer: S may be complete before the Q tile's threads have asked for the previous one
+    uint64_t* k_full = s_full + C::kBufs;
     uint64_t* k_empty = k_full + C::kKSlots;
     uint64_t* v_full = k_empty + C::kKSlots;
     uint64_t* v_empty = v_full + C::kVSlots;
@@ -1021,11 +1034,11 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         mbar_init(qdo_empty, 1);
         mbar_init(dq_done, 1);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&s_full[i], 1);
             mbar_init(&p_ready[i], kQTile);
             mbar_init(&dp_full[i], 1);
             mbar_init(&ds_full[i], kQTile);
         }
+        for (int s = 0; s < C::kBufs; ++s) mbar_init(&s_full[s], 1);
         for (int s = 0; s < C::kKSlots; ++s) {
             mbar_init(&k_full[s], 1);
             mbar_init(&k_empty[s], 1);
@@ -1122,24 +1135,25 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t kmaj_lo = (uint32_t)kmaj, mnmaj_lo = (uint32_t)mnmaj;
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
         const uint32_t lead = elect_one() ? 1u : 0u;
-        auto issue_r = [&](int i, int a_byte_off, int b_byte_off) {        // R_i = A B^T (contraction over d)
+        auto issue_r = [&](int buf, int a_byte_off, int b_byte_off) {        // R_buf = A B^T (contraction over d)
             const uint32_t a_lo = kmaj_lo + (uint32_t)(a_byte_off >> 4), b_lo = kmaj_lo + (uint32_t)(b_byte_off >> 4);
-            const uint32_t d = tmem_u + C::kColR + i * kTileN;
+            const uint32_t d = tmem_u + C::kColR + buf * kTileN;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t off16 = ((kk >> 2) * (kQTile * 128) + (kk & 3) * 32) >> 4;
                 mma_ss_lead(lead, d, a_lo + off16, b_lo + off16, desc_hi, idesc_s, kk > 0);
             }
         };
-        auto issue_dq = [&](int i, int k_byte_off, bool accumulate) {       // dQ_i += dS_i K (contraction over keys)
+        auto issue_dq = [&](int i, int buf, int k_byte_off, bool accumulate) {       // dQ_i += dS_i K (contraction over keys)
             const uint32_t b_lo = mnmaj_lo + (uint32_t)(k_byte_off >> 4);
-            const uint32_t d = tmem_u + C::kColDQ + i * D, a = tmem_u + C::kColR + i * kTileN;
+            const uint32_t d = tmem_u + C::kColDQ + i * D, a = tmem_u + C::kColR + buf * kTileN;
 #pragma unroll
             for (int kk = 0; kk < kTileN / 16; ++kk)
                 mma_ts_lead(lead, d, a + kk * 8, b_lo + kk * (2048 >> 4), desc_hi, idesc_dq, (accumulate || kk > 0) ? 1u : 0u);
         };
-        uint32_t kit = 0, vit = 0, seg_idx = 0;
+        uint32_t kit = 0, vit = 0, seg_idx = 0;                             // kit: first key tile of the segment, in the order of loading
         uint32_t n_step[2] = {0, 0};
+        uint32_t s_item = 0, r_item = 0, q_item = 0;                        // items whose S, dP, dQ have been issued
         bool ok = base_ok;
         std::conditional_t<kDeal, DealtWalker, SegmentWalker> walk(p, starts);
         Segment s;
@@ -1151,15 +1165,26 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const int cq[2] = {c0, c1};
             ok = __all_sync(0xffffffffu, mbar_wait(qdo_full, seg_idx & 1, abort_p));
             if (!ok) break;
-            uint32_t ks = kit % C::kKSlots;
-            ok = __all_sync(0xffffffffu, mbar_wait(&k_full[ks], (kit / C::kKSlots) & 1, abort_p));
-            if (!ok) break;
-            tc_fence_after();
-            for (int i = 0; i < 2; ++i)
-                if (cq[i] > 0) {
-                    issue_r(i, C::kOffQ + i * C::kTileBytes, C::kOffK + ks * C::kTileBytes);
-                    commit_lead(lead, &s_full[i]);
+            int js = 0, is = c0 > 0 ? 0 : 1, k_seen = 0;                    // next item to get its S; key tiles known to have arrived
+            // S of the next items, as far as buffers are free and K tiles up to j_most
+            auto issue_s = [&](int j_most) {
+                while (js < cnt && js <= j_most && s_item - q_item < (uint32_t)C::kBufs) {
+                    const uint32_t kt = kit + js, slot = kt % C::kKSlots, buf = s_item % C::kBufs;
+                    if (js >= k_seen) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&k_full[slot], (kt / C::kKSlots) & 1, abort_p));
+                        if (!ok) return;
+                        k_seen = js + 1;
+                    }
+                    tc_fence_after();
+                    issue_r(buf, C::kOffQ + is * C::kTileBytes, C::kOffK + slot * C::kTileBytes);
+                    commit_lead(lead, &s_full[buf]);
+                    ++s_item;
+                    do {
+                        if (++is == 2) is = 0, ++js;
+                    } while (js < cnt && js >= (is == 0 ? c0 : c1));
                 }
+            };
+            issue_s(C::kAhead);
             for (int j = 0; j < cnt && ok; ++j) {
                 const uint32_t vs = vit % C::kVSlots;
                 ok = __all_sync(0xffffffffu, mbar_wait(&v_full[vs], (vit / C::kVSlots) & 1, abort_p));
@@ -1170,40 +1195,31 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                         ok = __all_sync(0xffffffffu, mbar_wait(&p_ready[i], n_step[i] & 1, abort_p));
                         if (!ok) break;
                         tc_fence_after();
-                        issue_r(i, C::kOffDO + i * C::kTileBytes, C::kOffV + vs * C::kTileBytes);   // dP over S
+                        issue_r(r_item % C::kBufs, C::kOffDO + i * C::kTileBytes, C::kOffV + vs * C::kTileBytes);   // dP over S
                         commit_lead(lead, &dp_full[i]);
+                        ++r_item;
                     }
                 }
                 if (!ok) break;
                 commit_lead(lead, &v_empty[vs]);
-                const bool have_next = j + 1 < cnt;
-                if (!have_next) commit_lead(lead, qdo_empty);       // Q and dout of this segment have been read for the last time
-                uint32_t nks = 0;
-                if (have_next) {
-                    nks = (kit + 1) % C::kKSlots;
-                    ok = __all_sync(0xffffffffu, mbar_wait(&k_full[nks], ((kit + 1) / C::kKSlots) & 1, abort_p));
-                    if (!ok) break;
-                }
+                if (j + 1 == cnt) commit_lead(lead, qdo_empty);     // Q and dout of this segment have been read for the last time
+                const uint32_t ks = (kit + j) % C::kKSlots;
                 for (int i = 0; i < 2 && ok; ++i) {
                     if (j < cq[i]) {
                         ok = __all_sync(0xffffffffu, mbar_wait(&ds_full[i], n_step[i] & 1, abort_p));
                         if (!ok) break;
                         tc_fence_after();
-                        issue_dq(i, C::kOffK + ks * C::kTileBytes, j > 0);
+                        issue_dq(i, q_item % C::kBufs, C::kOffK + ks * C::kTileBytes, j > 0);
                         ++n_step[i];
-                    }
-                    if (have_next && j + 1 < cq[i]) {
-                        tc_fence_after();
-                        issue_r(i, C::kOffQ + i * C::kTileBytes, C::kOffK + nks * C::kTileBytes);
-                        commit_lead(lead, &s_full[i]);
+                        ++q_item;
+                        issue_s(j + C::kAhead);
                     }
                 }
                 if (!ok) break;
                 commit_lead(lead, &k_empty[ks]);
-                ++kit;
-                ks = nks;
             }
             if (!ok) break;
+            kit += cnt;
             commit_lead(lead, dq_done);
             ++seg_idx;
         }
@@ -1214,9 +1230,9 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int i = warp >> 2;
         const int r = (warp & 3) * 32 + lane;
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tR = tmem_base + lane_addr + C::kColR + i * kTileN;
+        const uint32_t tScores = tmem_base + lane_addr + C::kColR;
         const uint32_t tDQ = tmem_base + lane_addr + C::kColDQ + i * D;
-        uint32_t n = 0, seg_idx = 0;
+        uint32_t n = 0, seg_idx = 0, items = 0;               // items of the segments before
         bool ok = base_ok;
         std::conditional_t<kDeal, DealtWalker, SegmentWalker> walk(p, starts);
         int bh_first = 0;                                     // (b,h) of this CTA's first unit (used under schedule 0 only)
@@ -1242,7 +1258,9 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // a copy of the step for the tiles with masked columns (the last ones of a segment)
             auto step = [&](int j, auto masked_tag) {
                 constexpr bool kMasked = decltype(masked_tag)::value;
-                ok = __all_sync(0xffffffffu, mbar_wait(&s_full[i], n & 1, abort_p));
+                const uint32_t item = items + (j < c0 ? j + (uint32_t)i : c0) + (j < c1 ? j : c1);
+                const uint32_t tR = tScores + (item % C::kBufs) * kTileN;
+                ok = __all_sync(0xffffffffu, mbar_wait(&s_full[item % C::kBufs], (item / C::kBufs) & 1, abort_p));
                 if (!ok) return;
                 tc_fence_after();
                 const int nvalid = lim_row - (s.t_begin + j) * kTileN;
@@ -1268,11 +1286,13 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 ok = __all_sync(0xffffffffu, mbar_wait(&dp_full[i], n & 1, abort_p));
                 if (!ok) return;
                 tc_fence_after();
+                uint32_t dpb[2][16];
+                tmem_ld16_async(tR, dpb[0]);
 #pragma unroll
                 for (int c = 0; c < kTileN / 16; ++c) {
-                    uint32_t dp[16];
-                    tmem_ld16_async(tR + c * 16, dp);
+                    uint32_t (&dp)[16] = dpb[c & 1];
                     tmem_wait_ld16(dp);
+                    if (c + 1 < kTileN / 16) tmem_ld16_async(tR + (c + 1) * 16, dpb[(c + 1) & 1]);   // in flight during the arithmetic
                     uint32_t pk[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
@@ -1294,6 +1314,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             for (; j < n_open && ok; ++j) step(j, std::false_type{});
             for (; j < cnt_i && ok; ++j) step(j, std::true_type{});
             if (!ok) break;
+            items += c0 + c1;
             const uint32_t my_seg = seg_idx;
             if (!skipped) ++seg_idx;
             if (allowed_i == 0) continue;                      // this Q tile does not exist
