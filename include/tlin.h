@@ -304,9 +304,9 @@ typedef struct {
 } tlin_fwd_plan;
 
 typedef struct {
-    int32_t splits;        /* CTAs per (b,h)                                                 */
+    int32_t splits;        /* parts the keys of a (b,h) are cut into                         */
     int32_t keys_per_split;/* split s covers keys [s*keys_per_split, min(L, (s+1)*keys_per_split)) */
-    int32_t n_ctas;
+    int32_t n_ctas;        /* splits of all (b,h): one CTA each, or a run of them per CTA where more than fit on the chip */
     int64_t workspace_bytes;
 } tlin_decode_plan;
 

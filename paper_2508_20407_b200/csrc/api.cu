@@ -53,7 +53,7 @@ void log_fwd_plan(const char* what, int B, int H, int N, int W, int d, int causa
             p.uses_workspace ? " (split, merged by a second kernel)" : "");
 }
 void log_decode_plan(const char* what, int B, int H, int Ncap, int pos, int d, const tlin_decode_plan& p) {
-    fprintf(stderr, "libtlin: %s B=%d H=%d Ncap=%d pos=%d d=%d -> %d splits of %d keys, %d ctas, workspace %lld bytes\n",
+    fprintf(stderr, "libtlin: %s B=%d H=%d Ncap=%d pos=%d d=%d -> %d splits of %d keys, %d in all, workspace %lld bytes\n",
             what, B, H, Ncap, pos, d, p.splits, p.keys_per_split, p.n_ctas, (long long)p.workspace_bytes);
 }
 }  // namespace
@@ -339,7 +339,7 @@ extern "C" int tlin_decode_step(const void* q_new, const void* k_new, const void
     if (log_plans()) log_decode_plan("decode", B, H, Ncap, pos, d, plan);
     const Workspace w = workspace();
     if (!w.ptr || w.bytes < (size_t)plan.workspace_bytes) return TLIN_ERR_WORKSPACE;
-    return launch_decode(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, pos, nullptr, d, plan,
+    return launch_decode(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, pos, nullptr, d, plan, sms,
                          (float*)w.ptr, (cudaStream_t)stream);
 }
 
@@ -388,7 +388,7 @@ extern "C" int tlin_decode_step_fp8(const void* q_new, const void* k_new, const 
     if (rc != TLIN_OK) return rc;
     const Workspace w = workspace();
     if (!w.ptr || w.bytes < (size_t)plan.workspace_bytes) return TLIN_ERR_WORKSPACE;
-    return launch_decode_fp8(q_new, k_new, v_new, k_cache, v_cache, k_scale, v_scale, out, lse, B, H, Ncap, pos, d, plan,
+    return launch_decode_fp8(q_new, k_new, v_new, k_cache, v_cache, k_scale, v_scale, out, lse, B, H, Ncap, pos, d, plan, sms,
                              (float*)w.ptr, (cudaStream_t)stream);
 }
 
@@ -411,7 +411,7 @@ extern "C" int tlin_decode_step_ragged(const void* q_new, const void* k_new, con
     const Workspace w = workspace();
     if (!w.ptr || w.bytes < (size_t)plan.workspace_bytes) return TLIN_ERR_WORKSPACE;
     // the kernel checks every entry against max_pos (and Ncap) and reports a bad one through the status word
-    return launch_decode(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, max_pos, pos, d, plan,
+    return launch_decode(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, max_pos, pos, d, plan, sms,
                          (float*)w.ptr, (cudaStream_t)stream);
 }
 

@@ -303,8 +303,10 @@ extern "C" int tlin_plan_decode(int B, int H, int L, int d, int num_sms, tlin_de
     for (int s = 1; s <= max_s; ++s) {
         int64_t kps = (L + s - 1) / s;
         kps = (kps + 7) / 8 * 8;
-        const int64_t waves = (bh * s + slots - 1) / slots;
-        const int64_t cost = waves * (kps + 64);   // + a fixed per-CTA overhead, in keys
+        // A CTA takes one split, or a run of them read as one key range per (b,h); + a fixed overhead per range, in keys.  Runs make
+        // fine splits cheap, and these divide a ragged batch evenly (B16 H16, up to 8001 rows: 114 us with 8 splits, 104 with 15).
+        const int64_t run = (bh * s + slots - 1) / slots;
+        const int64_t cost = run * kps + 64 * ((run - 1) / s + 1 + (run > 1 && run % s != 0 ? 1 : 0));
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best_s = s; }
     }
     tlin_decode_plan p = {};

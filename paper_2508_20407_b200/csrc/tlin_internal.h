@@ -13,7 +13,7 @@ constexpr int kDefaultSMs = 148;       // B200
 constexpr int kTileN = 128;            // keys per tile on the tensor path
 constexpr int kSimtRows = 8;           // query rows per CTA on the CUDA-core path
 constexpr int kSimtKeys = 32;          // keys per staged tile on the CUDA-core path
-constexpr int kDecodeMaxSplits = 64;   // upper bound on CTAs per (b,h) in the decode step
+constexpr int kDecodeMaxSplits = 64;   // upper bound on the splits of a (b,h) in the decode step
 constexpr int kDecodeMinKeys = 256;    // do not split the cache finer than this
 constexpr int kDecodeCtasPerSM = 2;
 
@@ -149,7 +149,7 @@ int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float*
 int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long long* starts, int n_ctas, cudaStream_t st);
 int launch_decode(const void* q_new, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                   void* out, float* lse, int B, int H, int Ncap, int pos, const int* pos_per_seq, int d,
-                  const tlin_decode_plan& plan, float* ws, cudaStream_t st);
+                  const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st);
 int launch_bwd_simt(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                     void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, int is_f32, float* ws,
                     cudaStream_t st);
@@ -167,7 +167,7 @@ int decode_table_max_problems();
 int launch_decode_table(const tlin_decode_problem* problems, int n, int d, cudaStream_t st);
 int launch_decode_fp8(const void* q_new, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                       const float* k_scale, const float* v_scale, void* out, float* lse, int B, int H, int Ncap, int pos,
-                      int d, const tlin_decode_plan& plan, float* ws, cudaStream_t st);
+                      int d, const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st);
 int launch_merge_pair_bf16(const void* oa, const float* la, const void* ob, const float* lb,
                            void* out, float* lse, int64_t rows, int d, cudaStream_t st);
 int launch_merge_pair_f32(const float* oa, const float* la, const float* ob, const float* lb,

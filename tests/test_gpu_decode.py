@@ -445,3 +445,38 @@ def test_batched_decode_table_every_problem_against_the_oracle(d, n_problems):
     with pytest.raises(tl.TlinError):
         bad = list(problems[0]); bad[5] = problems[0][3].shape[2]                          # pos beyond the cache
         tl.tlin_decode_step_batched([tuple(bad)])
+
+
+# more splits than CTAs fit: a CTA takes a run of them, over the end of a (b,h) and (ragged) over sequences of one split or none beyond it
+@pytest.mark.parametrize("kind,B,H,N0,d", [("bf16", 45, 7, 2299, 128), ("fp8", 3, 120, 2499, 64), ("ragged", 40, 8, 2099, 64), ("ragged", 45, 7, 2299, 128)])
+def test_decode_runs_of_splits(kind, B, H, N0, d):
+    plan = tl.tlin_plan_decode(B, H, N0 + 1, d, 148)
+    assert plan.splits > 1 and plan.n_ctas > 2 * 148
+    if kind == "fp8":
+        kc_h, vc_h, ks, vs, qn, kn, vn = _fp8_cache(synth.Workload("dec8", B, H, d, N0, 1, seed=5, decode=True), pad=2)
+        kc, vc = kc_h.to(DEV), vc_h.to(DEV)
+        out, lse = tl.tlin_decode_step_fp8(qn[0].to(DEV), kn[0].to(DEV), vn[0].to(DEV), kc, vc, ks.to(DEV), vs.to(DEV), N0)
+        ref, ref_lse = oracle.decode_step_fp8(qn[0], kn[0], vn[0], kc_h, vc_h, ks, vs, N0)
+        parity.check(out.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", "fp8 runs")
+    else:
+        rng = torch.Generator(device="cpu").manual_seed(N0 + d)
+        kc_h, vc_h = (torch.randn((B, H, N0 + 3, d), generator=rng).to(torch.bfloat16) for _ in range(2))
+        q, kn, vn = (torch.randn((B, H, 1, d), generator=rng).to(torch.bfloat16) for _ in range(3))
+        kc, vc = kc_h.to(DEV), vc_h.to(DEV)
+        pos, bad = torch.full((B,), N0, dtype=torch.int32), 7
+        if kind == "ragged":
+            pos = torch.randint(0, N0 + 1, (B,), generator=rng, dtype=torch.int32)
+            pos[0], pos[1], pos[2], pos[bad] = 0, N0, plan.keys_per_split - 1, N0 + 1       # the last one is beyond the bound
+            out, lse = tl.tlin_decode_step_ragged(q.to(DEV), kn.to(DEV), vn.to(DEV), kc, vc, pos.to(DEV), N0)
+            assert tl.tlin_get_status() == tl.ERR_INVALID_ARG
+            assert float(out[bad].float().abs().max()) == 0.0 and bool((lse[bad] == float("-inf")).all())
+        else:
+            out, lse = tl.tlin_decode_step(q.to(DEV), kn.to(DEV), vn.to(DEV), kc, vc, N0)
+        for b in range(B):
+            if kind == "ragged" and b == bad:
+                continue
+            sl = slice(b, b + 1)
+            ref, ref_lse = oracle.decode_step(q[sl], kn[sl], vn[sl], kc_h[sl], vc_h[sl], int(pos[b]))
+            parity.check(out[sl].float().cpu().numpy(), lse[sl].cpu().numpy(), ref, ref_lse, "bf16", f"{kind} runs, sequence {b}")
+    assert tl.tlin_get_status() == 0
+    assert torch.equal(kc.cpu(), kc_h) and torch.equal(vc.cpu(), vc_h)
