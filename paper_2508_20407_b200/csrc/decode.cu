@@ -8,10 +8,12 @@
 // each warp-load covers 512 contiguous bytes (32/LPR rows); the LPR lanes that share a row reduce
 // their partial dot products with xor-shuffles.  Every row-group keeps its own running max/sum and
 // they are combined at the end; the CTA writes one normalised partial (o, lse) per (b,h) to the workspace and
-// a second kernel merges the splits (log-sum-exp weights).
+// a second kernel merges the splits (log-sum-exp weights).  Short steps merge inside a cluster instead (decode_cluster_kernel).
 #include "tlin_internal.h"
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 #include <math_constants.h>
+#include <atomic>
 #include <mutex>
 #include <string.h>
 
@@ -20,6 +22,7 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kUnroll = 4;
+constexpr int kMaxCluster = kDecodeMaxCluster;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -174,9 +177,11 @@ __device__ __forceinline__ int splits_of(int pos, int kps, int pos_all, int Ncap
 }
 // The splits of all (b,h), in order, dealt out as contiguous runs, one per CTA.  Neighbouring splits of one (b,h) are read as one
 // key range, so a CTA starts and ends a stream of loads once or twice instead of once per split: all CTAs of a wave of equal
-// splits end together, and draining, combining and starting anew idled the memory for about 3 us per wave.
-// B4 H32 d128, 8-bit cache of 15002 rows: 97 -> 87.5 us; B8 H32, 8-bit of 5001: 75.6 -> 62.0, bf16 of 4001: 94.2 -> 87.2.  Ragged, only
-// the splits that have keys are dealt: B3 H32 of up to 21489 rows 157 -> 137 us.
+// splits end together, and draining, combining and starting anew idled the memory for about 3 us per wave.  At two CTAs per SM,
+// B4 H32 d128, 8-bit cache of 15002 rows: 97 -> 87.5 us; B8 H32, 8-bit of 5001: 75.6 -> 62.0, bf16 of 4001: 94.2 -> 87.2.  Ragged,
+// only the splits that have keys are dealt: B3 H32 of up to 21489 rows 157 -> 137 us.
+// Three CTAs per SM (80 registers) have 98 KB of loads in flight per SM instead of 65: 87.5 -> 81.8, 62.0 -> 58.6, 87.2 -> 83.1,
+// 137 -> 128 us, and B8 H32 d128 65537 rows 1330 -> 1200 us = 7.1 TB/s (more than the copy bandwidth, which has writes in it).
 struct KeyRun {
     int bh, sp, left;                                      // first split, number of splits
     __device__ void single(int splits) {                   // one split per CTA
@@ -294,6 +299,79 @@ decode_splitk_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_new,
     }
 }
 
+// A short step: the splits of a (b,h) are the CTAs of a cluster, and the first of them merges the others' sums out of their shared
+// memory.  No second kernel and no trip of the partials through global memory, whose latencies are much of a step of 10 us:
+// B6 H12 d64 of up to 1778 rows 11.0 -> 10.3 us, B2 H16 d64 1401 rows 8.6 -> 6.5, B1 H32 d64 201 rows (one split) 5.4 -> 4.0.
+// kPerSM: where two CTAs per SM do not hold all clusters at a time, three may (the first of these: 72 clusters of 4, or of 6).
+template <int D, int kPerSM>
+__global__ void __launch_bounds__(kWarps * 32, kPerSM)
+decode_cluster_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_new, uint4* k_cache, uint4* v_cache,
+                      __nv_bfloat16* out, float* lse, int Ncap, int pos_all, const int* pos_per_seq, int H, int* status,
+                      int splits, int kps, float scale_log2e) {
+    namespace cg = cooperative_groups;
+    constexpr int LPR = D / 8;           // lanes (16-byte chunks) per row
+    const int bh = blockIdx.x / splits, sp = blockIdx.x - bh * splits;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    after_previous();
+    let_next_start();
+    int pos = pos_all;
+    if (pos_per_seq != nullptr) {
+        pos = pos_per_seq[bh / H];
+        if (!position_ok(pos, pos_all, Ncap)) {              // the same for every CTA of the cluster
+            if (threadIdx.x == 0) atomicExch(status, (int)TLIN_ERR_INVALID_ARG);
+            if (sp == 0 && threadIdx.x < D) {
+                out[(int64_t)bh * D + threadIdx.x] = __float2bfloat16_rn(0.f);
+                if (lse != nullptr && threadIdx.x == 0) lse[bh] = -CUDART_INF_F;
+            }
+            return;
+        }
+    }
+    const int j0 = sp * kps, j1 = min(pos + 1, j0 + kps);
+    const uint4* kn = k_new + (int64_t)bh * LPR;
+    const uint4* vn = v_new + (int64_t)bh * LPR;
+    uint4* kc = k_cache + (int64_t)bh * Ncap * LPR;
+    uint4* vc = v_cache + (int64_t)bh * Ncap * LPR;
+    if (pos >= j0 && pos < j1 && warp == 0 && lane < LPR) {  // append, as in decode_splitk_kernel
+        kc[(int64_t)pos * LPR + lane] = kn[lane];
+        vc[(int64_t)pos * LPR + lane] = vn[lane];
+    }
+    float a, ll, mm;
+    attend_key_range<D>(q_new + (int64_t)bh * LPR, kn, vn, kc, vc, j0, j1, pos, scale_log2e, a, ll, mm);
+
+    __shared__ float part[D + 2];                            // un-normalised sums, row sum, maximum (log2 units)
+    cg::cluster_group cl = cg::this_cluster();
+    if (sp != 0 && threadIdx.x < D) {
+        part[threadIdx.x] = a;
+        if (threadIdx.x == 0) part[D] = ll, part[D + 1] = mm;
+    }
+    cl.sync();
+    if (sp == 0 && threadIdx.x < D) {
+        float v[kMaxCluster], l[kMaxCluster], m[kMaxCluster];
+        v[0] = a, l[0] = ll, m[0] = mm;
+#pragma unroll
+        for (int r = 1; r < kMaxCluster; ++r) {
+            v[r] = 0.f, l[r] = 0.f, m[r] = -CUDART_INF_F;
+            if (r < splits) {
+                const float* other = cl.map_shared_rank(part, r);
+                v[r] = other[threadIdx.x], l[r] = other[D], m[r] = other[D + 1];
+            }
+        }
+        float top = m[0];
+#pragma unroll
+        for (int r = 1; r < kMaxCluster; ++r) top = fmaxf(top, m[r]);     // finite: the first split has a key
+        float sum = 0.f, z = 0.f;
+#pragma unroll
+        for (int r = 0; r < kMaxCluster; ++r) {
+            const float w = exp2f(m[r] - top);
+            z = fmaf(w, l[r], z);
+            sum = fmaf(w, v[r], sum);
+        }
+        out[(int64_t)bh * D + threadIdx.x] = __float2bfloat16_rn(sum / z);
+        if (lse != nullptr && threadIdx.x == 0) lse[bh] = (top + log2f(z)) * kLn2;
+    }
+    cl.sync();                                               // shared memory stays until it has been read
+}
+
 // A table of decode problems as one launch: one CTA per (problem, b*h), whole key range, result written directly (no
 // split, no second kernel).  Meant for the per-layer caches of a block, which are short (Appendix A, cache hit: the
 // (H+1) D W_oh term -- one row against the W_oh summary tokens of a layer -- and the row inside the window).
@@ -387,11 +465,6 @@ static_assert(kDecodeMaxSplits <= 64, "the merge reads two splits per lane");
 // each for K and V, codes widened in pairs by cvt.rn.f16x2.e4m3x2 (exact).  The key scale is folded into q, the value
 // scale into the final normalisation.  The new row is stored as encode(x / scale) (fp32 division, round to nearest
 // even, saturating) and every lane that meets it takes the same codes from k_new / v_new instead of the cache.
-__device__ __forceinline__ float2 e4m3x2_to_f32x2(uint32_t two_codes) {      // low byte -> x, next byte -> y
-    uint32_t h2;
-    asm("{\n\t.reg .b16 c;\n\tcvt.u16.u32 c, %1;\n\tcvt.rn.f16x2.e4m3x2 %0, c;\n\t}" : "=r"(h2) : "r"(two_codes));
-    return __half22float2(*reinterpret_cast<const __half2*>(&h2));
-}
 __device__ __forceinline__ uint32_t f32x2_to_e4m3x2(float lo, float hi) {     // lo -> low byte, hi -> next byte
     uint32_t r;
     asm("{\n\t.reg .b16 c;\n\tcvt.rn.satfinite.e4m3x2.f32 c, %1, %2;\n\tcvt.u32.u16 %0, c;\n\t}" : "=r"(r) : "f"(hi), "f"(lo));
@@ -431,14 +504,6 @@ __device__ __forceinline__ void axpy16_codes(uint32_t p2, const uint4& c, float 
             : "+f"(acc[4 * i]), "+f"(acc[4 * i + 1]), "+f"(acc[4 * i + 2]), "+f"(acc[4 * i + 3]) : "r"(w[i]), "r"(p2));
     }
 }
-__device__ __forceinline__ void widen16(const uint4& c, float (&x)[16]) {
-    const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 a = e4m3x2_to_f32x2(w[i] & 0xffffu), b = e4m3x2_to_f32x2(w[i] >> 16);
-        x[4 * i + 0] = a.x; x[4 * i + 1] = a.y; x[4 * i + 2] = b.x; x[4 * i + 3] = b.y;
-    }
-}
 // 16 bf16 values (two 16-byte words) divided by `scale` and encoded
 __device__ __forceinline__ uint4 quantise16(const uint4& lo8, const uint4& hi8, float scale) {
     const uint32_t w[8] = {lo8.x, lo8.y, lo8.z, lo8.w, hi8.x, hi8.y, hi8.z, hi8.w};
@@ -452,7 +517,7 @@ __device__ __forceinline__ uint4 quantise16(const uint4& lo8, const uint4& hi8, 
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-template <int D, bool kRuns>
+template <int D>
 __global__ void __launch_bounds__(kWarps * 32, kDecodeCtasPerSM)
 decode_fp8_splitk_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_new,
                          uint4* k_cache, uint4* v_cache,
@@ -470,10 +535,9 @@ decode_fp8_splitk_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_
     after_previous();
     let_next_start();
     KeyRun run;
-    if (kRuns) run.uniform(n_bh, splits);
-    else run.single(splits);
+    run.uniform(n_bh, splits);
     while (run.left > 0) {
-        const int bh = run.bh, take = kRuns ? min(run.left, splits - run.sp) : 1;
+        const int bh = run.bh, take = min(run.left, splits - run.sp);
         const int j0 = run.sp * kps, j1 = min(L, j0 + take * kps);
         const float ks = k_scale[bh], vs = v_scale[bh];
 
@@ -586,23 +650,64 @@ decode_fp8_splitk_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_
             part_o[slot * D + c] = ll > 0.f ? a * vs / ll : 0.f;          // the value scale applied once per output element
             if (c == 0) part_lse[slot] = ll > 0.f ? (mm + log2f(ll)) * kLn2 : -CUDART_INF_F;
         }
-        if (!kRuns) break;
         run.close(part_lse, splits, splits, take);
     }
 }
 
 // Runs where there are more splits than CTAs fit on the chip.  A single split per (b,h) leaves nothing to join, and the hardware's
-// own dealing of CTAs is then a little better (B64 H32 d128, 514 rows: 100 against 101.5 us).
+// own dealing of CTAs is then a little better (B64 H32 d128, 514 rows, at two CTAs per SM: 100 against 101.5 us).
 bool use_runs(const tlin_decode_plan& plan, int sms) { return plan.splits > 1 && plan.n_ctas > sms * kDecodeCtasPerSM; }
+
+// Clusters of `size` CTAs of decode_cluster_kernel that the device holds at a time (asked once per device, size and head size).
+template <int D, int kPerSM>
+int clusters_at_a_time(int size) {
+    static std::atomic<int> known[64][kMaxCluster + 1];
+    const int dev = current_device_slot();
+    if (dev < 0) return 0;
+    int n = known[dev][size].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)size);
+        cfg.blockDim = dim3(kWarps * 32);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<D, kPerSM>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        n += 1;                                              // 0: not asked yet
+        known[dev][size].store(n, std::memory_order_relaxed);
+    }
+    return n - 1;
+}
 
 template <int D>
 int launch_d(const void* q_new, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
              void* out, float* lse, int B, int H, int Ncap, int pos, const int* pos_per_seq, const tlin_decode_plan& plan,
-             int sms, float* ws, cudaStream_t st) {
+             int sms, float* ws, cudaStream_t st, bool two_kernels) {
     const int64_t bh = (int64_t)B * H;
     float* part_o = ws;
     float* part_lse = ws + bh * kDecodeMaxSplits * D;
     const float scale_log2e = kLog2e / sqrtf((float)D);
+    // The cluster kernel, with so many CTAs per SM; 0: two kernels.  Long splits are bound by the memory, and clusters fill the SMs
+    // less evenly (B3 H16 31756 rows as 6 splits: 142 us, two kernels 129).  A single split per (b,h) needs no merge at all; more of
+    // them than two per SM profit from the third (B64 H32 514 rows: 100 -> 89 us), fewer spread better without (B8 H32 983 rows: 24.6
+    // against 25.3 us).
+    int per_sm = 0;
+    if (!two_kernels && plan.splits == 1) per_sm = plan.n_ctas > 2 * sms ? 3 : 2;
+    else if (!two_kernels && plan.splits <= kMaxCluster && plan.keys_per_split <= kDecodeClusterKeys)
+        per_sm = bh <= clusters_at_a_time<D, 2>(plan.splits) ? 2 : bh <= clusters_at_a_time<D, 3>(plan.splits) ? 3 : 0;
+    if (per_sm > 0) {
+        TLIN_CUDA_CHECK(launch_overlapped_clusters(per_sm == 2 ? decode_cluster_kernel<D, 2> : decode_cluster_kernel<D, 3>, plan.n_ctas, plan.splits,
+            kWarps * 32, 0, st, (const uint4*)q_new, (const uint4*)k_new, (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache,
+            (__nv_bfloat16*)out, lse, Ncap, pos, pos_per_seq, H, status_word(), plan.splits, plan.keys_per_split, scale_log2e));
+        count_launch();
+        return TLIN_OK;
+    }
     const bool runs = use_runs(plan, sms);
     TLIN_CUDA_CHECK(launch_overlapped(runs ? decode_splitk_kernel<D, true> : decode_splitk_kernel<D, false>,
         (unsigned)(runs ? sms * kDecodeCtasPerSM : plan.n_ctas), kWarps * 32, 0, st,
@@ -622,7 +727,7 @@ int launch_fp8_d(const void* q_new, const void* k_new, const void* v_new, void* 
     float* part_lse = ws + bh * kDecodeMaxSplits * D;
     const float scale_log2e = kLog2e / sqrtf((float)D);
     const bool runs = use_runs(plan, sms);
-    TLIN_CUDA_CHECK(launch_overlapped(runs ? decode_fp8_splitk_kernel<D, true> : decode_fp8_splitk_kernel<D, false>,
+    TLIN_CUDA_CHECK(launch_overlapped(decode_fp8_splitk_kernel<D>,
         (unsigned)(runs ? sms * kDecodeCtasPerSM : plan.n_ctas), kWarps * 32, 0, st,
         (const uint4*)q_new, (const uint4*)k_new, (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, k_scale, v_scale,
         part_o, part_lse, Ncap, pos, (int)bh, plan.splits, plan.keys_per_split, scale_log2e));
@@ -672,9 +777,9 @@ int launch_decode_fp8(const void* q_new, const void* k_new, const void* v_new, v
 
 int launch_decode(const void* q_new, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                   void* out, float* lse, int B, int H, int Ncap, int pos, const int* pos_per_seq, int d,
-                  const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st) {
-    if (d == 128) return launch_d<128>(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, pos, pos_per_seq, plan, sms, ws, st);
-    if (d == 64) return launch_d<64>(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, pos, pos_per_seq, plan, sms, ws, st);
+                  const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st, bool two_kernels) {
+    if (d == 128) return launch_d<128>(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, pos, pos_per_seq, plan, sms, ws, st, two_kernels);
+    if (d == 64) return launch_d<64>(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, pos, pos_per_seq, plan, sms, ws, st, two_kernels);
     return TLIN_ERR_UNSUPPORTED;
 }
 
@@ -749,5 +854,5 @@ extern "C" int tlin_decode_step_static(const void* q_new, const void* k_new, con
     rc = tlin_plan_decode(B, H, pos + 1, d, sms, &plan);
     if (rc != TLIN_OK) return rc;
     return launch_decode(q_new, k_new, v_new, k_cache, v_cache, out, lse, B, H, Ncap, pos, nullptr, d, plan, sms, scratch,
-                         (cudaStream_t)stream);
+                         (cudaStream_t)stream, true);
 }

@@ -303,10 +303,17 @@ extern "C" int tlin_plan_decode(int B, int H, int L, int d, int num_sms, tlin_de
     for (int s = 1; s <= max_s; ++s) {
         int64_t kps = (L + s - 1) / s;
         kps = (kps + 7) / 8 * 8;
-        // A CTA takes one split, or a run of them read as one key range per (b,h); + a fixed overhead per range, in keys.  Runs make
-        // fine splits cheap, and these divide a ragged batch evenly (B16 H16, up to 8001 rows: 114 us with 8 splits, 104 with 15).
+        // In keys at the rate of a full SM.  A CTA takes one split, or a run of them read as one key range per (b,h); one or two CTAs
+        // on an SM get more than their third of its rate (4 x 32 heads, 15002 8-bit rows: 128 / 256 / 384 CTAs 142 / 93 / 83 us).
+        // + a fixed overhead per range, and about as much for the merge kernel where neither a cluster nor a single split does
+        // without it.  Runs make fine splits cheap, and these divide a ragged batch evenly (B16 H16, up to 8001 rows: 114 us with 8
+        // splits, 104 with 15).
         const int64_t run = (bh * s + slots - 1) / slots;
-        const int64_t cost = run * kps + 64 * ((run - 1) / s + 1 + (run > 1 && run % s != 0 ? 1 : 0));
+        const int64_t per_sm = (bh * s + num_sms - 1) / num_sms;
+        const int64_t rows = run > 1 || per_sm > 2 ? run * kps : kps * (per_sm == 1 ? 39 : 50) / 64;
+        const int64_t ranges = (run - 1) / s + 1 + (run > 1 && run % s != 0 ? 1 : 0);
+        const bool merge = s > 1 && (run > 1 || s > kDecodeMaxCluster || kps > kDecodeClusterKeys);
+        const int64_t cost = rows + 64 * (ranges + merge);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best_s = s; }
     }
     tlin_decode_plan p = {};

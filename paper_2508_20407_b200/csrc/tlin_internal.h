@@ -14,8 +14,10 @@ constexpr int kTileN = 128;            // keys per tile on the tensor path
 constexpr int kSimtRows = 8;           // query rows per CTA on the CUDA-core path
 constexpr int kSimtKeys = 32;          // keys per staged tile on the CUDA-core path
 constexpr int kDecodeMaxSplits = 64;   // upper bound on the splits of a (b,h) in the decode step
+constexpr int kDecodeMaxCluster = 8;   // up to this many splits are merged inside a cluster (the portable cluster size)
+constexpr int kDecodeClusterKeys = 1024;   // ... when they are no longer than this
 constexpr int kDecodeMinKeys = 256;    // do not split the cache finer than this
-constexpr int kDecodeCtasPerSM = 2;
+constexpr int kDecodeCtasPerSM = 3;    // 98 KB of loads in flight per SM (figures: KeyRun in decode.cu)
 
 struct Workspace { void* ptr; size_t bytes; };
 Workspace workspace();
@@ -114,18 +116,26 @@ __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 template <class... Params, class... Args>
-inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args) {
+inline cudaError_t launch_overlapped_clusters(void (*kernel)(Params...), unsigned grid, unsigned cluster, unsigned block, size_t smem, cudaStream_t st,
+                                              Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
+}
+template <class... Params, class... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args) {
+    return launch_overlapped_clusters(kernel, grid, 1, block, smem, st, static_cast<Args&&>(args)...);
 }
 
 #define TLIN_CUDA_CHECK(expr)                                                              \
@@ -149,7 +159,7 @@ int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float*
 int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long long* starts, int n_ctas, cudaStream_t st);
 int launch_decode(const void* q_new, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                   void* out, float* lse, int B, int H, int Ncap, int pos, const int* pos_per_seq, int d,
-                  const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st);
+                  const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st, bool two_kernels = false);
 int launch_bwd_simt(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                     void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, int is_f32, float* ws,
                     cudaStream_t st);

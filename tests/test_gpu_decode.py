@@ -480,3 +480,25 @@ def test_decode_runs_of_splits(kind, B, H, N0, d):
             parity.check(out[sl].float().cpu().numpy(), lse[sl].cpu().numpy(), ref, ref_lse, "bf16", f"{kind} runs, sequence {b}")
     assert tl.tlin_get_status() == 0
     assert torch.equal(kc.cpu(), kc_h) and torch.equal(vc.cpu(), vc_h)
+
+
+# short steps: the splits of a (b,h) are the CTAs of a cluster (1 to 8), some of them beyond the end of their sequence
+@pytest.mark.parametrize("splits", range(1, 9))
+@pytest.mark.parametrize("d", [64, 128])
+def test_decode_clusters_of_splits(splits, d):
+    B, H, N0 = 4, 2, 256 * splits - 4
+    plan = tl.tlin_plan_decode(B, H, N0 + 1, d, 148)
+    assert plan.splits == splits
+    rng = torch.Generator(device="cpu").manual_seed(splits)
+    kc_h, vc_h = (torch.randn((B, H, N0 + 3, d), generator=rng).to(torch.bfloat16) for _ in range(2))
+    q, kn, vn = (torch.randn((B, H, 1, d), generator=rng).to(torch.bfloat16) for _ in range(3))
+    kc, vc = kc_h.to(DEV), vc_h.to(DEV)
+    pos = [N0, 0, min(plan.keys_per_split, N0), N0 + 1]        # the last one is beyond the bound
+    out, lse = tl.tlin_decode_step_ragged(q.to(DEV), kn.to(DEV), vn.to(DEV), kc, vc, torch.tensor(pos, dtype=torch.int32, device=DEV), N0)
+    assert tl.tlin_get_status() == tl.ERR_INVALID_ARG and tl.tlin_last_launch_count() == 1
+    assert float(out[3].float().abs().max()) == 0.0 and bool((lse[3] == float("-inf")).all())
+    for b in range(3):
+        sl = slice(b, b + 1)
+        ref, ref_lse = oracle.decode_step(q[sl], kn[sl], vn[sl], kc_h[sl], vc_h[sl], pos[b])
+        parity.check(out[sl].float().cpu().numpy(), lse[sl].cpu().numpy(), ref, ref_lse, "bf16", f"cluster of {splits}, sequence {b}")
+    assert torch.equal(kc.cpu(), kc_h) and torch.equal(vc.cpu(), vc_h) and tl.tlin_get_status() == 0
