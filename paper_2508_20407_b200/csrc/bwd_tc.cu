@@ -988,7 +988,7 @@ struct BCfg {
     static constexpr int kBufs = D == 128 ? 2 : 3;
     static constexpr int kAhead = kBufs - 1;                   // S runs at most this many key tiles ahead (K slots: these and the current one)
     static_assert(kAhead < kKSlots, "S of a later key tile would wait for the slot of the current one");
-    static constexpr int kNumBars = 9 + kBufs + 2 * kKSlots + 2 * kVSlots;
+    static constexpr int kNumBars = 9 + 2 * kBufs + 2 * kKSlots + 2 * kVSlots;
     static constexpr int kSmemBytes = kOffBars + kNumBars * 8 + 32;   // + TMEM slot, abort flag, unit range
     // TMEM columns: the score buffers (S, then dP, then dS as bf16; 128 each), dQ0, dQ1 (D each)
     static constexpr uint32_t kColR = 0, kColDQ = kBufs * kTileN;
@@ -1017,8 +1017,10 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     uint64_t* p_ready = bars + 3;     // [2]  every thread of the Q tile has read S
     uint64_t* dp_full = bars + 5;     // [2]
     uint64_t* ds_full = bars + 7;     // [2]
-    uint64_t* s_full = bars + 9;      // [kBufs] by buffer: S may be complete before the Q tile's threads have asked for the previous one
-    uint64_t* k_full = s_full + C::kBufs;
+    // [2][kBufs] by Q tile and its step mod kBufs.  S may be complete before the tile's threads have asked for the previous one, so one
+    // barrier per tile would be a phase ahead; and by buffer, a warpgroup that skips a segment would ask for a phase beyond the next.
+    uint64_t* s_full = bars + 9;
+    uint64_t* k_full = s_full + 2 * C::kBufs;
     uint64_t* k_empty = k_full + C::kKSlots;
     uint64_t* v_full = k_empty + C::kKSlots;
     uint64_t* v_empty = v_full + C::kVSlots;
@@ -1038,7 +1040,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             mbar_init(&dp_full[i], 1);
             mbar_init(&ds_full[i], kQTile);
         }
-        for (int s = 0; s < C::kBufs; ++s) mbar_init(&s_full[s], 1);
+        for (int s = 0; s < 2 * C::kBufs; ++s) mbar_init(&s_full[s], 1);
         for (int s = 0; s < C::kKSlots; ++s) {
             mbar_init(&k_full[s], 1);
             mbar_init(&k_empty[s], 1);
@@ -1154,6 +1156,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         uint32_t kit = 0, vit = 0, seg_idx = 0;                             // kit: first key tile of the segment, in the order of loading
         uint32_t n_step[2] = {0, 0};
         uint32_t s_item = 0, r_item = 0, q_item = 0;                        // items whose S, dP, dQ have been issued
+        uint32_t s_step[2] = {0, 0};                                        // per Q tile: steps whose S has been issued
         bool ok = base_ok;
         std::conditional_t<kDeal, DealtWalker, SegmentWalker> walk(p, starts);
         Segment s;
@@ -1177,7 +1180,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     }
                     tc_fence_after();
                     issue_r(buf, C::kOffQ + is * C::kTileBytes, C::kOffK + slot * C::kTileBytes);
-                    commit_lead(lead, &s_full[buf]);
+                    commit_lead(lead, is == 0 ? &s_full[s_step[0]++ % C::kBufs] : &s_full[C::kBufs + s_step[1]++ % C::kBufs]);
                     ++s_item;
                     do {
                         if (++is == 2) is = 0, ++js;
@@ -1260,7 +1263,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 constexpr bool kMasked = decltype(masked_tag)::value;
                 const uint32_t item = items + (j < c0 ? j + (uint32_t)i : c0) + (j < c1 ? j : c1);
                 const uint32_t tR = tScores + (item % C::kBufs) * kTileN;
-                ok = __all_sync(0xffffffffu, mbar_wait(&s_full[item % C::kBufs], (item / C::kBufs) & 1, abort_p));
+                ok = __all_sync(0xffffffffu, mbar_wait(&s_full[i * C::kBufs + n % C::kBufs], (n / C::kBufs) & 1, abort_p));
                 if (!ok) return;
                 tc_fence_after();
                 const int nvalid = lim_row - (s.t_begin + j) * kTileN;

@@ -443,3 +443,13 @@ THREE_CHAINS = [(1, 300, 128, 128, 1), (4, 80, 257, 65, 0), (3, 60, 640, 200, 1)
 @pytest.mark.parametrize("B,H,N,W,causal", THREE_CHAINS)
 def test_backward_chains_of_key_tiles_at_head_size_64(B, H, N, W, causal):
     run_case(B, H, N, W, 64, causal, seed=1300 + N + W, impl=0, guarded=True, arrangement=1)
+
+
+# CTAs that go from query tile pairs with one 128-row half to pairs with both, in either order: the half without rows runs ahead
+HALF_PAIRS = [(1, 4, 512, 300, 64, 1), (1, 120, 1400, 640, 64, 1), (1, 160, 320, 300, 64, 1), (1, 160, 320, 300, 128, 1), (1, 100, 700, 300, 128, 0), (1, 90, 400, 330, 64, 0)]
+
+
+@pytest.mark.parametrize("B,H,N,W,d,causal", HALF_PAIRS)
+def test_backward_pairs_with_one_half(B, H, N, W, d, causal):
+    for _ in range(3):
+        run_case(B, H, N, W, d, causal, seed=1500 + N + W, impl=0, guarded=False, arrangement=1)
