@@ -127,7 +127,8 @@ typedef struct {
 int tlin_attn_forward_batched(const tlin_problem* problems, int n_problems, int d, tlin_stream_t stream);
 /* The split of a table's units among the CTAs of one launch (n_problems <= 24): starts[c] = first unit of CTA c,
  * starts[*n_ctas] = number of units; unit order = problem, then b*h, then query tile pair.  starts has room for
- * num_sms + 1 entries (num_sms <= 0: 148).  Pure host arithmetic. */
+ * num_sms + 1 entries (num_sms <= 0: 148).  Pure host arithmetic.  tlin_attn_forward_batched takes these runs, or, for up to 1024
+ * units, deals the units out singly where that makes the costliest CTA cheaper. */
 int tlin_plan_batched(const tlin_problem* problems, int n_problems, int num_sms, int64_t* starts, int32_t* n_ctas);
 
 /* Same as tlin_attn_forward with HOST input/output buffers (ideally pinned).  *_h are HOST

@@ -202,9 +202,11 @@ extern "C" int tlin_attn_forward_batched(const tlin_problem* problems, int n_pro
         if (log_plans())
             fprintf(stderr, "libtlin: batched forward, problems %d..%d of %d, d=%d -> %lld units on %d ctas\n", first, first + n - 1,
                     n_problems, d, (long long)starts[n_ctas], n_ctas);
-        long long st[kMaxGroups + 1];
-        for (int g = 0; g <= n_ctas; ++g) st[g] = starts[g];
-        rc = launch_fwd_tc_batched(problems + first, n, d, st, n_ctas, (cudaStream_t)stream);
+        long long runs[kMaxGroups + 1], lists[kMaxGroups + 1];
+        uint16_t order[kMaxListedUnits];
+        for (int g = 0; g <= n_ctas; ++g) runs[g] = starts[g];
+        const bool listed = deal_batched_units(problems + first, n, n_ctas, runs, lists, order);
+        rc = launch_fwd_tc_batched(problems + first, n, d, listed ? lists : runs, listed ? order : nullptr, n_ctas, (cudaStream_t)stream);
         if (rc != TLIN_OK) return rc;
     }
     return TLIN_OK;

@@ -110,6 +110,8 @@ template <> struct KernelMaps<true> {
     CUtensorMap q[kMaxBatch], k[kMaxBatch], v[kMaxBatch];
     ProblemDev prob[kMaxBatch];
     int n;
+    int listed;                        // the CTAs' units are order[u], not u
+    uint16_t order[kMaxListedUnits];
 };
 
 struct Params {
@@ -125,17 +127,19 @@ struct Params {
     float scale_log2e;
 };
 
-// Walks the units of a batched launch: whole problems, in table order.
+// Walks the units of a batched launch: whole problems, in table order (a contiguous run or a list).
 struct BatchWalker {
     long long u, u1;
     const ProblemDev* prob;
+    const uint16_t* order;
     int n, pi;
     __device__ BatchWalker(const KernelMaps<true>& m, const GroupStarts& starts)
-        : u(starts.u[blockIdx.x]), u1(starts.u[blockIdx.x + 1]), prob(m.prob), n(m.n), pi(0) {}
+        : u(starts.u[blockIdx.x]), u1(starts.u[blockIdx.x + 1]), prob(m.prob), order(m.listed ? m.order : nullptr), n(m.n), pi(0) {}
     __device__ bool next(Segment& s) {
         if (u >= u1) return false;
-        while (pi + 1 < n && u >= prob[pi + 1].unit0) ++pi;
-        const long long r = u - prob[pi].unit0;
+        const long long x = order != nullptr ? (long long)order[u] : u;
+        while (pi + 1 < n && x >= prob[pi + 1].unit0) ++pi;
+        const long long r = x - prob[pi].unit0;
         s.bh = (int)(r / prob[pi].q_tiles);
         s.qt = (int)(r - (long long)s.bh * prob[pi].q_tiles);
         s.t_begin = 0;
@@ -788,14 +792,18 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
     return TLIN_OK;
 }
 
-// A table of problems as one launch: every CTA walks a contiguous run of whole (problem, b*h, query tile pair) units.
+// A table of problems as one launch: every CTA walks a contiguous run or a list of whole (problem, b*h, query tile pair) units.
 template <int D>
-int launch_batched_d(const tlin_problem* problems, int n, const long long* starts_in, int n_ctas, cudaStream_t st) {
+int launch_batched_d(const tlin_problem* problems, int n, const long long* starts_in, const uint16_t* order, int n_ctas, cudaStream_t st) {
     using C = Cfg<D>;
     static_assert(sizeof(KernelMaps<true>) + sizeof(Params) + sizeof(GroupStarts) < 32000, "launch parameters exceed the limit");
     KernelMaps<true> maps;
     memset(&maps, 0, sizeof(maps));
     maps.n = n;
+    if (order != nullptr) {
+        maps.listed = 1;
+        memcpy(maps.order, order, sizeof(uint16_t) * (size_t)starts_in[n_ctas]);
+    }
     long long unit = 0;
     for (int i = 0; i < n; ++i) {
         const tlin_problem& pb = problems[i];
@@ -829,10 +837,10 @@ int launch_batched_d(const tlin_problem* problems, int n, const long long* start
 
 }  // namespace
 
-int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long long* starts, int n_ctas, cudaStream_t st) {
+int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long long* starts, const uint16_t* order, int n_ctas, cudaStream_t st) {
     if (n <= 0 || n > kMaxBatch) return TLIN_ERR_INVALID_ARG;
-    if (d == 128) return launch_batched_d<128>(problems, n, starts, n_ctas, st);
-    if (d == 64) return launch_batched_d<64>(problems, n, starts, n_ctas, st);
+    if (d == 128) return launch_batched_d<128>(problems, n, starts, order, n_ctas, st);
+    if (d == 64) return launch_batched_d<64>(problems, n, starts, order, n_ctas, st);
     return TLIN_ERR_UNSUPPORTED;
 }
 

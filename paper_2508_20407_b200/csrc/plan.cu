@@ -3,6 +3,7 @@
 // rule; Appendix A, cost terms), and every function here is tested against that count.
 #include "tlin_internal.h"
 #include <algorithm>
+#include <functional>
 #include <vector>
 
 using namespace tlin;
@@ -140,6 +141,56 @@ static int check_problem(const tlin_problem& pb) {
     return TLIN_OK;
 }
 
+static long long batched_unit_cost(const tlin_problem& pb, int key_tiles, int qt) {
+    return pb.causal_window ? fwd_problem_cost(pb.n_keys, pb.n_queries, key_tiles, qt) : key_tiles + 2;
+}
+
+bool tlin::deal_batched_units(const tlin_problem* problems, int n_problems, int n_ctas, const long long* runs, long long* starts, uint16_t* order) {
+    const long long U = runs[n_ctas];
+    if (U <= n_ctas || U > kMaxListedUnits) return false;
+    struct Class { long long cost; int first, step, count; };          // the units of one query tile pair of a problem, over its b*h
+    std::vector<Class> classes;
+    std::vector<long long> cost((size_t)U);
+    int unit = 0;
+    for (int i = 0; i < n_problems; ++i) {
+        const tlin_problem& pb = problems[i];
+        const int key_tiles = (pb.n_keys + kTileN - 1) / kTileN, q_tiles = (pb.n_queries + 255) / 256;
+        for (int qt = 0; qt < q_tiles; ++qt) {
+            const Class c = {batched_unit_cost(pb, key_tiles, qt), unit + qt, q_tiles, pb.BH};
+            for (int x = 0; x < c.count; ++x) cost[c.first + x * c.step] = c.cost;
+            classes.push_back(c);
+        }
+        unit += pb.BH * q_tiles;
+    }
+    long long costliest_run = 0;
+    for (int g = 0; g < n_ctas; ++g) {
+        long long sum = 0;
+        for (long long u = runs[g]; u < runs[g + 1]; ++u) sum += cost[u];
+        costliest_run = std::max(costliest_run, sum);
+    }
+    std::stable_sort(classes.begin(), classes.end(), [](const Class& a, const Class& b) { return a.cost > b.cost; });
+    typedef std::pair<long long, int> Load;                            // cost so far, CTA
+    std::vector<Load> heap((size_t)n_ctas);
+    for (int g = 0; g < n_ctas; ++g) heap[g] = Load(0, g);             // equal loads: already a heap
+    std::vector<int> owner((size_t)U), count((size_t)n_ctas + 1, 0);
+    long long costliest = 0;
+    for (const Class& c : classes)
+        for (int x = 0; x < c.count; ++x) {
+            std::pop_heap(heap.begin(), heap.end(), std::greater<Load>());
+            Load& least = heap.back();
+            least.first += c.cost;
+            costliest = std::max(costliest, least.first);
+            owner[c.first + x * c.step] = least.second;
+            ++count[least.second + 1];
+            std::push_heap(heap.begin(), heap.end(), std::greater<Load>());
+        }
+    if (costliest >= costliest_run) return false;
+    for (int g = 0; g < n_ctas; ++g) count[g + 1] += count[g];
+    for (int g = 0; g <= n_ctas; ++g) starts[g] = count[g];
+    for (long long u = 0; u < U; ++u) order[count[owner[u]]++] = (uint16_t)u;
+    return true;
+}
+
 extern "C" int tlin_plan_batched(const tlin_problem* problems, int n_problems, int num_sms, int64_t* starts, int32_t* n_ctas) {
     if (!problems || !starts || !n_ctas || n_problems <= 0 || n_problems > kMaxBatch) return TLIN_ERR_INVALID_ARG;
     if (num_sms <= 0) num_sms = kDefaultSMs;
@@ -153,7 +204,7 @@ extern "C" int tlin_plan_batched(const tlin_problem* problems, int n_problems, i
         if ((long long)pb.BH * pb.n_queries > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
         for (int bh = 0; bh < pb.BH; ++bh)
             for (int qt = 0; qt < q_tiles; ++qt)
-                prefix.push_back(prefix.back() + (pb.causal_window ? fwd_problem_cost(pb.n_keys, pb.n_queries, key_tiles, qt) : key_tiles + 2));
+                prefix.push_back(prefix.back() + batched_unit_cost(pb, key_tiles, qt));
     }
     const long long U = (long long)prefix.size() - 1;
     const int G = (int)std::min<long long>(num_sms, U);

@@ -105,6 +105,13 @@ __host__ __device__ inline long long bwd_first_unit_of_share(int N, int W, int c
 // fills starts[0 .. n_ctas], every CTA non-empty (n_ctas <= units).
 constexpr int kMaxBatch = 24;          // problems per launch of the batched kernel (its table travels as a launch parameter)
 void balanced_run_starts(const long long* prefix, long long units, int n_ctas, long long* starts);
+// With one to seven units per CTA a contiguous run is a coarse share.  Up to kMaxListedUnits units are dealt singly instead, each in
+// turn, costliest first, to the CTA with the least so far, if that makes the costliest CTA cheaper than `runs` (the starts of the
+// contiguous runs) does: CTA c then takes order[starts[c]] .. order[starts[c + 1] - 1], in ascending order.  Returns whether it does.
+// Four requests' inner layers at d = 128 (8 heads, 1024 + 1024 rows: 256 units of 10 to 19 on 148 CTAs): costliest 30 -> 27, 56.8 -> 52.1
+// us; 48 + 144 units of 6 requests (211 + 708 rows, d = 64) 28.3 -> 20.9 us; 4 x 32 heads of 300 + 1000 rows 96 -> 80 us.
+constexpr int kMaxListedUnits = 1024;
+bool deal_batched_units(const tlin_problem* problems, int n_problems, int n_ctas, const long long* runs, long long* starts, uint16_t* order);
 
 // Launches of one call, and of successive calls, overlap their starts: a kernel launched here may begin while the kernel before it
 // in the stream is still finishing (programmatic dependent launch), sets up what needs no memory, and waits in after_previous()
@@ -156,7 +163,8 @@ int launch_fwd_simt_f32(const float* q, const float* k, const float* v, float* o
 int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float* lse,
                   int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& plan,
                   float* ws, long long kv_rows_alloc, cudaStream_t st);   // kv_rows_alloc: rows per (b,h) of k, v (0 = N)
-int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long long* starts, int n_ctas, cudaStream_t st);
+// order: null, or the units in the order of the CTAs' lists (deal_batched_units)
+int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long long* starts, const uint16_t* order, int n_ctas, cudaStream_t st);
 int launch_decode(const void* q_new, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                   void* out, float* lse, int B, int H, int Ncap, int pos, const int* pos_per_seq, int d,
                   const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st, bool two_kernels = false);

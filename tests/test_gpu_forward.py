@@ -619,3 +619,18 @@ def test_forward_problems_dealt_by_cost(B, H, N, W, d, causal):
     plan = tl.tlin_plan_forward(B, H, N, W, d, causal)
     assert plan.schedule == 1 and plan.q_tiles > 1 and 4 * B * H * N * d <= 64 << 20      # what the dispatch asks
     guarded_compare(synth.Workload("dealt", B, H, d, N, W, seed=70 + N, causal_window=causal), 2)
+
+
+# units dealt singly to the CTAs: a few more than CTAs, the most a list holds, and one more (contiguous runs)
+@pytest.mark.parametrize("d,specs", [(128, [(1, 60, 500, 500, 300, 1), (1, 40, 600, 600, 100, 0)]), (64, [(1, 12, 200, 200, 700, 0), (1, 100, 1000, 900, 300, 1), (1, 3, 3000, 3000, 129, 1)]),
+                                     (64, [(4, 127, 320, 320, 257, 1), (1, 8, 900, 900, 64, 0)]), (64, [(4, 127, 320, 320, 257, 1), (1, 9, 900, 900, 64, 0)])])
+def test_batched_forward_units_dealt_singly(d, specs):
+    problems, guards = _batched_case(d, specs, seed=40 + d)
+    tl.tlin_attn_forward_batched(problems)
+    torch.cuda.synchronize()
+    assert tl.tlin_get_status() == 0 and tl.tlin_last_launch_count() == 1
+    for i, ((q, k, v, out, lse, n_keys, causal), (og, lg)) in enumerate(zip(problems, guards)):
+        og.check(f"problem {i} out")
+        lg.check(f"problem {i} lse")
+        ref, ref_lse = oracle.attn_forward(q.cpu(), k[:, :, :n_keys].contiguous().cpu(), v[:, :, :n_keys].contiguous().cpu(), causal)
+        parity.check(out.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", f"problem {i} {specs[i]}")
