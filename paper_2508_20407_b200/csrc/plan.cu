@@ -290,7 +290,7 @@ int tlin::plan_forward(int B, int H, int N, int W, int d, int causal_window, int
         const int64_t problems = bh * p.q_tiles;
         const int64_t ctas1 = num_sms < problems ? num_sms : problems;
         const int64_t kv_bytes = 2 * bh * (int64_t)N * d * 2;
-        const bool kv_in_l2 = p.q_tiles == 1 || kv_bytes <= (int64_t)64 << 20;
+        const bool kv_in_l2 = p.q_tiles == 1 || kv_bytes <= kKVInL2;
         int64_t cost1 = ((problems + ctas1 - 1) / ctas1) * ((int64_t)p.key_tiles + 2);
         bool allow1 = kv_in_l2;
         if (causal_window && p.q_tiles > 1) {

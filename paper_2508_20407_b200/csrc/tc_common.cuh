@@ -120,7 +120,7 @@ inline EncodeTiledFn encode_fn() {
 // Does a launch that follows this plan deal its problems out by cost?  K and V are read by the query tiles of a (b,h) at unrelated
 // times, so they have to stay in L2 (the bound the planner uses for schedule 1).
 inline bool dealt(const tlin_fwd_plan& plan, long long bh, int d) {
-    return plan.schedule == 1 && plan.causal_window && plan.q_tiles > 1 && 2 * bh * plan.n_keys * (long long)d * 2 <= (64LL << 20);
+    return plan.schedule == 1 && plan.causal_window && plan.q_tiles > 1 && 2 * bh * plan.n_keys * (long long)d * 2 <= kKVInL2;
 }
 
 // [BH, rows, D] bf16, box = 64 elements x box_rows rows x 1, 128-byte swizzle, zero fill outside.  rows_alloc > rows: only
