@@ -14,12 +14,15 @@
 // CTAs are numbered group*q_tiles + q_tile: the q_tiles CTAs of a group walk the same (b,h,key-tile)
 // units at the same time, so K/V tiles are fetched from HBM once and re-read from L2.  A group's unit
 // range may start or end in the middle of a (b,h); such partial results (normalised o, lse) go to the
-// workspace and fwd_merge_kernel combines them with log-sum-exp weights.
+// workspace and fwd_merge_kernel combines them with log-sum-exp weights.  Few, short problems are merged inside
+// clusters instead (kCluster).
 //
 // Every wait is bounded: on expiry the CTA sets the library's error word, drains and exits.
 #include "tlin_internal.h"
 #include "sm100_ptx.cuh"
 #include "tc_common.cuh"
+#include <atomic>
+#include <cooperative_groups.h>
 #include <math_constants.h>
 #include <mutex>
 #include <string.h>
@@ -78,7 +81,12 @@ __device__ __forceinline__ void exp2_poly2(uint64_t x2, float& p0, float& p1) {
 // W1000 d256 3952 -> 56 us, B4 H12 N370 W96 d32 96 -> 12 us.
 // kDealt and kAnyDealt are the first and the last with problems dealt out by cost (DealtWalker; a form of their own because the
 // choice at run time costs the others 1 to 2 %).
-enum { kOneProblem = 0, kTable = 1, kAnyHead = 2, kDealt = 3, kAnyDealt = 4 };
+// kCluster is the first for few, short problems: the CTAs of a cluster share the keys of one (b,h,query tile pair), leave their rows in
+// their shared memory, and each merges a share of the rows from all of them; no merge kernel, no partials in global memory.
+// Against split groups and the merge kernel: B2 H4 N3000 W100 d64 17.2 -> 11.9 us, B1 H16 N2000 W200 d64 17.9 -> 13.9, B4 H8 N1000 W64 d128
+// 18.1 -> 14.3, B2 H16 N4000 W250 d128 33.6 -> 29.4, B1 H4 N1024 W128 d64 8.5 -> 8.3.
+enum { kOneProblem = 0, kTable = 1, kAnyHead = 2, kDealt = 3, kAnyDealt = 4, kCluster = 5 };
+constexpr int kMaxCluster = 8;             // the portable size
 
 template <int D>
 struct Cfg {
@@ -123,6 +131,7 @@ struct Params {
     int n_groups, q_tiles, key_tiles;
     int N, W, causal;
     int d;                // head size (row length of every tensor)
+    int cluster;          // CTAs that share a problem's keys (kCluster)
     int schedule;         // 0: groups of q_tiles CTAs stream key ranges; 1: every CTA walks whole (b,h,q-tile) problems
     float scale_log2e;
 };
@@ -149,10 +158,31 @@ struct BatchWalker {
         return true;
     }
 };
+// The one segment of a CTA of a cluster: its share of the key tiles that the pair may use.
+struct ClusterWalker {
+    Segment seg;
+    bool more;
+    __device__ ClusterWalker(const Params& p) : more(true) {
+        const int problem = blockIdx.x / p.cluster, rank = blockIdx.x - problem * p.cluster;
+        seg.prob = 0;
+        seg.bh = problem / p.q_tiles;
+        seg.qt = problem - seg.bh * p.q_tiles;
+        const int a0 = tiles_allowed(p, seg.qt * kTileM, 0), a1 = tiles_allowed(p, seg.qt * kTileM, 1), tiles = a0 > a1 ? a0 : a1;
+        seg.t_begin = tiles * rank / p.cluster;
+        seg.t_end = tiles * (rank + 1) / p.cluster;
+    }
+    __device__ bool next(Segment& s) {
+        s = seg;
+        const bool had = more;
+        more = false;
+        return had;
+    }
+};
 template <int kForm>
 __device__ __forceinline__ auto make_walker(const KernelMaps<kForm == kTable>& m, const Params& p, const GroupStarts& starts) {
     if constexpr (kForm == kTable) return BatchWalker(m, starts);
     else if constexpr (kForm == kDealt || kForm == kAnyDealt) return DealtWalker(p, starts);
+    else if constexpr (kForm == kCluster) return ClusterWalker(p);
     else return SegmentWalker(p, starts);
 }
 // shape (N, W, causal, key_tiles) and result pointers of the problem a segment belongs to
@@ -403,6 +433,11 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             }
         }
     }
+    if constexpr (kForm == kCluster) {          // the two barriers of the merge below
+        __syncwarp();
+        cluster_sync();
+        cluster_sync();
+    }
     } else {
         // ------------------------------------------------------------------ softmax warpgroups (one per Q tile)
         setmaxnreg_inc<kSoftmaxRegs>();
@@ -531,6 +566,82 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             int j = 0;
             for (; j < n_open && ok; ++j) step(j, std::false_type{});
             for (; j < cnt_i && ok; ++j) step(j, std::true_type{});
+            if constexpr (kForm == kCluster) {
+                // -------------------------------------------------------- merge inside the cluster
+                if (ok && cnt_i > 0) {
+                    ok = mbar_wait(&pv_done[i], (n - 1) & 1, abort_p);
+                    ok = __all_sync(0xffffffffu, ok);
+                    tc_fence_after();
+                }
+                float x0, x1, x2, x3;
+                f2_unpack(l2[0], x0, x1);
+                f2_unpack(l2[1], x2, x3);
+                const float l = (x0 + x1) + (x2 + x3);
+                const bool have = ok && l > 0.f;
+                float* sO = reinterpret_cast<float*>(smem);       // 256 rows of D, 16-byte pieces at (piece xor row mod 8)
+                float* sLse = sO + kTileM * D;
+                static_assert(kForm != kCluster || kTileM * (D + 1) * 4 <= C::kSmemTiles, "the rows lie over Q and the ring");
+                named_barrier(1, 256);             // both Q tiles' products are complete: Q and the ring are free
+                const int rl = i * kQTile + r;
+                sLse[rl] = have ? (m_ref + log2f(l)) * kLn2 : -CUDART_INF_F;
+                const float inv_l = have ? 1.f / l : 0.f;
+                if (ok && cnt_i > 0) {
+#pragma unroll
+                    for (int c = 0; c < D / 16; ++c) {
+                        uint32_t o[16];
+                        tmem_ld16_async(tO + c * 16, o);
+                        tmem_wait_ld16(o);
+#pragma unroll
+                        for (int v4 = 0; v4 < 4; ++v4)
+                            *reinterpret_cast<float4*>(sO + rl * D + (((c * 4 + v4) ^ (rl & 7)) << 2)) =
+                                make_float4(__uint_as_float(o[v4 * 4]) * inv_l, __uint_as_float(o[v4 * 4 + 1]) * inv_l,
+                                            __uint_as_float(o[v4 * 4 + 2]) * inv_l, __uint_as_float(o[v4 * 4 + 3]) * inv_l);
+                    }
+                }
+                __syncwarp();
+                cluster_sync();
+                namespace cg = cooperative_groups;
+                cg::cluster_group cl = cg::this_cluster();
+                constexpr int kLanes = D / 4 < 32 ? D / 4 : 32;     // lanes per row
+                const int rank = (int)cl.block_rank(), piece = lane % kLanes;
+                const int rr_end = kTileM * (rank + 1) / p.cluster;
+                for (int rr = kTileM * rank / p.cluster + warp * (32 / kLanes) + lane / kLanes; rr < rr_end; rr += 8 * (32 / kLanes)) {
+                    const int out_row = row0 + rr;
+                    float part[kMaxCluster];
+                    float4 x[kMaxCluster];
+                    float top = -CUDART_INF_F;
+#pragma unroll
+                    for (int c = 0; c < kMaxCluster; ++c) {
+                        part[c] = c < p.cluster ? cl.map_shared_rank(sLse, c)[rr] : -CUDART_INF_F;
+                        top = fmaxf(top, part[c]);
+                    }
+#pragma unroll
+                    for (int c = 0; c < kMaxCluster; ++c) {         // a share without keys for the row has left nothing there
+                        x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (part[c] != -CUDART_INF_F) x[c] = *reinterpret_cast<const float4*>(cl.map_shared_rank(sO, c) + rr * D + ((piece ^ (rr & 7)) << 2));
+                    }
+                    const float ref = top == -CUDART_INF_F ? 0.f : top;
+                    float z = 0.f;
+                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int c = 0; c < kMaxCluster; ++c) {
+                        const float w = ex2((part[c] - ref) * kLog2e);
+                        z += w;
+                        sum.x = fmaf(w, x[c].x, sum.x); sum.y = fmaf(w, x[c].y, sum.y);
+                        sum.z = fmaf(w, x[c].z, sum.z); sum.w = fmaf(w, x[c].w, sum.w);
+                    }
+                    if (out_row < p.W) {
+                        const float f = z > 0.f ? 1.f / z : 0.f;
+                        const long long at = (long long)s.bh * p.W + out_row;
+                        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + at * D + piece * 4) =
+                            make_uint2(pack_bf16x2(sum.x * f, sum.y * f), pack_bf16x2(sum.z * f, sum.w * f));
+                        if (piece == 0 && p.lse != nullptr) p.lse[at] = top + logf(z);
+                    }
+                }
+                __syncwarp();
+                cluster_sync();                    // nobody leaves while its rows are still being read
+                break;
+            }
             if (!ok) break;
             if (allowed_i == 0) continue;                  // this Q tile does not exist: nothing to write
             // ---------------------------------------------------------------- epilogue of the segment
@@ -759,7 +870,7 @@ fwd_merge_kernel(const __grid_constant__ Params p, const __grid_constant__ Group
 
 template <int D, int kForm>
 int launch_d(const void* q, const void* k, const void* v, void* out, float* lse, int B, int H, int N, int W,
-             int d, int causal, const tlin_fwd_plan& plan, float* ws, long long kv_rows_alloc, cudaStream_t st) {
+             int d, int causal, const tlin_fwd_plan& plan, float* ws, long long kv_rows_alloc, cudaStream_t st, int cluster = 1) {
     using C = Cfg<D>;
     const long long bh = (long long)B * H;
     KernelMaps<false> maps;
@@ -771,10 +882,16 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
     p.out = out; p.lse = lse; p.ws = ws; p.status = status_word();
     if (!p.status) return TLIN_ERR_CUDA;
     p.total_units = plan.total_units; p.n_groups = plan.n_groups; p.q_tiles = plan.q_tiles; p.key_tiles = plan.key_tiles;
-    p.N = N; p.W = W; p.causal = causal; p.d = d; p.schedule = plan.schedule;
+    p.N = N; p.W = W; p.causal = causal; p.d = d; p.schedule = plan.schedule; p.cluster = cluster;
     p.scale_log2e = kLog2e / sqrtf((float)d);
     static bool smem_allowed[64] = {};
     TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_tc_kernel<D, kForm>, C::kSmemBytes, smem_allowed));
+    if constexpr (kForm == kCluster) {
+        GroupStarts none = {};              // not read
+        TLIN_CUDA_CHECK(launch_overlapped_clusters(fwd_tc_kernel<D, kForm>, (unsigned)(bh * plan.q_tiles * cluster), cluster, kThreads, C::kSmemBytes, st, maps, p, none));
+        count_launch();
+        return TLIN_OK;
+    }
     if (plan.n_groups > kMaxGroups) return TLIN_ERR_UNSUPPORTED;
     GroupStarts starts;
     fwd_group_starts(plan, &starts);
@@ -790,6 +907,57 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
         count_launch();
     }
     return TLIN_OK;
+}
+
+// Clusters of `size` CTAs that the device holds at a time (asked once per device and size).
+template <int D>
+int clusters_at_a_time(int size) {
+    static std::atomic<int> known[64][kMaxCluster + 1];
+    static bool smem_allowed[64] = {};
+    const int dev = current_device_slot();
+    if (dev < 0) return 0;
+    int n = known[dev][size].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)size);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (allow_dynamic_smem(fwd_tc_kernel<D, kCluster>, Cfg<D>::kSmemBytes, smem_allowed) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, fwd_tc_kernel<D, kCluster>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        n += 1;                                              // 0: not asked yet
+        known[dev][size].store(n, std::memory_order_relaxed);
+    }
+    return n - 1;
+}
+// Into how many shares a cluster cuts the keys of a call whose plan splits them (1: the plan's own groups and the merge kernel).  In
+// key-tile times: a share, 2 to start and finish and 2 for the merge, against the groups' steps and segments and, for the merge kernel,
+// 4, more with the parts that it merges and with the row's length.  Fewer, longer shares lose what the merge saves: B4 H16 N8192 W256
+// d64 (2 shares of 32 against 148 groups of 28) 57.0 -> 59.8 us, B8 H8 N6000 W200 d64 46.7 -> 48.0; the rule leaves both.
+template <int D>
+int cluster_shares(const tlin_fwd_plan& plan, long long bh) {
+    if (plan.schedule != 0 || !plan.uses_workspace) return 1;
+    const long long problems = bh * plan.q_tiles, T = plan.key_tiles;
+    if (problems > kDefaultSMs / 2) return 1;
+    const long long steps = (plan.total_units + plan.n_groups - 1) / plan.n_groups;
+    long long best_cost = steps + 2 * (steps / T + 1) + 4 + (plan.n_groups / bh + 2) / 4 + (D == 128 ? 1 : 0);
+    int best = 1;
+    for (int shares = 2; shares <= kMaxCluster; ++shares) {
+        const long long cost = (T + shares - 1) / shares + 4;
+        if (cost < best_cost && problems <= clusters_at_a_time<D>(shares)) {
+            best_cost = cost;
+            best = shares;
+        }
+    }
+    return best;
 }
 
 // A table of problems as one launch: every CTA walks a contiguous run or a list of whole (problem, b*h, query tile pair) units.
@@ -855,6 +1023,11 @@ int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float*
         if (d < 64) return launch_d<64, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
         if (d < 128) return launch_d<128, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
         return launch_d<256, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
+    }
+    if (d == 64 || d == 128) {
+        const int shares = d == 128 ? cluster_shares<128>(plan, (long long)B * H) : cluster_shares<64>(plan, (long long)B * H);
+        if (shares > 1 && d == 128) return launch_d<128, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
+        if (shares > 1) return launch_d<64, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
     }
     if (d == 128) return launch_d<128, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
     if (d == 64) return launch_d<64, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);

@@ -634,3 +634,22 @@ def test_batched_forward_units_dealt_singly(d, specs):
         lg.check(f"problem {i} lse")
         ref, ref_lse = oracle.attn_forward(q.cpu(), k[:, :, :n_keys].contiguous().cpu(), v[:, :, :n_keys].contiguous().cpu(), causal)
         parity.check(out.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", f"problem {i} {specs[i]}")
+
+
+# few short problems whose keys the CTAs of a cluster share: 2 to 8 shares, shares without keys (window rule), pairs with one half
+CLUSTERS = [(1, 4, 1024, 128, 64, 1), (2, 4, 3000, 100, 64, 1), (1, 16, 2000, 200, 64, 0), (1, 32, 3000, 200, 64, 1), (2, 12, 2500, 250, 128, 0), (2, 16, 4000, 250, 128, 1),
+            (1, 20, 2000, 130, 128, 1), (1, 30, 1700, 1, 128, 0), (1, 2, 800, 800, 64, 1), (1, 3, 1500, 1100, 128, 1)]
+
+
+@pytest.mark.parametrize("B,H,N,W,d,causal", CLUSTERS)
+def test_forward_keys_shared_by_a_cluster(B, H, N, W, d, causal):
+    assert tl.tlin_plan_forward(B, H, N, W, d, causal).uses_workspace
+    wl = synth.Workload("cluster", B, H, d, N, W, seed=2100 + N + W, causal_window=causal)
+    q, k, v = synth.forward_inputs(wl, device=DEV)
+    out, lse = tl.tlin_attn_forward(q, k, v, causal_window=causal)
+    torch.cuda.synchronize()
+    assert tl.tlin_get_status() == 0 and tl.tlin_last_launch_count() <= 2       # 1, unless the device cannot hold the clusters at a time
+    again, lse_again = tl.tlin_attn_forward(q, k, v, causal_window=causal)
+    ref, ref_lse = oracle.attn_forward(q.cpu(), k.cpu(), v.cpu(), causal)
+    parity.check(out.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", f"{(B, H, N, W, d, causal)}")
+    assert torch.equal(out, again) and torch.equal(lse, lse_again)
