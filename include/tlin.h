@@ -299,8 +299,8 @@ typedef struct {
                               focused attention and the generation window);
                               1: every CTA works through whole (b,h,query tile) problems, keys never split
                               (many query rows, short context: the restoring cross-attention of Section 3).
-                              A call of few, short problems whose plan is schedule 0 with splits may let clusters of up to 8
-                              CTAs share each (b,h,query tile)'s keys instead of the groups (d = 64 and 128) */
+                              A call of few, short problems whose plan is schedule 0 with splits (at head sizes other than 64
+                              and 128: any plan) may let clusters of up to 8 CTAs share each (b,h,query tile)'s keys instead */
     int32_t causal_window; /* the call's mask, N and W: the group boundaries of schedule 1 depend on them              */
     int32_t n_keys;
     int32_t n_queries;

@@ -81,11 +81,13 @@ __device__ __forceinline__ void exp2_poly2(uint64_t x2, float& p0, float& p1) {
 // W1000 d256 3952 -> 56 us, B4 H12 N370 W96 d32 96 -> 12 us.
 // kDealt and kAnyDealt are the first and the last with problems dealt out by cost (DealtWalker; a form of their own because the
 // choice at run time costs the others 1 to 2 %).
-// kCluster is the first for few, short problems: the CTAs of a cluster share the keys of one (b,h,query tile pair), leave their rows in
+// kCluster and kAnyCluster are the first and the third for few, short problems: the CTAs of a cluster share the keys of one (b,h,query tile pair), leave their rows in
 // their shared memory, and each merges a share of the rows from all of them; no merge kernel, no partials in global memory.
-// Against split groups and the merge kernel: B2 H4 N3000 W100 d64 17.2 -> 11.9 us, B1 H16 N2000 W200 d64 17.9 -> 13.9, B4 H8 N1000 W64 d128
-// 18.1 -> 14.3, B2 H16 N4000 W250 d128 33.6 -> 29.4, B1 H4 N1024 W128 d64 8.5 -> 8.3.
-enum { kOneProblem = 0, kTable = 1, kAnyHead = 2, kDealt = 3, kAnyDealt = 4, kCluster = 5 };
+// Against split groups and the merge kernel: B2 H4 N3000 W100 d64 17.2 -> 11.6 us, B1 H16 N2000 W200 d64 17.9 -> 14.0, B4 H8 N1000 W64 d128
+// 17.9 -> 13.1, B2 H16 N4000 W250 d128 33.7 -> 28.8, B1 H4 N1024 W128 d64 8.5 -> 8.3; B1 H9 N4000 W100 d80 23.7 -> 16.8, B2 H4 N2000
+// W500 d160 26.6 -> 21.3; against whole problems B1 H3 N700 W500 d96 18.2 -> 12.0.  The merge has several rows and shares on their way
+// at a time: one row after the other, 128 rows of two shares took 8 us.
+enum { kOneProblem = 0, kTable = 1, kAnyHead = 2, kDealt = 3, kAnyDealt = 4, kCluster = 5, kAnyCluster = 6 };
 constexpr int kMaxCluster = 8;             // the portable size
 
 template <int D>
@@ -159,6 +161,7 @@ struct BatchWalker {
     }
 };
 // The one segment of a CTA of a cluster: its share of the key tiles that the pair may use.
+template <int D>
 struct ClusterWalker {
     Segment seg;
     bool more;
@@ -167,7 +170,8 @@ struct ClusterWalker {
         seg.prob = 0;
         seg.bh = problem / p.q_tiles;
         seg.qt = problem - seg.bh * p.q_tiles;
-        const int a0 = tiles_allowed(p, seg.qt * kTileM, 0), a1 = tiles_allowed(p, seg.qt * kTileM, 1), tiles = a0 > a1 ? a0 : a1;
+        const int row0 = seg.qt * Cfg<D>::kRows;
+        const int a0 = tiles_allowed(p, row0, 0), a1 = Cfg<D>::kTiles > 1 ? tiles_allowed(p, row0, 1) : 0, tiles = a0 > a1 ? a0 : a1;
         seg.t_begin = tiles * rank / p.cluster;
         seg.t_end = tiles * (rank + 1) / p.cluster;
     }
@@ -178,11 +182,11 @@ struct ClusterWalker {
         return had;
     }
 };
-template <int kForm>
+template <int D, int kForm>
 __device__ __forceinline__ auto make_walker(const KernelMaps<kForm == kTable>& m, const Params& p, const GroupStarts& starts) {
     if constexpr (kForm == kTable) return BatchWalker(m, starts);
     else if constexpr (kForm == kDealt || kForm == kAnyDealt) return DealtWalker(p, starts);
-    else if constexpr (kForm == kCluster) return ClusterWalker(p);
+    else if constexpr (kForm == kCluster || kForm == kAnyCluster) return ClusterWalker<D>(p);
     else return SegmentWalker(p, starts);
 }
 // shape (N, W, causal, key_tiles) and result pointers of the problem a segment belongs to
@@ -197,7 +201,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __grid_constant__ Params p,
               const __grid_constant__ GroupStarts starts) {
     using C = Cfg<D>;
-    constexpr bool kBatched = kForm == kTable, kAny = kForm == kAnyHead || kForm == kAnyDealt, kWhole = kForm == kTable || kForm >= kDealt;   // kWhole: no split keys
+    constexpr bool kBatched = kForm == kTable, kAny = kForm == kAnyHead || kForm == kAnyDealt || kForm == kAnyCluster, kShared = kForm == kCluster || kForm == kAnyCluster, kWhole = kForm == kTable || kForm >= kDealt;   // kWhole: no split keys
     constexpr int kTileM = C::kRows;
     const int d = kAny ? p.d : D;                              // row length; everything below folds where it is D
     const int boxes = kAny ? (d + 63) / 64 : C::kBoxes;
@@ -264,7 +268,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             uint32_t it = 0;           // ring counter
             uint32_t seg_idx = 0;
             bool ok = true;
-            auto walk = make_walker<kForm>(maps, p, starts);
+            auto walk = make_walker<D, kForm>(maps, p, starts);
             Segment s;
             while (ok && walk.next(s)) {
                 const auto& pr = problem_of<kBatched>(maps, p, s);
@@ -359,7 +363,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             constexpr std::integral_constant<int, 0> k_begin{};
             constexpr std::integral_constant<int, kFirstKeys / 16> k_first{};
             constexpr std::integral_constant<int, kTileN / 16> k_end{};
-            auto walk = make_walker<kForm>(maps, p, starts);
+            auto walk = make_walker<D, kForm>(maps, p, starts);
             Segment s;
             while (ok && walk.next(s)) {
                 const auto& pr = problem_of<kBatched>(maps, p, s);
@@ -433,7 +437,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             }
         }
     }
-    if constexpr (kForm == kCluster) {          // the two barriers of the merge below
+    if constexpr (kShared) {                    // the two barriers of the merge below
         __syncwarp();
         cluster_sync();
         cluster_sync();
@@ -449,7 +453,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
         const uint32_t tO = tmem_base + lane_addr + C::kColO + i * D;
         uint32_t n = 0;     // tiles processed by this warpgroup (phase counter of s_full/p_full/pv_done)
         bool ok = true;
-        auto walk = make_walker<kForm>(maps, p, starts);
+        auto walk = make_walker<D, kForm>(maps, p, starts);
         int bh_first = 0;                                  // (b,h) of this CTA's first unit (used under schedule 0 only)
         if constexpr (!kWhole) bh_first = (int)(walk.u / p.key_tiles);
         Segment s;
@@ -566,7 +570,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             int j = 0;
             for (; j < n_open && ok; ++j) step(j, std::false_type{});
             for (; j < cnt_i && ok; ++j) step(j, std::true_type{});
-            if constexpr (kForm == kCluster) {
+            if constexpr (kShared) {
                 // -------------------------------------------------------- merge inside the cluster
                 if (ok && cnt_i > 0) {
                     ok = mbar_wait(&pv_done[i], (n - 1) & 1, abort_p);
@@ -578,16 +582,17 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 f2_unpack(l2[1], x2, x3);
                 const float l = (x0 + x1) + (x2 + x3);
                 const bool have = ok && l > 0.f;
-                float* sO = reinterpret_cast<float*>(smem);       // 256 rows of D, 16-byte pieces at (piece xor row mod 8)
+                float* sO = reinterpret_cast<float*>(smem);       // rows of D, 16-byte pieces at (piece xor row mod 8)
                 float* sLse = sO + kTileM * D;
-                static_assert(kForm != kCluster || kTileM * (D + 1) * 4 <= C::kSmemTiles, "the rows lie over Q and the ring");
-                named_barrier(1, 256);             // both Q tiles' products are complete: Q and the ring are free
+                static_assert(kTileM * (D + 1 + kMaxCluster / 2) * 4 <= C::kSmemTiles, "the rows lie over Q and the ring");
+                named_barrier(1, kTileM);          // all Q tiles' products are complete: Q and the ring are free
                 const int rl = i * kQTile + r;
                 sLse[rl] = have ? (m_ref + log2f(l)) * kLn2 : -CUDART_INF_F;
                 const float inv_l = have ? 1.f / l : 0.f;
                 if (ok && cnt_i > 0) {
 #pragma unroll
                     for (int c = 0; c < D / 16; ++c) {
+                        if (kAny && c * 16 >= d) break;
                         uint32_t o[16];
                         tmem_ld16_async(tO + c * 16, o);
                         tmem_wait_ld16(o);
@@ -603,41 +608,69 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 namespace cg = cooperative_groups;
                 cg::cluster_group cl = cg::this_cluster();
                 constexpr int kLanes = D / 4 < 32 ? D / 4 : 32;     // lanes per row
-                const int rank = (int)cl.block_rank(), piece = lane % kLanes;
-                const int rr_end = kTileM * (rank + 1) / p.cluster;
-                for (int rr = kTileM * rank / p.cluster + warp * (32 / kLanes) + lane / kLanes; rr < rr_end; rr += 8 * (32 / kLanes)) {
-                    const int out_row = row0 + rr;
-                    float part[kMaxCluster];
-                    float4 x[kMaxCluster];
-                    float top = -CUDART_INF_F;
+                const int rank = (int)cl.block_rank(), rr_begin = kTileM * rank / p.cluster, rr_end = kTileM * (rank + 1) / p.cluster;
+                const long long at0 = (long long)s.bh * p.W + row0;
+                // the shares' weights, one row per thread; 0 where a share has no keys for the row and has left nothing
+                float* sW = sLse + kTileM;                          // [row - rr_begin][kMaxCluster]
+                if (rr_begin + (int)threadIdx.x < rr_end) {
+                    const int rr = rr_begin + threadIdx.x;
+                    float part[kMaxCluster], top = -CUDART_INF_F, z = 0.f;
 #pragma unroll
                     for (int c = 0; c < kMaxCluster; ++c) {
                         part[c] = c < p.cluster ? cl.map_shared_rank(sLse, c)[rr] : -CUDART_INF_F;
                         top = fmaxf(top, part[c]);
                     }
-#pragma unroll
-                    for (int c = 0; c < kMaxCluster; ++c) {         // a share without keys for the row has left nothing there
-                        x[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (part[c] != -CUDART_INF_F) x[c] = *reinterpret_cast<const float4*>(cl.map_shared_rank(sO, c) + rr * D + ((piece ^ (rr & 7)) << 2));
-                    }
                     const float ref = top == -CUDART_INF_F ? 0.f : top;
-                    float z = 0.f;
-                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int c = 0; c < kMaxCluster; ++c) {
-                        const float w = ex2((part[c] - ref) * kLog2e);
-                        z += w;
-                        sum.x = fmaf(w, x[c].x, sum.x); sum.y = fmaf(w, x[c].y, sum.y);
-                        sum.z = fmaf(w, x[c].z, sum.z); sum.w = fmaf(w, x[c].w, sum.w);
+                        part[c] = ex2((part[c] - ref) * kLog2e);
+                        z += part[c];
                     }
-                    if (out_row < p.W) {
-                        const float f = z > 0.f ? 1.f / z : 0.f;
-                        const long long at = (long long)s.bh * p.W + out_row;
-                        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + at * D + piece * 4) =
-                            make_uint2(pack_bf16x2(sum.x * f, sum.y * f), pack_bf16x2(sum.z * f, sum.w * f));
-                        if (piece == 0 && p.lse != nullptr) p.lse[at] = top + logf(z);
-                    }
+                    const float f = z > 0.f ? 1.f / z : 0.f;
+#pragma unroll
+                    for (int c = 0; c < kMaxCluster; ++c) sW[(rr - rr_begin) * kMaxCluster + c] = part[c] * f;
+                    if (row0 + rr < p.W && p.lse != nullptr) p.lse[at0 + rr] = top + logf(z);
                 }
+                named_barrier(1, kTileM);
+                // kU rows per lane and kE shares of each on their way at a time
+                constexpr int kRowStep = 4 * C::kTiles * (32 / kLanes);     // rows of all softmax warps
+                auto merge_rows = [&](auto rows_at_once, auto shares_at_once) {
+                    constexpr int kU = decltype(rows_at_once)::value, kE = decltype(shares_at_once)::value;
+                    for (int r0 = rr_begin + warp * (32 / kLanes) + lane / kLanes; r0 < rr_end; r0 += kU * kRowStep) {
+#pragma unroll
+                        for (int v = 0; v < D / 4 / kLanes; ++v) {
+                            const int piece = lane % kLanes + v * kLanes;
+                            if (kAny && piece * 4 >= d) break;
+                            float w[kU][kE];
+                            float4 x[kU][kE];
+#pragma unroll
+                            for (int u = 0; u < kU; ++u) {
+                                const int rr = r0 + u * kRowStep;
+#pragma unroll
+                                for (int e = 0; e < kE; ++e) {
+                                    w[u][e] = rr < rr_end ? sW[(rr - rr_begin) * kMaxCluster + e] : 0.f;
+                                    x[u][e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                    if (w[u][e] > 0.f) x[u][e] = *reinterpret_cast<const float4*>(cl.map_shared_rank(sO, e) + rr * D + ((piece ^ (rr & 7)) << 2));
+                                }
+                            }
+#pragma unroll
+                            for (int u = 0; u < kU; ++u) {
+                                const int rr = r0 + u * kRowStep;
+                                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                                for (int e = 0; e < kE; ++e) {
+                                    sum.x = fmaf(w[u][e], x[u][e].x, sum.x); sum.y = fmaf(w[u][e], x[u][e].y, sum.y);
+                                    sum.z = fmaf(w[u][e], x[u][e].z, sum.z); sum.w = fmaf(w[u][e], x[u][e].w, sum.w);
+                                }
+                                if (rr < rr_end && row0 + rr < p.W)
+                                    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (at0 + rr) * d + piece * 4) =
+                                        make_uint2(pack_bf16x2(sum.x, sum.y), pack_bf16x2(sum.z, sum.w));
+                            }
+                        }
+                    }
+                };
+                if (p.cluster > 4) merge_rows(std::integral_constant<int, 2>{}, std::integral_constant<int, 8>{});
+                else merge_rows(std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{});
                 __syncwarp();
                 cluster_sync();                    // nobody leaves while its rows are still being read
                 break;
@@ -745,6 +778,9 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             }
             tc_fence_before();      // TMEM reads of O are complete before the next segment's arrive lets PV overwrite it
         }
+        } else if constexpr (kShared) {                    // one Q tile: these warps only take part in the merge's barriers
+            cluster_sync();
+            cluster_sync();
         }
     }
 
@@ -886,7 +922,7 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
     p.scale_log2e = kLog2e / sqrtf((float)d);
     static bool smem_allowed[64] = {};
     TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_tc_kernel<D, kForm>, C::kSmemBytes, smem_allowed));
-    if constexpr (kForm == kCluster) {
+    if constexpr (kForm == kCluster || kForm == kAnyCluster) {
         GroupStarts none = {};              // not read
         TLIN_CUDA_CHECK(launch_overlapped_clusters(fwd_tc_kernel<D, kForm>, (unsigned)(bh * plan.q_tiles * cluster), cluster, kThreads, C::kSmemBytes, st, maps, p, none));
         count_launch();
@@ -910,7 +946,7 @@ int launch_d(const void* q, const void* k, const void* v, void* out, float* lse,
 }
 
 // Clusters of `size` CTAs that the device holds at a time (asked once per device and size).
-template <int D>
+template <int D, int kForm>
 int clusters_at_a_time(int size) {
     static std::atomic<int> known[64][kMaxCluster + 1];
     static bool smem_allowed[64] = {};
@@ -928,8 +964,8 @@ int clusters_at_a_time(int size) {
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (allow_dynamic_smem(fwd_tc_kernel<D, kCluster>, Cfg<D>::kSmemBytes, smem_allowed) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, fwd_tc_kernel<D, kCluster>, &cfg) != cudaSuccess) {
+        if (allow_dynamic_smem(fwd_tc_kernel<D, kForm>, Cfg<D>::kSmemBytes, smem_allowed) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, fwd_tc_kernel<D, kForm>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
             n = 0;
         }
@@ -940,19 +976,27 @@ int clusters_at_a_time(int size) {
 }
 // Into how many shares a cluster cuts the keys of a call whose plan splits them (1: the plan's own groups and the merge kernel).  In
 // key-tile times: a share, 2 to start and finish and 2 for the merge, against the groups' steps and segments and, for the merge kernel,
-// 4, more with the parts that it merges and with the row's length.  Fewer, longer shares lose what the merge saves: B4 H16 N8192 W256
+// 4, more with the parts that it merges and with the row's length, less where a step is longer (two PV products).  Fewer, longer shares lose what the merge saves: B4 H16 N8192 W256
 // d64 (2 shares of 32 against 148 groups of 28) 57.0 -> 59.8 us, B8 H8 N6000 W200 d64 46.7 -> 48.0; the rule leaves both.
-template <int D>
+// At other head sizes also instead of whole problems, of which there are few enough here for one per CTA (at 64 and 128 a call that is
+// planned whole stays whole: its result is that of the same problem in a table).
+template <int D, int kForm>
 int cluster_shares(const tlin_fwd_plan& plan, long long bh) {
-    if (plan.schedule != 0 || !plan.uses_workspace) return 1;
     const long long problems = bh * plan.q_tiles, T = plan.key_tiles;
     if (problems > kDefaultSMs / 2) return 1;
-    const long long steps = (plan.total_units + plan.n_groups - 1) / plan.n_groups;
-    long long best_cost = steps + 2 * (steps / T + 1) + 4 + (plan.n_groups / bh + 2) / 4 + (D == 128 ? 1 : 0);
+    constexpr bool kAny = kForm == kAnyCluster;
+    long long best_cost = T;
+    if (plan.schedule == 0) {
+        if (!plan.uses_workspace) return 1;
+        const long long steps = (plan.total_units + plan.n_groups - 1) / plan.n_groups, parts = plan.n_groups / bh;
+        best_cost = steps + 2 * (steps / T + 1) + (parts + 2) / (D == 256 ? 8 : 4) + (kAny ? 3 : D == 128 ? 5 : 4);
+    } else if (!kAny) {
+        return 1;
+    }
     int best = 1;
     for (int shares = 2; shares <= kMaxCluster; ++shares) {
         const long long cost = (T + shares - 1) / shares + 4;
-        if (cost < best_cost && problems <= clusters_at_a_time<D>(shares)) {
+        if (cost < best_cost && problems <= clusters_at_a_time<D, kForm>(shares)) {
             best_cost = cost;
             best = shares;
         }
@@ -1017,17 +1061,22 @@ int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float*
                   float* ws, long long kv_rows_alloc, cudaStream_t st) {
     if (plan.tile_m != (d > 128 ? kQTile : kTileM) || plan.tile_n != kTileN) return TLIN_ERR_UNSUPPORTED;
     if ((long long)B * H * W > 0x7fffffffLL || d % 8 != 0 || d > 256) return TLIN_ERR_UNSUPPORTED;
+    const long long bh = (long long)B * H;
+    const int shares = d == 128 ? cluster_shares<128, kCluster>(plan, bh) : d == 64 ? cluster_shares<64, kCluster>(plan, bh)
+                     : d < 64 ? cluster_shares<64, kAnyCluster>(plan, bh) : d < 128 ? cluster_shares<128, kAnyCluster>(plan, bh) : cluster_shares<256, kAnyCluster>(plan, bh);
+    if (shares > 1) {
+        if (d == 128) return launch_d<128, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
+        if (d == 64) return launch_d<64, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
+        if (d < 64) return launch_d<64, kAnyCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
+        if (d < 128) return launch_d<128, kAnyCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
+        return launch_d<256, kAnyCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
+    }
     if (dealt(plan, (long long)B * H, d)) {
         if (d == 128) return launch_d<128, kDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
         if (d == 64) return launch_d<64, kDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
         if (d < 64) return launch_d<64, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
         if (d < 128) return launch_d<128, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
         return launch_d<256, kAnyDealt>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
-    }
-    if (d == 64 || d == 128) {
-        const int shares = d == 128 ? cluster_shares<128>(plan, (long long)B * H) : cluster_shares<64>(plan, (long long)B * H);
-        if (shares > 1 && d == 128) return launch_d<128, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
-        if (shares > 1) return launch_d<64, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
     }
     if (d == 128) return launch_d<128, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
     if (d == 64) return launch_d<64, kOneProblem>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st);
