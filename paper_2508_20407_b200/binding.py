@@ -98,7 +98,8 @@ SIGNATURES = {
 }
 
 _lib = None
-_workspace_tensor = None  # keeps the registered workspace alive
+_workspaces = {}          # device index -> the buffer that the library holds the address of: alive as long as it is registered
+_workspace_tensor = None  # the one registered last
 
 
 def lib():
@@ -193,27 +194,44 @@ def workspace_bytes_backward(B, H, N, W, d) -> int:
     return int(lib().tlin_workspace_bytes_backward(B, H, N, W, d))
 
 
+def _device_slot() -> int:
+    """The entry of the current device, under which the library files a workspace (0 where no device can be asked)."""
+    try:
+        return _current_device()
+    except RuntimeError:
+        return 0
+
+
 def set_workspace(t: torch.Tensor | None):
-    """Registers a device buffer (any dtype) as split-K scratch; the tensor is kept alive here."""
+    """Registers a device buffer (any dtype) as split-K scratch of the current device; the tensor is kept alive here until
+    another one takes its place there.  The other devices keep theirs: the library goes on using them."""
     global _workspace_tensor
+    slot = _device_slot()
     if t is None:
         _check(lib().tlin_set_workspace(None, 0), "tlin_set_workspace")
+        _workspaces.pop(slot, None)
     else:
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("workspace must be a contiguous CUDA tensor")
         _check(lib().tlin_set_workspace(_ptr(t), t.numel() * t.element_size()), "tlin_set_workspace")
+        _workspaces[slot] = t
     _workspace_tensor = t
 
 
 def ensure_workspace(nbytes: int, device="cuda"):
-    """Grows the registered workspace to at least ``nbytes`` (allocation happens here, in torch)."""
-    global _workspace_tensor
-    cur = 0 if _workspace_tensor is None else _workspace_tensor.numel()
-    if cur > 0 and nbytes <= cur and _workspace_tensor.device == device:
-        return _workspace_tensor
-    if nbytes > cur or (_workspace_tensor is not None and str(_workspace_tensor.device) != str(torch.device(device)) and torch.device(device).index is not None):
+    """Grows the current device's workspace to at least ``nbytes`` (allocation happens here, in torch)."""
+    t = _workspaces.get(_device_slot())
+    if t is not None and nbytes <= t.numel() and t.device == device:
+        return t
+    if t is None:
+        grow = nbytes > 0
+    else:
+        wanted = torch.device(device)
+        grow = nbytes > t.numel() or (wanted.index is not None and wanted != t.device)
+    if grow:
         set_workspace(torch.empty(max(nbytes, 1 << 20), dtype=torch.uint8, device=device))
-    return _workspace_tensor
+        t = _workspace_tensor
+    return t
 
 
 # ------------------------------------------------------------------ compute
