@@ -32,9 +32,10 @@ int as_int(int64_t x) {
     if (x > INT32_MAX) bad("a dimension exceeds 2^31 - 1");
     return (int)x;
 }
+// Asked for once the tensors have been checked: without a device there is no current stream, and a CPU tensor is the caller's error.
+tlin_stream_t current_stream() { return (tlin_stream_t)c10::cuda::getCurrentCUDAStream().stream(); }
 tlin_stream_t stream_of(const py::object& stream) {
-    if (stream.is_none()) return (tlin_stream_t)c10::cuda::getCurrentCUDAStream().stream();
-    return reinterpret_cast<tlin_stream_t>(stream.attr("cuda_stream").cast<uintptr_t>());
+    return stream.is_none() ? current_stream() : reinterpret_cast<tlin_stream_t>(stream.attr("cuda_stream").cast<uintptr_t>());
 }
 Tensor fresh(at::IntArrayRef shape, at::ScalarType dtype, const Tensor& like) {
     return at::detail::empty_cuda(shape, dtype, like.device(), std::nullopt);
@@ -60,8 +61,9 @@ size_t workspace_forward(const Tensor& q, const Tensor& k, int64_t n_keys, int c
                                         as_int(q.size(3)), causal);
 }
 // kind: 0 bf16, 1 fp32, 2 bf16 over the first n_keys rows of a cache
+template <class StreamFn>
 Result run_forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, int64_t n_keys, const Opt& out_, const Opt& lse_, int causal,
-                   tlin_stream_t st) {
+                   StreamFn&& stream) {
     const int64_t B = four_dims(q, "q").size(0), H = q.size(1), W = q.size(2), d = q.size(3), N = four_dims(k, "k").size(2);
     const at::ScalarType dt = kind == 1 ? at::kFloat : at::kBFloat16;
     check(q, dt, {B, H, W, d}, "q");
@@ -69,6 +71,7 @@ Result run_forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, 
     check(v, dt, {B, H, N, d}, kind == 2 ? "v_cache" : "v");
     const Tensor out = given_or_fresh(out_, {B, H, W, d}, dt, q, "out"), lse = given_or_fresh(lse_, {B, H, W}, at::kFloat, q, "lse");
     const int b = as_int(B), h = as_int(H), n = as_int(N), w = as_int(W), dd = as_int(d), nk = as_int(n_keys);
+    const tlin_stream_t st = stream();
     const int rc = without_gil([&] {
         const void *qp = q.data_ptr(), *kp = k.data_ptr(), *vp = v.data_ptr();
         float* lp = (float*)lse.data_ptr();
@@ -81,12 +84,13 @@ Result run_forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, 
 
 Result forward(int kind, const Tensor& q, const Tensor& k, const Tensor& v, int64_t n_keys, const Opt& out, const Opt& lse, int causal,
                const py::object& stream) {
-    return run_forward(kind, q, k, v, n_keys, out, lse, causal, stream_of(stream));
+    return run_forward(kind, q, k, v, n_keys, out, lse, causal, [&] { return stream_of(stream); });
 }
 
 using Gradients = std::tuple<int, Tensor, Tensor, Tensor>;
-Gradients run_backward(bool f32, const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out, const Tensor& lse,
-                                                 const Tensor& dout, const Opt& dq_, const Opt& dk_, const Opt& dv_, int causal, tlin_stream_t st) {
+template <class StreamFn>
+Gradients run_backward(bool f32, const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out, const Tensor& lse, const Tensor& dout,
+                       const Opt& dq_, const Opt& dk_, const Opt& dv_, int causal, StreamFn&& stream) {
     const int64_t B = four_dims(q, "q").size(0), H = q.size(1), W = q.size(2), d = q.size(3), N = four_dims(k, "k").size(2);
     const at::ScalarType dt = f32 ? at::kFloat : at::kBFloat16;
     check(q, dt, {B, H, W, d}, "q");
@@ -98,6 +102,7 @@ Gradients run_backward(bool f32, const Tensor& q, const Tensor& k, const Tensor&
     const Tensor dq = given_or_fresh(dq_, {B, H, W, d}, dt, q, "dq"), dk = given_or_fresh(dk_, {B, H, N, d}, dt, q, "dk"),
                  dv = given_or_fresh(dv_, {B, H, N, d}, dt, q, "dv");
     const int b = as_int(B), h = as_int(H), n = as_int(N), w = as_int(W), dd = as_int(d);
+    const tlin_stream_t st = stream();
     const int rc = without_gil([&] {
         if (f32)
             return tlin_attn_backward_f32((const float*)q.data_ptr(), (const float*)k.data_ptr(), (const float*)v.data_ptr(), (const float*)out.data_ptr(),
@@ -111,7 +116,7 @@ Gradients run_backward(bool f32, const Tensor& q, const Tensor& k, const Tensor&
 
 Gradients backward(bool f32, const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out, const Tensor& lse, const Tensor& dout, const Opt& dq,
                    const Opt& dk, const Opt& dv, int causal, const py::object& stream) {
-    return run_backward(f32, q, k, v, out, lse, dout, dq, dk, dv, causal, stream_of(stream));
+    return run_backward(f32, q, k, v, out, lse, dout, dq, dk, dv, causal, [&] { return stream_of(stream); });
 }
 size_t workspace_backward(const Tensor& q, const Tensor& k) {
     four_dims(q, "q");
@@ -139,7 +144,7 @@ struct Attention : public torch::autograd::Function<Attention> {
         const Tensor q = q_in.contiguous(), k = k_in.contiguous(), v = v_in.contiguous();
         const bool f32 = q.scalar_type() == at::kFloat;
         if (!f32 && q.is_cuda()) ensure_workspace(workspace_forward(q, k, -1, (int)causal), q);
-        const auto [rc, out, lse] = run_forward(f32 ? 1 : 0, q, k, v, 0, std::nullopt, std::nullopt, (int)causal, (tlin_stream_t)c10::cuda::getCurrentCUDAStream().stream());
+        const auto [rc, out, lse] = run_forward(f32 ? 1 : 0, q, k, v, 0, std::nullopt, std::nullopt, (int)causal, current_stream);
         raise(rc, f32 ? "tlin_attn_forward_f32" : "tlin_attn_forward");
         ctx->save_for_backward({q, k, v, out, lse});
         ctx->saved_data["causal"] = causal;
@@ -152,11 +157,10 @@ struct Attention : public torch::autograd::Function<Attention> {
         const bool f32 = q.scalar_type() == at::kFloat;
         const Tensor dout = grads[0].defined() ? grads[0].contiguous() : at::zeros_like(saved[3]);
         const int causal = (int)ctx->saved_data["causal"].toInt();
-        const auto st = (tlin_stream_t)c10::cuda::getCurrentCUDAStream().stream();
-        auto [rc, dq, dk, dv] = run_backward(f32, q, k, saved[2], saved[3], saved[4], dout, std::nullopt, std::nullopt, std::nullopt, causal, st);
+        auto [rc, dq, dk, dv] = run_backward(f32, q, k, saved[2], saved[3], saved[4], dout, std::nullopt, std::nullopt, std::nullopt, causal, current_stream);
         if (rc == TLIN_ERR_WORKSPACE) {      // too small so far: asking first would cost this thread a turn of the interpreter (20 us)
             ensure_workspace(workspace_backward(q, k), q);
-            std::tie(rc, dq, dk, dv) = run_backward(f32, q, k, saved[2], saved[3], saved[4], dout, dq, dk, dv, causal, st);
+            std::tie(rc, dq, dk, dv) = run_backward(f32, q, k, saved[2], saved[3], saved[4], dout, dq, dk, dv, causal, current_stream);
         }
         raise(rc, f32 ? "tlin_attn_backward_f32" : "tlin_attn_backward");
         return {dq, dk, dv, Tensor()};
@@ -202,13 +206,15 @@ Result decode(int kind, const Tensor& q, const Tensor& kn, const Tensor& vn, con
     return {rc, out, lse};
 }
 
-// problems: a sequence of (q, k, v, out, lse, n_keys, causal_window)
+// problems: a sequence of (q, k, v, out, lse, n_keys, causal_window), each any iterable; the numbers whatever int() takes
+int64_t number(const py::handle& x) { return py::int_(py::reinterpret_borrow<py::object>(x)).cast<int64_t>(); }
 int forward_batched(const py::sequence& problems, const py::object& stream) {
+    if (problems.size() == 0) throw py::index_error("a table needs at least one problem");
     std::vector<tlin_problem> table;
     table.reserve(problems.size());
     int d_first = 0, i = 0;
     for (const py::handle item : problems) {
-        const py::sequence pr = py::reinterpret_borrow<py::sequence>(item);
+        const py::tuple pr(py::reinterpret_borrow<py::object>(item));
         if (pr.size() != 7) bad("problem " + std::to_string(i) + ": expected (q, k, v, out, lse, n_keys, causal_window)");
         const Tensor q = pr[0].cast<Tensor>(), k = pr[1].cast<Tensor>(), v = pr[2].cast<Tensor>(), out = pr[3].cast<Tensor>();
         const Tensor* all[4] = {&q, &k, &v, &out};
@@ -218,7 +224,7 @@ int forward_batched(const py::sequence& problems, const py::object& stream) {
             if (!all[x]->is_cuda() || all[x]->scalar_type() != at::kBFloat16 || !all[x]->is_contiguous()) bad(here + ": " + names[x] + " must be a contiguous bf16 CUDA tensor");
         if (q.dim() < 2 || k.dim() < 2) bad(here + ": shape mismatch");
         const int64_t d = q.size(-1), W = q.size(-2), rows = k.size(-2), bh = W * d > 0 ? q.numel() / (W * d) : 0;
-        const int64_t n_keys = pr[5].is_none() ? rows : pr[5].cast<int64_t>();
+        const int64_t n_keys = pr[5].is_none() ? rows : number(pr[5]);
         if (k.numel() != bh * rows * d || !v.sizes().equals(k.sizes()) || !out.sizes().equals(q.sizes())) bad(here + ": shape mismatch");
         tlin_problem t = {};
         t.q = q.data_ptr(); t.k = k.data_ptr(); t.v = v.data_ptr(); t.out = out.data_ptr();
@@ -228,7 +234,7 @@ int forward_batched(const py::sequence& problems, const py::object& stream) {
             t.lse = (float*)lse.data_ptr();
         }
         t.BH = as_int(bh); t.n_keys = as_int(n_keys); t.kv_rows = rows != n_keys ? as_int(rows) : 0; t.n_queries = as_int(W);
-        t.causal_window = (int)pr[6].cast<int64_t>();
+        t.causal_window = (int)number(pr[6]);
         table.push_back(t);
         if (i++ == 0) d_first = as_int(d);
     }
