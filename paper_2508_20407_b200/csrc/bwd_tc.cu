@@ -793,9 +793,8 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             order.unit(p, u, bh, t);
             for (int i = first_q_tile(p, t); i < p.q_tiles128; ++i, ++g) {
                 ok = __all_sync(0xffffffffu, mbar_wait(dq_full, g & 1, abort_p));
-                if (!ok) break;
                 tc_fence_after();
-                uint32_t o[4][32];
+                uint32_t o[4][32];                                // of no use, and not stored, when the wait has run out
 #pragma unroll
                 for (int c = 0; c < 4; ++c) tmem_ld32_async(tDQ + c * 32, o[c]);
 #pragma unroll
@@ -804,11 +803,18 @@ bwd_fused_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 mbar_arrive(dq_drained);
                 // rows of dQ (consecutive in the workspace) through shared memory, 16 at a time, added by the copy engine
                 float* drow = p.ws + ((long long)bh * p.Wpad + i * kQTile) * D;
+                if (issuer) bulk_wait_read<3>();                  // the first buffer's previous rows have been read
+                // a wait that ran out is each warp's own finding (the phase may complete between two of them): the four warps go on,
+                // or leave, together
+                ok = named_barrier_all(1, 128, ok);
+                if (!ok) break;
 #pragma unroll
                 for (int c = 0; c < kQTile / C::kDqRows; ++c) {
                     float* buf = reinterpret_cast<float*>(smem + C::kOffDQ + (c & 3) * (C::kDqRows * D * 4));
-                    if (issuer) bulk_wait_read<3>();              // the buffer's previous rows have been read
-                    named_barrier(1, 128);
+                    if (c > 0) {
+                        if (issuer) bulk_wait_read<3>();          // the buffer's previous rows have been read
+                        named_barrier(1, 128);
+                    }
 #pragma unroll
                     for (int e = 0; e < C::kDqRows; ++e) buf[e * D + r] = __uint_as_float(o[c >> 1][(c & 1) * 16 + e]);
                     fence_proxy_async_smem();

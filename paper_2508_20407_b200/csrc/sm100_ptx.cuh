@@ -99,12 +99,19 @@ __device__ __forceinline__ void bulk_add_f32(float* gdst, const void* smem_src, 
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// barrier of `threads` threads of the CTA (id 1 .. 15)
 // every thread of every CTA of the cluster; what they wrote to shared memory before is visible after
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// barrier of `threads` threads of the CTA (id 1 .. 15)
 __device__ __forceinline__ void named_barrier(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+// the same, and whether `mine` holds in all of them: warps that stop together ask this, since one that leaves alone keeps the others waiting
+__device__ __forceinline__ bool named_barrier_all(int id, int threads, bool mine) {
+    uint32_t all;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbar.red.and.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(all) : "r"(id), "r"(threads), "r"(mine ? 1u : 0u) : "memory");
+    return all != 0;
+}
 
 // ---------------------------------------------------------------- tcgen05: TMEM allocation
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_result, uint32_t ncols) {   // whole warp
