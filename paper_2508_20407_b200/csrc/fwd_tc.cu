@@ -23,6 +23,7 @@
 #include "tc_common.cuh"
 #include <atomic>
 #include <cooperative_groups.h>
+#include <float.h>
 #include <math_constants.h>
 #include <mutex>
 #include <string.h>
@@ -581,14 +582,14 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 f2_unpack(l2[0], x0, x1);
                 f2_unpack(l2[1], x2, x3);
                 const float l = (x0 + x1) + (x2 + x3);
-                const bool have = ok && l > 0.f;
+                const bool none = !ok || l == 0.f;                // no keys here, or none that counts; a NaN is passed on
                 float* sO = reinterpret_cast<float*>(smem);       // rows of D, 16-byte pieces at (piece xor row mod 8)
                 float* sLse = sO + kTileM * D;
                 static_assert(kTileM * (D + 1 + kMaxCluster / 2) * 4 <= C::kSmemTiles, "the rows lie over Q and the ring");
                 named_barrier(1, kTileM);          // all Q tiles' products are complete: Q and the ring are free
                 const int rl = i * kQTile + r;
-                sLse[rl] = have ? (m_ref + log2f(l)) * kLn2 : -CUDART_INF_F;
-                const float inv_l = have ? 1.f / l : 0.f;
+                sLse[rl] = none ? -CUDART_INF_F : (m_ref + log2f(l)) * kLn2;
+                const float inv_l = none ? 0.f : 1.f / l;
                 if (ok && cnt_i > 0) {
 #pragma unroll
                     for (int c = 0; c < D / 16; ++c) {
@@ -610,7 +611,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 constexpr int kLanes = D / 4 < 32 ? D / 4 : 32;     // lanes per row
                 const int rank = (int)cl.block_rank(), rr_begin = kTileM * rank / p.cluster, rr_end = kTileM * (rank + 1) / p.cluster;
                 const long long at0 = (long long)s.bh * p.W + row0;
-                // the shares' weights, one row per thread; 0 where a share has no keys for the row and has left nothing
+                // the shares' weights, one row per thread; negative where a share has no keys for the row and has left nothing
                 float* sW = sLse + kTileM;                          // [row - rr_begin][kMaxCluster]
                 if (rr_begin + (int)threadIdx.x < rr_end) {
                     const int rr = rr_begin + threadIdx.x;
@@ -620,15 +621,16 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                         part[c] = c < p.cluster ? cl.map_shared_rank(sLse, c)[rr] : -CUDART_INF_F;
                         top = fmaxf(top, part[c]);
                     }
-                    const float ref = top == -CUDART_INF_F ? 0.f : top;
+                    const float ref = fmaxf(top, -FLT_MAX);
+                    float weight[kMaxCluster];
 #pragma unroll
                     for (int c = 0; c < kMaxCluster; ++c) {
-                        part[c] = ex2((part[c] - ref) * kLog2e);
-                        z += part[c];
+                        weight[c] = ex2((part[c] - ref) * kLog2e);
+                        z += weight[c];
                     }
-                    const float f = z > 0.f ? 1.f / z : 0.f;
+                    const float f = 1.f / z;                    // not used where no share has anything
 #pragma unroll
-                    for (int c = 0; c < kMaxCluster; ++c) sW[(rr - rr_begin) * kMaxCluster + c] = part[c] * f;
+                    for (int c = 0; c < kMaxCluster; ++c) sW[(rr - rr_begin) * kMaxCluster + c] = part[c] == -CUDART_INF_F ? -1.f : weight[c] * f;
                     if (row0 + rr < p.W && p.lse != nullptr) p.lse[at0 + rr] = top + logf(z);
                 }
                 named_barrier(1, kTileM);
@@ -648,9 +650,9 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                                 const int rr = r0 + u * kRowStep;
 #pragma unroll
                                 for (int e = 0; e < kE; ++e) {
-                                    w[u][e] = rr < rr_end ? sW[(rr - rr_begin) * kMaxCluster + e] : 0.f;
+                                    w[u][e] = rr < rr_end ? sW[(rr - rr_begin) * kMaxCluster + e] : -1.f;
                                     x[u][e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                    if (w[u][e] > 0.f) x[u][e] = *reinterpret_cast<const float4*>(cl.map_shared_rank(sO, e) + rr * D + ((piece ^ (rr & 7)) << 2));
+                                    if (!(w[u][e] < 0.f)) x[u][e] = *reinterpret_cast<const float4*>(cl.map_shared_rank(sO, e) + rr * D + ((piece ^ (rr & 7)) << 2));
                                 }
                             }
 #pragma unroll
@@ -692,8 +694,8 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 f2_unpack(l2[1], c, d2);
                 l = (a + b) + (c + d2);
             }
-            const float inv_l = l > 0.f ? 1.f / l : 0.f;
-            const float lse_val = l > 0.f ? (m_ref + log2f(l)) * kLn2 : -CUDART_INF_F;
+            const float inv_l = l == 0.f ? 0.f : 1.f / l;      // a NaN is passed on, in the row and in its lse
+            const float lse_val = l == 0.f ? -CUDART_INF_F : (m_ref + log2f(l)) * kLn2;
             const bool store = row < pr.W;
             // partial result -> workspace slot (0: first segment of this CTA's range, 1: a later one)
             float* pbase = p.ws + ((long long)blockIdx.x * 2 + (s.bh == bh_first ? 0 : 1)) * (long long)kTileM * (d + 1);
@@ -866,9 +868,13 @@ fwd_merge_kernel(const __grid_constant__ Params p, const __grid_constant__ Group
                 }
             }
             float mn = m[ps];
+            bool empty = mn == -CUDART_INF_F;             // every part so far: the maximum alone would not see a NaN
 #pragma unroll
-            for (int i = 0; i < kMergeParts; ++i) mn = fmaxf(mn, ls[i]);
-            if (mn == -CUDART_INF_F) continue;            // every part so far is empty
+            for (int i = 0; i < kMergeParts; ++i) {
+                mn = fmaxf(mn, ls[i]);
+                empty = empty && ls[i] == -CUDART_INF_F;
+            }
+            if (empty) continue;
             const float old = expf(m[ps] - mn);
             m[ps] = mn;
             z[ps] *= old;

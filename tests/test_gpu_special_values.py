@@ -1,0 +1,56 @@
+"""Values at the ends of the formats through every form of the kernels: a NaN reaches what depends on it and nothing else."""
+import pytest
+import torch
+
+from paper_2508_20407_b200 import binding as tl
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+NAN, INF = float("nan"), float("inf")
+
+
+def normal(seed, *shape, dtype=torch.bfloat16):
+    g = torch.Generator(device="cpu").manual_seed(seed)
+    return torch.randn(*shape, generator=g).to(dtype).to(DEV)
+
+
+def forward(q, k, v, causal):
+    fn = tl.tlin_attn_forward_f32 if q.dtype == torch.float32 else tl.tlin_attn_forward
+    out, lse = fn(q, k, v, causal_window=causal)
+    assert tl.tlin_get_status() == 0
+    return out, lse
+
+
+# keys shared in a cluster, split and merged by a second kernel (few and many parts), whole problems, one key tile
+FORMS = [(1, 4, 1024, 128), (5, 16, 2048, 256), (1, 2, 60000, 64), (8, 16, 512, 300), (2, 3, 100, 60)]
+
+
+@pytest.mark.parametrize("d,dtype", [(64, torch.bfloat16), (128, torch.bfloat16), (96, torch.bfloat16), (160, torch.bfloat16), (36, torch.float32)])
+@pytest.mark.parametrize("B,H,N,W", FORMS)
+def test_forward_passes_a_nan_on(B, H, N, W, d, dtype):
+    q, k, v = normal(1, B, H, W, d, dtype=dtype), normal(2, B, H, N, d, dtype=dtype), normal(3, B, H, N, d, dtype=dtype)
+    clean = forward(q, k, v, 0)
+    assert all(bool(torch.isfinite(t).all()) for t in clean)
+    hit = (B - 1, H - 1)
+
+    def check(got, rows, with_lse):
+        for t, ref, depends in zip(got, clean, (True, with_lse)):
+            t, ref = t.clone(), ref.clone()
+            if depends:
+                assert bool(t[hit][rows].isnan().all())
+                t[hit][rows] = ref[hit][rows] = 0
+            assert torch.equal(t, ref)
+
+    # single keys in columns that every form gives to the special-function unit: the cubic that d = 64 and 128 use for some of the
+    # others takes a NaN for the lower end of its range, and that key then counts for nothing
+    everywhere = slice(None)
+    for keys in (slice(3, 4), slice(N // 10, N * 9 // 10), slice((N - 1) // 32 * 32, (N - 1) // 32 * 32 + 1)):
+        bad = k.clone()
+        bad[hit][keys] = NAN                        # every row's sum
+        check(forward(q, bad, v, 0), everywhere, True)
+        bad = v.clone()
+        bad[hit][keys] = NAN                        # every row's result, not its sum
+        check(forward(q, k, bad, 0), everywhere, False)
+    bad = q.clone()
+    bad[hit][W // 2] = NAN
+    check(forward(bad, k, v, 0), slice(W // 2, W // 2 + 1), True)
