@@ -54,3 +54,23 @@ def test_forward_passes_a_nan_on(B, H, N, W, d, dtype):
     bad = q.clone()
     bad[hit][W // 2] = NAN
     check(forward(bad, k, v, 0), slice(W // 2, W // 2 + 1), True)
+
+
+# a score of -inf masks a key (an extra column of q at 1, of k at -inf); with every key masked there is nothing to attend to
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,pos", [(2, 4, 600), (2, 16, 1401), (1, 1, 30), (64, 32, 300), (4, 32, 8000)])
+def test_decode_step_with_masked_scores(B, H, pos, d):
+    q, kn, vn = normal(1, B, H, 1, d), normal(2, B, H, 1, d), normal(3, B, H, 1, d)
+    kc, vc = normal(4, B, H, pos + 3, d), normal(5, B, H, pos + 3, d)
+    q[..., 0] = 1
+    kc[..., 0] = -INF
+    kn[..., 0] = -INF
+    at = torch.full((B,), pos, dtype=torch.int32, device=DEV)
+    for out, lse in (tl.tlin_decode_step(q, kn, vn, kc, vc, pos), tl.tlin_decode_step_ragged(q, kn, vn, kc, vc, at, pos)):
+        assert float(out.float().abs().max()) == 0.0 and bool((lse == -INF).all())
+    kn[..., 0] = 0                                  # only the new row counts: the step returns its value
+    for out, lse in (tl.tlin_decode_step(q, kn, vn, kc, vc, pos), tl.tlin_decode_step_ragged(q, kn, vn, kc, vc, at, pos)):
+        assert torch.equal(out, vn)
+        want = (q.float() * kn.float()).sum(-1)[..., 0] / d ** 0.5
+        assert float((lse - want).abs().max()) <= 1e-5
+    assert tl.tlin_get_status() == 0
