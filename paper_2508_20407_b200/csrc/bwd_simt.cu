@@ -207,14 +207,23 @@ __global__ void bwd_round_kernel(const float* __restrict__ src, T* __restrict__ 
     if (x < n) from_f(dst[x], src[x]);
 }
 
+bool overlap(const void* a, int64_t a_bytes, const void* b, int64_t b_bytes) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x < y + (uint64_t)b_bytes && y < x + (uint64_t)a_bytes;
+}
+
 template <typename T, int BT, int TC, int CM>
 int launch_t(const T* q, const T* k, const T* v, const T* out, const float* lse, const T* dout, T* dq, T* dk, T* dv,
              int B, int H, int N, int W, int d, int causal, float* ws, cudaStream_t st) {
     const int64_t n_bh = (int64_t)B * H, rows = n_bh * W;
     float* delta = ws;                                  // [B*H*W]
     constexpr bool kF32 = sizeof(T) == 4;
-    // fp32: the sums go straight into the result; bf16: [B*H*W*d] fp32 behind delta, 16-byte aligned
-    float* dq_acc = kF32 ? reinterpret_cast<float*>(dq) : ws + ((rows + 3) / 4) * 4;
+    // fp32: the sums go straight into the result, unless the main kernel still reads an input there (dq written over q, say);
+    // otherwise [B*H*W*d] fp32 behind delta, 16-byte aligned
+    const int64_t q_bytes = rows * d * (int64_t)sizeof(T), k_bytes = n_bh * N * (int64_t)d * (int64_t)sizeof(T);
+    const bool in_place = kF32 && !overlap(dq, q_bytes, q, q_bytes) && !overlap(dq, q_bytes, dout, q_bytes) && !overlap(dq, q_bytes, k, k_bytes) &&
+                          !overlap(dq, q_bytes, v, k_bytes) && !overlap(dq, q_bytes, lse, rows * (int64_t)sizeof(float));
+    float* dq_acc = in_place ? reinterpret_cast<float*>(dq) : ws + ((rows + 3) / 4) * 4;
     const float scale = 1.f / sqrtf((float)d);
     static bool allowed[64] = {};
     TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_simt_kernel<T, BT, TC, CM>, (int)bwd_smem_bytes<BT>(TC * CM, column_slack<TC, CM>()), allowed));
@@ -227,7 +236,7 @@ int launch_t(const T* q, const T* k, const T* v, const T* out, const float* lse,
         q, k, v, dout, lse, delta, dq_acc, dk, dv, N, W, d, causal, n_bh, scale);
     TLIN_CUDA_CHECK(cudaGetLastError());
     count_launch(2);
-    if constexpr (!kF32) {
+    if (!in_place) {
         bwd_round_kernel<T><<<(unsigned)((rows * d + 255) / 256), 256, 0, st>>>(dq_acc, dq, rows * d);
         TLIN_CUDA_CHECK(cudaGetLastError());
         count_launch();
