@@ -15,6 +15,7 @@
 #include "tlin_internal.h"
 #include "simt_tiles.cuh"
 #include <cooperative_groups.h>
+#include <float.h>
 #include <math_constants.h>
 
 namespace tlin {
@@ -169,12 +170,13 @@ fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
         if (row >= W) break;
         float mm = -CUDART_INF_F;
         for (int c = 0; c < cluster; ++c) mm = fmaxf(mm, cl.map_shared_rank(ms, c)[rr]);
+        const float ref = fmaxf(mm, -FLT_MAX);                  // no share may have a finite score
         float ll = 0.f, w[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             w[c] = 0.f;
             if (c < cluster) {
-                w[c] = exp2f((cl.map_shared_rank(ms, c)[rr] - mm) * kLog2e);
+                w[c] = exp2f((cl.map_shared_rank(ms, c)[rr] - ref) * kLog2e);
                 ll += w[c] * cl.map_shared_rank(ls, c)[rr];
             }
         }

@@ -57,6 +57,20 @@ def test_forward_passes_a_nan_on(B, H, N, W, d, dtype):
 
 
 # a score of -inf masks a key (an extra column of q at 1, of k at -inf); with every key masked there is nothing to attend to
+@pytest.mark.parametrize("d", [36, 64])
+@pytest.mark.parametrize("B,H,N,W", [(1, 4, 1024, 128), (8, 16, 512, 300)])
+def test_fp32_rows_without_a_finite_score_have_a_sum_of_nothing(B, H, N, W, d):
+    q, k, v = (normal(i, B, H, rows, d, dtype=torch.float32) for i, rows in enumerate((W, N, N)))
+    q[..., 0] = 1
+    k[..., 0] = -INF
+    _, lse = forward(q, k, v, 0)
+    assert bool((lse == -INF).all())
+    k[:, :, N // 2:, 0] = 0                         # half of the keys are back, in the second shares only
+    out, lse = forward(q, k, v, 0)
+    alone, lse_alone = forward(q, k[:, :, N // 2:].contiguous(), v[:, :, N // 2:].contiguous(), 0)
+    assert float((out - alone).abs().max()) <= 1e-5 and float((lse - lse_alone).abs().max()) <= 1e-5
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("B,H,pos", [(2, 4, 600), (2, 16, 1401), (1, 1, 30), (64, 32, 300), (4, 32, 8000)])
 def test_decode_step_with_masked_scores(B, H, pos, d):
