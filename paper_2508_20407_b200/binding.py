@@ -99,6 +99,7 @@ SIGNATURES = {
 
 _lib = None
 _workspaces = {}          # device index -> the buffer that the library holds the address of: alive as long as it is registered
+_workspace_sizes = {}     # device index -> its elements, if it lies on that device
 _workspace_tensor = None  # the one registered last
 
 
@@ -210,19 +211,21 @@ def set_workspace(t: torch.Tensor | None):
     if t is None:
         _check(lib().tlin_set_workspace(None, 0), "tlin_set_workspace")
         _workspaces.pop(slot, None)
+        _workspace_sizes.pop(slot, None)
     else:
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("workspace must be a contiguous CUDA tensor")
         _check(lib().tlin_set_workspace(_ptr(t), t.numel() * t.element_size()), "tlin_set_workspace")
         _workspaces[slot] = t
+        _workspace_sizes[slot] = t.numel() if t.device.index == slot else -1
     _workspace_tensor = t
 
 
 def ensure_workspace(nbytes: int, device="cuda"):
     """Grows the current device's workspace to at least ``nbytes`` (allocation happens here, in torch)."""
+    if type(device) is torch.device and nbytes <= _workspace_sizes.get(device.index, -1):
+        return _workspaces[device.index]
     t = _workspaces.get(_device_slot())
-    if t is not None and nbytes <= t.numel() and t.device == device:
-        return t
     if t is None:
         grow = nbytes > 0
     else:

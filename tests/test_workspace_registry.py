@@ -66,6 +66,7 @@ def machine(monkeypatch):
     monkeypatch.setattr(tl, "lib", m.lib)
     monkeypatch.setattr(tl, "_current_device", lambda: m.current)
     monkeypatch.setattr(tl, "_workspaces", {}, raising=False)
+    monkeypatch.setattr(tl, "_workspace_sizes", {}, raising=False)
     monkeypatch.setattr(tl, "_workspace_tensor", None)
     monkeypatch.setattr(torch, "empty", m.empty)
     return m
