@@ -55,7 +55,7 @@ typedef enum {
  *                    "Causal Attention", j <= i, aligned to the end).  One softmax runs over the
  *                    union of both key sets.  Requires N >= W.
  * bf16 path: d a multiple of 8 up to 256, on the tensor cores (64 and 128 in tiles of their own, the others in zero-padded
- * ones).  f32 path: d a multiple of 4 up to 256 (covers the paper's d = 36), CUDA cores.
+ * ones; many (b,h) of a few rows and keys at those others on the CUDA cores).  f32 path: d a multiple of 4 up to 256 (covers the paper's d = 36), CUDA cores.
  * Uses the workspace when the plan splits the key range (see tlin_workspace_bytes_forward); head sizes other than 64 and 128
  * also run without one, with whole key ranges.
  */

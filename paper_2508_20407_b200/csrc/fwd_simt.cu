@@ -1,6 +1,6 @@
 // CUDA-core forward kernel: exact softmax attention, fp32 arithmetic, any head dimension up to 256.
-// Serves the fp32 entry point (error bar 1e-4), and bf16 where tlin_set_forward_impl(1) asks for it or the call has 2^31 query
-// rows or more at a head size other than 64 and 128.
+// Serves the fp32 entry point (error bar 1e-4), and bf16 where tlin_set_forward_impl(1) asks for it or, at a head size other than 64 and
+// 128, the call has very few rows and keys per (b,h) (rows_beat_tensor_cores) or 2^31 query rows or more.
 // Section 3 attention formula; causal rule j <= N-W+i; online (running max / running sum) softmax.
 //
 // Bound by the FFMA rate (128 per clock and SM, 72 TFLOP/s at 1.9 GHz).  A CTA of 128 threads (16 row groups x 8 column
@@ -14,6 +14,7 @@
 // distributed shared memory, so that no workspace is needed.
 #include "tlin_internal.h"
 #include "simt_tiles.cuh"
+#include <algorithm>
 #include <cooperative_groups.h>
 #include <float.h>
 #include <math_constants.h>
@@ -198,6 +199,14 @@ fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
     cl.sync();                                  // nobody leaves while its rows are still being read
 }
 
+// Keys shared between CTAs while there are fewer CTAs than twice the SMs, at least four tiles each.
+int cluster_size(int64_t items, int N) {
+    int cluster = 1;
+    const int tiles = (N + kBN - 1) / kBN;
+    while (cluster < 8 && items * cluster * 2 <= 2 * kDefaultSMs && tiles >= 8 * cluster) cluster *= 2;
+    return cluster;
+}
+
 template <typename T, int ROWS, int CM>
 int launch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H, int N, int W, int d,
            int causal, long long kv_rows_alloc, cudaStream_t st) {
@@ -207,10 +216,7 @@ int launch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H,
     const size_t smem = sizeof(float) * smem_floats<ROWS>(d, column_slack<kTC, CM>());
     static bool allowed[64] = {};
     TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_simt_kernel<T, ROWS, CM>, (int)(sizeof(float) * smem_floats<ROWS>(8 * CM, column_slack<kTC, CM>())), allowed));
-    // Keys shared between CTAs while there are fewer CTAs than twice the SMs, at least four tiles each.
-    int cluster = 1;
-    const int tiles = (N + kBN - 1) / kBN;
-    while (cluster < 8 && items * cluster * 2 <= 2 * kDefaultSMs && tiles >= 8 * cluster) cluster *= 2;
+    const int cluster = cluster_size(items, N);
     if (items * cluster > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(items * cluster));
@@ -229,14 +235,156 @@ int launch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H,
     return TLIN_OK;
 }
 
+// Few query rows, or few keys: one warp per row instead of a register tile.  The tiles above are at least 64 rows x 64 keys whatever
+// the call has, and for 1 to 8 rows most of that is work on padding.  Eight rows per CTA; keys and values are staged 32 at a time (fp32),
+// lane l scores key l, the warp reduces maximum and sum with shuffles, and lane c accumulates the output columns c, c + 32, ...
+constexpr int kWarpRows = 8, kWarpKeys = 32, kWarpColumns = 8;      // columns per lane: d <= 256
+
+__device__ __forceinline__ float to_f32(float x) { return x; }
+__device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
+
+__device__ __forceinline__ float warp_max(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+}
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kWarpRows * 32)
+fwd_row_per_warp_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ out, float* __restrict__ lse,
+                        int N, int W, int d, int causal, int q_tiles, float scale, int64_t kv_rows) {
+    extern __shared__ __align__(16) float smem[];
+    const int kstride = d + 4;                 // padded: lanes reading different rows hit different banks
+    float* Qs = smem;                          // [kWarpRows][d]
+    float* Ks = Qs + kWarpRows * d;            // [kWarpKeys][d+4]
+    float* Vs = Ks + kWarpKeys * kstride;      // [kWarpKeys][d]
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t bh = blockIdx.x / q_tiles;
+    const int row0 = (blockIdx.x % q_tiles) * kWarpRows;
+    const int i = row0 + warp;
+    const bool row_ok = i < W;
+    const T* qb = q + (bh * W + row0) * (int64_t)d;
+    const T* kb = k + bh * kv_rows * d;        // kv_rows >= N: rows per (b,h) of the key/value allocation
+    const T* vb = v + bh * kv_rows * d;
+
+    const int rows_here = min(kWarpRows, W - row0);
+    for (int idx = threadIdx.x; idx < rows_here * d; idx += blockDim.x) Qs[idx] = to_f32(qb[idx]);
+
+    // keys this CTA needs: up to the limit of its last row
+    const int64_t last_i = row0 + rows_here - 1;
+    const int64_t klimit_blk = causal ? min((int64_t)N, (int64_t)(N - W) + last_i + 1) : (int64_t)N;
+    const int64_t klimit_row = causal ? (int64_t)(N - W) + i + 1 : (int64_t)N;  // keys j < klimit_row allowed
+
+    float m = -CUDART_INF_F, l = 0.f;
+    float acc[kWarpColumns];
+#pragma unroll
+    for (int r = 0; r < kWarpColumns; ++r) acc[r] = 0.f;
+
+    for (int64_t t0 = 0; t0 < klimit_blk; t0 += kWarpKeys) {
+        __syncthreads();
+        const int nk = (int)min((int64_t)kWarpKeys, (int64_t)N - t0);
+        for (int idx = threadIdx.x; idx < kWarpKeys * d; idx += blockDim.x) {
+            const int r = idx / d, c = idx - r * d;
+            float kv = 0.f, vv = 0.f;
+            if (r < nk) {
+                kv = to_f32(kb[(t0 + r) * d + c]);
+                vv = to_f32(vb[(t0 + r) * d + c]);
+            }
+            Ks[r * kstride + c] = kv;
+            Vs[r * d + c] = vv;
+        }
+        __syncthreads();
+        if (!row_ok) continue;
+        const int64_t j = t0 + lane;
+        const bool ok = j < N && j < klimit_row;
+        float s = 0.f;
+        const float4* q4 = reinterpret_cast<const float4*>(Qs + warp * d);
+        const float4* k4 = reinterpret_cast<const float4*>(Ks + lane * kstride);
+        for (int c = 0; c < d / 4; ++c) {
+            const float4 a = q4[c], b = k4[c];
+            s = fmaf(a.x, b.x, s); s = fmaf(a.y, b.y, s); s = fmaf(a.z, b.z, s); s = fmaf(a.w, b.w, s);
+        }
+        s = ok ? s * scale : -CUDART_INF_F;
+        const float m_new = fmaxf(m, warp_max(s));
+        if (m_new == -CUDART_INF_F) continue;          // nothing that counts so far
+        const float corr = expf(m - m_new);            // m = -inf -> 0
+        const float p = ok ? expf(s - m_new) : 0.f;
+        l = l * corr + warp_sum(p);
+        m = m_new;
+#pragma unroll
+        for (int r = 0; r < kWarpColumns; ++r) acc[r] *= corr;
+        for (int jj = 0; jj < kWarpKeys; ++jj) {
+            const float pj = __shfl_sync(0xffffffffu, p, jj);
+#pragma unroll
+            for (int r = 0; r < kWarpColumns; ++r) {
+                const int c = lane + 32 * r;
+                if (c < d) acc[r] = fmaf(pj, Vs[jj * d + c], acc[r]);
+            }
+        }
+    }
+    if (!row_ok) return;
+    const float inv_l = 1.f / l;
+    T* ob = out + (bh * W + i) * (int64_t)d;
+#pragma unroll
+    for (int r = 0; r < kWarpColumns; ++r) {
+        const int c = lane + 32 * r;
+        if (c < d) store1(ob + c, acc[r] * inv_l);
+    }
+    if (lse != nullptr && lane == 0) lse[bh * W + i] = m + logf(l);
+}
+
+template <typename T>
+int launch_row_per_warp(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H, int N, int W, int d,
+                        int causal, long long kv_rows_alloc, cudaStream_t st) {
+    const int q_tiles = (W + kWarpRows - 1) / kWarpRows;
+    const int64_t ctas = (int64_t)B * H * q_tiles;
+    if (ctas > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
+    auto smem_bytes = [](int d) { return (int)sizeof(float) * (kWarpRows * d + kWarpKeys * (d + 4) + kWarpKeys * d); };
+    static bool allowed[64] = {};
+    TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_row_per_warp_kernel<T>, smem_bytes(32 * kWarpColumns), allowed));
+    fwd_row_per_warp_kernel<T><<<(unsigned)ctas, kWarpRows * 32, smem_bytes(d), st>>>(q, k, v, out, lse, N, W, d, causal, q_tiles, 1.0f / sqrtf((float)d),
+                                                                                 kv_rows_alloc > 0 ? (int64_t)kv_rows_alloc : (int64_t)N);
+    TLIN_CUDA_CHECK(cudaGetLastError());
+    count_launch();
+    return TLIN_OK;
+}
+
+// Which of the two: time of each in units of about 0.6 us, the longer of one CTA's chain of key tiles and the SMs' share of all of them,
+// fitted to 10000 calls (fp32; d 4 to 256, 4 to 1024 keys, 1 to 512 rows, 1 to 6000 (b,h)).  Tiles / rows, microseconds: d64 1500 (b,h) W4
+// N32 55 / 21, W16 N64 55 / 98; d128 1500 W8 N64 150 / 86, 400 W1 N128 76 / 35; d256 64 W8 N8 27 / 13; d100 400 W9 N256 125 / 159; d36 148
+// W8 N1024 55 / 139.  On the tiles alone 3710 of those calls are more than 5 % slower than on the rows alone, with the choice 154; more
+// than 5 % slower than on the tiles alone are 109.
+bool rows_are_cheaper(int64_t n_bh, int N, int W, int d, int tile_rows, int64_t items, int cluster) {
+    const double sms = kDefaultSMs, beyond128 = d > 128 ? d - 128 : 0;
+    const double tiles = (N + kBN - 1) / kBN, steps = (N + kWarpKeys - 1) / kWarpKeys, ctas = (double)n_bh * ((W + kWarpRows - 1) / kWarpRows);
+    const double staged = N < kWarpKeys ? N / (double)kWarpKeys : steps;          // a step of fewer keys stages fewer
+    const bool from_hbm = 8.0 * n_bh * N * d > 80e6;                              // K and V do not stay in L2: a step waits longer
+    const double row_chain = (6.4 + 0.1 * d) * steps * (from_hbm ? 1.6 : 1);
+    const double row_share = (0.87 * n_bh * W * steps + ctas * staged * (0.024 * d + 0.03 * beyond128)) / sms;
+    const double tile_chain = 0.2 * d * (((int)tiles + cluster - 1) / cluster);
+    const double tile_share = (double)items * (tile_rows / 64) * tiles * (4.6 + 0.165 * d) / sms;
+    return std::max(row_chain, row_share) < std::max(tile_chain, tile_share) + 4;
+}
+
 // 8 columns per CM.  Eight rows per thread instead of four halve the shared-memory reads but need 128 query rows per CTA: worth it
-// for 40 < d <= 64 when that leaves few SMs without a CTA (128 CTAs at B4 H8 N2000 W500 d64: 261 against 285 us); at d <= 40, with three CTAs of
+// for 40 < d <= 64 and more than 64 rows when that leaves few SMs without a CTA (128 CTAs at B4 H8 N2000 W500 d64: 261 against 285 us); at d <= 40, with three CTAs of
 // either kind per SM, the finer split wins (B8 H12 N1024 W512 d36: 210 against 218 us, B8 H4 N327 W327: 42 against 52 us), and
 // beyond d = 64 the registers do not suffice.
 template <typename T>
 int dispatch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H, int N, int W, int d,
              int causal, long long kv, cudaStream_t st) {
-    if (d > 40 && d <= 64 && (int64_t)B * H * ((W + 127) / 128) >= kDefaultSMs * 3 / 4)
+    const int64_t n_bh = (int64_t)B * H;
+    const int tile_rows = d > 40 && d <= 64 && W > 64 && n_bh * ((W + 127) / 128) >= kDefaultSMs * 3 / 4 ? 128 : 64;
+    const int64_t items = n_bh * ((W + tile_rows - 1) / tile_rows);
+    if (rows_are_cheaper(n_bh, N, W, d, tile_rows, items, cluster_size(items, N)))
+        return launch_row_per_warp<T>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
+    if (tile_rows == 128)
         return launch<T, 8, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
     if (d <= 40) return launch<T, 4, 5>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
     if (d <= 64) return launch<T, 4, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);

@@ -231,6 +231,20 @@ extern "C" int tlin_plan_forward(int B, int H, int N, int W, int d, int causal_w
     return tlin::plan_forward(B, H, N, W, d, causal_window, is_f32, num_sms, false, plan);
 }
 
+// Head sizes other than 64 and 128: a tensor-core CTA takes about 6 us for a problem whatever its size, so many (b,h) of a few rows and
+// at most about 100 keys are done sooner by the CUDA cores, one warp per row.  In units of 0.26 us, as rows_are_cheaper in fwd_simt.cu,
+// fitted to 5600 calls.  Tensor cores / rows, microseconds: d96 1500 (b,h) W1 N8 62 / 19, W16 N8 62 / 56, W1 N64 62 / 39, W1 N128 54 / 75;
+// d8 6000 W8 N32 198 / 72; d256 400 W4 N4 24 / 15; d96 400 W8 N64 19 / 23.
+static bool rows_beat_tensor_cores(int64_t bh, int N, int W, int d) {
+    const int64_t problems = bh * ((W + (d <= 128 ? 255 : 127)) / (d <= 128 ? 256 : 128));
+    const int64_t waves = (problems + kDefaultSMs - 1) / kDefaultSMs;
+    if (waves < 2) return false;
+    const double steps = (N + 31) / 32, staged = N < 32 ? N / 32.0 : steps, ctas = (double)bh * ((W + 7) / 8);
+    const double chain = (14 + 0.05 * d) * steps;
+    const double share = (1.1 * bh * W * steps + ctas * staged * (0.06 * d + (d > 128 ? 0.11 * (d - 128) : 0))) / kDefaultSMs;
+    return std::max(chain, share) + 14 < 23.0 * waves;
+}
+
 // whole_only: schedule 1 whatever it costs (a tensor-path call whose caller has registered no workspace)
 int tlin::plan_forward(int B, int H, int N, int W, int d, int causal_window, int is_f32, int num_sms, bool whole_only,
                        tlin_fwd_plan* plan) {
@@ -243,7 +257,7 @@ int tlin::plan_forward(int B, int H, int N, int W, int d, int causal_window, int
     const bool tc_shape = !is_f32 && (d == 64 || d == 128 || (d % 8 == 0 && d <= 256 && (int64_t)B * H * W <= INT32_MAX));
     if (impl == 2 && !tc_shape) return TLIN_ERR_UNSUPPORTED;
     if (is_f32 ? (d % 4 != 0 || d > 256) : (d % 8 != 0 || d > 256)) return TLIN_ERR_UNSUPPORTED;
-    const bool tc = tc_shape && impl != 1;
+    const bool tc = tc_shape && impl != 1 && (impl == 2 || d == 64 || d == 128 || !rows_beat_tensor_cores((int64_t)B * H, N, W, d));
     tlin_fwd_plan p = {};
     const int64_t bh = (int64_t)B * H;
     p.tensor_path = tc ? 1 : 0;
