@@ -12,7 +12,6 @@
 #include "tlin_internal.h"
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
-#include <float.h>
 #include <math_constants.h>
 #include <atomic>
 #include <mutex>
@@ -360,16 +359,20 @@ decode_cluster_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_new
         float top = m[0];
 #pragma unroll
         for (int r = 1; r < kMaxCluster; ++r) top = fmaxf(top, m[r]);
-        const float ref = fmaxf(top, -FLT_MAX);                           // every score is -inf: zeros, as from the merge kernel
-        float sum = 0.f, z = 0.f;
+        if (top == -CUDART_INF_F) {                          // every score is -inf: zeros, as from the merge kernel
+            out[(int64_t)bh * D + threadIdx.x] = __float2bfloat16_rn(0.f);
+            if (lse != nullptr && threadIdx.x == 0) lse[bh] = -CUDART_INF_F;
+        } else {                                             // (a branch: a guard on z below costs a step of 4.6 us 0.2)
+            float sum = 0.f, z = 0.f;
 #pragma unroll
-        for (int r = 0; r < kMaxCluster; ++r) {
-            const float w = exp2f(m[r] - ref);
-            z = fmaf(w, l[r], z);
-            sum = fmaf(w, v[r], sum);
+            for (int r = 0; r < kMaxCluster; ++r) {
+                const float w = exp2f(m[r] - top);
+                z = fmaf(w, l[r], z);
+                sum = fmaf(w, v[r], sum);
+            }
+            out[(int64_t)bh * D + threadIdx.x] = __float2bfloat16_rn(sum / z);
+            if (lse != nullptr && threadIdx.x == 0) lse[bh] = (top + log2f(z)) * kLn2;
         }
-        out[(int64_t)bh * D + threadIdx.x] = __float2bfloat16_rn(sum / fmaxf(z, FLT_MIN));      // (otherwise the largest weight is 1)
-        if (lse != nullptr && threadIdx.x == 0) lse[bh] = (top + log2f(z)) * kLn2;
     }
     cl.sync();                                               // shared memory stays until it has been read
 }
