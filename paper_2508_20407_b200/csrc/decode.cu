@@ -371,7 +371,7 @@ decode_cluster_kernel(const uint4* q_new, const uint4* k_new, const uint4* v_new
                 sum = fmaf(w, v[r], sum);
             }
             out[(int64_t)bh * D + threadIdx.x] = __float2bfloat16_rn(sum / z);
-            if (lse != nullptr && threadIdx.x == 0) lse[bh] = (top + log2f(z)) * kLn2;
+            if (lse != nullptr && threadIdx.x == 0) lse[bh] = fmaf(top, kLn2, logf(z));
         }
     }
     cl.sync();                                               // shared memory stays until it has been read
