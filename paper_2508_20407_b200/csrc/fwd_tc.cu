@@ -49,6 +49,12 @@ constexpr int kPolyPairs = 5;                // of every 16 column pairs, this m
 // B1 H32 N131072 W1024 d128, 262 -> 257 us at N32768 W512, 437 -> 429 us at B4 H32 N=W=4096 d64).
 constexpr int kFirstKeys = 96;
 constexpr float kRescaleThreshold = 32.0f;  // base-2 units: P stays below 2^32, far inside bf16/fp32 range
+// An exponent is one fma, s * scale - m with m = round(s_max * scale).  That rounding is the same for all of a row and cancels, but where
+// scores pass 2^31, as those of keys masked with the lowest finite value, it is a power of two that P cannot hold.  Other head sizes,
+// whose P stands in for one kept in fp32, turn to differences of scores when a row's reference lies beyond this (base-2 units); the
+// step that finds it is done again by another copy of the code.  Differences in every step cost 3 % (packed) to 9 % (single), a branch
+// inside the step 4 %, this 0.6 %, over 50 calls.
+constexpr float kFusedScores = 1024.f;
 
 // 2^x for a packed pair without the special-function unit: x = n + f with n = floor(x) (taken by adding
 // 1.5*2^23 rounding down, which leaves n in the low mantissa bits), 2^f on [0,1) by a cubic fitted for
@@ -472,13 +478,15 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             const int lim_warp = (int)(lim_warp_ll < pr.N ? lim_warp_ll : pr.N);
             const int cnt_i = seg_count(s, allowed_i);
             float m_ref = -CUDART_INF_F;
+            float s_ref = -CUDART_INF_F;            // kAny: the score that m_ref is of
+            bool beyond = false;                    // kAny: the reference of some row of the warp is beyond kFusedScores
             uint64_t l2[2] = {0ull, 0ull};          // four partial row sums as two packed fp32 pairs
             // One key tile.  The steps with masked columns (the last ones of a segment, if any) are a second copy of the code:
             // conditions inside the exponential loop cut it into short blocks that each wait for their own results.  One copy with
             // conditions and the row sums inside the loop against this: B1 H32 N131072 W1024 d128 2.15 -> 1.89 ms,
             // N32768 W512 298 -> 265 us, B1 H32 N32768 W1024 d64 416 -> 380 us (back to back, under the power cap).
-            auto step = [&](int j, auto masked_tag) {
-                constexpr bool kMasked = decltype(masked_tag)::value;
+            auto step = [&](int j, auto masked_tag, auto exact_tag) {
+                constexpr bool kMasked = decltype(masked_tag)::value, kExact = decltype(exact_tag)::value;
                 ok = mbar_wait(&s_full[i], n & 1, abort_p);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
@@ -501,9 +509,13 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                     mx[e & 3] = max3(mx[e & 3], __uint_as_float(sv[e >> 4][(2 * e) & 31]), __uint_as_float(sv[e >> 4][(2 * e + 1) & 31]));
                 const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
                 const float m_new = fmaxf(m_ref, tmax * p.scale_log2e);
-                const bool need = m_new > m_ref + kRescaleThreshold;
+                const bool need = kExact ? tmax > s_ref : m_new > m_ref + kRescaleThreshold;
                 if (__any_sync(0xffffffffu, need)) {
-                    const float alpha = need ? ex2(m_ref - m_new) : 1.f;     // m_ref = -inf -> 0
+                    if constexpr (kAny && !kExact) {       // nothing of this step has been written yet
+                        beyond = __any_sync(0xffffffffu, need && fabsf(m_new) > kFusedScores);
+                        if (beyond) return;
+                    }
+                    const float alpha = need ? ex2(kExact ? (s_ref - tmax) * p.scale_log2e : m_ref - m_new) : 1.f;     // m_ref = -inf -> 0
                     if (j > 0) {
                         ok = mbar_wait(&pv_done[i], (n - 1) & 1, abort_p);
                         ok = __all_sync(0xffffffffu, ok);
@@ -522,20 +534,25 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                     const uint64_t alpha2 = f2_pack(alpha, alpha);
                     l2[0] = f2_mul(l2[0], alpha2);
                     l2[1] = f2_mul(l2[1], alpha2);
-                    if (need) m_ref = m_new;
+                    if (need) {
+                        m_ref = m_new;
+                        if constexpr (kAny) s_ref = tmax;
+                    }
                 }
                 const float m_use = m_ref == -CUDART_INF_F ? 0.f : m_ref;
                 // P = 2^(s*scale - m) as bf16 over the columns of S; kPolyPairs of every 16 pairs take the polynomial route (FMA
                 // pipe), the rest the special-function unit.  A masked tile takes the special-function unit only: it gives an
                 // exact 0 for -inf, the polynomial 2^-126.  The fp32 values stay in the registers of S and are summed after P has
                 // been handed over, off the path the tensor pipe waits for.
-                const uint64_t scale2 = f2_pack(p.scale_log2e, p.scale_log2e), negm2 = f2_pack(-m_use, -m_use);
+                const float s_use = s_ref == -CUDART_INF_F ? 0.f : s_ref;
+                const uint64_t scale2 = f2_pack(p.scale_log2e, p.scale_log2e), negm2 = kExact ? f2_pack(-s_use, -s_use) : f2_pack(-m_use, -m_use);
 #pragma unroll
                 for (int c = 0; c < kTileN / 32; ++c) {
                     uint32_t pk[16], pk_low[kAny ? 16 : 1];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
-                        const uint64_t x2 = f2_fma(f2_pack_bits(sv[c][2 * e], sv[c][2 * e + 1]), scale2, negm2);
+                        const uint64_t s2 = f2_pack_bits(sv[c][2 * e], sv[c][2 * e + 1]);
+                        const uint64_t x2 = kExact ? f2_mul(f2_add(s2, negm2), scale2) : f2_fma(s2, scale2, negm2);
                         float p0, p1;
                         if (!kMasked && !kAny && e * kPolyPairs / 16 != (e + 1) * kPolyPairs / 16) {
                             exp2_poly2(x2, p0, p1);
@@ -571,8 +588,16 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
             int n_open = lim_warp / kTileN - s.t_begin;
             n_open = n_open < 0 ? 0 : (n_open < cnt_i ? n_open : cnt_i);
             int j = 0;
-            for (; j < n_open && ok; ++j) step(j, std::false_type{});
-            for (; j < cnt_i && ok; ++j) step(j, std::true_type{});
+            for (; j < n_open && ok && !beyond; ++j) {
+                step(j, std::false_type{}, std::false_type{});
+                if (kAny && beyond) break;
+            }
+            for (; j >= n_open && j < cnt_i && ok && !beyond; ++j) {
+                step(j, std::true_type{}, std::false_type{});
+                if (kAny && beyond) break;
+            }
+            if constexpr (kAny)                            // from the step that found it on, that one again
+                for (; beyond && j < cnt_i && ok; ++j) step(j, std::true_type{}, std::true_type{});
             if constexpr (kShared) {
                 // -------------------------------------------------------- merge inside the cluster
                 if (ok && cnt_i > 0) {

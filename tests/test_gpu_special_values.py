@@ -88,3 +88,28 @@ def test_decode_step_with_masked_scores(B, H, pos, d):
         want = (q.float() * kn.float()).sum(-1)[..., 0] / d ** 0.5
         assert float((lse - want).abs().max()) <= 1e-5
     assert tl.tlin_get_status() == 0
+
+
+# scores far beyond anything that a model has, as from keys masked with the lowest finite value instead of -inf: the forms that keep P
+# beyond 8 bits (fp32, and bf16 at head sizes other than 64 and 128) stay exact there.  Forms: clusters, split and merged, whole
+@pytest.mark.parametrize("d,dtype", [(40, torch.bfloat16), (96, torch.bfloat16), (160, torch.bfloat16), (36, torch.float32), (128, torch.float32)])
+@pytest.mark.parametrize("B,H,N,W", [(1, 4, 1024, 128), (1, 2, 20000, 64), (8, 16, 512, 300), (2, 3, 100, 60)])
+def test_scores_of_any_finite_size(B, H, N, W, d, dtype):
+    q, k, v = (normal(i, B, H, rows, d, dtype=dtype) for i, rows in enumerate((W, N, N)))
+    q[..., 0], k[..., 0] = 1, 0
+    lowest = torch.finfo(torch.bfloat16).min
+    tol = 2e-2 if dtype == torch.bfloat16 else 1e-4
+    half = N // 2
+    masked = k.clone()
+    masked[:, :, :half, 0] = lowest
+    out, lse = forward(q, masked, v, 0)
+    alone, lse_alone = forward(q, k[:, :, half:].contiguous(), v[:, :, half:].contiguous(), 0)
+    assert float((out.float() - alone.float()).abs().max()) <= tol and float((lse - lse_alone).abs().max()) <= 1e-4
+    masked[..., 0] = lowest                         # every key alike: their mean
+    out, lse = forward(q, masked, v, 0)
+    mean = v.float().mean(2, keepdim=True)
+    assert float((out.float() - mean).abs().max()) <= tol / 2 and bool(torch.isfinite(lse).all())
+    huge = (k.float() * 1e12).to(dtype)             # one key takes all
+    out, _ = forward(q, huge, v, 0)
+    best = (q.double() @ huge.double().transpose(2, 3)).argmax(3)
+    assert torch.equal(out, torch.gather(v, 2, best[..., None].expand(-1, -1, -1, d)))
