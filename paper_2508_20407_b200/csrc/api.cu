@@ -197,8 +197,10 @@ extern "C" int tlin_attn_forward_batched(const tlin_problem* problems, int n_pro
     if (rc != TLIN_OK) return rc;
     for (int first = 0; first < n_problems; first += kMaxBatch) {
         const int n = n_problems - first < kMaxBatch ? n_problems - first : kMaxBatch;
-        rc = tlin_plan_batched(problems + first, n, sms, starts, &n_ctas);
-        if (rc != TLIN_OK) return rc;
+        if (sms != kDefaultSMs || n_problems > kMaxBatch) {           // else the check above has made it
+            rc = tlin_plan_batched(problems + first, n, sms, starts, &n_ctas);
+            if (rc != TLIN_OK) return rc;
+        }
         if (log_plans())
             fprintf(stderr, "libtlin: batched forward, problems %d..%d of %d, d=%d -> %lld units on %d ctas\n", first, first + n - 1,
                     n_problems, d, (long long)starts[n_ctas], n_ctas);

@@ -3,7 +3,6 @@
 // rule; Appendix A, cost terms), and every function here is tested against that count.
 #include "tlin_internal.h"
 #include <algorithm>
-#include <functional>
 #include <vector>
 
 using namespace tlin;
@@ -162,27 +161,38 @@ bool tlin::deal_batched_units(const tlin_problem* problems, int n_problems, int 
         }
         unit += pb.BH * q_tiles;
     }
-    long long costliest_run = 0;
+    long long costliest_run = 0, total = 0, biggest = 0;
     for (int g = 0; g < n_ctas; ++g) {
         long long sum = 0;
         for (long long u = runs[g]; u < runs[g + 1]; ++u) sum += cost[u];
         costliest_run = std::max(costliest_run, sum);
+        total += sum;
     }
+    for (const Class& c : classes) biggest = std::max(biggest, c.cost);
+    if (costliest_run <= std::max(biggest, (total + n_ctas - 1) / n_ctas)) return false;      // no shares can be cheaper
     std::stable_sort(classes.begin(), classes.end(), [](const Class& a, const Class& b) { return a.cost > b.cost; });
-    typedef std::pair<long long, int> Load;                            // cost so far, CTA
-    std::vector<Load> heap((size_t)n_ctas);
-    for (int g = 0; g < n_ctas; ++g) heap[g] = Load(0, g);             // equal loads: already a heap
+    // Heap of (cost so far, CTA), the least on top, where it grows in place and sinks: the host's time is part of a small table's
+    // (256 units on 148 CTAs 5.7 -> 4.2 us against popping and pushing).
+    static_assert(kMaxGroups <= 256, "eight bits of the key are the CTA");
+    std::vector<uint64_t> heap((size_t)n_ctas);
+    for (int g = 0; g < n_ctas; ++g) heap[g] = (uint64_t)g;            // equal loads: already a heap
     std::vector<int> owner((size_t)U), count((size_t)n_ctas + 1, 0);
     long long costliest = 0;
     for (const Class& c : classes)
         for (int x = 0; x < c.count; ++x) {
-            std::pop_heap(heap.begin(), heap.end(), std::greater<Load>());
-            Load& least = heap.back();
-            least.first += c.cost;
-            costliest = std::max(costliest, least.first);
-            owner[c.first + x * c.step] = least.second;
-            ++count[least.second + 1];
-            std::push_heap(heap.begin(), heap.end(), std::greater<Load>());
+            const int cta = (int)(heap[0] & 255u);
+            const uint64_t load = heap[0] + ((uint64_t)c.cost << 8);
+            costliest = std::max(costliest, (long long)(load >> 8));
+            owner[c.first + x * c.step] = cta;
+            ++count[cta + 1];
+            int at = 0;
+            for (int child = 1; child < n_ctas; child = 2 * at + 1) {
+                if (child + 1 < n_ctas && heap[child + 1] < heap[child]) ++child;
+                if (load <= heap[child]) break;
+                heap[at] = heap[child];
+                at = child;
+            }
+            heap[at] = load;
         }
     if (costliest >= costliest_run) return false;
     for (int g = 0; g < n_ctas; ++g) count[g + 1] += count[g];
