@@ -80,10 +80,6 @@ struct DealtWalker {
     }
 };
 
-__device__ __forceinline__ void commit_elected(uint64_t* bar) {
-    if (elect_one()) tc_commit(bar);
-}
-
 // Number of key tiles Q tile `i` of this CTA may use at all (0 if the tile lies beyond W).
 template <class P>
 __device__ __forceinline__ int tiles_allowed(const P& p, int row0, int i) {
