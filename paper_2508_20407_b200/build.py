@@ -2,6 +2,7 @@
 that marshals its hot entry points."""
 from __future__ import annotations
 
+import importlib.metadata
 import importlib.util
 import os
 import subprocess
@@ -59,7 +60,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if r.returncode != 0:
             raise RuntimeError("link failed:\n" + r.stdout + r.stderr)
     source = os.path.join(CSRC, "fastcall.cpp")
-    if force or _stale(FASTCALL, [source, headers[-1]]):
+    # the extension is linked to PyTorch's C++ interface, which changes with its version
+    stamp, torch_version = os.path.join(OBJ, "fastcall.torch"), importlib.metadata.version("torch")
+    built_for = open(stamp).read() if os.path.exists(stamp) else ""
+    if force or built_for != torch_version or _stale(FASTCALL, [source, headers[-1]]):
         torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
         cuda = os.path.dirname(os.path.dirname(nvcc)) if os.path.sep in nvcc else "/usr/local/cuda"
         cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-o", FASTCALL, source,
@@ -70,6 +74,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("g++ failed: " + " ".join(cmd) + "\n" + r.stdout + r.stderr)
+        with open(stamp, "w") as f:
+            f.write(torch_version)
     return LIB
 
 
