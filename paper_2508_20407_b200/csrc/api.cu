@@ -45,12 +45,16 @@ bool log_plans() {
     }();
     return on;
 }
-void log_fwd_plan(const char* what, int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& p) {
+// shares: CTAs per cluster that share a problem's keys instead of the plan's groups (1: none do)
+void log_fwd_plan(const char* what, int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& p, int shares = 1) {
+    char how[64] = "";
+    if (shares > 1) snprintf(how, sizeof how, " (keys shared by clusters of %d, merged in them)", shares);
+    else if (p.uses_workspace) snprintf(how, sizeof how, " (split, merged by a second kernel)");
     fprintf(stderr, "libtlin: %s B=%d H=%d N=%d W=%d d=%d causal_window=%d -> %s, schedule %d, tile %dx%d, q_tiles %d, key_tiles %d, "
                     "groups %d, ctas %d, units %lld, workspace %lld bytes%s\n",
             what, B, H, N, W, d, causal, p.tensor_path ? "tensor cores" : "CUDA cores", p.schedule, p.tile_m, p.tile_n, p.q_tiles,
             p.key_tiles, p.n_groups, p.n_ctas, (long long)p.total_units, (long long)p.workspace_bytes,
-            p.uses_workspace ? " (split, merged by a second kernel)" : "");
+            how);
 }
 void log_decode_plan(const char* what, int B, int H, int Ncap, int pos, int d, const tlin_decode_plan& p) {
     fprintf(stderr, "libtlin: %s B=%d H=%d Ncap=%d pos=%d d=%d -> %d splits of %d keys, %d in all, workspace %lld bytes\n",
@@ -114,7 +118,7 @@ static int forward_common(const void* q, const void* k, const void* v, void* out
         rc = tlin_plan_forward(B, H, N, W, d, causal_window, is_f32, sms, &plan);
         if (rc != TLIN_OK) return rc;
     }
-    if (log_plans()) log_fwd_plan(is_f32 ? "forward (fp32)" : "forward", B, H, N, W, d, causal_window, plan);
+    if (log_plans() && !plan.tensor_path) log_fwd_plan(is_f32 ? "forward (fp32)" : "forward", B, H, N, W, d, causal_window, plan);
     if (is_f32)
         return launch_fwd_simt_f32((const float*)q, (const float*)k, (const float*)v, (float*)out, lse, B, H, N, W, d, causal_window,
                                    kv_rows_alloc, st);
@@ -131,6 +135,7 @@ static int forward_common(const void* q, const void* k, const void* v, void* out
         }
         ws = (float*)w.ptr;
     }
+    if (log_plans()) log_fwd_plan("forward", B, H, N, W, d, causal_window, plan, fwd_cluster_shares(plan, (long long)B * H, d));
     return launch_fwd_tc(q, k, v, out, lse, B, H, N, W, d, causal_window, plan, ws, kv_rows_alloc, st);
 }
 

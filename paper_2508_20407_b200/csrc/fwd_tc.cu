@@ -1089,14 +1089,18 @@ int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long
     return TLIN_ERR_UNSUPPORTED;
 }
 
+int fwd_cluster_shares(const tlin_fwd_plan& plan, long long bh, int d) {
+    return d == 128 ? cluster_shares<128, kCluster>(plan, bh) : d == 64 ? cluster_shares<64, kCluster>(plan, bh)
+         : d < 64 ? cluster_shares<64, kAnyCluster>(plan, bh) : d < 128 ? cluster_shares<128, kAnyCluster>(plan, bh) : cluster_shares<256, kAnyCluster>(plan, bh);
+}
+
 int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float* lse,
                   int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& plan,
                   float* ws, long long kv_rows_alloc, cudaStream_t st) {
     if (plan.tile_m != (d > 128 ? kQTile : kTileM) || plan.tile_n != kTileN) return TLIN_ERR_UNSUPPORTED;
     if ((long long)B * H * W > 0x7fffffffLL || d % 8 != 0 || d > 256) return TLIN_ERR_UNSUPPORTED;
     const long long bh = (long long)B * H;
-    const int shares = d == 128 ? cluster_shares<128, kCluster>(plan, bh) : d == 64 ? cluster_shares<64, kCluster>(plan, bh)
-                     : d < 64 ? cluster_shares<64, kAnyCluster>(plan, bh) : d < 128 ? cluster_shares<128, kAnyCluster>(plan, bh) : cluster_shares<256, kAnyCluster>(plan, bh);
+    const int shares = fwd_cluster_shares(plan, bh, d);
     if (shares > 1) {
         if (d == 128) return launch_d<128, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);
         if (d == 64) return launch_d<64, kCluster>(q, k, v, out, lse, B, H, N, W, d, causal, plan, ws, kv_rows_alloc, st, shares);

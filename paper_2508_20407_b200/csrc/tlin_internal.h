@@ -166,11 +166,14 @@ int launch_fwd_simt_f32(const float* q, const float* k, const float* v, float* o
 int launch_fwd_tc(const void* q, const void* k, const void* v, void* out, float* lse,
                   int B, int H, int N, int W, int d, int causal, const tlin_fwd_plan& plan,
                   float* ws, long long kv_rows_alloc, cudaStream_t st);   // kv_rows_alloc: rows per (b,h) of k, v (0 = N)
+// CTAs per cluster that share the keys of a problem of this plan (the plan's groups are then not used), 1 without clusters
+int fwd_cluster_shares(const tlin_fwd_plan& plan, long long bh, int d);
 // order: null, or the units in the order of the CTAs' lists (deal_batched_units)
 int launch_fwd_tc_batched(const tlin_problem* problems, int n, int d, const long long* starts, const uint16_t* order, int n_ctas, cudaStream_t st);
 int launch_decode(const void* q_new, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                   void* out, float* lse, int B, int H, int Ncap, int pos, const int* pos_per_seq, int d,
-                  const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st, bool two_kernels = false);
+                  const tlin_decode_plan& plan, int sms, float* ws, cudaStream_t st,
+                  bool two_kernels = false);   // two_kernels: short steps as well (decode.cu, tlin_decode_step_static)
 int launch_bwd_simt(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                     void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, int is_f32, float* ws,
                     cudaStream_t st);

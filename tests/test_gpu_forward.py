@@ -1,6 +1,10 @@
 """GPU parity of the forward entry points against the CPU oracle (element by element on the same
 seeded inputs; sampled rows at the full benchmark sizes).  Everything goes through the C-ABI."""
 import ctypes
+import os
+import re
+import subprocess
+import sys
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -642,13 +646,38 @@ CLUSTERS = [(1, 4, 1024, 128, 64, 1), (2, 4, 3000, 100, 64, 1), (1, 16, 2000, 20
             (1, 4, 3000, 100, 40, 0), (1, 4, 2500, 300, 80, 1), (1, 3, 700, 500, 96, 0), (2, 4, 2000, 500, 160, 1), (2, 3, 5000, 200, 256, 0)]
 
 
+_SHARES = """
+import torch
+from paper_2508_20407_b200 import binding as tl
+for B, H, N, W, d, causal in {cases}:
+    q, k = (torch.zeros((B, H, n, d), dtype=torch.bfloat16, device="cuda") for n in (W, N))
+    tl.tlin_attn_forward(q, k, k, causal_window=causal)
+"""
+
+
+@pytest.fixture(scope="module")
+def cluster_shares():
+    """CTAs per cluster that the library's log names for each of CLUSTERS (0: another form served the call)."""
+    r = subprocess.run([sys.executable, "-c", _SHARES.format(cases=CLUSTERS)], capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, TLIN_LOG="1"), cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0, r.stderr[-2000:]
+    lines = [line for line in r.stderr.splitlines() if line.startswith("libtlin: forward ")]
+    assert len(lines) == len(CLUSTERS)
+    found = [re.search(r"clusters of (\d+)", line) for line in lines]
+    return {case: int(m.group(1)) if m else 0 for case, m in zip(CLUSTERS, found)}
+
+
 @pytest.mark.parametrize("B,H,N,W,d,causal", CLUSTERS)
-def test_forward_keys_shared_by_a_cluster(B, H, N, W, d, causal):
+def test_forward_keys_shared_by_a_cluster(cluster_shares, B, H, N, W, d, causal):
+    assert 2 <= cluster_shares[(B, H, N, W, d, causal)] <= 8
     wl = synth.Workload("cluster", B, H, d, N, W, seed=2100 + N + W, causal_window=causal)
     q, k, v = synth.forward_inputs(wl, device=DEV)
-    out, lse = tl.tlin_attn_forward(q, k, v, causal_window=causal)
+    out_g, lse_g = Guarded(q.shape, torch.bfloat16, DEV), Guarded(q.shape[:3], torch.float32, DEV)
+    out, lse = tl.tlin_attn_forward(q, k, v, out_g.t, lse_g.t, causal_window=causal)
     torch.cuda.synchronize()
-    assert tl.tlin_get_status() == 0 and tl.tlin_last_launch_count() <= 2       # 1, unless the device cannot hold the clusters at a time
+    assert tl.tlin_get_status() == 0 and tl.tlin_last_launch_count() == 1
+    out_g.check("out")
+    lse_g.check("lse")
     again, lse_again = tl.tlin_attn_forward(q, k, v, causal_window=causal)
     ref, ref_lse = oracle.attn_forward(q.cpu(), k.cpu(), v.cpu(), causal)
     parity.check(out.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", f"{(B, H, N, W, d, causal)}")
