@@ -451,11 +451,12 @@ def test_batched_decode_table_every_problem_against_the_oracle(d, n_problems):
 @pytest.mark.parametrize("kind,B,H,N0,d", [("bf16", 45, 7, 2299, 128), ("fp8", 3, 120, 2499, 64), ("ragged", 40, 8, 2099, 64), ("ragged", 45, 7, 2299, 128)])
 def test_decode_runs_of_splits(kind, B, H, N0, d):
     plan = tl.tlin_plan_decode(B, H, N0 + 1, d, 148)
-    assert plan.splits > 1 and plan.n_ctas > 2 * 148
+    assert plan.splits > 1 and plan.n_ctas > 3 * 148       # CTAs that an SM holds at a time
     if kind == "fp8":
         kc_h, vc_h, ks, vs, qn, kn, vn = _fp8_cache(synth.Workload("dec8", B, H, d, N0, 1, seed=5, decode=True), pad=2)
         kc, vc = kc_h.to(DEV), vc_h.to(DEV)
         out, lse = tl.tlin_decode_step_fp8(qn[0].to(DEV), kn[0].to(DEV), vn[0].to(DEV), kc, vc, ks.to(DEV), vs.to(DEV), N0)
+        assert tl.tlin_last_launch_count() == 2             # the splits and their merge: no clusters
         ref, ref_lse = oracle.decode_step_fp8(qn[0], kn[0], vn[0], kc_h, vc_h, ks, vs, N0)
         parity.check(out.float().cpu().numpy(), lse.cpu().numpy(), ref, ref_lse, "bf16", "fp8 runs")
     else:
@@ -468,10 +469,11 @@ def test_decode_runs_of_splits(kind, B, H, N0, d):
             pos = torch.randint(0, N0 + 1, (B,), generator=rng, dtype=torch.int32)
             pos[0], pos[1], pos[2], pos[bad] = 0, N0, plan.keys_per_split - 1, N0 + 1       # the last one is beyond the bound
             out, lse = tl.tlin_decode_step_ragged(q.to(DEV), kn.to(DEV), vn.to(DEV), kc, vc, pos.to(DEV), N0)
-            assert tl.tlin_get_status() == tl.ERR_INVALID_ARG
+            assert tl.tlin_last_launch_count() == 2 and tl.tlin_get_status() == tl.ERR_INVALID_ARG
             assert float(out[bad].float().abs().max()) == 0.0 and bool((lse[bad] == float("-inf")).all())
         else:
             out, lse = tl.tlin_decode_step(q.to(DEV), kn.to(DEV), vn.to(DEV), kc, vc, N0)
+            assert tl.tlin_last_launch_count() == 2
         for b in range(B):
             if kind == "ragged" and b == bad:
                 continue
