@@ -14,8 +14,8 @@ constexpr int kTileN = 128;            // keys per tile on the tensor path
 // K and V of a call that stay in L2 (126 MB) while its CTAs read them at unrelated times.  64 / 112 MiB, microseconds: 256 heads of 780
 // keys, 277 rows, d = 128 (102 MB) 91 / 76; 128 x 1500, 800 rows (98 MB) 132 / 107; 64 x 3000, 2000 rows (98 MB) 156 / 145.
 constexpr int64_t kKVInL2 = 112ll << 20;
-constexpr int kSimtRows = 8;           // query rows per CTA on the CUDA-core path
-constexpr int kSimtKeys = 32;          // keys per staged tile on the CUDA-core path
+constexpr int kSimtRows = 8;           // query rows and keys per tile that plans of the CUDA-core path report; its kernels take
+constexpr int kSimtKeys = 32;          // tiles of their own (fwd_simt.cu: by d, the rows and the number of (b,h))
 constexpr int kDecodeMaxSplits = 64;   // upper bound on the splits of a (b,h) in the decode step
 constexpr int kDecodeMaxCluster = 8;   // up to this many splits are merged inside a cluster (the portable cluster size)
 constexpr int kDecodeClusterKeys = 1024;   // ... when they are no longer than this
