@@ -55,7 +55,8 @@ typedef enum {
  *                    "Causal Attention", j <= i, aligned to the end).  One softmax runs over the
  *                    union of both key sets.  Requires N >= W.
  * bf16 path: d a multiple of 8 up to 256, on the tensor cores (64 and 128 in tiles of their own, the others in zero-padded
- * ones; many (b,h) of a few rows and keys at those others on the CUDA cores).  f32 path: d a multiple of 4 up to 256 (covers the paper's d = 36), CUDA cores.
+ * ones; many (b,h) of a few rows and keys at those others on the CUDA cores).  f32 path: d a multiple of 4 up to 256
+ * (covers the paper's d = 36), CUDA cores.
  * Uses the workspace when the plan splits the key range (see tlin_workspace_bytes_forward); head sizes other than 64 and 128
  * also run without one, with whole key ranges.
  */
@@ -326,7 +327,7 @@ int64_t tlin_plan_backward_share_start(int B, int H, int N, int W, int causal_wi
  * (b,h,query tile) problem costs the key tiles its rows may use (+3 for starting and finishing it and for its masked steps), which grows with the
  * query tile, and when there are at least three problems per group the groups take contiguous runs of problems whose
  * costliest run is as cheap as contiguous runs allow (long problems) and which stay close to equal shares of the cost.  A launch
- * whose K and V stay in L2 (64 MiB) takes the problems of that schedule in descending order of cost instead, one round of CTAs
+ * whose K and V stay in L2 (112 MiB) takes the problems of that schedule in descending order of cost instead, one round of CTAs
  * after the other, every other round backwards: the same problems, more evenly shared. */
 int64_t tlin_plan_group_start(const tlin_fwd_plan* plan, int g);
 /* Mask predicate: may query i (0 <= i < W) use key j?  1 or 0. */
@@ -366,9 +367,10 @@ int tlin_set_forward_impl(int impl);
  *       contribution of every (128-key, 64-query) block is added to an fp32 buffer in the workspace by reductions in L2 and
  *       rounded to bf16 at the end, so dQ repeats only up to the order of those fp32 additions (dK, dV stay bitwise
  *       repeatable); needs B*H*ceil(W/128)*128*(d+2)*4 bytes of workspace, which tlin_workspace_bytes_backward includes;
- *   0 (the default) = the library chooses: arrangement 2 at d = 128 while that fp32 dQ buffer is at most 64 MiB (2 to 13 %
- *       faster on B200), arrangement 1 otherwise (beyond that size the two are level: the reductions, not the matrix
- *       products, bound arrangement 2).
+ *   0 (the default) = the library chooses: arrangement 2 at d = 128 while that fp32 dQ buffer is at most 64 MiB (level for
+ *       1024 queries over 1024 keys at that size, up to 36 % faster otherwise on B200), arrangement 1 beyond (up to 12 % faster
+ *       there for short sequences over themselves; arrangement 2 is 7 to 26 % faster from 128 MiB on where a (b,h) has 16 key
+ *       tiles or more, so set 2 there if dQ need not be bitwise repeatable).
  * Set 1 where bitwise repeatable gradients are needed.  Returns the old value; TLIN_ERR_INVALID_ARG for another argument.
  * tlin_backward_arrangement: the arrangement (1 or 2) a call with these sizes gets under the current setting; host-only. */
 int tlin_set_backward_impl(int impl);

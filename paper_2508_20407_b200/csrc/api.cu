@@ -253,9 +253,15 @@ extern "C" int tlin_attn_forward_host(const void* q_h, const void* k_h, const vo
 }
 
 // Which arrangement of the tensor-core backward a bf16 call with these sizes gets.  The one-kernel arrangement pays for its
-// two saved matrix products with fp32 reductions into a B*H*ceil(W/128)*128*d*4-byte dQ buffer.  Measured against the two
-// kernels it is 2 to 13 % faster while that buffer is at most 64 MiB and level with them beyond (its CTAs take the key
-// tiles in turn, so the rows being added to stay in L2 at any size); beyond 64 MiB the bitwise repeatable two kernels run.
+// two saved matrix products with fp32 reductions into a B*H*ceil(W/128)*128*d*4-byte dQ buffer.  Measured, two kernels / one,
+// microseconds, by the MiB of that buffer (d = 128; the first three under the window rule):
+//                                     16           32           64            96            128           256
+//   1024 queries, 1024 keys        56 / 44      95 / 89     191 / 193     283 / 309     374 / 399     786 / 825
+//   4096 queries, 4096 keys       148 / 95     241 / 214    492 / 436     715 / 705     965 / 898    2153 / 1837
+//   1024 queries, 8192 keys       469 / 349    955 / 709   1842 / 1400   2874 / 2200   3760 / 2845   7736 / 6040
+//   2048 queries, 2048 keys, no   127 / 100    262 / 209    527 / 383     803 / 609    1048 / 780    2090 / 1598
+// So up to 64 MiB the one kernel is never the slower one by more than about 1 %.  Beyond, the bitwise repeatable two kernels run: faster
+// for short sequences over themselves, slower where a (b,h) has many key tiles.
 extern "C" int tlin_backward_arrangement(int B, int H, int N, int W, int d) {
     if (B <= 0 || H <= 0 || N <= 0 || W <= 0) return TLIN_ERR_INVALID_ARG;
     if (d != 64 && d != 128) return TLIN_ERR_UNSUPPORTED;

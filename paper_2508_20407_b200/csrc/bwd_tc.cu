@@ -194,8 +194,11 @@ struct UnitOrder {
 };
 // Dealing pays where runs and turns come out uneven, i.e. with few units per CTA and a window that is a large part of the keys (units
 // per CTA x N / W up to 32: costliest CTA 8 to 100 % above the mean against 1 to 10 %), and costs about 5 % of locality otherwise
-// (B1 H32 N32768 W512 817 -> 867 us); it needs the tensors that the units of a (b,h) share in L2 for all (b,h) at once.
-// Measured: B3 H12 N=W=1999 d64 161 -> 119 us (two kernels), B1 H16 N=W=2000 d128 84 -> 61 us (one kernel).
+// (B1 H32 N32768 W512 817 -> 867 us).  Measured: B3 H12 N=W=1999 d64 161 -> 119 us (two kernels), B1 H16 N=W=2000 d128 84 -> 61 us
+// (one kernel).  What dealing gives shrinks as the tensors that the units of a (b,h) share (one kernel: dQ sums, Q and dout; two: Q or
+// dout) outgrow L2, hence the bound, which lies where the one kernel stops gaining (d128, turns / dealt, us): 100 MiB N=W=4096 404 / 333,
+// N4096 W2048 511 / 498; 136 MiB 490 / 456, 692 / 689; 144 MiB 503 / 485, 695 / 738; 200 MiB 731 / 689, 1032 / 1080.  The two kernels
+// mostly gain 5 to 12 % on either side of it (d64 N=W=4096: 136 MiB 1449 / 1286, 160 MiB 1694 / 1511, 200 MiB 2140 / 1917).
 bool deal_units(long long bh, int N, int W, int causal, int key_tiles, long long shared_bytes, int num_sms) {
     return causal && shared_bytes <= (140LL << 20) && bh * key_tiles * N <= 32LL * num_sms * W;
 }
