@@ -491,7 +491,7 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
                 tc_fence_after();
-                // the whole row of S (128 fp32) comes into registers once (at other head sizes its chunks once more for the exponentials)
+                // the whole row of S (128 fp32) comes into registers once (in the form with a loop below, its chunks once more for the exponentials)
                 const int nvalid = kMasked ? lim_row - (s.t_begin + j) * kTileN : 0;   // columns [0, nvalid) of this tile are allowed for this row
                 uint32_t sv[kTileN / 32][32];
 #pragma unroll
@@ -546,10 +546,14 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 // been handed over, off the path the tensor pipe waits for.
                 const float s_use = s_ref == -CUDART_INF_F ? 0.f : s_ref;
                 const uint64_t scale2 = f2_pack(p.scale_log2e, p.scale_log2e), negm2 = kExact ? f2_pack(-s_use, -s_use) : f2_pack(-m_use, -m_use);
-                if constexpr (kAny) {
+                if constexpr (kAny && (D > 64 || kForm == kAnyDealt)) {
                     // A loop over chunks of 32 keys: unrolled, the three copies of the step (open, masked, exact) and the MMA warp's code did
-                    // not fit the instruction cache together, 1.9 of 8.2 stall cycles per instruction (B2 H9 N3001 W517 d96 41.5 -> 37.2 us,
-                    // B8 H9 N1000 W300 d80 36 -> 33).  At d = 64 and 128 the loop is the slower form (56.8 -> 60.0, 230 -> 240 us).
+                    // not fit the instruction cache together, 1.9 of 8.2 stall cycles per instruction.  Unrolled / loop, microseconds: B2 H9
+                    // N3001 W517 d96 41.4 / 37.1, d160 53.5 / 51.3, d256 67.2 / 64.4; B1 H12 N8000 W700 d112 61.1 / 55.1, d192 90.9 / 91.6.
+                    // Up to 64 columns the code is half as long and long runs of open tiles fit: there the loop only where whole problems
+                    // are dealt out (d32: B4 H16 N512 W512 14.9 / 14.1, B16 H16 N1200 W600 118.3 / 116.1); elsewhere B1 H8 N16000 W1024 60.8 /
+                    // 66.3, B2 H9 N3001 W517 28.9 / 30.0, B1 H12 N8000 W700 42.2 / 44.8, against B16 H16 N400 W256 29.5 / 28.2.  At d = 64
+                    // and 128 the loop is the slower form (56.8 / 60.0, 230 / 240).
 #pragma unroll 1
                     for (int c = 0; c < kTileN / 32; ++c) {
                         uint32_t x[32], pk[16], pk_low[16];
@@ -586,13 +590,13 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                 }
 #pragma unroll
                 for (int c = 0; c < kTileN / 32; ++c) {
-                    uint32_t pk[16];
+                    uint32_t pk[16], pk_low[kAny ? 16 : 1];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
                         const uint64_t s2 = f2_pack_bits(sv[c][2 * e], sv[c][2 * e + 1]);
-                        const uint64_t x2 = f2_fma(s2, scale2, negm2);
+                        const uint64_t x2 = kExact ? f2_mul(f2_add(s2, negm2), scale2) : f2_fma(s2, scale2, negm2);
                         float p0, p1;
-                        if (!kMasked && e * kPolyPairs / 16 != (e + 1) * kPolyPairs / 16) {
+                        if (!kMasked && !kAny && e * kPolyPairs / 16 != (e + 1) * kPolyPairs / 16) {
                             exp2_poly2(x2, p0, p1);
                         } else {
                             float x0, x1;
@@ -603,8 +607,11 @@ fwd_tc_kernel(const __grid_constant__ KernelMaps<kForm == kTable> maps, const __
                         sv[c][2 * e] = __float_as_uint(p0);
                         sv[c][2 * e + 1] = __float_as_uint(p1);
                         pk[e] = pack_bf16x2(p0, p1);
+                        if constexpr (kAny)
+                            pk_low[e] = pack_bf16x2(p0 - __uint_as_float(pk[e] << 16), p1 - __uint_as_float(pk[e] & 0xffff0000u));
                     }
-                    tmem_st16(tS + c * 16, pk);
+                    tmem_st16(tS + c * (kAny ? 32 : 16), pk);
+                    if constexpr (kAny) tmem_st16(tS + c * 32 + 16, pk_low);
                     if (c == kFirstKeys / 32 - 1) {    // the first keys are in place: let the PV MMAs start on them
                         tc_wait_st();
                         tc_fence_before();
