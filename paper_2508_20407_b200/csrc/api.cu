@@ -247,7 +247,7 @@ extern "C" int tlin_attn_forward_f32(const float* q, const float* k, const float
 
 extern "C" size_t tlin_scratch_bytes_forward_f32(int B, int H, int N, int W, int d, int causal_window) {
     if (B <= 0 || H <= 0 || N <= 0 || W <= 0 || d <= 0 || forward_impl() != 0) return 0;
-    return fwd_f32_tensor_path(B, H, N, W, d, causal_window) ? fwd_f32_scratch_bytes(B, H, N, W, d) : 0;
+    return fwd_f32_tensor_path(B, H, N, W, d, causal_window) ? fwd_f32_scratch_bytes(B, H, N, W, d, causal_window) : 0;
 }
 
 extern "C" int tlin_attn_forward_f32_scratch(const float* q, const float* k, const float* v, float* out, float* lse,

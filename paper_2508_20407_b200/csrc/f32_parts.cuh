@@ -44,6 +44,11 @@ struct SplitJobs {
     long long zero_n;
 };
 int launch_split(const SplitJobs& jobs, cudaStream_t st);
+// No call takes more scratch than this, which an allocator keeps once it has been asked for it.  Few query tiles over long histories are
+// what would: forward, unbounded / 2 GiB / 1 GiB / on the CUDA cores, microseconds: B1 H32 N131072 W128 d128 (6.0 GiB) 3500 / 4890 / 7170 /
+// 11720, B8 H32 N65536 W100 d36 (7.5) 4590 / 6020 / 6320 / 14990, B1 H16 N131072 W128 d128 (3.0) 2450 / 2440 / 3970 / 8780, B1 H32
+// N131072 W1024 d64 (3.0) 5750 / 5750 / 5770 / 31700.
+constexpr size_t kMaxScratch = (size_t)2 << 30;
 // Parts of `rows` rows in all, in bytes
 inline size_t part_bytes(long long rows, int d) { return (size_t)kParts * 2 * rows * padded_head(d); }
 

@@ -173,7 +173,7 @@ double fwd_simt_us(long long n_bh, int N, int W, int d, int causal);
 // fp32 on the tensor cores (fwd_f32_tc.cu, bwd_f32_tc.cu): whether a call is better served there, its scratch, and the call.  It returns
 // TLIN_ERR_UNSUPPORTED, with nothing launched, for several launches whose results lie over inputs.
 bool fwd_f32_tensor_path(int B, int H, int N, int W, int d, int causal);
-size_t fwd_f32_scratch_bytes(int B, int H, int N, int W, int d);
+size_t fwd_f32_scratch_bytes(int B, int H, int N, int W, int d, int causal);
 int launch_fwd_f32_tc(const float* q, const float* k, const float* v, float* out, float* lse, int B, int H, int N, int W, int d, int causal,
                       void* scratch, int sms, cudaStream_t st);
 bool bwd_f32_tensor_path(int B, int H, int N, int W, int d, int causal);

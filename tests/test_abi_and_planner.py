@@ -348,3 +348,19 @@ def test_batched_plan_rejects_bad_problems_on_the_host():
     assert L.tlin_attn_forward_batched(None, 1, 64, None) == tl.ERR_INVALID_ARG
     assert L.tlin_attn_forward_cache(ctypes.c_void_p(16), ctypes.c_void_p(16), ctypes.c_void_p(16), ctypes.c_void_p(16), None,
                                      1, 1, 100, 101, 8, 64, 0, None) == tl.ERR_INVALID_ARG
+
+
+# (B, H, N, W, d): few query tiles over long histories are what would take the most, in the forward for want of tiles to fill the chip
+# with, in the backward for one (b,h) alone; the last row of each side of 2 GiB
+@pytest.mark.parametrize("B,H,N,W,d", [(8, 32, 65536, 128, 128), (1, 32, 131072, 64, 128), (1, 32, 131072, 128, 128), (1, 32, 131072, 1024, 64),
+                                       (8, 32, 65536, 100, 36), (1, 20, 262144, 128, 36), (1, 2, 1300000, 300, 128), (1, 1, 1300000, 40000, 64)])
+def test_scratch_of_an_fp32_call_is_bounded(B, H, N, W, d):
+    for causal in (0, 1):
+        fwd, bwd = tl.lib().tlin_scratch_bytes_forward_f32(B, H, N, W, d, causal), tl.lib().tlin_scratch_bytes_backward_f32(B, H, N, W, d, causal)
+        assert 0 < fwd <= 2 << 30
+        assert 0 <= bwd <= 2 << 30 and (d > 64 or W < 500 or bwd > 0)
+
+
+def test_an_fp32_call_whose_single_heads_outgrow_the_bound_takes_no_scratch():
+    assert tl.lib().tlin_scratch_bytes_forward_f32(1, 2, 2000000, 300, 128, 1) == 0
+    assert tl.lib().tlin_scratch_bytes_backward_f32(1, 2, 3000000, 1000, 64, 1) == 0

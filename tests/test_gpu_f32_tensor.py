@@ -119,3 +119,25 @@ def test_one_call_in_several_launches():
     assert fwd and bwd
     for a, b in zip(got, ref):
         assert float((a - b).double().norm()) <= 2e-6 * float(b.double().norm())
+
+
+def test_a_long_history_goes_in_chunks_of_no_more_than_the_bound():
+    """24 heads of 131072 keys are 2.3 GiB of parts for one query tile each: several launches, the last of fewer heads or not."""
+    B, H, N, W, d = 1, 24, 131072, 20, 64
+    lib, sizes, stream = tl.lib(), (B, H, N, W, d, 1), torch.cuda.current_stream().cuda_stream
+    need = lib.tlin_scratch_bytes_forward_f32(*sizes)
+    assert 0 < need <= 2 << 30
+    g = torch.Generator(device=DEV).manual_seed(1)
+    q, k, v = (torch.randn(B, H, rows, d, generator=g, device=DEV) for rows in (W, N, N))
+    results = []
+    for s in (scratch(need), None):
+        out, lse = torch.empty_like(q), torch.empty(B, H, W, device=DEV)
+        assert lib.tlin_attn_forward_f32_scratch(*pointers(q, k, v, out, lse), *sizes, s.data_ptr() if s is not None else None, need if s is not None else 0, stream) == 0
+        results.append((out, lse, tl.tlin_last_launch_count()))
+    assert tl.tlin_get_status() == 0 and results[0][2] > 3
+    scores = q.double() @ k.double().transpose(-1, -2) / math.sqrt(d)
+    scores.masked_fill_(torch.arange(N, device=DEV)[None] > (N - W + torch.arange(W, device=DEV))[:, None], -math.inf)
+    lse = torch.logsumexp(scores, -1)
+    out = scores.sub_(lse[..., None]).exp_() @ v.double()
+    for x, a, b in zip((out, lse), results[0], results[1]):      # as test_as_exact_as_the_cuda_cores
+        assert float((a - x).norm()) <= max(1.2 * float((b - x).norm()), 4 * 2.0 ** -24 * float(x.norm()))
