@@ -141,3 +141,41 @@ def test_a_long_history_goes_in_chunks_of_no_more_than_the_bound():
     out = scores.sub_(lse[..., None]).exp_() @ v.double()
     for x, a, b in zip((out, lse), results[0], results[1]):      # as test_as_exact_as_the_cuda_cores
         assert float((a - x).norm()) <= max(1.2 * float((b - x).norm()), 4 * 2.0 ** -24 * float(x.norm()))
+
+
+def forward_lse(q, k):
+    """lse of the tensor cores for values that do not matter, and the 64-bit scores."""
+    B, H, W, d = q.shape
+    N, lib = k.shape[2], tl.lib()
+    need = lib.tlin_scratch_bytes_forward_f32(B, H, N, W, d, 0)
+    assert need > 0
+    s, out, lse = scratch(need), torch.empty_like(q), torch.empty(B, H, W, device=DEV)
+    assert lib.tlin_attn_forward_f32_scratch(*pointers(q, k, k, out, lse), B, H, N, W, d, 0, s.data_ptr(), need, torch.cuda.current_stream().cuda_stream) == 0
+    assert tl.tlin_get_status() == 0
+    return lse, q.double() @ k.double().transpose(-1, -2) / math.sqrt(d)
+
+
+# what the tensor pipe cuts off a score is put back only where something was cut off: the mean of 7200 roundings to nearest is far below an
+# eighth of 2^-24
+@pytest.mark.parametrize("d", [36, 64, 100, 128])
+@pytest.mark.parametrize("sign", [0, -1])
+def test_lse_of_whole_scores(d, sign):
+    q, k = (torch.randint(-8, 9, (2, 12, rows, d), generator=torch.Generator().manual_seed(rows)).float().to(DEV) for rows in (300, 1500))
+    if sign:
+        q, k = -q.abs(), k.abs()
+    lse, scores = forward_lse(q, k)
+    want = torch.logsumexp(scores, -1)
+    assert abs(float(((lse - want) / want.abs()).mean())) <= 2.0 ** -27
+
+
+# and it is put back in the direction it was cut, towards zero.  With products of one sign the partial sums of a score grow evenly over its
+# n products of 16 columns, each cut by half of a last place, 2^-24.5 of it on average, at most: (n + 1) / 2 * 2^-24.5 of the
+# score less the 0.94e-8 n that are put back
+@pytest.mark.parametrize("d", [36, 64, 100, 128])
+@pytest.mark.parametrize("sign", [1, -1])
+def test_lse_of_scores_of_one_sign(d, sign):
+    q, k = sign * normal(1, 2, 12, 300, d).abs(), normal(2, 2, 12, 1500, d).abs()
+    lse, scores = forward_lse(q, k)
+    want, n = torch.logsumexp(scores, -1), (d + 15) // 16
+    size = float((torch.softmax(scores, -1) * scores.abs()).sum(-1).mean())
+    assert abs(float((lse - want).mean())) <= ((n + 1) / 2 * 2.0 ** -24.5 - 0.94e-8 * n) * size
