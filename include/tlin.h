@@ -69,7 +69,8 @@ int tlin_attn_forward_f32(const float* q, const float* k, const float* v, float*
 /* The same on the tensor cores, with numbers as sums of three bf16 parts and the accuracy of fp32 arithmetic: `scratch` is device
  * memory of tlin_scratch_bytes_forward_f32 bytes, 16-byte aligned, that the call alone uses until it has completed on `stream` (the
  * workspace is not touched).  At most 2 GiB; 0 bytes: the call is served better by the CUDA cores.  With less scratch, or NULL, it is served by them
- * too, and so it is where a tensor holds a number outside [2^-100, 2^30] in magnitude other than 0 (found on the device). */
+ * too, and so are the (b,h) in which a tensor holds a number outside [2^-100, 2^30] in magnitude other than 0, or a NaN that masked
+ * keys would let through (found on the device; all of the call where a result lies over an input of another (b,h)). */
 size_t tlin_scratch_bytes_forward_f32(int B, int H, int N, int W, int d, int causal_window);
 int tlin_attn_forward_f32_scratch(const float* q, const float* k, const float* v, float* out, float* lse,
                                   int B, int H, int N, int W, int d, int causal_window,

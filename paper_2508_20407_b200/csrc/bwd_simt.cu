@@ -83,9 +83,9 @@ template <typename T, int BT, int TC, int CM>
 __global__ void __launch_bounds__(kTR * TC, CM * TC <= 40 ? 3 : CM * TC <= 64 ? 2 : 1)
 bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const T* __restrict__ dout,
                 const float* __restrict__ lse, const float* __restrict__ delta, float* __restrict__ dq_acc, T* __restrict__ dk,
-                T* __restrict__ dv, int N, int W, int d, int causal, int64_t n_bh, float scale, const int* wanted) {
+                T* __restrict__ dv, int N, int W, int d, int causal, int64_t n_bh, float scale, const Heads heads) {
     after_previous();
-    if (wanted != nullptr && *wanted == 0) return;         // the tensor-core kernel before this one has computed the call
+    if (heads.any != nullptr && !heads.has(blockIdx.x % n_bh)) return;       // the tensor-core kernel before this one has computed it
     constexpr int NT = kTR * TC;
     constexpr int RI = BT / kTR, KJ = BT / TC, KA = BT / kTR;    // rows and keys of a thread's scores; keys of its dk / dv rows
     constexpr int LDP = ld_p<BT>();
@@ -205,10 +205,10 @@ bwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
 }
 
 template <typename T>
-__global__ void bwd_round_kernel(const float* __restrict__ src, T* __restrict__ dst, long long n, const int* wanted) {
-    if (wanted != nullptr && *wanted == 0) return;
+__global__ void bwd_round_kernel(const float* __restrict__ src, T* __restrict__ dst, long long n, long long per_bh, const Heads heads) {
+    if (heads.none()) return;
     const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < n) from_f(dst[x], src[x]);
+    if (x < n && heads.has(x / per_bh)) from_f(dst[x], src[x]);
 }
 
 // Where dq is summed.  fp32: straight in the result, unless the main kernel still reads an input there (dq written over q, say);
@@ -223,7 +223,7 @@ float* dq_sums(const void* q, const void* k, const void* v, const float* lse, co
 
 template <typename T, int BT, int TC, int CM>
 int launch_t(const T* q, const T* k, const T* v, const T* out, const float* lse, const T* dout, T* dq, T* dk, T* dv,
-             int B, int H, int N, int W, int d, int causal, float* ws, cudaStream_t st, const int* wanted) {
+             int B, int H, int N, int W, int d, int causal, float* ws, cudaStream_t st, const Heads& heads) {
     const int64_t n_bh = (int64_t)B * H, rows = n_bh * W;
     float* delta = ws;                                  // [B*H*W]
     float* dq_acc = dq_sums<T>(q, k, v, lse, dout, dq, n_bh, N, W, d, ws);
@@ -232,21 +232,21 @@ int launch_t(const T* q, const T* k, const T* v, const T* out, const float* lse,
     TLIN_CUDA_CHECK(allow_dynamic_smem(bwd_simt_kernel<T, BT, TC, CM>, (int)bwd_smem_bytes<BT>(TC * CM, column_slack<TC, CM>()), allowed));
     const int64_t ctas = n_bh * ((N + BT - 1) / BT);
     if (ctas > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
-    if (wanted == nullptr) {                            // else the tensor-core kernel has prepared both, if this call is to run
+    if (heads.any == nullptr) {                            // else the tensor-core kernels have prepared both for the heads that are to run
         bwd_delta_kernel<T><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(out, dout, delta, rows, d);
         TLIN_CUDA_CHECK(cudaGetLastError());
         count_launch();
         TLIN_CUDA_CHECK(cudaMemsetAsync(dq_acc, 0, (size_t)rows * d * sizeof(float), st));
         bwd_simt_kernel<T, BT, TC, CM><<<(unsigned)ctas, kTR * TC, bwd_smem_bytes<BT>(d, column_slack<TC, CM>()), st>>>(
-            q, k, v, dout, lse, delta, dq_acc, dk, dv, N, W, d, causal, n_bh, scale, nullptr);
+            q, k, v, dout, lse, delta, dq_acc, dk, dv, N, W, d, causal, n_bh, scale, heads);
         TLIN_CUDA_CHECK(cudaGetLastError());
     } else {
         TLIN_CUDA_CHECK(launch_overlapped(bwd_simt_kernel<T, BT, TC, CM>, (unsigned)ctas, kTR * TC, bwd_smem_bytes<BT>(d, column_slack<TC, CM>()), st,
-                                          q, k, v, dout, lse, (const float*)delta, dq_acc, dk, dv, N, W, d, causal, n_bh, scale, wanted));
+                                          q, k, v, dout, lse, (const float*)delta, dq_acc, dk, dv, N, W, d, causal, n_bh, scale, heads));
     }
     count_launch();
     if ((void*)dq_acc != (void*)dq) {
-        bwd_round_kernel<T><<<(unsigned)((rows * d + 255) / 256), 256, 0, st>>>(dq_acc, dq, rows * d, wanted);
+        bwd_round_kernel<T><<<(unsigned)((rows * d + 255) / 256), 256, 0, st>>>(dq_acc, dq, rows * d, (long long)W * d, heads);
         TLIN_CUDA_CHECK(cudaGetLastError());
         count_launch();
     }
@@ -255,15 +255,15 @@ int launch_t(const T* q, const T* k, const T* v, const T* out, const float* lse,
 
 template <typename T>
 int launch_any(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
-               void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, float* ws, cudaStream_t st, const int* wanted) {
+               void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, float* ws, cudaStream_t st, const Heads& heads) {
     if ((long long)B * H * W * d > (1LL << 40) || (long long)N > 0x7fffffffLL - 64) return TLIN_ERR_UNSUPPORTED;
     const T *qt = (const T*)q, *kt = (const T*)k, *vt = (const T*)v, *ot = (const T*)out, *dot = (const T*)dout;
     T *dqt = (T*)dq, *dkt = (T*)dk, *dvt = (T*)dv;
-    if (d <= 40) return launch_t<T, 64, 8, 5>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, wanted);
-    if (d <= 64) return launch_t<T, 64, 8, 8>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, wanted);
-    if (d <= 112) return launch_t<T, 64, 16, 7>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, wanted);
-    if (d <= 128) return launch_t<T, 64, 16, 8>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, wanted);
-    if (d <= 256) return launch_t<T, 32, 16, 16>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, wanted);
+    if (d <= 40) return launch_t<T, 64, 8, 5>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, heads);
+    if (d <= 64) return launch_t<T, 64, 8, 8>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, heads);
+    if (d <= 112) return launch_t<T, 64, 16, 7>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, heads);
+    if (d <= 128) return launch_t<T, 64, 16, 8>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, heads);
+    if (d <= 256) return launch_t<T, 32, 16, 16>(qt, kt, vt, ot, lse, dot, dqt, dkt, dvt, B, H, N, W, d, causal, ws, st, heads);
     return TLIN_ERR_UNSUPPORTED;
 }
 
@@ -286,9 +286,9 @@ size_t bwd_workspace_bytes(long long B, long long H, long long W, int d) {
 
 int launch_bwd_simt(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                     void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, int is_f32, float* ws,
-                    cudaStream_t st, const int* wanted) {
-    if (is_f32) return launch_any<float>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, st, wanted);
-    return launch_any<__nv_bfloat16>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, st, nullptr);
+                    cudaStream_t st, const Heads& heads) {
+    if (is_f32) return launch_any<float>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, st, heads);
+    return launch_any<__nv_bfloat16>(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal, ws, st, {});
 }
 
 }  // namespace tlin

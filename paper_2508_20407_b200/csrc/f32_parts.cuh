@@ -5,9 +5,10 @@
 //
 // The parts of the tensors are made by one pass over them (split_kernel) into scratch that the caller provides, [part][b h][row][d8]
 // with d8 = d rounded up to 8, which the tensor maps then read with zero fill beyond d8.  Numbers outside [2^-100, 2^30] other than 0
-// (infinities, what would lose its low parts or overflow on the way) are found there: such a call runs on the CUDA cores
-// instead, decided on the device.  The split kernel's blocks leave one word each, the tensor kernels read them and return at once
-// if any is set, and the CUDA-core kernels behind them return at once if none is.
+// (infinities, what would lose its low parts or overflow on the way) are found there: a (b,h) with such a number runs on the CUDA cores
+// instead, decided on the device.  The split kernel's blocks leave one word each, several blocks to a (b,h); the tensor kernels read the
+// words and pass the (b,h) by that have one set, and the CUDA-core kernel behind them computes those and returns at once if there
+// are none.
 #pragma once
 #include "tlin_internal.h"
 #include "sm100_ptx.cuh"
@@ -18,8 +19,7 @@ namespace f32 {
 
 constexpr int kParts = 3;
 constexpr int kSplitThreads = 256;
-constexpr int kMaxSplitBlocks = 4 * kDefaultSMs;
-constexpr int kFlagWords = kMaxSplitBlocks + 8;        // one per block, then the word that the CUDA-core kernels look at
+constexpr int kSplitBlocks = 6 * kDefaultSMs;          // up to; more (b,h) get one each
 // partial products in ascending size, so that the small ones are added while the sum is small: (part of A, part of B)
 __host__ __device__ constexpr int product_a(int i) { return i == 0 ? 0 : i == 1 ? 1 : i == 2 ? 2 : i == 3 ? 0 : i == 4 ? 1 : 0; }
 __host__ __device__ constexpr int product_b(int i) { return i == 0 ? 2 : i == 1 ? 1 : i == 3 ? 1 : 0; }
@@ -28,21 +28,28 @@ constexpr int kProducts = 6;
 inline long long padded_head(int d) { return ((long long)d + 7) / 8 * 8; }
 inline int padded_rows(int W) { return (W + 127) / 128 * 128; }
 
-// What the split kernel makes: the parts of up to four tensors of n_bh blocks of rows, and for the backward the row statistics.
+// What the split kernel makes: the parts of up to four tensors of n_bh (b,h), and for the backward the row statistics.
 struct SplitJobs {
     const float* src[4];
     __nv_bfloat16* dst[4];
-    long long rows[4];            // of all (b,h)
-    int n, d, blocks;
+    int rows[4];                  // per (b,h)
+    int n, d;
+    long long n_bh;
+    int per_bh;                   // blocks
     int nan_too;                  // bit t: a NaN in tensor t is one of the numbers that the parts do not hold
-    int* flags;                   // one per block
+    int* words;                   // one per block
     const float *out, *dout, *lse;
     float *neg_lse, *delta;       // [n_bh][Wpad]: -lse (beyond W: -inf) and out . dout (beyond W: 0); null in the forward
+    float* plain_delta;           // [n_bh][W]: the same as the CUDA-core kernel sums and reads it
     int W, Wpad;
-    long long rows_padded;
-    float* zero;                  // zero_n floats to clear (a multiple of 4), or null
-    long long zero_n;
+    float* zero;                  // [n_bh][W][d] to clear, or null
 };
+// Blocks per (b,h), with `groups` groups of eight numbers each.  An even number: B8 H12 N1024 W512 d36 backward, with 6, 8 or 10 of them
+// 275 us, with 7 or 9 285, of which the split itself is 1 to 3.
+inline int split_blocks(long long n_bh, long long groups) {
+    const long long share = kSplitBlocks / n_bh < 2 ? kSplitBlocks / n_bh : kSplitBlocks / n_bh / 2 * 2, most = (groups + kSplitThreads - 1) / kSplitThreads;
+    return (int)(share < 1 ? 1 : share < most ? share : most);
+}
 int launch_split(const SplitJobs& jobs, cudaStream_t st);
 // No call takes more scratch than this, which an allocator keeps once it has been asked for it.  Few query tiles over long histories are
 // what would: forward, unbounded / 2 GiB / 1 GiB / on the CUDA cores, microseconds: B1 H32 N131072 W128 d128 (6.0 GiB) 3500 / 4890 / 7170 /

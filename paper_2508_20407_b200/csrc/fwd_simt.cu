@@ -39,10 +39,10 @@ __host__ __device__ constexpr size_t smem_floats(int d, int slack) {
 template <typename T, int ROWS, int CM>
 __global__ void __launch_bounds__(kNT, CM * ROWS <= 40 ? 3 : 2)
 fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ out, float* __restrict__ lse,
-                int N, int W, int d, int causal, int q_tiles, int64_t n_bh, int cluster, float scale, int64_t kv_rows, const int* wanted) {
+                int N, int W, int d, int causal, int q_tiles, int64_t n_bh, int cluster, float scale, int64_t kv_rows, const Heads heads) {
     constexpr int BM = kTR * ROWS;
     after_previous();
-    if (wanted != nullptr && *wanted == 0) return;         // the tensor-core kernel before this one has computed the call
+    if (heads.none()) return;                              // the tensor-core kernel before this one has computed the call
     extern __shared__ __align__(16) float smem[];
     const int ld = row_stride(d);
     float* Qs = smem;                           // [BM][ld]
@@ -56,6 +56,7 @@ fwd_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
     const int rank = (int)(blockIdx.x - item * cluster);
     const int qt = q_tiles - 1 - (int)(item / n_bh);
     const int64_t bh = item % n_bh;
+    if (!heads.has(bh)) return;                            // the same for all CTAs of a cluster
     const int row0 = qt * BM;
     const T* kb = k + bh * kv_rows * d;         // kv_rows >= N: rows per (b,h) of the key/value allocation
     const T* vb = v + bh * kv_rows * d;
@@ -211,7 +212,7 @@ int cluster_size(int64_t items, int N) {
 
 template <typename T, int ROWS, int CM>
 int launch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H, int N, int W, int d,
-           int causal, long long kv_rows_alloc, cudaStream_t st, const int* wanted) {
+           int causal, long long kv_rows_alloc, cudaStream_t st, const Heads& heads) {
     constexpr int BM = kTR * ROWS;
     const int q_tiles = (W + BM - 1) / BM;
     const int64_t n_bh = (int64_t)B * H, items = n_bh * q_tiles;
@@ -232,9 +233,9 @@ int launch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H,
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = wanted != nullptr ? 2 : 1;
+    cfg.numAttrs = heads.any != nullptr ? 2 : 1;
     TLIN_CUDA_CHECK(cudaLaunchKernelEx(&cfg, fwd_simt_kernel<T, ROWS, CM>, q, k, v, out, lse, N, W, d, causal, q_tiles, n_bh, cluster,
-                                       1.0f / sqrtf((float)d), kv_rows_alloc > 0 ? (int64_t)kv_rows_alloc : (int64_t)N, wanted));
+                                       1.0f / sqrtf((float)d), kv_rows_alloc > 0 ? (int64_t)kv_rows_alloc : (int64_t)N, heads));
     count_launch();
     return TLIN_OK;
 }
@@ -261,7 +262,8 @@ __device__ __forceinline__ float warp_sum(float x) {
 template <typename T>
 __global__ void __launch_bounds__(kWarpRows * 32)
 fwd_row_per_warp_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ out, float* __restrict__ lse,
-                        int N, int W, int d, int causal, int q_tiles, float scale, int64_t kv_rows) {
+                        int N, int W, int d, int causal, int q_tiles, float scale, int64_t kv_rows, const Heads heads) {
+    if (!heads.has(blockIdx.x / q_tiles)) return;
     extern __shared__ __align__(16) float smem[];
     const int kstride = d + 4;                 // padded: lanes reading different rows hit different banks
     float* Qs = smem;                          // [kWarpRows][d]
@@ -345,7 +347,7 @@ fwd_row_per_warp_kernel(const T* __restrict__ q, const T* __restrict__ k, const 
 
 template <typename T>
 int launch_row_per_warp(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H, int N, int W, int d,
-                        int causal, long long kv_rows_alloc, cudaStream_t st) {
+                        int causal, long long kv_rows_alloc, cudaStream_t st, const Heads& heads) {
     const int q_tiles = (W + kWarpRows - 1) / kWarpRows;
     const int64_t ctas = (int64_t)B * H * q_tiles;
     if (ctas > 0x7fffffffLL) return TLIN_ERR_UNSUPPORTED;
@@ -353,7 +355,7 @@ int launch_row_per_warp(const T* q, const T* k, const T* v, T* out, float* lse, 
     static bool allowed[64] = {};
     TLIN_CUDA_CHECK(allow_dynamic_smem(fwd_row_per_warp_kernel<T>, smem_bytes(32 * kWarpColumns), allowed));
     fwd_row_per_warp_kernel<T><<<(unsigned)ctas, kWarpRows * 32, smem_bytes(d), st>>>(q, k, v, out, lse, N, W, d, causal, q_tiles, 1.0f / sqrtf((float)d),
-                                                                                 kv_rows_alloc > 0 ? (int64_t)kv_rows_alloc : (int64_t)N);
+                                                                                 kv_rows_alloc > 0 ? (int64_t)kv_rows_alloc : (int64_t)N, heads);
     TLIN_CUDA_CHECK(cudaGetLastError());
     count_launch();
     return TLIN_OK;
@@ -388,20 +390,20 @@ bool rows_are_cheaper(int64_t n_bh, int N, int W, int d, int tile_rows, int64_t 
 int tile_rows_of(int64_t n_bh, int W, int d) { return d > 40 && d <= 64 && W > 64 && n_bh * ((W + 127) / 128) >= kDefaultSMs * 3 / 4 ? 128 : 64; }
 template <typename T>
 int dispatch(const T* q, const T* k, const T* v, T* out, float* lse, int B, int H, int N, int W, int d,
-             int causal, long long kv, cudaStream_t st, const int* wanted = nullptr) {
+             int causal, long long kv, cudaStream_t st, const Heads& heads = {}) {
     const int64_t n_bh = (int64_t)B * H;
     const int tile_rows = tile_rows_of(n_bh, W, d);
     const int64_t items = n_bh * ((W + tile_rows - 1) / tile_rows);
-    if (wanted == nullptr && rows_are_cheaper(n_bh, N, W, d, tile_rows, items, cluster_size(items, N)))
-        return launch_row_per_warp<T>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st);
+    if (rows_are_cheaper(n_bh, N, W, d, tile_rows, items, cluster_size(items, N)))
+        return launch_row_per_warp<T>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
     if (tile_rows == 128)
-        return launch<T, 8, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, wanted);
-    if (d <= 40) return launch<T, 4, 5>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, wanted);
-    if (d <= 64) return launch<T, 4, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, wanted);
-    if (d <= 104) return launch<T, 4, 13>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, wanted);
-    if (d <= 128) return launch<T, 4, 16>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, wanted);
-    if (d <= 192) return launch<T, 4, 24>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, wanted);
-    return launch<T, 4, 32>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, wanted);
+        return launch<T, 8, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
+    if (d <= 40) return launch<T, 4, 5>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
+    if (d <= 64) return launch<T, 4, 8>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
+    if (d <= 104) return launch<T, 4, 13>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
+    if (d <= 128) return launch<T, 4, 16>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
+    if (d <= 192) return launch<T, 4, 24>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
+    return launch<T, 4, 32>(q, k, v, out, lse, B, H, N, W, d, causal, kv, st, heads);
 }
 
 }  // namespace
@@ -424,8 +426,8 @@ int launch_fwd_simt_bf16(const void* q, const void* k, const void* v, void* out,
                                    (__nv_bfloat16*)out, lse, B, H, N, W, d, causal, kv_rows_alloc, st);
 }
 int launch_fwd_simt_f32(const float* q, const float* k, const float* v, float* out, float* lse,
-                        int B, int H, int N, int W, int d, int causal, long long kv_rows_alloc, cudaStream_t st, const int* wanted) {
-    return dispatch<float>(q, k, v, out, lse, B, H, N, W, d, causal, kv_rows_alloc, st, wanted);
+                        int B, int H, int N, int W, int d, int causal, long long kv_rows_alloc, cudaStream_t st, const Heads& heads) {
+    return dispatch<float>(q, k, v, out, lse, B, H, N, W, d, causal, kv_rows_alloc, st, heads);
 }
 
 }  // namespace tlin

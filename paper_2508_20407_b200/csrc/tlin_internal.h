@@ -163,12 +163,34 @@ inline bool overlap(const void* a, int64_t a_bytes, const void* b, int64_t b_byt
     return x < y + (uint64_t)b_bytes && y < x + (uint64_t)a_bytes;
 }
 
+// The (b,h) of a call that the CUDA-core kernels are to compute after the tensor cores, found on the device: with `any` null all of them;
+// otherwise none while *any is 0, else all (`all`) or those that have one of their per_bh words set.
+struct Heads {
+    const int* any = nullptr;
+    const int* words = nullptr;
+    int per_bh = 0, all = 0;
+#ifdef __CUDACC__
+    __device__ __forceinline__ bool none() const { return any != nullptr && *any == 0; }
+    __device__ __forceinline__ bool special(long long bh) const {
+        bool found = all != 0;
+        const int* w = words + bh * per_bh;
+#pragma unroll 1
+        for (int i = 0; i < per_bh && !found; ++i) found = w[i] != 0;
+        return found;
+    }
+    __device__ __forceinline__ bool has(long long bh) const { return any == nullptr || (*any != 0 && special(bh)); }
+#endif
+};
+// results over an input otherwise than one (b,h) over the same (b,h) of a tensor of the same size
+inline bool crosses(const void* to, int64_t to_bytes, const void* from, int64_t from_bytes) {
+    return overlap(to, to_bytes, from, from_bytes) && !(to == from && to_bytes == from_bytes);
+}
+
 // ---- launchers (one per kernel family); all validate nothing: api.cu has done it ----------
 int launch_fwd_simt_bf16(const void* q, const void* k, const void* v, void* out, float* lse,
                          int B, int H, int N, int W, int d, int causal, long long kv_rows_alloc, cudaStream_t st);
 int launch_fwd_simt_f32(const float* q, const float* k, const float* v, float* out, float* lse,
-                        int B, int H, int N, int W, int d, int causal, long long kv_rows_alloc, cudaStream_t st,
-                        const int* wanted = nullptr);    // device word: 0 and the kernel returns at once
+                        int B, int H, int N, int W, int d, int causal, long long kv_rows_alloc, cudaStream_t st, const Heads& heads = {});
 double fwd_simt_us(long long n_bh, int N, int W, int d, int causal);
 // fp32 on the tensor cores (fwd_f32_tc.cu, bwd_f32_tc.cu): whether a call is better served there, its scratch, and the call.  It returns
 // TLIN_ERR_UNSUPPORTED, with nothing launched, for several launches whose results lie over inputs.
@@ -193,7 +215,7 @@ int launch_decode(const void* q_new, const void* k_new, const void* v_new, void*
                   bool two_kernels = false);   // two_kernels: short steps as well (decode.cu, tlin_decode_step_static)
 int launch_bwd_simt(const void* q, const void* k, const void* v, const void* out, const float* lse, const void* dout,
                     void* dq, void* dk, void* dv, int B, int H, int N, int W, int d, int causal, int is_f32, float* ws,
-                    cudaStream_t st, const int* wanted = nullptr);       // as for the forward; delta and cleared sums are then in place
+                    cudaStream_t st, const Heads& heads = {});           // some heads only: delta and their cleared sums are in place
 // where that kernel sums dq of an fp32 call: dq itself, or behind delta in ws
 float* bwd_simt_sums(const float* q, const float* k, const float* v, const float* lse, const float* dout, float* dq, long long n_bh, int N, int W, int d, float* ws);
 double bwd_simt_us(long long n_bh, int N, int W, int d, int causal);

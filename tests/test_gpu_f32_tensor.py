@@ -74,23 +74,99 @@ def test_as_exact_as_the_cuda_cores(B, H, N, W, d, causal):
         assert float((a - x).norm()) <= max(1.2 * float((b - x).norm()), 4 * 2.0 ** -24 * size)
 
 
+def forward(q, k, v, causal, with_scratch=True, out=None):
+    """(out, lse) of the C entry point: on the tensor cores, which the sizes have to be for, or without scratch on the CUDA cores."""
+    (B, H, W, d), N, lib = q.shape, k.shape[2], tl.lib()
+    need = lib.tlin_scratch_bytes_forward_f32(B, H, N, W, d, causal) if with_scratch else 0
+    assert not with_scratch or need
+    s, out, lse = scratch(need), torch.empty_like(q) if out is None else out, torch.empty(B, H, W, device=DEV)
+    assert lib.tlin_attn_forward_f32_scratch(*pointers(q, k, v, out, lse), B, H, N, W, d, causal, s.data_ptr() if need else None, need,
+                                             torch.cuda.current_stream().cuda_stream) == 0
+    return out, lse
+
+
+def backward(q, k, v, out, lse, dout, causal, with_scratch=True, grads=None):
+    (B, H, W, d), N, lib = q.shape, k.shape[2], tl.lib()
+    tl.ensure_workspace(tl.workspace_bytes_backward(B, H, N, W, d))
+    need = lib.tlin_scratch_bytes_backward_f32(B, H, N, W, d, causal) if with_scratch else 0
+    assert not with_scratch or need
+    s, grads = scratch(need), [torch.empty_like(t) for t in (q, k, v)] if grads is None else grads
+    assert lib.tlin_attn_backward_f32_scratch(*pointers(q, k, v, out, lse, dout, *grads), B, H, N, W, d, causal, s.data_ptr() if need else None, need,
+                                              torch.cuda.current_stream().cuda_stream) == 0
+    return grads
+
+
+def same(a, b):
+    return torch.equal(a.isnan(), b.isnan()) and torch.equal(a.nan_to_num(), b.nan_to_num())
+
+
+def check_that_one_head_goes_to_the_cuda_cores(t, what, head, value, causal=1, in_place=False):
+    """`value` in one (b,h) of t[what]: that one as the CUDA cores compute it, all others as without it, bit for bit.  dq of more than one
+    addition in any order (the CUDA cores', and the tensor cores' over more than 1536 keys) to the rounding of its sums."""
+    clean = forward(t["q"], t["k"], t["v"], causal)
+    clean_grads = backward(t["q"], t["k"], t["v"], *clean, t["dout"], causal)
+    t = dict(t)
+    t[what] = t[what].clone()
+    t[what][head][min(17, t[what].shape[2] - 1), 3] = value
+    q, k, v, dout = (t[x] for x in ("q", "k", "v", "dout"))
+    others = torch.ones(q.shape[:2], dtype=torch.bool, device=DEV)
+    others[head] = False
+    got, cores = forward(q, k, v, causal, out=q.clone() if in_place else None), forward(q, k, v, causal, False)
+    if in_place:
+        over = q.clone()
+        assert all(same(x, y) for x, y in zip(forward(over, k, v, causal, out=over), got))
+    for x, y, z in zip(got, cores, clean):
+        assert torch.equal(x[others], z[others])
+        assert same(x[head], y[head]) if what != "dout" else torch.equal(x, z)
+    cores_grads = backward(q, k, v, *got, dout, causal, False)
+    if in_place:
+        over = [q.clone(), k.clone(), v.clone()]
+        grads = backward(*over, *got, dout, causal, grads=over)
+    else:
+        grads = backward(q, k, v, *got, dout, causal)
+    for x, y, z, name in zip(grads, cores_grads, clean_grads, ("dq", "dk", "dv")):
+        if name == "dq":
+            ok = torch.isfinite(y[head])
+            assert torch.equal(torch.isfinite(x[head]), ok)
+            if not (what in ("q", "k") and abs(value) > 1):           # one key takes all there: ds is 0, and its rounding is multiplied by the value
+                assert float((x[head] - y[head])[ok].double().norm()) <= 1e-6 * float(y[head][ok].double().norm())
+        else:
+            assert same(x[head], y[head])
+        if name == "dq" and k.shape[2] > 1536:
+            assert float((x[others] - z[others]).double().norm()) <= 1e-6 * float(z[others].double().norm())
+        else:
+            assert torch.equal(x[others], z[others])
+    assert tl.tlin_get_status() == 0
+
+
+def tensors(B, H, N, W, d):
+    return dict(q=normal(1, B, H, W, d), dout=normal(2, B, H, W, d), k=normal(3, B, H, N, d), v=normal(4, B, H, N, d))
+
+
 @pytest.mark.parametrize("what", ["q", "k", "v", "dout"])
 @pytest.mark.parametrize("value", [math.inf, -3e38, 1e-35, 2e9])
 def test_numbers_that_the_parts_do_not_hold_go_to_the_cuda_cores(what, value):
-    B, H, N, W, d = 2, 16, 500, 300, 36
-    t = dict(q=normal(1, B, H, W, d), dout=normal(2, B, H, W, d), k=normal(3, B, H, N, d), v=normal(4, B, H, N, d))
-    t[what][1, 3, 17, 5] = value
-    (got, fwd, bwd), (ref, _, _) = both_sides(t["q"], t["k"], t["v"], t["dout"], 1)
-    assert fwd and bwd
-    for name, a, b in zip(("out", "lse", "dq", "dk", "dv"), got, ref):
-        if what != "dout" and name in ("out", "lse"):
-            assert torch.equal(a.isnan(), b.isnan()) and torch.equal(a.nan_to_num(), b.nan_to_num())
-        # sums of additions in any order (dq), and with dout alone outside, over another forward's out and lse
-        ok = torch.isfinite(b) & torch.isfinite(a)
-        assert torch.equal(torch.isfinite(a), torch.isfinite(b))
-        if what in ("q", "k") and abs(value) > 1 and name in ("dq", "dk"):
-            continue                              # one key takes all: their exact ds is 0, and its rounding is multiplied by the value
-        assert float((a.double() - b.double())[ok].norm()) <= 1e-5 * float(b[ok].double().norm())
+    check_that_one_head_goes_to_the_cuda_cores(tensors(2, 16, 500, 300, 36), what, (1, 3), value)
+
+
+# keys shared in a cluster (forward) and dq in several pieces; several pieces without clusters; several launches, the head in the last and in
+# the first; results over inputs
+@pytest.mark.parametrize("B,H,N,W,d,head,in_place", [(1, 3, 3000, 200, 64, (0, 1), False), (1, 40, 2100, 640, 36, (0, 39), False), (2, 160, 2000, 300, 64, (1, 159), False),
+                                                     (2, 160, 2000, 300, 64, (0, 0), False), (2, 16, 500, 500, 36, (1, 3), True), (1, 3, 3000, 200, 64, (0, 2), True)])
+@pytest.mark.parametrize("what,value", [("v", math.nan), ("k", math.inf)])
+def test_one_head_on_the_cuda_cores_in_every_form(B, H, N, W, d, head, in_place, what, value):
+    check_that_one_head_goes_to_the_cuda_cores(tensors(B, H, N, W, d), what, head, value, in_place=in_place)
+
+
+def test_one_head_on_one_warp_per_row():
+    """A call that the CUDA cores compute with the kernel of one warp per row, when they compute all of it."""
+    q, k, v = (normal(i, 1, 1000, rows, 128) for i, rows in enumerate((19, 27, 27)))
+    clean = forward(q, k, v, 1)
+    v[0, 501, 20, 7] = math.nan
+    got, cores = forward(q, k, v, 1), forward(q, k, v, 1, False)
+    for x, y, z in zip(got, cores, clean):
+        assert same(x[0, 501], y[0, 501]) and torch.equal(x[0, :501], z[0, :501]) and torch.equal(x[0, 502:], z[0, 502:])
+    assert tl.tlin_get_status() == 0
 
 
 def test_results_over_inputs_and_too_little_scratch():
