@@ -263,8 +263,9 @@ int tlin_attn_backward_f32(const float* q, const float* k, const float* v, const
                            const float* dout, float* dq, float* dk, float* dv,
                            int B, int H, int N, int W, int d, int causal_window, tlin_stream_t stream);
 
-/* The same on the tensor cores for d up to 64, as tlin_attn_forward_f32_scratch.  Where the CUDA cores serve the call for want of
- * scratch, they use the workspace. */
+/* The same on the tensor cores for d up to 64, as tlin_attn_forward_f32_scratch (dout: up to 2^20 in magnitude).  Where the CUDA cores serve
+ * the call for want of scratch, or because its scratch holds less than the whole call and a result lies over an input, they use the
+ * workspace.  dq of more than 1536 keys is summed in any order, and so does not repeat bit for bit. */
 size_t tlin_scratch_bytes_backward_f32(int B, int H, int N, int W, int d, int causal_window);
 int tlin_attn_backward_f32_scratch(const float* q, const float* k, const float* v, const float* out, const float* lse,
                                    const float* dout, float* dq, float* dk, float* dv,

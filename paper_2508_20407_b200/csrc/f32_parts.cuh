@@ -4,7 +4,7 @@
 // TFLOP/s nominal where the CUDA cores have 72.
 //
 // The parts of the tensors are made by one pass over them (split_kernel) into scratch that the caller provides, [part][b h][row][d8]
-// with d8 = d rounded up to 8, which the tensor maps then read with zero fill beyond d8.  Numbers outside [2^-100, 2^30] other than 0
+// with d8 = d rounded up to 8, which the tensor maps then read with zero fill beyond d8.  Numbers outside [2^-100, 2^30] (dout: 2^20) other than 0
 // (infinities, what would lose its low parts or overflow on the way) are found there: a (b,h) with such a number runs on the CUDA cores
 // instead, decided on the device.  The split kernel's blocks leave one word each, several blocks to a (b,h); the tensor kernels read the
 // words and pass the (b,h) by that have one set, and the CUDA-core kernel behind them computes those and returns at once if there
@@ -24,11 +24,17 @@ constexpr int kSplitBlocks = 6 * kDefaultSMs;          // up to; more (b,h) get 
 __host__ __device__ constexpr int product_a(int i) { return i == 0 ? 0 : i == 1 ? 1 : i == 2 ? 2 : i == 3 ? 0 : i == 4 ? 1 : 0; }
 __host__ __device__ constexpr int product_b(int i) { return i == 0 ? 2 : i == 1 ? 1 : i == 3 ? 1 : 0; }
 constexpr int kProducts = 6;
+// ds is split into parts too, and a bf16 part below 2^-133 is lost.  The backward therefore runs on 2^19 dout (exactly that times the
+// gradients), which dout up to 2^20 leaves room for: 64 * 2^39 * 2^30 = 2^75 in dp, 2^106 in a product with q or k.  Relative error of
+// dk, dout 2^-90 and v 2^-20 times normal: without 9.1e-6, so 3.4e-7.
+constexpr float kDoutScale = 524288.f;
 
 inline long long padded_head(int d) { return ((long long)d + 7) / 8 * 8; }
 inline int padded_rows(int W) { return (W + 127) / 128 * 128; }
 
-// What the split kernel makes: the parts of up to four tensors of n_bh (b,h), and for the backward the row statistics.
+// What the split kernel makes: the parts of up to four tensors of n_bh (b,h), and for the backward (kDoutTensor is dout there, its parts of
+// kDoutScale times it) the row statistics.
+constexpr int kDoutTensor = 1;
 struct SplitJobs {
     const float* src[4];
     __nv_bfloat16* dst[4];
@@ -39,8 +45,8 @@ struct SplitJobs {
     int nan_too;                  // bit t: a NaN in tensor t is one of the numbers that the parts do not hold
     int* words;                   // one per block
     const float *out, *dout, *lse;
-    float *neg_lse, *delta;       // [n_bh][Wpad]: -lse (beyond W: -inf) and out . dout (beyond W: 0); null in the forward
-    float* plain_delta;           // [n_bh][W]: the same as the CUDA-core kernel sums and reads it
+    float *neg_lse, *delta;       // [n_bh][Wpad]: -lse (beyond W: -inf) and kDoutScale out . dout (beyond W: 0); null in the forward
+    float* plain_delta;           // [n_bh][W]: out . dout as the CUDA-core kernel sums and reads it
     int W, Wpad;
     float* zero;                  // [n_bh][W][d] to clear, or null
 };

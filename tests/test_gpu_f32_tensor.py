@@ -255,3 +255,18 @@ def test_lse_of_scores_of_one_sign(d, sign):
     want, n = torch.logsumexp(scores, -1), (d + 15) // 16
     size = float((torch.softmax(scores, -1) * scores.abs()).sum(-1).mean())
     assert abs(float((lse - want).mean())) <= ((n + 1) / 2 * 2.0 ** -24.5 - 0.94e-8 * n) * size
+
+
+# ds is split into parts as well: gradients of the same accuracy wherever dout and v lie inside the range, here with products down to 2^-116
+# (fp32 itself has less than 24 bits left below 2^-126).  dq of the CUDA cores is no measure there: their additions in memory flush to zero
+@pytest.mark.parametrize("of_dout,of_v", [(-96, -20), (-90, -20), (-60, -50), (-96, 0), (19, 28), (0, 0)])
+def test_gradients_at_the_ends_of_the_range(of_dout, of_v):
+    B, H, N, W, d = 2, 12, 1500, 300, 36
+    q, k, v, dout = normal(1, B, H, W, d), normal(2, B, H, N, d), normal(3, B, H, N, d), normal(4, B, H, W, d)
+    v, dout = (t.sign() * t.abs().clamp(0.25, 2.0) * 2.0 ** e for t, e in ((v, of_v), (dout, of_dout - 1)))
+    out, lse = forward(q, k, v, 1)
+    got, cores = backward(q, k, v, out, lse, dout, 1), backward(q, k, v, out, lse, dout, 1, False)
+    for x, a, b in zip(exact(q, k, v, dout, 1)[2:], got, cores):
+        size = float(x.norm())
+        assert float((a - x).norm()) <= max(min(1.2 * float((b - x).norm()), 2.0 ** -20 * size), 4 * 2.0 ** -24 * size)
+    assert tl.tlin_get_status() == 0
