@@ -69,7 +69,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-o", FASTCALL, source,
                "-I" + os.path.join(torch_dir, "include"), "-I" + os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
                "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"], "-L" + os.path.join(torch_dir, "lib"),
-               "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lc10", "-lc10_cuda", "-L" + HERE, "-l:libtlin.so",
+               "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lc10", "-lc10_cuda", "-L" + os.path.join(cuda, "lib64"), "-lcudart", "-L" + HERE, "-l:libtlin.so",
                "-Wl,-rpath,$ORIGIN"]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:

@@ -5,6 +5,8 @@
 #include <torch/csrc/utils/pybind.h>
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAGraphsC10Utils.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <optional>
@@ -55,13 +57,25 @@ int without_gil(F&& f) {                 // called with the lock held (from Pyth
 }
 using Result = std::tuple<int, Tensor, Tensor>;
 
+// Whether `t` lies in memory that a graph's capture keeps for it (or in another pool of its own): what PyTorch allocates under its own
+// captures.
+bool in_a_pool(const Tensor& t) {
+    const size_t at = (size_t)t.data_ptr();
+    for (const auto& s : c10::cuda::CUDACachingAllocator::snapshot({0, 0}, false).segments)
+        if (s.device == t.device().index() && at >= s.address && at < s.address + s.total_size)
+            return s.owner_private_pool_id != c10::MempoolId_t{0, 0};
+    return false;
+}
 // Scratch of one call, from PyTorch's allocator on the call's stream: its memory is not given out again before the call is over there.
-// Undefined where none is wanted or there is no memory for it.
+// Undefined where none is wanted or there is no memory for it, and under a capture that PyTorch does not know of (cudaStreamBeginCapture
+// by the caller): there the memory would be given out again while the graph still writes to it at every launch.
 Tensor scratch_for(size_t bytes, const Tensor& like, tlin_stream_t st) {
     if (bytes == 0) return Tensor();
     try {
         const c10::cuda::CUDAStreamGuard guard(c10::cuda::getStreamFromExternal((cudaStream_t)st, like.device().index()));
-        return at::detail::empty_cuda({(int64_t)bytes}, at::kByte, like.device(), std::nullopt);
+        const Tensor t = at::detail::empty_cuda({(int64_t)bytes}, at::kByte, like.device(), std::nullopt);
+        if (c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None && !in_a_pool(t)) return Tensor();
+        return t;
     } catch (const c10::OutOfMemoryError&) {
         return Tensor();
     }

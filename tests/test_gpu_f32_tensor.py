@@ -1,5 +1,6 @@
 """fp32 calls on the tensor cores, three bf16 parts per number: sizes at the edges of their tiles, results against 64-bit sums, and the
 numbers that the parts do not hold."""
+import ctypes
 import math
 
 import pytest
@@ -269,4 +270,63 @@ def test_gradients_at_the_ends_of_the_range(of_dout, of_v):
     for x, a, b in zip(exact(q, k, v, dout, 1)[2:], got, cores):
         size = float(x.norm())
         assert float((a - x).norm()) <= max(min(1.2 * float((b - x).norm()), 2.0 ** -20 * size), 4 * 2.0 ** -24 * size)
+    assert tl.tlin_get_status() == 0
+
+
+def test_replay_of_a_capture():
+    """PyTorch's captures keep the scratch for the graph: the tensor cores serve the call there too."""
+    t = tensors(2, 16, 500, 300, 36)
+    other = {x: normal(7 + i, *t[x].shape) for i, x in enumerate(t)}
+
+    def call():
+        out, lse = tl.tlin_attn_forward_f32(t["q"], t["k"], t["v"])
+        return [out, lse] + list(tl.tlin_attn_backward_f32(t["q"], t["k"], t["v"], out, lse, t["dout"]))
+
+    call()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        recorded = call()
+    for values in (other, tensors(2, 16, 500, 300, 36)):
+        for x in t:
+            t[x].copy_(values[x])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(recorded, call()))
+    assert tl.tlin_get_status() == 0
+
+
+def test_a_capture_that_pytorch_does_not_know_of_takes_no_scratch():
+    """Its memory would be given out again while the graph still writes to it: the call is recorded on the CUDA cores."""
+    rt = ctypes.CDLL("libcudart.so.12")
+    t = tensors(2, 16, 500, 300, 36)
+    q, k, v, dout = (t[x] for x in ("q", "k", "v", "dout"))
+    stream = torch.cuda.Stream()
+    out, lse, grads = torch.empty_like(q), torch.empty(2, 16, 300, device=DEV), [torch.empty_like(x) for x in (q, k, v)]
+    need = max(tl.lib().tlin_scratch_bytes_forward_f32(2, 16, 500, 300, 36, 1), tl.lib().tlin_scratch_bytes_backward_f32(2, 16, 500, 300, 36, 1))
+
+    def call():
+        tl.tlin_attn_forward_f32(q, k, v, out, lse, stream=stream)
+        tl.tlin_attn_backward_f32(q, k, v, out, lse, dout, *grads, stream=stream)
+
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        call()
+        torch.cuda.synchronize()
+        handle, graph, run = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_void_p()
+        assert rt.cudaStreamBeginCapture(handle, 1) == 0              # of this thread
+        call()
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) == 0
+        assert rt.cudaGraphInstantiate(ctypes.byref(run), graph, ctypes.c_ulonglong(0)) == 0
+        taken = [torch.zeros(need, dtype=torch.uint8, device=DEV) for _ in range(4)]        # what the warm call's scratch left
+        for x in [out, lse] + grads:
+            x.zero_()
+        assert rt.cudaGraphLaunch(run, handle) == 0
+        torch.cuda.synchronize()
+    assert rt.cudaGraphExecDestroy(run) == 0 and rt.cudaGraphDestroy(graph) == 0
+    assert not any(bool(x.any()) for x in taken)
+    want = forward(q, k, v, 1, False)
+    assert torch.equal(out, want[0]) and torch.equal(lse, want[1])
+    want = backward(q, k, v, *want, dout, 1, False)
+    assert torch.equal(grads[1], want[1]) and torch.equal(grads[2], want[2])
+    assert float((grads[0] - want[0]).double().norm()) <= 1e-6 * float(want[0].double().norm())
     assert tl.tlin_get_status() == 0
