@@ -60,6 +60,9 @@ void log_decode_plan(const char* what, int B, int H, int Ncap, int pos, int d, c
     fprintf(stderr, "libtlin: %s B=%d H=%d Ncap=%d pos=%d d=%d -> %d splits of %d keys, %d in all, workspace %lld bytes\n",
             what, B, H, Ncap, pos, d, p.splits, p.keys_per_split, p.n_ctas, (long long)p.workspace_bytes);
 }
+void log_bwd(const char* what, int B, int H, int N, int W, int d, int causal, const char* how, size_t bytes) {
+    fprintf(stderr, "libtlin: backward %sB=%d H=%d N=%d W=%d d=%d causal_window=%d -> %s %lld bytes\n", what, B, H, N, W, d, causal, how, (long long)bytes);
+}
 }  // namespace
 
 // Index of the current device in the per-device tables; 0 where no device can be asked (registering a workspace is
@@ -315,6 +318,7 @@ static int backward_common(const void* q, const void* k, const void* v, const vo
         const size_t need = tlin_scratch_bytes_backward_f32(B, H, N, W, d, causal_window);
         if (need > 0 && scratch_bytes >= need) {
             if (!aligned16(scratch)) return TLIN_ERR_INVALID_ARG;
+            if (log_plans()) log_bwd("(fp32) ", B, H, N, W, d, causal_window, "tensor cores, three bf16 parts, scratch", need);
             rc = launch_bwd_f32_tc((const float*)q, (const float*)k, (const float*)v, (const float*)out, lse, (const float*)dout, (float*)dq, (float*)dk,
                                    (float*)dv, B, H, N, W, d, causal_window, scratch, sms, st);
             if (rc != TLIN_ERR_UNSUPPORTED) return rc;
@@ -324,10 +328,12 @@ static int backward_common(const void* q, const void* k, const void* v, const vo
     const bool tc = !is_f32 && (d == 64 || d == 128) && forward_impl() != 1;
     if (!tc) {
         if (!w.ptr || w.bytes < bwd_workspace_bytes(B, H, W, d)) return TLIN_ERR_WORKSPACE;
+        if (log_plans()) log_bwd(is_f32 ? "(fp32) " : "", B, H, N, W, d, causal_window, "CUDA cores, workspace", bwd_workspace_bytes(B, H, W, d));
         return launch_bwd_simt(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal_window, is_f32, (float*)w.ptr, st);
     }
     if (tlin_backward_arrangement(B, H, N, W, d) == 2) {
         if (!w.ptr || w.bytes < bwd_fused_workspace_bytes(B, H, W, d)) return TLIN_ERR_WORKSPACE;
+        if (log_plans()) log_bwd("", B, H, N, W, d, causal_window, "tensor cores, one kernel, workspace", bwd_fused_workspace_bytes(B, H, W, d));
         return launch_bwd_fused(q, k, v, out, lse, dout, dq, dk, dv, B, H, N, W, d, causal_window, (float*)w.ptr, sms, st);
     }
     tlin_fwd_plan plan;

@@ -2,6 +2,9 @@
 numbers that the parts do not hold."""
 import ctypes
 import math
+import os
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -330,3 +333,22 @@ def test_a_capture_that_pytorch_does_not_know_of_takes_no_scratch():
     assert torch.equal(grads[1], want[1]) and torch.equal(grads[2], want[2])
     assert float((grads[0] - want[0]).double().norm()) <= 1e-6 * float(want[0].double().norm())
     assert tl.tlin_get_status() == 0
+
+
+_LOGGED = """
+import torch
+from paper_2508_20407_b200 import binding as tl
+for d, dtype in ((36, torch.float32), (100, torch.float32), (64, torch.bfloat16), (96, torch.bfloat16), (128, torch.bfloat16)):
+    q, k, v = (torch.randn(2, 16, n, d, device="cuda").to(dtype).requires_grad_() for n in (300, 500, 500))
+    tl.attention(q, k, v)[0].sum().backward()
+torch.cuda.synchronize()
+"""
+
+
+def test_the_plan_log_names_every_call():
+    r = subprocess.run([sys.executable, "-c", _LOGGED], capture_output=True, text=True, timeout=300, env=dict(os.environ, TLIN_LOG="1"),
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0, r.stderr
+    lines = [line for line in r.stderr.splitlines() if line.startswith("libtlin:")]
+    assert [("forward" in line, "backward" in line) for line in lines] == [(True, False), (False, True)] * 5, r.stderr
+    assert "three bf16 parts" in lines[0] and "three bf16 parts" in lines[1] and "CUDA cores" in lines[3] and "CUDA cores" in lines[7]
