@@ -352,3 +352,43 @@ def test_the_plan_log_names_every_call():
     lines = [line for line in r.stderr.splitlines() if line.startswith("libtlin:")]
     assert [("forward" in line, "backward" in line) for line in lines] == [(True, False), (False, True)] * 5, r.stderr
     assert "three bf16 parts" in lines[0] and "three bf16 parts" in lines[1] and "CUDA cores" in lines[3] and "CUDA cores" in lines[7]
+
+
+def test_calls_in_several_launches_whose_results_lie_over_inputs():
+    """They go to the CUDA cores with nothing launched before."""
+    B, H, N, W, d = 2, 160, 2000, 2000, 36
+    t = tensors(B, H, N, W, d)
+    q, k, v, dout = (t[x] for x in ("q", "k", "v", "dout"))
+    assert tl.lib().tlin_scratch_bytes_forward_f32(B, H, N, W, d, 1) and tl.lib().tlin_scratch_bytes_backward_f32(B, H, N, W, d, 1)
+    out, lse = forward(q, k, v, 1, False)
+    over = q.clone()
+    got = forward(over, k, v, 1, out=over)
+    assert tl.tlin_last_launch_count() == 1 and torch.equal(got[0], out) and torch.equal(got[1], lse)
+    want = backward(q, k, v, out, lse, dout, 1, False)
+    launches = tl.tlin_last_launch_count()
+    over = k.clone()
+    dq, dk, dv = backward(q, over, v, out, lse, dout, 1, grads=[torch.empty_like(q), over, torch.empty_like(v)])
+    assert tl.tlin_last_launch_count() == launches and torch.equal(dk, want[1]) and torch.equal(dv, want[2])
+    assert float((dq - want[0]).double().norm()) <= 1e-6 * float(want[0].double().norm())          # summed in any order
+    assert tl.tlin_get_status() == 0
+
+
+def test_two_streams_at_once():
+    sizes = [(2, 16, 500, 300, 36), (1, 12, 1500, 513, 64)]
+    inputs = [tensors(*s) for s in sizes]
+
+    def call(t):
+        out, lse = tl.tlin_attn_forward_f32(t["q"], t["k"], t["v"])
+        return [out, lse] + list(tl.tlin_attn_backward_f32(t["q"], t["k"], t["v"], out, lse, t["dout"]))
+
+    want = [call(t) for t in inputs]
+    torch.cuda.synchronize()
+    streams, got = [torch.cuda.Stream(), torch.cuda.Stream()], []
+    for _ in range(10):
+        for s, t in zip(streams, inputs):
+            with torch.cuda.stream(s):
+                got.append(call(t))
+    torch.cuda.synchronize()
+    for i, results in enumerate(got):
+        assert all(torch.equal(a, b) for a, b in zip(results, want[i % 2]))
+    assert tl.tlin_get_status() == 0
