@@ -56,7 +56,7 @@ typedef enum {
  *                    union of both key sets.  Requires N >= W.
  * bf16 path: d a multiple of 8 up to 256, on the tensor cores (64 and 128 in tiles of their own, the others in zero-padded
  * ones; many (b,h) of a few rows and keys at those others on the CUDA cores).  f32 path: d a multiple of 4 up to 256
- * (covers the paper's d = 36), CUDA cores.
+ * (covers the paper's d = 36), on the CUDA cores; with scratch also on the tensor cores (tlin_attn_forward_f32_scratch).
  * Uses the workspace when the plan splits the key range (see tlin_workspace_bytes_forward); head sizes other than 64 and 128
  * also run without one, with whole key ranges.
  */
@@ -252,7 +252,8 @@ int tlin_decode_step_static(const void* q_new, const void* k_new, const void* v_
  * bf16: d in {64,128} runs on the tensor cores (two kernels that recompute p, no atomics, bitwise repeatable; or one kernel
  * at d = 128 with dq summed by fp32 reductions, which small calls get by default: tlin_set_backward_impl); any other
  * d that is a multiple of 8 up to 256 runs on the CUDA-core kernels (dq summed with fp32 atomics).  f32: d a multiple
- * of 4 up to 256 (covers the paper's d = 36), CUDA-core kernels.
+ * of 4 up to 256 (covers the paper's d = 36), CUDA-core kernels; with scratch also on the tensor cores up to d = 64
+ * (tlin_attn_backward_f32_scratch).
  * Needs a workspace of tlin_workspace_bytes_backward bytes (row sums, partial or accumulated dq in fp32).
  * Errors as for tlin_attn_forward.
  */
@@ -333,7 +334,7 @@ typedef struct {
     int64_t workspace_bytes;
 } tlin_decode_plan;
 
-/* num_sms <= 0 means "use the value of the B200 (148)". */
+/* num_sms <= 0 means "use the value of the B200 (148)".  In fp32 the plan of a call without scratch. */
 int tlin_plan_forward(int B, int H, int N, int W, int d, int causal_window, int is_f32, int num_sms, tlin_fwd_plan* plan);
 int tlin_plan_decode(int B, int H, int L, int d, int num_sms, tlin_decode_plan* plan);
 /* Work sharing of the tensor-core dK/dV kernel of tlin_attn_backward: its units are (b,h,128-key tile) in that order and
@@ -376,7 +377,7 @@ const char* tlin_status_string(int status);
 const char* tlin_version(void);
 /* Which kernel serves tlin_attn_forward: 0 = automatic, 1 = always the CUDA-core kernel,
  * 2 = tensor-core kernel (TLIN_ERR_UNSUPPORTED if the shape does not allow it, i.e. in fp32).  tlin_attn_backward follows the same
- * switch (1 = CUDA-core kernels for every head size).  Returns the old value. */
+ * switch (1 = CUDA-core kernels for every head size).  With 1 or 2 no fp32 call takes scratch.  Returns the old value. */
 int tlin_set_forward_impl(int impl);
 /* How the tensor-core kernels of tlin_attn_backward (bf16, d = 64 or 128) are arranged; the chain rule of the Section 3
  * attention formula is the same in both (the paper gives no gradient algorithm of its own):

@@ -9,6 +9,7 @@ import sys
 import pytest
 import torch
 
+from guards import Guarded
 from paper_2508_20407_b200 import binding as tl
 
 pytestmark = pytest.mark.gpu
@@ -391,4 +392,34 @@ def test_two_streams_at_once():
     torch.cuda.synchronize()
     for i, results in enumerate(got):
         assert all(torch.equal(a, b) for a, b in zip(results, want[i % 2]))
+    assert tl.tlin_get_status() == 0
+
+
+# in a cluster, in several launches, at one d8 beyond d, with more (b,h) than blocks of the split; some of them with a head for the CUDA cores
+@pytest.mark.parametrize("B,H,N,W,d,special", [(1, 3, 3000, 200, 64, True), (2, 160, 2000, 300, 64, True), (1, 5, 2100, 640, 68, False), (8, 32, 520, 512, 20, False),
+                                               (2, 600, 60, 50, 36, False), (2, 16, 385, 129, 36, True)])
+def test_scratch_of_the_documented_size_between_guards(B, H, N, W, d, special):
+    """Nothing is written beyond it and nothing in it is read before it is written: it starts as NaNs, and words that are set."""
+    t = tensors(B, H, N, W, d)
+    if special:
+        t["v"][B - 1, H - 1, N // 2, 1] = math.inf
+    q, k, v, dout = (t[x] for x in ("q", "k", "v", "dout"))
+    lib, sizes, stream = tl.lib(), (B, H, N, W, d, 0), torch.cuda.current_stream().cuda_stream
+    if lib.tlin_scratch_bytes_forward_f32(*sizes):
+        want = forward(q, k, v, 0)
+        s, out, lse = Guarded((lib.tlin_scratch_bytes_forward_f32(*sizes),), torch.uint8), torch.empty_like(q), torch.empty(B, H, W, device=DEV)
+        assert lib.tlin_attn_forward_f32_scratch(*pointers(q, k, v, out, lse), *sizes, s.t.data_ptr(), s.nbytes, stream) == 0
+        s.check("forward")
+        assert same(out, want[0]) and same(lse, want[1])
+    else:
+        out, lse = tl.tlin_attn_forward_f32(q, k, v, causal_window=0)
+    if lib.tlin_scratch_bytes_backward_f32(*sizes):
+        want = backward(q, k, v, out, lse, dout, 0)
+        s, grads = Guarded((lib.tlin_scratch_bytes_backward_f32(*sizes),), torch.uint8), [torch.empty_like(x) for x in (q, k, v)]
+        assert lib.tlin_attn_backward_f32_scratch(*pointers(q, k, v, out, lse, dout, *grads), *sizes, s.t.data_ptr(), s.nbytes, stream) == 0
+        s.check("backward")
+        assert same(grads[1], want[1]) and same(grads[2], want[2])
+        ok = torch.isfinite(want[0])                   # dq of several additions in any order
+        assert torch.equal(torch.isfinite(grads[0]), ok)
+        assert float((grads[0] - want[0])[ok].double().norm()) <= 1e-6 * float(want[0][ok].double().norm())
     assert tl.tlin_get_status() == 0
