@@ -7,7 +7,7 @@
 // with d8 = d rounded up to 8, which the tensor maps then read with zero fill beyond d8.  Numbers outside [2^-100, 2^30] (dout: 2^20) other than 0
 // (infinities, what would lose its low parts or overflow on the way) are found there: a (b,h) with such a number runs on the CUDA cores
 // instead, decided on the device.  The split kernel's blocks leave one word each, several blocks to a (b,h); the tensor kernels read the
-// words and pass the (b,h) by that have one set, and the CUDA-core kernel behind them computes those and returns at once if there
+// words and leave those (b,h) out that have one set, and the CUDA-core kernel behind them computes these and returns at once if there
 // are none.
 #pragma once
 #include "tlin_internal.h"
